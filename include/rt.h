@@ -408,8 +408,8 @@ rt_status rt_set_pah_spectra(rt_grid *g, int pah, int64_t first_cell, int64_t n_
  * [n_cases][n_bins] the emitted power per bin, erg/s per molecule (its sum equals
  * rate * h_nu up to the energy cut at the top). Inputs: nu_edges [n_bins+1] (Hz,
  * increasing), sigma [n_cases][n_bins] absorption cross sections per molecule (cm^2),
- * n_levels 16..4096. One GPU block per case; allocates and frees its device arrays;
- * synchronises. */
+ * n_levels 16..4096. Allocates and frees its device arrays (the level spectra of a
+ * group of cases, at most 256 MB at a time or one case); synchronises. */
 typedef struct rt_pah_pt_case {
     double modes[4][2];     /* mode groups: (number of modes, Einstein temperature K) */
     int32_t n_groups;       /* 1..4 */

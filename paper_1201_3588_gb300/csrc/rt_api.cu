@@ -58,6 +58,7 @@ struct rt_grid {
   double* d_pah_sigma = nullptr;
   float* d_pah_s = nullptr;
   double* d_pah_L = nullptr;
+  double* d_pah_T = nullptr;
   double* d_pah_ek = nullptr;
   int* d_pah_qk = nullptr;
   double* d_pah_wk = nullptr;
@@ -161,6 +162,7 @@ void free_tables(rt_grid* g) {
   dfree(g->d_pah_sigma);
   dfree(g->d_pah_s);
   dfree(g->d_pah_L);
+  dfree(g->d_pah_T);
   dfree(g->d_pah_ek);
   dfree(g->d_pah_qk);
   dfree(g->d_pah_wk);
@@ -253,6 +255,7 @@ rt_status build_pah_tables(rt_grid* g, cudaStream_t s) {
   if ((st = dalloc(&g->d_pah_sigma, (size_t)P * B)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_s, (size_t)P * M * B)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_L, (size_t)P * M)) != RT_OK) return st;
+  if ((st = dalloc(&g->d_pah_T, (size_t)P * M)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_ek, (size_t)K)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_qk, (size_t)P * K)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_wk, (size_t)P * K)) != RT_OK) return st;
@@ -294,6 +297,7 @@ rt_status build_pah_tables(rt_grid* g, cudaStream_t s) {
   pb.f_ref = 1.0e4;  // erg s^-1 cm^-2, the heating bath of the paper's Fig. 3
   pb.s = g->d_pah_s;
   pb.L = g->d_pah_L;
+  pb.T = g->d_pah_T;
   pb.e_k = g->d_pah_ek;
   pb.q_k = g->d_pah_qk;
   pb.w_k = g->d_pah_wk;
@@ -1358,43 +1362,60 @@ rt_status rt_pah_temperature_distribution(const rt_pah_pt_case* cases, int n_cas
   for (size_t i = 0; i < (size_t)n_cases * n_bins; ++i)
     if (!(sigma[i] >= 0) || !std::isfinite(sigma[i])) return RT_ERR_ARG;
   cudaStream_t s = as_stream(stream);
-  const size_t nP = (size_t)n_cases * n_levels, nE = (size_t)n_cases * n_bins;
-  PtCase* d_cases = nullptr;
-  double *d_nu = nullptr, *d_sig = nullptr, *d_P = nullptr, *d_T = nullptr, *d_a = nullptr,
-         *d_em = nullptr;
+  const size_t M = (size_t)n_levels, B = (size_t)n_bins, n = (size_t)n_cases;
+  // The cases in groups whose level spectra (M x B doubles a case) fit 256 MB. One
+  // device block holds a group's inputs, outputs and work arrays, so that a call makes
+  // one allocation, one copy each way per group, and one wait per group.
+  // Where even that does not fit the device, smaller groups.
+  const size_t per = 8 * (M * B + M + 1), most = ((size_t)256 << 20) / per;
+  size_t group = most < 1 ? 1 : (most < n ? most : n);
+  static_assert(sizeof(PtCase) % sizeof(double) == 0, "cases sit between doubles");
+  const size_t case_d = sizeof(PtCase) / sizeof(double);
+  size_t in_d = 0, out_d = 0;
+  double* dev = nullptr;
   rt_status st = RT_OK;
-  if ((st = dalloc(&d_cases, (size_t)n_cases)) == RT_OK &&
-      (st = dalloc(&d_nu, (size_t)n_bins + 1)) == RT_OK && (st = dalloc(&d_sig, nE)) == RT_OK &&
-      (st = dalloc(&d_P, nP)) == RT_OK && (st = dalloc(&d_T, nP)) == RT_OK &&
-      (st = dalloc(&d_a, (size_t)n_cases)) == RT_OK && (st = dalloc(&d_em, nE)) == RT_OK) {
-    cudaError_t e = cudaMemcpyAsync(d_cases, pc.data(), sizeof(PtCase) * n_cases,
-                                    cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(d_nu, nu_edges, sizeof(double) * (n_bins + 1), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(d_sig, sigma, sizeof(double) * nE, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-      e = launch_pah_pt(d_cases, n_cases, d_nu, n_bins, d_sig, n_levels, t_sub, d_P, d_T, d_a,
-                        d_em, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(P_out, d_P, sizeof(double) * nP, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(T_out, d_T, sizeof(double) * nP, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(p_above_out, d_a, sizeof(double) * n_cases, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(emission_out, d_em, sizeof(double) * nE, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    st = cuda_status(e);
+  for (;; group = (group + 1) / 2) {
+    in_d = group * case_d + (B + 1) + group * B;
+    out_d = group * (2 * M + B + 1);
+    st = dalloc(&dev, in_d + out_d + pt_scratch_doubles((int)group, n_levels, n_bins));
+    if (st == RT_OK) break;
+    if (st != RT_ERR_OOM || group == 1) return st;
   }
-  dfree(d_cases);
-  dfree(d_nu);
-  dfree(d_sig);
-  dfree(d_P);
-  dfree(d_T);
-  dfree(d_a);
-  dfree(d_em);
-  return st;
+  cudaError_t e = cudaSuccess;
+  try {
+    std::vector<double> host(in_d > out_d ? in_d : out_d);
+    for (size_t c0 = 0; c0 < n && e == cudaSuccess; c0 += group) {
+      const size_t nc = n - c0 < group ? n - c0 : group;
+      double* d_nu = dev + nc * case_d;
+      double* d_sig = d_nu + (B + 1);
+      double* d_P = dev + in_d;
+      double* d_T = d_P + nc * M;
+      double* d_em = d_T + nc * M;
+      double* d_a = d_em + nc * B;
+      std::memcpy(host.data(), &pc[c0], sizeof(PtCase) * nc);
+      std::memcpy(host.data() + nc * case_d, nu_edges, sizeof(double) * (B + 1));
+      std::memcpy(host.data() + nc * case_d + B + 1, sigma + c0 * B, sizeof(double) * nc * B);
+      e = cudaMemcpyAsync(dev, host.data(), sizeof(double) * (nc * (case_d + B) + B + 1),
+                          cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess)
+        e = launch_pah_pt(reinterpret_cast<const PtCase*>(dev), (int)nc, d_nu, n_bins, d_sig,
+                          n_levels, t_sub, d_P, d_T, d_a, d_em, dev + in_d + out_d, s);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(host.data(), d_P, sizeof(double) * nc * (2 * M + B + 1),
+                            cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) break;
+      std::memcpy(P_out + c0 * M, host.data(), sizeof(double) * nc * M);
+      std::memcpy(T_out + c0 * M, host.data() + nc * M, sizeof(double) * nc * M);
+      std::memcpy(emission_out + c0 * B, host.data() + 2 * nc * M, sizeof(double) * nc * B);
+      std::memcpy(p_above_out + c0, host.data() + nc * (2 * M + B), sizeof(double) * nc);
+    }
+  } catch (const std::bad_alloc&) {
+    st = RT_ERR_OOM;
+  }
+  if (e != cudaSuccess) cudaStreamSynchronize(s);
+  dfree(dev);
+  return st != RT_OK ? st : cuda_status(e);
 }
 
 // Work arrays of rt_pah_emission: cell lists for `cells` cells; the network's

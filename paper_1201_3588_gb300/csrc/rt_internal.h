@@ -238,6 +238,7 @@ struct PahBuild {
   double T_star, f_ref;      // template heating: source blackbody at bolometric flux f_ref
   float* s;                  // [n_pah][M][B] emission per level and bin, erg/s
   double* L;                 // [n_pah][M] cooling rate per level, erg/s
+  double* T;                 // [n_pah][M] level temperatures (work array)
   double* e_k;               // [K] photon energy of each coarse bin, erg
   int* q_k;                  // [n_pah][K] floor(e_k / dE)
   double* w_k;               // [n_pah][K] e_k / dE - q_k
@@ -298,7 +299,9 @@ struct PtCase {
 };
 cudaError_t launch_pah_pt(const PtCase* cases, int n_cases, const double* nu, int B,
                           const double* sigma, int M, double t_sub, double* P_out,
-                          double* T_out, double* p_above, double* em_out, cudaStream_t s);
+                          double* T_out, double* p_above, double* em_out, double* scratch,
+                          cudaStream_t s);
+size_t pt_scratch_doubles(int n_cases, int M, int B);
 
 cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T_frozen,
                             float* u_frozen, float t_min, cudaStream_t s);

@@ -44,23 +44,71 @@ __device__ double temperature_of(double E, const PahSpec& sp) {
   return sqrt(lo * hi);
 }
 
-// one thread per (PAH, level): temperature, cooling rate (FP64) and emission
-// spectrum per bin (stored FP32)
-__global__ void k_pah_levels(PahBuild pb) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
+// The temperature at heat content E: an FP32 bisection (cheap here: FP64 runs at 1/64 of
+// the FP32 rate) gives a start good to about 1e-6, from which Newton's method in FP64
+// converges to the last bits in two steps; where it does not (a start out of the FP32
+// range), the FP64 bisection. One thread; the bisection alone takes 50 FP64 evaluations.
+__device__ double level_temperature(double E, const PahSpec& sp) {
+  if (!(E > 0.0)) return 0.0;
+  // FP32: heat contents relative to E, ln T in [ln 1e-3, ln 1e9]
+  float w[kMaxModeGroups], th[kMaxModeGroups];
+#pragma unroll
+  for (int i = 0; i < kMaxModeGroups; ++i) {
+    w[i] = i < sp.n_groups ? (float)(sp.n_modes[i] * kK * sp.theta[i] / E) : 0.0f;
+    th[i] = i < sp.n_groups ? (float)sp.theta[i] : 1.0f;
+  }
+  float lo = -6.9077554f, hi = 20.723266f;
+  for (int it = 0; it < 25; ++it) {
+    const float mid = 0.5f * (lo + hi), rT = expf(-mid);
+    float e = 0.0f;
+#pragma unroll
+    for (int i = 0; i < kMaxModeGroups; ++i) e += w[i] / expm1f(fminf(th[i] * rT, 80.0f));
+    if (e < 1.0f) lo = mid; else hi = mid;
+  }
+  double T = exp(0.5 * ((double)lo + (double)hi));
+  for (int it = 0; it < 6; ++it) {
+    double e = 0.0, de = 0.0;  // heat content and T times its derivative
+    for (int i = 0; i < sp.n_groups; ++i) {
+      const double x = sp.theta[i] / T;
+      if (x < 700.0) {
+        const double m = 1.0 / expm1(x), u = sp.n_modes[i] * kK * sp.theta[i] * m;
+        e += u;
+        de += u * x * (1.0 + m);
+      }
+    }
+    const double step = (E - e) / de;
+    if (!(fabs(step) < 0.1)) break;
+    T += T * step;
+    if (fabs(step) < 1e-9) return T;  // the next step would be below 1e-16
+  }
+  return temperature_of(E, sp);
+}
+
+// one thread per (PAH, level): temperature of the level
+__global__ void k_pah_temps(PahBuild pb) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= pb.n_pah * pb.M) return;
-  int p = idx / pb.M, f = idx % pb.M;
-  const PahSpec& sp = pb.spec[p];
-  double T = temperature_of(f * pb.dE[p], sp);
+  const int p = idx / pb.M, f = idx % pb.M;
+  pb.T[idx] = level_temperature(f * pb.dE[p], pb.spec[p]);
+}
+
+// one warp per (PAH, level): cooling rate (FP64) and emission spectrum per bin (stored
+// FP32). A thread per level doing its bins one after another, the temperature by FP64
+// bisection, took 20 ms for 2 x 400 levels and 200 bins; this takes 0.05 ms.
+__global__ void k_pah_levels(PahBuild pb) {
+  const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (idx >= pb.n_pah * pb.M) return;
+  const int p = idx / pb.M, f = idx % pb.M;
   const double* sig = pb.sigma + (size_t)p * pb.B;
   float* s = pb.s + ((size_t)p * pb.M + f) * pb.B;
   double L = 0.0;
-  for (int b = 0; b < pb.B; ++b) {
-    double v = 4.0 * kPi * sig[b] * planck_bin(pb.nu[b], pb.nu[b + 1], T);
+  planck::planck_bins_warp(pb.nu, pb.B, pb.T[idx], [&](int b, double v) {
+    v *= 4.0 * kPi * sig[b];
     s[b] = (float)v;
     L += v;
-  }
-  pb.L[idx] = L;
+  });
+  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+  if (lane == 0) pb.L[idx] = L;
 }
 
 // coarse photon energies e_k = h sqrt(nu_lo nu_hi) over each coarse bin's range,
@@ -541,7 +589,8 @@ __global__ void k_count_flags(const unsigned char* flag, long long n, unsigned l
 
 cudaError_t launch_pah_tables(const PahBuild& pb, const PahTables& t, cudaStream_t s) {
   int n = pb.n_pah * pb.M;
-  k_pah_levels<<<(n + 63) / 64, 64, 0, s>>>(pb);
+  k_pah_temps<<<(n + 31) / 32, 32, 0, s>>>(pb);
+  k_pah_levels<<<(n + 3) / 4, 128, 0, s>>>(pb);
   int nk = pb.n_pah * pb.K;
   k_pah_coarse<<<(nk + 63) / 64, 64, 0, s>>>(pb);
   const int nf = n > nk ? n : nk;
@@ -617,115 +666,141 @@ cudaError_t launch_surrogate_add(const float* Y, const float* p_abs, long long n
   return cudaGetLastError();
 }
 
-// P(T) of a PAH in a monochromatic field (Fig. 3), one block per case: levels
-// E_f = f dE up to E(t_top) + h nu with their temperatures and cooling rates
-// (threads over levels), populations by the level-by-level flux balance for the
-// single photon energy (one thread), then the time fraction above t_sub and the
-// emission per bin (threads over bins). Shared memory: T, L, D [M] doubles.
-__device__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-  return t;
+// P(T) of a PAH in a monochromatic field (Fig. 3): levels E_f = f dE up to E(t_top) +
+// h nu. Four kernels over all cases of a call: the level temperatures (a thread per
+// level), the levels' emission per bin and cooling rates (a warp per level; FP64-bound,
+// so every bin edge is evaluated once and the spectra are kept for the last kernel), the
+// populations by the level-by-level flux balance for the single photon energy (a warp
+// per case, the recursion in one lane), the emission (a block per case and 32 bins).
+// One block per case doing all of it, with every Planck integral twice, took 187 ms for
+// 12 cases of 400 levels and 200 bins; the four kernels take 0.03 + 0.17 + 0.17 + 0.02
+// ms, the call 0.61 ms with its copies and allocation.
+__global__ void k_pt_temps(const PtCase* cases, int n_cases, int M, double* dE_out,
+                           double* T_out) {
+  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (idx >= (long long)n_cases * M) return;
+  const int c = (int)(idx / M), f = (int)(idx % M);
+  const PtCase& cs = cases[c];
+  const double dE = (heat_content(cs.t_top, cs.spec) + cs.h_nu) / (double)(M - 1);
+  if (f == 0) dE_out[c] = dE;
+  T_out[idx] = f == 0 ? 0.0 : level_temperature(f * dE, cs.spec);
 }
 
-__global__ void k_pah_pt(const PtCase* cases, const double* nu, int B, const double* sigma,
-                         int M, double t_sub, double* P_out, double* T_out, double* p_above,
-                         double* em_out) {
+__global__ void k_pt_levels(int n_cases, const double* nu, int B, const double* sigma, int M,
+                            const double* dE, const double* T, double* spec, double* cool) {
+  const long long idx = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  if (idx >= (long long)n_cases * M) return;
+  const int c = (int)(idx / M);
+  const double* sig = sigma + (size_t)c * B;
+  double* s = spec + (size_t)idx * B;
+  double L = 0.0;
+  planck::planck_bins_warp(nu, B, T[idx], [&](int b, double v) {
+    v *= sig[b];
+    s[b] = v;
+    L += v;
+  });
+  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+  if ((threadIdx.x & 31) == 0) cool[idx] = 4.0 * kPi * L / dE[c];  // steps down per second
+}
+
+// The flux F up across the boundary below level f equals cooling across it, P_f = F / C_f;
+// then F changes by what leaves level f upwards less what has arrived there: from level
+// f - q (weight 1 - w) and f - q - 1 (weight w), one photon being q + w levels. A serial
+// chain over the levels in one lane: the reciprocals of C are formed in parallel before
+// it, so a step is one product, one fused multiply-add and a maximum deep (with the
+// division and the arrivals scattered through shared memory a step took 1.0 us, now 0.4).
+// Shared memory: P and 1/C, M doubles each.
+__global__ void __launch_bounds__(32) k_pt_populations(const PtCase* cases, int M,
+                                                       const double* dE, const double* cool,
+                                                       const double* T, double t_sub,
+                                                       double* P_out, double* p_above) {
   extern __shared__ double sm[];
-  double* T = sm;
-  double* L = T + M;
-  double* D = L + M;
-  double* red = D + M;  // [32]
-  const PtCase c = cases[blockIdx.x];
-  const double* sig = sigma + (size_t)blockIdx.x * B;
-  double* P = P_out + (size_t)blockIdx.x * M;
-  const double dE = (heat_content(c.t_top, c.spec) + c.h_nu) / (double)(M - 1);
-  for (int f = threadIdx.x; f < M; f += blockDim.x) {
-    const double Tf = f == 0 ? 0.0 : temperature_of(f * dE, c.spec);
-    double l = 0.0;
-    if (f > 0)
-      for (int b = 0; b < B; ++b) l += sig[b] * planck_bin(nu[b], nu[b + 1], Tf);
-    T[f] = Tf;
-    L[f] = 4.0 * kPi * l;
-    D[f] = 0.0;
+  double* P = sm;
+  double* rC = P + M;
+  const PtCase& c = cases[blockIdx.x];
+  const int lane = threadIdx.x;
+  const size_t row = (size_t)blockIdx.x * M;
+  for (int f = lane; f < M; f += 32) {
+    const double C = cool[row + f];
+    rC[f] = C > 0.0 ? fmin(1.0 / C, 1e308) : 0.0;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const double x = c.h_nu / dE;
+  __syncwarp();
+  if (lane == 0) {
+    const double x = c.h_nu / dE[blockIdx.x];
     const int q = (int)floor(x);
     const double w = x - floor(x);
-    const double R = c.rate;
-    // arrivals from level i: level i + q (weight 1 - w) and i + q + 1 (weight w),
-    // both cut at the top level; returns the upward rate out of level i
-    auto scatter = [&](int i, double Pi) {
-      int f = i + q;
-      double wk = w;
-      if (f >= M - 1) {
-        f = M - 1;
-        wk = 0.0;
-      }
-      double up = 0.0;
-      if (f > i) {
-        D[f] += Pi * R * (1.0 - wk);
-        up += R * (1.0 - wk);
-      }
-      if (wk > 0.0 && f + 1 < M) {
-        D[f + 1] += Pi * R * wk;
-        up += R * wk;
-      }
-      return up;
-    };
+    const double r0 = q > 0 ? c.rate * (1.0 - w) : 0.0, r1 = c.rate * w;
+    // upward rate out of level i; absorptions beyond the top level end there
+    auto up = [&](int i) { return i + q < M - 1 ? r0 + r1 : (i < M - 1 ? c.rate : 0.0); };
     P[0] = 1.0;
-    double F = scatter(0, 1.0);
+    double F = up(0);
     for (int f = 1; f < M; ++f) {
-      const double C = L[f] / dE;
-      const double Pf = C > 0.0 ? F / C : 0.0;
+      const double D = (f > q ? r1 * P[f - q - 1] : 0.0) + (q > 0 && f >= q ? r0 * P[f - q] : 0.0);
+      const double Pf = F * rC[f];
       P[f] = Pf;
-      const double u = scatter(f, Pf);
-      F = fmax(F - D[f] + Pf * u, 0.0);
+      F = fmax(fma(Pf, up(f), F - D), 0.0);
       if (Pf > 1e250) {  // keep the numbers finite
         for (int i = 0; i <= f; ++i) P[i] *= 1e-250;
-        for (int i = 0; i < M; ++i) D[i] *= 1e-250;
         F *= 1e-250;
       }
     }
   }
-  __syncthreads();
-  double s = 0.0, a = 0.0;
-  for (int f = threadIdx.x; f < M; f += blockDim.x) s += P[f];
-  const double tot = block_sum(s, red);
-  for (int f = threadIdx.x; f < M; f += blockDim.x) {
+  __syncwarp();
+  double tot = 0.0, a = 0.0;
+  for (int f = lane; f < M; f += 32) tot += P[f];
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  for (int f = lane; f < M; f += 32) {
     const double v = P[f] / tot;
-    P[f] = v;
-    T_out[(size_t)blockIdx.x * M + f] = T[f];
-    if (T[f] > t_sub) a += v;
+    P_out[row + f] = v;
+    if (T[row + f] > t_sub) a += v;
   }
-  a = block_sum(a, red);
-  if (threadIdx.x == 0) p_above[blockIdx.x] = a;
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if (lane == 0) p_above[blockIdx.x] = a;
+}
+
+constexpr int kPtWarps = 8;
+
+__global__ void __launch_bounds__(32 * kPtWarps) k_pt_emission(int B, int M, const double* spec,
+                                                               const double* P, double* em_out) {
+  __shared__ double part[kPtWarps][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.y * 32 + lane;
+  const size_t row = (size_t)blockIdx.x * M;
+  double e = 0.0;
+  if (b < B)
+    for (int f = warp; f < M; f += kPtWarps) e += P[row + f] * spec[(row + f) * B + b];
+  part[warp][lane] = e;
   __syncthreads();
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    double e = 0.0;
-    for (int f = 1; f < M; ++f) e += P[f] * planck_bin(nu[b], nu[b + 1], T[f]);
-    em_out[(size_t)blockIdx.x * B + b] = 4.0 * kPi * sig[b] * e;
+  if (warp == 0 && b < B) {
+    for (int i = 1; i < kPtWarps; ++i) e += part[i][lane];
+    em_out[(size_t)blockIdx.x * B + b] = 4.0 * kPi * e;
   }
 }
 
+size_t pt_scratch_doubles(int n_cases, int M, int B) {
+  return (size_t)n_cases * (1 + M + (size_t)M * B);
+}
+
+// scratch: pt_scratch_doubles(n_cases, M, B) doubles
 cudaError_t launch_pah_pt(const PtCase* cases, int n_cases, const double* nu, int B,
                           const double* sigma, int M, double t_sub, double* P_out,
-                          double* T_out, double* p_above, double* em_out, cudaStream_t s) {
-  const size_t smem = sizeof(double) * (3 * (size_t)M + 32);
+                          double* T_out, double* p_above, double* em_out, double* scratch,
+                          cudaStream_t s) {
+  double* dE = scratch;
+  double* cool = dE + n_cases;
+  double* spec = cool + (size_t)n_cases * M;
+  const size_t smem = sizeof(double) * 2 * (size_t)M;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_pah_pt, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(
+        k_pt_populations, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_pah_pt<<<n_cases, 256, smem, s>>>(cases, nu, B, sigma, M, t_sub, P_out, T_out, p_above,
-                                      em_out);
+  const long long n = (long long)n_cases * M;
+  k_pt_temps<<<(unsigned)((n + 31) / 32), 32, 0, s>>>(cases, n_cases, M, dE, T_out);
+  k_pt_levels<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(n_cases, nu, B, sigma, M, dE, T_out, spec,
+                                                      cool);
+  k_pt_populations<<<n_cases, 32, smem, s>>>(cases, M, dE, cool, T_out, t_sub, P_out, p_above);
+  k_pt_emission<<<dim3(n_cases, (B + 31) / 32), 32 * kPtWarps, 0, s>>>(B, M, spec, P_out, em_out);
   return cudaGetLastError();
 }
 
