@@ -261,16 +261,17 @@ rt_status rt_image_profile(rt_grid *g, int plane_a, int plane_b, int half_rows, 
 
 /* ---------------------------------------------------------------------------
  * Batches: many models (grids) of uneven size, optical depth and package count in
- * one persistent launch. Warps take chunks of `chunk` packages (model, index range)
- * from a device queue, interleaved over the models, and run the packet pool on the
- * chunk's model. The plan holds every device array the launch needs, so running it
- * allocates nothing and can be captured in a CUDA graph.
+ * one persistent launch. Every warp works on one model at a time, taking `chunk` of
+ * its packages at a time from the model's device counter, and turns to another model
+ * (picked by the packages left) when that one is handed out. The plan holds every
+ * device array the launch needs, so running it allocates nothing and can be captured
+ * in a CUDA graph.
  * ------------------------------------------------------------------------- */
 typedef struct rt_batch rt_batch;
 
 /* Plan packages 0 .. n_packages[m]-1 of every grid m (seed + m keys model m's Philox
  * streams; o: as rt_transport, pool kernel only, o->threads the threads per block
- * of the batched launch; chunk 0: 4096). Builds missing
+ * of the batched launch; chunk 0: 64, values below 32 act as 32). Builds missing
  * tables (synchronising) and allocates the plan's device arrays. The grids must
  * outlive the plan and stay on the current device. */
 rt_status rt_batch_create(rt_grid *const *grids, int n, const uint64_t *n_packages,

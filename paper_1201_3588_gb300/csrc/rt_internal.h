@@ -130,26 +130,20 @@ constexpr unsigned long long kPeelCapacityDefault = 1ull << 24;
 constexpr unsigned long long kPeelCapacityMax = 1ull << 31;
 constexpr size_t kMaxImagePixels = (size_t)1 << 28;  // all planes together (2 GiB of FP64)
 
-// One model of a batched launch, and one chunk of its packages.
+// One model of a batched launch.
 struct ModelDesc {
   DevGrid g;
   DevTables t;
   DevRun r;
 };
 
-struct BatchChunk {
-  int model;
-  int pad;
-  unsigned long long first, count;  // package indices [first, first + count)
-};
-
 // Kernel launchers (rt_transport.cu, rt_tables.cu).
-// s_fixed: the species count all models share (2 has a walk compiled for it,
-// without the path-length tally), 0 otherwise
-cudaError_t launch_transport_batch(const ModelDesc* models, const BatchChunk* chunks,
-                                   long long n_chunks, unsigned long long* next_chunk,
-                                   int blocks_per_sm, int s_fixed, int threads,
-                                   cudaStream_t s);
+// next [n_models]: packages of each model handed out so far (zeros); chunk >= 32: how
+// many a warp takes at a time. s_fixed: the species count all models share (2 has a walk
+// compiled for it, without the path-length tally), 0 otherwise
+cudaError_t launch_transport_batch(const ModelDesc* models, int n_models,
+                                   unsigned long long* next, int chunk, int blocks_per_sm,
+                                   int s_fixed, int threads, cudaStream_t s);
 cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const DevRun& r,
                                   int blocks_per_sm, int threads, cudaStream_t s,
                                   const DevPeel* peel = nullptr, bool path = false);

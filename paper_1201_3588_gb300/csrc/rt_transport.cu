@@ -1001,24 +1001,41 @@ __global__ void __launch_bounds__(256) k_transport_plain(DevGrid g, DevTables t,
 }
 
 // ---------------------------------------------------------------- pool loop
-// Where a warp's package indices come from: one global counter shared by all warps
-// (one model), or a range owned by the warp (one chunk of a batch). take() returns
-// the first of nd consecutive indices to every lane of the warp.
+// Where a warp's package indices come from: one counter of the launch (one model), or
+// the counter of the model the warp works on (a batch). take() gives the lane of rank
+// `rank` among the warp's nd dead lanes its index; indices at or beyond the end mean that
+// there is none left.
 struct GlobalIds {
   unsigned long long* next;
-  __device__ __forceinline__ unsigned long long take(int nd, int lane, int leader) {
+  __device__ __forceinline__ unsigned long long take(int nd, int rank, int lane, int leader) {
     unsigned long long b = 0;
     if (lane == leader) b = atomicAdd(next, (unsigned long long)nd);
-    return __shfl_sync(kFull, b, leader);
+    return __shfl_sync(kFull, b, leader) + (unsigned long long)rank;
   }
 };
 
-struct RangeIds {
-  unsigned long long pos;
-  __device__ __forceinline__ unsigned long long take(int nd, int, int) {
-    unsigned long long b = pos;
-    pos += (unsigned long long)nd;
-    return b;
+// Reserves `chunk` >= 32 indices at a time, [pos, pos + left) being what remains of the
+// warp's reservation.
+struct ModelIds {
+  unsigned long long* next;
+  unsigned long long pos, end;  // end: the model's number of packages
+  int left, chunk;
+  __device__ __forceinline__ unsigned long long take(int nd, int rank, int lane, int leader) {
+    unsigned long long j = pos + (unsigned long long)rank;
+    if (nd <= left) {
+      pos += (unsigned long long)nd;
+      left -= nd;
+      return j;
+    }
+    unsigned long long b = end;
+    if (pos < end) {  // until a reservation came back empty
+      if (lane == leader) b = atomicAdd(next, (unsigned long long)chunk);
+      b = __shfl_sync(kFull, b, leader);
+    }
+    if (rank >= left) j = b + (unsigned long long)(rank - left);
+    pos = b + (unsigned long long)(nd - left);
+    left = chunk - (nd - left);
+    return j;
   }
 };
 
@@ -1031,9 +1048,9 @@ struct RangeIds {
 // one atomic. `sed` is the escaped-spectrum histogram (shared or global memory).
 // kPeel: scatterings and re-emissions at image bins are recorded (position, w,
 // bin) in the peel-off event buffer, one slot range per warp and phase; point-source
-// emissions are counted per bin in s_nemit.
+// emissions are counted per bin in s_nemit. Returns false when the time budget ran out.
 template <bool kPeel, class Ids, int kS = 0, bool kPath = false>
-__device__ __forceinline__ void pool_warp(const DevGrid& g, const DevTables& t, const DevRun& r,
+__device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, const DevRun& r,
                                           const Kappa* kap, const float* star_cdf,
                                           unsigned long long* sed, unsigned long long n_end,
                                           Ids& ids, Tally& tl, unsigned long long t0,
@@ -1060,9 +1077,9 @@ __device__ __forceinline__ void pool_warp(const DevGrid& g, const DevTables& t, 
     unsigned dead = __ballot_sync(kFull, !alive);
     if (dead) {
       const int nd = __popc(dead);
-      const unsigned long long base = ids.take(nd, lane, __ffs(dead) - 1);
+      const unsigned long long j =
+          ids.take(nd, __popc(dead & lt_mask), lane, __ffs(dead) - 1);
       if (!alive) {
-        unsigned long long j = base + __popc(dead & lt_mask);
         if (j < n_end) {
           emit<float>(k, r.first_id + j, r, star_cdf, B);
           ++tl.emitted;
@@ -1088,7 +1105,7 @@ __device__ __forceinline__ void pool_warp(const DevGrid& g, const DevTables& t, 
         }
       }
     }
-    if (!__any_sync(kFull, alive)) break;
+    if (!__any_sync(kFull, alive)) return true;
     if (__any_sync(kFull, tl.crossings >= kTallyFlushAt || tl.levels >= kTallyFlushAt))
       flush_tally(tl, r.counters);
     bool stop = false;
@@ -1096,7 +1113,7 @@ __device__ __forceinline__ void pool_warp(const DevGrid& g, const DevTables& t, 
     stop = __shfl_sync(kFull, stop, 0);
     if (stop) {
       if (lane == 0) atomicOr(r.status, kStatusTimeout);
-      break;
+      return false;
     }
     for (int step = 0; step < K; ++step) {
       // walk phase: lanes not waiting for an interaction cross one cell
@@ -1262,35 +1279,82 @@ __global__ void __launch_bounds__(256, kMinBlocks)
 }
 
 // ---------------------------------------------------------------- batch kernel
-// Many models in one persistent launch: warps take chunks (model, package range)
-// from a global queue, stage that model's descriptor in shared memory and run the
-// pool loop over the chunk (tables in global memory / L2, spectrum by global
-// atomics). Counters are flushed to the chunk's model when the chunk ends.
+// Many models in one persistent launch. A warp picks a model, stages its descriptor in
+// shared memory and runs the pool loop on it, drawing packages from the model's counter
+// until that is exhausted and its own lanes have run dry; then it picks the next. The
+// pick is weighted by the packages each model has left: the first one stratified over
+// the warps (so that neighbouring warps share a model's rows in L1), later ones at
+// random. A warp's lanes therefore run dry once per model it works on. (Fixed chunks of
+// 4096 packages, a warp's lanes drained at the end of each, left three quarters of the
+// warps without work for a batch of 24 models and 6.5e6 packages -- 1600 chunks for 4864
+// warps -- and took 28.7 ms; this takes 8.0.) Tables in global memory / L2, spectrum by global atomics;
+// counters are flushed to the model when the warp leaves it.
+__device__ __forceinline__ int pick_model(const ModelDesc* models, int n,
+                                          const unsigned long long* next, unsigned warp_id,
+                                          unsigned n_warps, unsigned pick) {
+  const int lane = threadIdx.x & 31;
+  auto remaining = [&](int m) {
+    if (m >= n) return 0ull;
+    const unsigned long long all = models[m].r.n_packages;
+    const unsigned long long out = *reinterpret_cast<const volatile unsigned long long*>(&next[m]);
+    return out < all ? all - out : 0ull;
+  };
+  unsigned long long tot = 0;
+  for (int m = lane; m < n; m += 32) tot += remaining(m);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(kFull, tot, o);
+  if (tot == 0) return -1;
+  // a point in [0, tot) as a 64-bit fraction: the warp's place, or a hash
+  unsigned long long frac = (((unsigned long long)warp_id << 1 | 1) << 31) / n_warps << 32;
+  if (pick > 0) {
+    frac = ((unsigned long long)warp_id << 32 | pick) * 0x9E3779B97F4A7C15ull;
+    frac ^= frac >> 29;
+    frac *= 0xBF58476D1CE4E5B9ull;
+  }
+  unsigned long long point = __umul64hi(frac, tot);
+  int last = -1;  // the counters move meanwhile: the last model that had any left
+  for (int m0 = 0; m0 < n; m0 += 32) {
+    const unsigned long long r = remaining(m0 + lane);
+    unsigned long long c = r;  // inclusive sum over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(kFull, c, o);
+      if (lane >= o) c += u;
+    }
+    const unsigned above = __ballot_sync(kFull, c > point), any = __ballot_sync(kFull, r > 0);
+    if (above) return m0 + __ffs(above) - 1;
+    if (any) last = m0 + 31 - __clz(any);
+    point -= __shfl_sync(kFull, c, 31);
+  }
+  return last;
+}
+
+// Two species: held to 64 registers (56 bytes of spills) for four blocks per SM, 8.0 ms
+// against 8.7 with the three blocks of 74 registers; the generic form would spill 180.
 template <int kS>
-__global__ void __launch_bounds__(256) k_transport_batch(const ModelDesc* models,
-                                                         const BatchChunk* chunks,
-                                                         long long n_chunks,
-                                                         unsigned long long* next_chunk) {
+__global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const ModelDesc* models, int n_models,
+                                                         unsigned long long* next, int chunk) {
   __shared__ ModelDesc sdesc[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned per_block = blockDim.x >> 5;
   const unsigned long long t0 = global_ns();
-  for (;;) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(next_chunk, 1ull);
-    c = __shfl_sync(kFull, c, 0);
-    if ((long long)c >= n_chunks) break;
-    const BatchChunk ch = chunks[c];
-    const int* src = reinterpret_cast<const int*>(&models[ch.model]);
+  for (unsigned pick = 0;; ++pick) {
+    const int m = pick_model(models, n_models, next, blockIdx.x * per_block + warp,
+                             gridDim.x * per_block, pick);
+    if (m < 0) break;
+    const int* src = reinterpret_cast<const int*>(&models[m]);
     int* dst = reinterpret_cast<int*>(&sdesc[warp]);
     for (int i = lane; i < (int)(sizeof(ModelDesc) / sizeof(int)); i += 32) dst[i] = src[i];
     __syncwarp();
     const ModelDesc& md = sdesc[warp];
     Tally tl = {};
-    RangeIds ids{ch.first};
-    pool_warp<false, RangeIds, kS>(md.g, md.t, md.r, md.t.kap, md.t.star_cdf, md.r.sed,
-                                    ch.first + ch.count, ids, tl, t0);
+    ModelIds ids{next + m, 0ull, md.r.n_packages, 0, chunk};
+    const bool in_time =
+        pool_warp<false, ModelIds, kS>(md.g, md.t, md.r, md.t.kap, md.t.star_cdf, md.r.sed,
+                                        md.r.n_packages, ids, tl, t0);
     flush_tally(tl, md.r.counters);
     __syncwarp();
+    if (!in_time) break;
   }
 }
 
@@ -1562,9 +1626,9 @@ cudaError_t launch_transport_plain(const DevGrid& g, const DevTables& t, const D
 }
 
 template <int kS>
-static cudaError_t launch_batch_variant(const ModelDesc* models, const BatchChunk* chunks,
-                                        long long n_chunks, unsigned long long* next_chunk,
-                                        int blocks_per_sm, int threads, cudaStream_t s) {
+static cudaError_t launch_batch_variant(const ModelDesc* models, int n_models,
+                                        unsigned long long* next, int chunk, int blocks_per_sm,
+                                        int threads, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1575,21 +1639,18 @@ static cudaError_t launch_batch_variant(const ModelDesc* models, const BatchChun
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   int bps = blocks_per_sm > 0 && blocks_per_sm < occ ? blocks_per_sm : occ;
-  k_transport_batch<kS><<<sms * bps, threads, 0, s>>>(models, chunks, n_chunks, next_chunk);
+  k_transport_batch<kS><<<sms * bps, threads, 0, s>>>(models, n_models, next, chunk);
   return cudaGetLastError();
 }
 
-cudaError_t launch_transport_batch(const ModelDesc* models, const BatchChunk* chunks,
-                                   long long n_chunks, unsigned long long* next_chunk,
-                                   int blocks_per_sm, int s_fixed, int threads,
-                                   cudaStream_t s) {
+cudaError_t launch_transport_batch(const ModelDesc* models, int n_models,
+                                   unsigned long long* next, int chunk, int blocks_per_sm,
+                                   int s_fixed, int threads, cudaStream_t s) {
   if (threads <= 0) threads = 256;
   if (threads % 32 != 0 || threads > 256) return cudaErrorInvalidValue;
   if (s_fixed == 2)
-    return launch_batch_variant<2>(models, chunks, n_chunks, next_chunk, blocks_per_sm,
-                                   threads, s);
-  return launch_batch_variant<0>(models, chunks, n_chunks, next_chunk, blocks_per_sm, threads,
-                                 s);
+    return launch_batch_variant<2>(models, n_models, next, chunk, blocks_per_sm, threads, s);
+  return launch_batch_variant<0>(models, n_models, next, chunk, blocks_per_sm, threads, s);
 }
 
 cudaError_t launch_trace(const DevGrid& g, const DevTables& t, const DevRun& r,
