@@ -380,15 +380,18 @@ def path_walk_runs(walk, N, S, L, n_slots, images=False):
     if images or not fits:
         return False
     if walk == 0:
-        return S == 4 or 32 * N > 4e9
+        if 32 * N > 4e9:
+            return True
+        # a block turns one cell into eight: N = n^3 + 7 blocks, slots = n^3 + 8 blocks
+        refined = 8 * (n_slots - N) > 0.5 * N
+        return S == 4 and not (refined and 48 * N <= 0.5e9)
     return walk == 2
 
 
-def walk_label(choice, N, S, L):
+def walk_label(choice, N, S, L, n_slots):
     """The pool walk the library runs for this grid (the same rule as rt_transport)."""
     if choice == "auto":
-        choice = "path" if L <= 4 and (S == 4 or 32 * N > 4e9) else "linked"
-        return f"{choice} (automatic)"
+        return f"{'path' if path_walk_runs(0, N, S, L, n_slots) else 'linked'} (automatic)"
     return choice
 
 
@@ -651,7 +654,8 @@ def run_ours(args):
                        "packages_full_workload": FULL_PACKAGES.get(args.workload),
                        "leaves": N, "bins": B, "species": S, "levels": L,
                        "reemission": "bjorkman-wood",
-                       "walk": walk_label(args.walk, N, S, L) if "walk" not in opts else
+                       "walk": walk_label(args.walk, N, S, L, model.tree.n_base ** 3 +
+                                          8 * model.tree.n_blocks) if "walk" not in opts else
                        {1: "linked", 2: "path"}[opts["walk"]] + " (autotuned)",
                        "launch": opts or "defaults",
                        "form": "FP32 packet-pool transport" +

@@ -49,6 +49,7 @@ struct rt_grid {
   unsigned short* d_cdf_guide = nullptr;
   int* d_u_guide = nullptr;
   Kappa* d_kap = nullptr;
+  float* d_kext = nullptr;
   float* d_star_cdf = nullptr;
   double* d_star_frac = nullptr;
   float* d_Tfrozen = nullptr;
@@ -68,7 +69,7 @@ struct rt_grid {
   float* d_pah_cell_cdf = nullptr;  // [n_pah][N][B] per-cell re-emission spectra
   unsigned* d_pahabs = nullptr;
   unsigned* d_pah_flag = nullptr;  // [N] PAH-active bits per cell (bit p: PAH p)
-  float* d_pathabs = nullptr;  // path-length tallies [S][N]
+  float* d_pathabs = nullptr;  // path-length tallies [N][S]
   // peel-off images
   int* d_plane_of_bin = nullptr;         // [B]
   double* d_image = nullptr;             // [n_planes][ny][nx]
@@ -157,6 +158,7 @@ void free_tables(rt_grid* g) {
   dfree(g->d_cdf_guide);
   dfree(g->d_u_guide);
   dfree(g->d_kap);
+  dfree(g->d_kext);
   dfree(g->d_star_cdf);
   dfree(g->d_star_frac);
   dfree(g->d_pah_sigma);
@@ -177,6 +179,26 @@ void free_tables(rt_grid* g) {
 static bool path_walk_fits(const rt_grid_desc* d) {
   const double nb = (double)d->n_base * d->n_base * d->n_base;
   return d->max_level <= 4 && nb + 8.0 * (double)d->n_blocks < 2147483647.0;
+}
+
+// The automatic walk. The linked walk finds the next leaf with one read wherever the
+// neighbour is not finer; the path walk descends through the tree at every change of a
+// refined block, but reads one array of (slots x species) floats where the linked walk
+// reads 32-byte records and, for more than two species, a row of densities.
+//  - Two species (densities in the record), and species counts without a compiled path
+//    walk: linked until the records exceed 4 GB.
+//  - Four species: linked where most cells sit in refined blocks and records and densities
+//    are within 0.5 GB, a few times L2. 1e7 packages, linked and path: 8.0e6 cells, all but
+//    a tenth refined, 16.2 and 22.1 ms; 6.0e6 cells, a third refined, 21.8 and 21.0; 1.9e7
+//    cells, refined (0.9 GB), 40.7 and 34.6; 2.6e7 cells 46.8 and 36.0; 5.4e7 cells 84.6
+//    and 52.9.
+static bool path_walk_auto(const rt_grid_desc* d) {
+  if (!path_walk_fits(d)) return false;
+  const double rec = 4.0 * kRec * (double)d->n_leaves;
+  if (rec > 4.0e9) return true;
+  if (d->n_species != 4) return false;
+  const bool refined = 8.0 * (double)d->n_blocks > 0.5 * (double)d->n_leaves;
+  return !(refined && rec + 16.0 * (double)d->n_leaves <= 0.5e9);
 }
 
 void free_all(rt_grid* g) {
@@ -338,6 +360,7 @@ rt_status build_tables(rt_grid* g, cudaStream_t s) {
   ALLOC(g->d_cdf_guide, (size_t)S * (nT - 1) * B);
   ALLOC(g->d_u_guide, (size_t)S * nT);
   ALLOC(g->d_kap, (size_t)S * B);
+  ALLOC(g->d_kext, (size_t)S * B);
   ALLOC(g->d_star_cdf, (size_t)B);
   ALLOC(g->d_star_frac, 1);
 #undef ALLOC
@@ -368,6 +391,7 @@ rt_status build_tables(rt_grid* g, cudaStream_t s) {
   tb.cdf_guide = g->d_cdf_guide;
   tb.u_guide = g->d_u_guide;
   tb.kap = g->d_kap;
+  tb.kext = g->d_kext;
   tb.star_cdf = g->d_star_cdf;
   tb.star_frac = g->d_star_frac;
   RT_CUDA(launch_build_tables(tb, s));
@@ -383,6 +407,7 @@ rt_status build_tables(rt_grid* g, cudaStream_t s) {
   DevTables& t = g->tab;
   t = DevTables{};
   t.kap = g->d_kap;
+  t.kext = g->d_kext;
   t.star_cdf = g->d_star_cdf;
   t.S32 = g->d_S32;
   t.S64 = g->d_S64;
@@ -501,7 +526,7 @@ rt_status rt_grid_create(const rt_grid_desc* d, rt_grid** out) {
   // face links only where the automatic walk reads them (built below); otherwise on
   // the first call that needs them (ensure_links). The path walk's densities by tree
   // slot likewise: now where it is the automatic walk, else on first use.
-  const bool path_auto = path_walk_fits(d) && (S == 4 || 4.0 * kRec * (double)N > 4.0e9);
+  const bool path_auto = path_walk_auto(d);
   const bool links_now = !path_auto;
   if (links_now) ALLOC(g->d_links, (size_t)N * kRec);
   if (path_auto) ALLOC(g->d_rho_slot, (size_t)S * (nb + 8 * d->n_blocks));
@@ -832,17 +857,14 @@ static rt_status fill_run(rt_grid* g, uint64_t n_packages, uint64_t seed, uint64
   return RT_OK;
 }
 
-// The pool walk for this grid: the path walk when asked for, or (automatic) for four
-// species (the link record holds no densities then, and the path walk measured faster
-// from 1.9e7 to 1.7e8 cells) and whenever the face-link records exceed 4 GB; grids
-// deeper than the path walk serves keep the links.
+// The pool walk for this grid: the one asked for, or the automatic choice; grids deeper
+// than the path walk serves keep the links.
 static bool use_path_walk(const rt_grid* g, const rt_run_opts* o) {
   if (!path_walk_fits(&g->desc)) return false;
   const int w = o ? o->walk : RT_WALK_AUTO;
   if (w == RT_WALK_PATH) return true;
   if (w == RT_WALK_LINKED) return false;
-  const double rec_bytes = 4.0 * kRec * (double)g->desc.n_leaves;
-  return g->desc.n_species == 4 || rec_bytes > 4.0e9;
+  return path_walk_auto(&g->desc);
 }
 
 rt_status rt_transport(rt_grid* g, uint64_t n_packages, uint64_t seed,
@@ -936,11 +958,17 @@ rt_status rt_pathlength(rt_grid* g, float* out, int mem, void* stream) {
   cudaStream_t s = as_stream(stream);
   RT_CUDA(cudaSetDevice(g->dev));
   const size_t n = (size_t)g->desc.n_species * g->desc.n_leaves;
-  RT_CUDA(cudaMemcpyAsync(out, g->d_pathabs, sizeof(float) * n,
-                          mem == RT_MEM_DEVICE ? cudaMemcpyDeviceToDevice
-                                               : cudaMemcpyDeviceToHost,
-                          s));
-  if (mem != RT_MEM_DEVICE) return sync_status(g, s);
+  float* dst = out;
+  if (mem != RT_MEM_DEVICE) {
+    rt_status st;
+    if (!g->d_Tscratch && (st = dalloc(&g->d_Tscratch, n)) != RT_OK) return st;
+    dst = g->d_Tscratch;
+  }
+  RT_CUDA(launch_tally_out(g->g, g->d_pathabs, dst, s));
+  if (mem != RT_MEM_DEVICE) {
+    RT_CUDA(cudaMemcpyAsync(out, dst, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
+    return sync_status(g, s);
+  }
   return RT_OK;
 }
 
@@ -1665,6 +1693,7 @@ struct rt_batch {
   int blocks_per_sm = 0;
   int threads = 256;  // threads per block of the batched launch
   int s_fixed = 0;  // the species count every model shares (walk compiled for it), else 0
+  bool tally = false;  // path-length tallies kept
   cudaStream_t capture_stream = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1731,8 +1760,9 @@ rt_status rt_batch_create(rt_grid* const* grids, int n, const uint64_t* n_packag
   b->blocks_per_sm = o ? o->blocks_per_sm : 0;
   b->threads = (o && o->threads > 0) ? o->threads : 256;
   b->s_fixed = grids[0]->desc.n_species;
-  for (int m = 0; m < n; ++m)  // the fixed-count walk runs without the path-length tally
-    if (grids[m]->desc.n_species != b->s_fixed || desc[(size_t)m].r.pathabs) b->s_fixed = 0;
+  b->tally = desc[0].r.pathabs != nullptr;  // one choice of estimators for all models
+  for (int m = 0; m < n; ++m)
+    if (grids[m]->desc.n_species != b->s_fixed) b->s_fixed = 0;
   if ((st = dalloc(&b->d_models, (size_t)n)) != RT_OK ||
       (st = dalloc(&b->d_next, (size_t)n)) != RT_OK) {
     rt_batch_destroy(b);
@@ -1759,7 +1789,7 @@ rt_status rt_batch_run(rt_batch* b, int reset, int temperatures, void* stream) {
     }
   RT_CUDA(cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long) * b->grids.size(), s));
   RT_CUDA(launch_transport_batch(b->d_models, (int)b->grids.size(), b->d_next, b->chunk,
-                                 b->blocks_per_sm, b->s_fixed, b->threads, s));
+                                 b->blocks_per_sm, b->s_fixed, b->tally, b->threads, s));
   if (temperatures)
     for (rt_grid* g : b->grids)
       RT_CUDA(launch_temperatures(g->g, g->tab, g->d_count, g->d_Tscratch, g->d_counters, s));

@@ -26,10 +26,12 @@ enum Counter {
 // Face links of a leaf (record of 8 int32 per leaf: faces -x,+x,-y,+y,-z,+z, then
 // the densities of species 0 and 1 as float bits when S <= 2). A link is
 //   kLinkEscape                the face is the domain boundary;
-//   id | (level << 28)         the neighbouring leaf (same size or coarser);
+//   id | (levels up << 28)     the neighbouring leaf: 0 levels up a leaf of the same size
+//                              (so links below kLinkSame need no decoding), else coarser;
 //   -(block + 1)               the same-size neighbour is split: descend into block.
 constexpr int32_t kLinkEscape = (int32_t)0x80000000;
 constexpr int32_t kLinkLeafMask = 0x0FFFFFFF;
+constexpr int32_t kLinkSame = 1 << 28;
 constexpr long long kMaxLinkedLeaves = 1ll << 28;
 
 // Geometry and densities (device pointers), passed by value.
@@ -51,14 +53,15 @@ struct DevGrid {
 // then the densities of species 0 and 1 when S <= 2 (zero otherwise).
 constexpr int kRec = 8;
 
-// Per-bin opacity record for one species, kept in shared memory during transport.
-struct Kappa {
+// Per-bin opacity record for one species.
+struct alignas(16) Kappa {
   float kext, ksca, kabs, g;  // cm^2 g^-1, cm^2 g^-1, cm^2 g^-1, HG asymmetry
 };
 
 // Tables built in FP64 on the device and stored for transport.
 struct DevTables {
   const Kappa* kap;           // [B][S]
+  const float* kext;          // [B][S] the records' extinction opacities alone
   const float* star_cdf;      // [B] normalised cumulative stellar spectrum
   const float* S32;           // [S][n_T] emitted power per gram at the table rows
   const double* S64;          // [S][n_T]
@@ -90,7 +93,7 @@ struct DevRun {
   unsigned int* status;
   unsigned* pahabs;               // [n_pah][n_leaves][n_coarse] PAH absorptions
   unsigned* pah_flag;             // [n_leaves] bit p set: PAH p absorbed in the cell
-  float* pathabs;                 // [S][n_leaves] path-length tallies, or null
+  float* pathabs;                 // [n_leaves][S] path-length tallies, or null
   float src[3];                   // source position, base-cube units
   float beam[3];
   double src64[3];
@@ -140,10 +143,10 @@ struct ModelDesc {
 // Kernel launchers (rt_transport.cu, rt_tables.cu).
 // next [n_models]: packages of each model handed out so far (zeros); chunk >= 32: how
 // many a warp takes at a time. s_fixed: the species count all models share (2 has a walk
-// compiled for it, without the path-length tally), 0 otherwise
+// compiled for it), 0 otherwise; tally: the path-length tallies (of every model)
 cudaError_t launch_transport_batch(const ModelDesc* models, int n_models,
                                    unsigned long long* next, int chunk, int blocks_per_sm,
-                                   int s_fixed, int threads, cudaStream_t s);
+                                   int s_fixed, bool tally, int threads, cudaStream_t s);
 cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const DevRun& r,
                                   int blocks_per_sm, int threads, cudaStream_t s,
                                   const DevPeel* peel = nullptr, bool path = false);
@@ -211,6 +214,7 @@ struct TableBuild {
   unsigned short* cdf_guide; // [S][n_T-1][B]
   int* u_guide;              // [S][n_T]
   Kappa* kap;                // [B][S]
+  float* kext;               // [B][S]
   float* star_cdf;           // [B]
   double* star_frac;         // [1] in-range fraction of the stellar blackbody
 };
@@ -299,6 +303,8 @@ size_t pt_scratch_doubles(int n_cases, int M, int B);
 
 cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T_frozen,
                             float* u_frozen, float t_min, cudaStream_t s);
+// out [S][n_leaves] from tallies [n_leaves][S]
+cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out, cudaStream_t s);
 cudaError_t launch_temperatures(const DevGrid& g, const DevTables& t,
                                 const unsigned long long* count, float* T_out,
                                 unsigned long long* counters, cudaStream_t s,

@@ -162,6 +162,7 @@ __global__ void k_opacity(TableBuild tb) {
       k.kext = (float)(tb.kabs[j] + tb.ksca[j]);
       k.g = (float)tb.ghg[j];
       tb.kap[(size_t)b * tb.S + s] = k;
+      tb.kext[(size_t)b * tb.S + s] = k.kext;
     }
   }
 }
@@ -229,7 +230,7 @@ __global__ void k_temperatures(DevGrid g, DevTables t, const unsigned long long*
     int s = (int)(idx / g.n_leaves);
     long long c = idx - (long long)s * g.n_leaves;
     // absorbed energy in units of eps: the count, or the path-length tally
-    const double n = pathabs ? (double)pathabs[idx] : (double)count[idx];
+    const double n = pathabs ? (double)pathabs[c * g.S + s] : (double)count[idx];
     float rho_d0 = g.rho[c * g.S + s];
     float Tv = 0.0f;
     if (n > 0.0 && rho_d0 > 0.0f) {
@@ -270,6 +271,13 @@ __global__ void k_temperatures(DevGrid g, DevTables t, const unsigned long long*
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(&counters[kCClamped], (unsigned long long)__popc(m));
 }
 
+// Path-length tallies, species within a cell adjacent, to one array per species.
+__global__ void k_tally_out(const float* pathabs, long long N, int S, float* out) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (c >= N) return;
+  for (int s = 0; s < S; ++s) out[(size_t)s * N + c] = pathabs[(size_t)c * S + s];
+}
+
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -288,6 +296,12 @@ cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T
                             float* u_frozen, float t_min, cudaStream_t s) {
   long long n = (long long)g.S * g.n_leaves;
   k_frozen_u<<<nblk(n, 256), 256, 0, s>>>(g, t, T_frozen, u_frozen, t_min);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out,
+                             cudaStream_t s) {
+  k_tally_out<<<nblk(g.n_leaves, 256), 256, 0, s>>>(pathabs, g.n_leaves, g.S, out);
   return cudaGetLastError();
 }
 

@@ -198,19 +198,29 @@ struct Pkg {
   R inv[3];  // 1/d; +inf where d == 0 (of either sign)
   R tau;
   int bin;
-  unsigned event;
+  unsigned event;  // interactions so far
   unsigned long long id;
-  bool touched;  // interacted at least once
+  unsigned dirs;  // the pool's walks: signs of the direction (see orient)
 };
 
-struct Tally {  // per-thread counters, flushed to the 64-bit device totals
+struct Tally {  // per-thread counters (plain kernel), flushed to the 64-bit device totals
   unsigned emitted, escaped, capped, absorptions, scatters, crossings, errors, clamped;
   unsigned levels;  // child-table reads of the walk
   unsigned peel_events, peel_crossings;  // peel-off sight lines and the cells they cross
 };
 
-// a flush is forced before any per-thread counter could pass 2^31
-constexpr unsigned kTallyFlushAt = 1u << 31;
+// The pool counts crossings and tree reads per lane and everything rarer per warp in
+// shared memory (nine counters in registers made the walks spill).
+struct LaneTally {
+  unsigned crossings, levels;
+};
+
+constexpr int kTallyWords = 16;  // per warp: kNumCounters words
+static_assert(kNumCounters <= kTallyWords, "the counters fit a warp's words");
+
+// a flush is forced once a counter passes 2^30: one round of the pool adds at most
+// 32 x refill_period to a warp's
+constexpr unsigned kTallyFlushAt = 1u << 30;
 
 enum Adv { kCrossed = 0, kInteract = 1, kEscaped = 2, kError = 3 };
 
@@ -226,7 +236,6 @@ __device__ __forceinline__ void emit(Pkg<R>& k, unsigned long long id, const Dev
   uint4 w = draw(r.seed, id, 0u, 0u);
   k.id = id;
   k.event = 0;
-  k.touched = false;
   k.bin = search_cdf(star_cdf, B, unit<float>(w.x));
   if (r.source_kind == 1) {
 #pragma unroll
@@ -280,7 +289,7 @@ __device__ __forceinline__ int advance(Pkg<R>& k, const DevGrid& g, const Kappa*
     const R seg = (kx > (R)0 && dtau > k.tau) ? k.tau / kx : tex;
     for (int s = 0; s < g.S; ++s) {
       const float v = (float)((R)__ldg(&rho[s]) * (R)kb[s].kabs * seg);
-      if (v > 0.f) atomicAdd(&pathabs[(size_t)s * g.n_leaves + leaf], v);
+      if (v > 0.f) atomicAdd(&pathabs[(size_t)leaf * g.S + s], v);
     }
   }
   if (kx > (R)0 && dtau > k.tau) {
@@ -298,9 +307,114 @@ __device__ __forceinline__ int advance(Pkg<R>& k, const DevGrid& g, const Kappa*
   return kCrossed;
 }
 
+// ---------------------------------------------------------------- forward frame
+// The pool's walks run in a frame in which the package moves forward along every axis:
+// an axis with d < 0 is mirrored (p -> -p, d -> -d; a cell [lo, hi] -> [-hi, -lo]), which
+// FP32 does exactly, and every operation of the walk commutes with the sign, so the
+// positions are bit for bit those of the unmirrored walk. The face ahead is then always
+// lo + edge, a position can only pass its cell's upper bound (one minimum instead of a
+// clamp), the neighbour's corner is the face itself, and the child of a point is a plain
+// floor. Pkg::p, d, inv and the cell's corner are kept mirrored between interactions;
+// the frame changes with the direction (orient).
+// Together with what moved out of the step (the move to an interaction point into the
+// interaction phase, the spectrum of escaped packages into the refill, the rarer counters
+// into shared memory) it took the linked walk on the disk of 2.4e6 cells from 11.5 to 8.3
+// warp instructions per crossing and 5e6 packages from 5.08 to 4.17 ms at four blocks per
+// SM; the path walk on 8.0e6 cells, 1e7 packages, from 22.8 to 22.1 ms.
+//
+// Pkg::dirs: bits 24-26, the mirrored axes; byte a (a = 0, 1, 2), what the walk looks up
+// by the exit axis: linked, the byte offset of the face's link in the record; path, 0x80
+// where the axis is mirrored.
+__device__ __forceinline__ unsigned mirrored(const Pkg<float>& k) { return (k.dirs >> 24) & 7u; }
+
+template <bool kPath, class CellT>
+__device__ __forceinline__ void orient(Pkg<float>& k, CellT& c, unsigned was) {
+  unsigned dirs = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const bool neg = k.d[a] < 0.f;
+    if (neg != (((was >> a) & 1u) != 0u)) {
+      k.p[a] = -k.p[a];
+      c.lo[a] = -(c.lo[a] + c.sz);
+    }
+    k.d[a] = fabsf(k.d[a]);
+    k.inv[a] = fabsf(k.inv[a]);
+    if (neg) dirs |= 1u << (24 + a);
+    if (kPath)
+      dirs |= neg ? 0x80u << (8 * a) : 0u;
+    else
+      dirs |= (unsigned)(8 * a + (neg ? 0 : 4)) << (8 * a);
+  }
+  k.dirs = dirs;
+}
+
+// the direction with its signs back (k.d only), and one component of a position
+__device__ __forceinline__ void restore_direction(Pkg<float>& k) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    if ((k.dirs >> (24 + a)) & 1u) k.d[a] = -k.d[a];
+}
+
+__device__ __forceinline__ float true_component(const Pkg<float>& k, float v, int a) {
+  return (k.dirs >> (24 + a)) & 1u ? -v : v;
+}
+
+// What byte a of k.dirs says of the exit axis: for the linked walk the byte, for the path
+// walk its top bit over all 32 bits. (prmt itself: the intrinsic for it ignores the
+// selector bit that spreads the sign.)
+__device__ __forceinline__ unsigned pick_byte(unsigned x, unsigned sel) {
+  unsigned r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "r"(sel));
+  return r;
+}
+
+// Distance to the nearest face ahead and its axis (the lowest on ties): ax0, ax1 or
+// neither. An axis with d == 0 has inv = +inf and gives +inf, or NaN on its upper face,
+// which the minimum never picks.
+struct Exit {
+  float F[3], t;
+  bool ax0, ax1;
+};
+
+template <class CellT>
+__device__ __forceinline__ Exit exit_of(const Pkg<float>& k, const CellT& c) {
+  Exit e;
+  float t[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    e.F[a] = c.lo[a] + c.sz;
+    t[a] = (e.F[a] - k.p[a]) * k.inv[a];
+  }
+  e.t = fminf(fminf(t[0], t[1]), t[2]);
+  e.ax0 = t[0] == e.t;
+  e.ax1 = !e.ax0 && t[1] == e.t;
+  return e;
+}
+
+// onto the face ahead; the corner becomes that of the same-size neighbour
+template <class CellT>
+__device__ __forceinline__ void cross(Pkg<float>& k, CellT& c, const Exit& e) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const bool here = a == 0 ? e.ax0 : (a == 1 ? e.ax1 : !(e.ax0 || e.ax1));
+    const float v = fminf(e.F[a], fmaf(e.t, k.d[a], k.p[a]));
+    k.p[a] = here ? e.F[a] : v;
+    c.lo[a] = here ? e.F[a] : c.lo[a];
+  }
+}
+
+// to the interaction point: tau spent inside the cell at extinction kx
+template <class CellT>
+__device__ __forceinline__ void to_point(Pkg<float>& k, const CellT& c, float kx) {
+  const float sd = k.tau / kx;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    k.p[a] = fminf(c.lo[a] + c.sz, fmaf(sd, k.d[a], k.p[a]));
+}
+
 // ---------------------------------------------------------------- linked walk
-// The leaf a package is in, with its level, its lower corner and its edge (base-cube
-// units; both exact in FP32: multiples of 2^-level below 2^13).
+// The leaf a package is in, with its lower corner (in the package's forward frame) and
+// its edge (base-cube units; both exact in FP32: multiples of 2^-level below 2^13).
 struct Cell {
   int leaf;
   float lo[3];
@@ -308,138 +422,192 @@ struct Cell {
   __device__ __forceinline__ int level() const { return 127 - (__float_as_int(sz) >> 23); }
 };
 
-__device__ __forceinline__ void set_corner(Cell& c, const int I[3], int level) {
+template <class CellT>
+__device__ __forceinline__ void set_corner(CellT& c, const int I[3], int level) {
   c.sz = __int_as_float((127 - level) << 23);
 #pragma unroll
   for (int a = 0; a < 3; ++a) c.lo[a] = (float)I[a] * c.sz;
 }
 
 // Enter the grid at the package's position (full descent from the base cube).
-__device__ __forceinline__ int enter(const Pkg<float>& k, const DevGrid& g, Cell& c,
+__device__ __forceinline__ int enter(Pkg<float>& k, const DevGrid& g, Cell& c,
                                      unsigned& child_reads) {
   int I[3], level;
   int rc = locate<float>(g, k.p, k.d, c.leaf, level, I);
   if (rc == 0) {
     child_reads += level;
     set_corner(c, I, level);
+    orient<false>(k, c, 0u);
   }
   return rc;
+}
+
+// The densities of a leaf as one vector (kS = 2: from its face-link record, 4: from the
+// density rows), and the sum of densities times a bin's opacities.
+template <int kS>
+__device__ __forceinline__ float4 leaf_rho(const DevGrid& g, int leaf) {
+  if constexpr (kS == 2) {
+    const float2 r = __ldg(reinterpret_cast<const float2*>(g.links + (size_t)leaf * kRec + 6));
+    return make_float4(r.x, r.y, 0.f, 0.f);
+  } else if constexpr (kS == 4) {
+    return __ldg(reinterpret_cast<const float4*>(g.rho) + leaf);
+  } else {
+    return make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// A bin's opacities of kS species as one vector, from a table [B][kS].
+template <int kS>
+__device__ __forceinline__ float4 bin_vec(const float* table, int bin) {
+  if constexpr (kS == 4) {
+    return reinterpret_cast<const float4*>(table)[bin];
+  } else if constexpr (kS == 2) {
+    const float2 e = reinterpret_cast<const float2*>(table)[bin];
+    return make_float4(e.x, e.y, 0.f, 0.f);
+  } else {
+    return make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// Extinction of a leaf per base-cube unit of path at a bin. kS: the species count when
+// fixed at compile time (2 or 4: the densities r, the bin's opacities as one vector from
+// kext), 0 when read from the grid (densities from the face-link record for one or two
+// species). kInOrder: summed species by species as the generic form does (the launches with
+// the path-length tally, whose histories are those of the generic walk to the last bit).
+template <int kS, bool kInOrder = false>
+__device__ __forceinline__ float leaf_ext(const DevGrid& g, int leaf, float4 r, int bin,
+                                          const Kappa* kap, const float* kext) {
+  if constexpr (kS == 2) {
+    const float4 e = bin_vec<2>(kext, bin);
+    if constexpr (kInOrder) return fmaf(r.y, e.y, r.x * e.x);
+    return r.x * e.x + r.y * e.y;
+  } else if constexpr (kS == 4) {
+    const float4 e = bin_vec<4>(kext, bin);
+    if constexpr (kInOrder)
+      return fmaf(r.w, e.w, fmaf(r.z, e.z, fmaf(r.y, e.y, r.x * e.x)));
+    return r.x * e.x + r.y * e.y + r.z * e.z + r.w * e.w;
+  } else {
+    const Kappa* kb = kap + bin * g.S;
+    if (g.S <= 2) {
+      const int* rec = g.links + (size_t)leaf * kRec;
+      float kx = __int_as_float(__ldg(rec + 6)) * kb[0].kext;
+      if (g.S == 2) kx += __int_as_float(__ldg(rec + 7)) * kb[1].kext;
+      return kx;
+    }
+    const float* rho = g.rho + (size_t)leaf * g.S;
+    float kx = 0.f;
+    for (int s = 0; s < g.S; ++s) kx += __ldg(&rho[s]) * kb[s].kext;
+    return kx;
+  }
+}
+
+// Path-length tallies of a segment of length seg in a leaf, [n_leaves][S]: rho_s
+// kappa_abs,s seg is added for every species. With the species of a cell side by side two
+// or four of them are one vector reduction to one sector. 2e6 packages through 1.06e6
+// cells of two species: 3.9 ms with an atomic per species into arrays apart (and the
+// generic species loop), 2.7 ms.
+template <int kS>
+__device__ __forceinline__ void tally_segment(const DevGrid& g, float* pathabs, int leaf,
+                                              float4 r, int bin, float seg, const Kappa* kap,
+                                              const float* kabs) {
+  if constexpr (kS == 2) {
+    const float4 a = bin_vec<2>(kabs, bin);
+    const float v0 = r.x * a.x * seg, v1 = r.y * a.y * seg;
+    if (v0 > 0.f || v1 > 0.f)
+      asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(
+                       __cvta_generic_to_global(pathabs + 2 * (size_t)leaf)),
+                   "f"(v0), "f"(v1)
+                   : "memory");
+  } else if constexpr (kS == 4) {
+    const float4 a = bin_vec<4>(kabs, bin);
+    const float v0 = r.x * a.x * seg, v1 = r.y * a.y * seg, v2 = r.z * a.z * seg,
+                v3 = r.w * a.w * seg;
+    if (v0 > 0.f || v1 > 0.f || v2 > 0.f || v3 > 0.f)
+      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                       __cvta_generic_to_global(pathabs + 4 * (size_t)leaf)),
+                   "f"(v0), "f"(v1), "f"(v2), "f"(v3)
+                   : "memory");
+  } else {
+    const float* rho = g.rho + (size_t)leaf * g.S;
+    const Kappa* kb = kap + bin * g.S;
+    for (int s = 0; s < g.S; ++s) {
+      const float v = __ldg(&rho[s]) * kb[s].kabs * seg;
+      if (v > 0.f) atomicAdd(&pathabs[(size_t)leaf * g.S + s], v);
+    }
+  }
 }
 
 // One cell of the walk using the face links: the exit face follows from the
 // geometry alone, so the face link and the densities come from one record read;
 // the next leaf is the linked one (same size or coarser), or is found by a short
-// descent when the neighbouring region is finer. kLos: a sight line, which never
-// interacts and adds the cell's optical depth to *tau_los instead.
-template <bool kLos = false, int kS = 0>
+// descent when the neighbouring region is finer. Where the optical depth runs out
+// inside the cell nothing is changed (to_point follows in the interaction phase, which
+// runs with more lanes). kLos: a sight line, which never interacts and adds the cell's
+// optical depth to *tau_los instead. kTally: the path-length tallies, into pathabs (kabs:
+// the absorption opacities [B][kS]).
+template <bool kLos = false, int kS = 0, bool kTally = false>
 __device__ __forceinline__ int advance_linked(Pkg<float>& k, Cell& c, const DevGrid& g,
-                                              const Kappa* kap,
-                                              unsigned& child_reads, float* pathabs,
-                                              float* tau_los = nullptr) {
-  // every array below is indexed with constants only, so it stays in registers
-  const float sz = c.sz;
-  const float lo0 = c.lo[0], lo1 = c.lo[1], lo2 = c.lo[2];
-  const float hi0 = lo0 + sz, hi1 = lo1 + sz, hi2 = lo2 + sz;
-  const float d0 = k.d[0], d1 = k.d[1], d2 = k.d[2];
-  // distance to the face ahead on each axis; an axis with d == 0 has inv = +inf and
-  // gives +inf, or NaN on its upper face, which the minimum below never picks
-  const float t0 = ((k.inv[0] > 0.f ? hi0 : lo0) - k.p[0]) * k.inv[0];
-  const float t1 = ((k.inv[1] > 0.f ? hi1 : lo1) - k.p[1]) * k.inv[1];
-  const float t2 = ((k.inv[2] > 0.f ? hi2 : lo2) - k.p[2]) * k.inv[2];
-  // exit axis: the nearest face, the lowest axis on ties
-  const float tmin = fminf(fminf(t0, t1), t2);
-  const int ax = t0 == tmin ? 0 : (t1 == tmin ? 1 : 2);
-  const float tex = fmaxf(tmin, 0.f);
-  const float dax = ax == 0 ? d0 : (ax == 1 ? d1 : d2);
-  const bool up = dax > 0.f;
-  const int* rec = g.links + (size_t)c.leaf * kRec;
-  const int link = __ldg(rec + 2 * ax + (up ? 1 : 0));
-  // kS: the species count when fixed at compile time (2: both densities in the
-  // record), 0 when read from the grid
-  const Kappa* kb = kap + k.bin * (kS > 0 ? kS : g.S);
-  float kx;
-  if (kS == 2 || (kS == 0 && g.S <= 2)) {
-    kx = __int_as_float(__ldg(rec + 6)) * kb[0].kext;
-    if (kS == 2 || g.S == 2) kx += __int_as_float(__ldg(rec + 7)) * kb[1].kext;
-  } else {
-    const float* rho = g.rho + (size_t)c.leaf * g.S;
-    kx = 0.f;
-    for (int s = 0; s < g.S; ++s) kx += __ldg(&rho[s]) * kb[s].kext;
-  }
-  const float dtau = kx * tex;
+                                              const Kappa* kap, const float* kext,
+                                              unsigned& child_reads, float* tau_los = nullptr,
+                                              float* pathabs = nullptr,
+                                              const float* kabs = nullptr) {
+  const Exit e = exit_of(k, c);
+  const float4 r = leaf_rho<kS>(g, c.leaf);
+  const float kx = leaf_ext<kS, kTally>(g, c.leaf, r, k.bin, kap, kext);
+  const unsigned off =
+      pick_byte(k.dirs, e.ax0 ? 0x4440u : (e.ax1 ? 0x4441u : 0x4442u));
+  const int link = __ldg(reinterpret_cast<const int*>(
+      reinterpret_cast<const char*>(g.links + (size_t)c.leaf * kRec) + off));
+  const float dtau = kx * e.t;
   bool hit;
   if constexpr (kLos) {
     *tau_los += dtau;
     hit = false;
   } else {
-    hit = kx > 0.f && dtau > k.tau;
+    hit = dtau > k.tau;  // only where kx > 0
   }
-  if (!kLos && pathabs) {  // path-length tally of the segment inside this cell
-    const float seg = hit ? k.tau / kx : tex;
-    const float* rho = g.rho + (size_t)c.leaf * g.S;
-    for (int s = 0; s < g.S; ++s) {
-      const float v = __ldg(&rho[s]) * kb[s].kabs * seg;
-      if (v > 0.f) atomicAdd(&pathabs[(size_t)s * g.n_leaves + c.leaf], v);
-    }
-  }
-  if (hit) {
-    const float sd = k.tau / kx;
-    k.p[0] = fminf(hi0, fmaxf(lo0, k.p[0] + sd * d0));
-    k.p[1] = fminf(hi1, fmaxf(lo1, k.p[1] + sd * d1));
-    k.p[2] = fminf(hi2, fmaxf(lo2, k.p[2] + sd * d2));
-    return kInteract;
-  }
+  if constexpr (kTally)
+    tally_segment<kS>(g, pathabs, c.leaf, r, k.bin, hit ? k.tau / kx : e.t, kap, kabs);
+  if (hit) return kInteract;
   if constexpr (!kLos) k.tau -= dtau;
-  const float f0 = d0 > 0.f ? hi0 : lo0, f1 = d1 > 0.f ? hi1 : lo1, f2 = d2 > 0.f ? hi2 : lo2;
-  k.p[0] = ax == 0 ? f0 : fminf(hi0, fmaxf(lo0, k.p[0] + tex * d0));
-  k.p[1] = ax == 1 ? f1 : fminf(hi1, fmaxf(lo1, k.p[1] + tex * d1));
-  k.p[2] = ax == 2 ? f2 : fminf(hi2, fmaxf(lo2, k.p[2] + tex * d2));
-  if (link == kLinkEscape) return kEscaped;
-  // the same-size neighbour's corner
-  const float step = up ? sz : -sz;
-  const float n0 = ax == 0 ? lo0 + step : lo0;
-  const float n1 = ax == 1 ? lo1 + step : lo1;
-  const float n2 = ax == 2 ? lo2 + step : lo2;
-  if (link >= 0) {
-    const int nl = link >> 28;
-    const float nsz = __int_as_float((127 - nl) << 23);
-    c.leaf = link & kLinkLeafMask;
-    if (nsz == sz) {
-      c.lo[0] = n0;
-      c.lo[1] = n1;
-      c.lo[2] = n2;
-    } else {  // a coarser leaf: round the corner down to its edge (exact)
-      c.sz = nsz;
-      const float isz = __int_as_float((127 + nl) << 23);
-      c.lo[0] = floorf(n0 * isz) * c.sz;
-      c.lo[1] = floorf(n1 * isz) * c.sz;
-      c.lo[2] = floorf(n2 * isz) * c.sz;
-    }
+  cross(k, c, e);
+  if ((unsigned)link < (unsigned)kLinkSame) {  // a leaf of the same size
+    c.leaf = link;
     return kCrossed;
   }
+  if (link >= 0) {  // a coarser leaf: round the corner down to its edge (exact)
+    c.leaf = link & kLinkLeafMask;
+    const int bits = __float_as_int(c.sz) + ((link >> 28) << 23);
+    c.sz = __int_as_float(bits);
+    const float isz = __int_as_float((254 << 23) - bits);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) c.lo[a] = floorf(c.lo[a] * isz) * c.sz;
+    return kCrossed;
+  }
+  if (link == kLinkEscape) return kEscaped;
   // the same-size neighbour is split: descend, staying inside that node
   int lev = c.level();
   const float iz = __int_as_float((127 + lev) << 23);  // 2^level
-  int J0 = (int)(n0 * iz), J1 = (int)(n1 * iz), J2 = (int)(n2 * iz);
+  int J[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) J[a] = (int)(c.lo[a] * iz);
   long long blk = -(long long)link - 1;
   for (;;) {
     if (blk >= g.n_blocks || lev >= g.max_level) return kError;
     ++lev;
     ++child_reads;
-    const float sc = (float)(1 << lev);
-    const int j0 = min(max(cell_index(k.p[0] * sc, d0), 2 * J0), 2 * J0 + 1);
-    const int j1 = min(max(cell_index(k.p[1] * sc, d1), 2 * J1), 2 * J1 + 1);
-    const int j2 = min(max(cell_index(k.p[2] * sc, d2), 2 * J2), 2 * J2 + 1);
-    const int oct = (j0 - 2 * J0) | ((j1 - 2 * J1) << 1) | ((j2 - 2 * J2) << 2);
-    J0 = j0;
-    J1 = j1;
-    J2 = j2;
+    const float sc = __int_as_float((127 + lev) << 23);
+    unsigned oct = mirrored(k);  // a mirrored axis numbers its children backwards
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      J[a] = min(max(__float2int_rd(k.p[a] * sc), 2 * J[a]), 2 * J[a] + 1);
+      oct ^= (unsigned)(J[a] & 1) << a;
+    }
     const int node = __ldg(&g.child[blk * 8 + oct]);
     if (node >= 0) {
       if ((long long)node >= g.n_leaves) return kError;
       c.leaf = node;
-      const int I[3] = {J0, J1, J2};
-      set_corner(c, I, lev);
+      set_corner(c, J, lev);
       return kCrossed;
     }
     blk = -(long long)node - 1;
@@ -461,10 +629,11 @@ __device__ __forceinline__ int advance_linked(Pkg<float>& k, Cell& c, const DevG
 constexpr int kPathLevels = 4;  // the path walk serves grids of at most 4 levels
 
 struct PathCell {
-  int slot;  // tree slot of the leaf: its row in rho_slot
-  float kx;  // the leaf's extinction at the package's bin, or -1 when not yet read
-  int J[3];  // integer coordinates of the leaf's lower corner at its level
-  float sz;  // 2^-level
+  int slot;     // tree slot of the leaf: its row in rho_slot
+  float kx;     // the leaf's extinction at the package's bin
+  float lo[3];  // lower corner, in the package's forward frame
+  float sz;     // 2^-level
+  int b0;       // base cube the package is in
   int b1, b2, b3, b4;
   __device__ __forceinline__ int level() const { return 127 - (__float_as_int(sz) >> 23); }
   __device__ __forceinline__ int blk(int l) const {
@@ -481,7 +650,7 @@ struct PathCell {
 // Enter the grid at the package's position: descent from the base cube, recording
 // the blocks on the path. 0 inside, 1 outside, -1 malformed (or deeper than the
 // walk serves).
-__device__ __forceinline__ int enter_path(const Pkg<float>& k, const DevGrid& g, PathCell& c,
+__device__ __forceinline__ int enter_path(Pkg<float>& k, const DevGrid& g, PathCell& c,
                                           unsigned& child_reads) {
   const int n = g.n_base;
   int I[3];
@@ -491,6 +660,7 @@ __device__ __forceinline__ int enter_path(const Pkg<float>& k, const DevGrid& g,
     if (I[a] < 0 || I[a] >= n) return 1;
   }
   int slot = I[0] + n * (I[1] + n * I[2]);
+  c.b0 = slot;
   int node = __ldg(&g.base[slot]);
   int lev = 0;
   while (node < 0) {
@@ -514,10 +684,8 @@ __device__ __forceinline__ int enter_path(const Pkg<float>& k, const DevGrid& g,
   }
   if ((long long)node >= g.n_leaves) return -1;
   c.slot = slot;
-  c.kx = -1.f;
-  c.sz = __int_as_float((127 - lev) << 23);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) c.J[a] = I[a];
+  set_corner(c, I, lev);
+  orient<true>(k, c, 0u);
   return 0;
 }
 
@@ -545,21 +713,6 @@ __device__ __forceinline__ int path_leaf(const DevGrid& g, int slot) {
   return node >= 0 && (long long)node < g.n_leaves ? node : -1;
 }
 
-// The extinction opacities of a bin as one vector (kS = 4 or 2: from the block's
-// shared-memory copy, one 16- or 8-byte read; zeros for the generic form, which reads
-// them from the opacity records kb in slot_ext).
-template <int kS>
-__device__ __forceinline__ float4 bin_ext(const float* kext, int bin) {
-  if constexpr (kS == 4) {
-    return reinterpret_cast<const float4*>(kext)[bin];
-  } else if constexpr (kS == 2) {
-    const float2 e = reinterpret_cast<const float2*>(kext)[bin];
-    return make_float4(e.x, e.y, 0.f, 0.f);
-  } else {
-    return make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-}
-
 template <int kS>
 __device__ __forceinline__ float slot_ext(const DevGrid& g, float4 v, int slot, float4 e,
                                           const Kappa* kb) {
@@ -575,96 +728,94 @@ __device__ __forceinline__ float slot_ext(const DevGrid& g, float4 v, int slot, 
   }
 }
 
+// The extinction of the cell a package is in, at its bin.
+template <int kS>
+__device__ __forceinline__ float path_ext(const DevGrid& g, int slot, int bin, const Kappa* kap,
+                                          const float* kext) {
+  return slot_ext<kS>(g, slot_row<kS>(g, slot), slot, bin_vec<kS>(kext, bin),
+                      kap + bin * (kS > 0 ? kS : g.S));
+}
+
 // One cell of the path walk (kS: 2 or 4 species read as one vector, 0 the generic
 // loop). The next cell is found from the rows alone: the slot of the first node off
-// the package's path is known from the block ids it carries, and that slot's row is
-// either the leaf's densities or the code of the block to descend into -- one read
-// per crossing (one more per level descended). The extinction at the package's bin
+// the package's path is known from the block ids it carries (the next base cube is a
+// stride away from its own), and that slot's row is either the leaf's densities or the
+// code of the block to descend into -- one read per crossing (one more per level
+// descended). Integer coordinates are formed only in refined cubes; between base cubes,
+// most of a large grid's crossings, there are none. The extinction at the package's bin
 // is kept in the cell for the next step.
 template <int kS>
 __device__ __forceinline__ int advance_path(Pkg<float>& k, PathCell& c, const DevGrid& g,
                                             const Kappa* kap, const float* kext,
                                             unsigned& child_reads) {
-  const float sz = c.sz;
-  int J0 = c.J[0], J1 = c.J[1], J2 = c.J[2];
-  const float lo0 = (float)J0 * sz, lo1 = (float)J1 * sz, lo2 = (float)J2 * sz;
-  const float hi0 = lo0 + sz, hi1 = lo1 + sz, hi2 = lo2 + sz;
-  const float d0 = k.d[0], d1 = k.d[1], d2 = k.d[2];
-  const float t0 = ((k.inv[0] > 0.f ? hi0 : lo0) - k.p[0]) * k.inv[0];
-  const float t1 = ((k.inv[1] > 0.f ? hi1 : lo1) - k.p[1]) * k.inv[1];
-  const float t2 = ((k.inv[2] > 0.f ? hi2 : lo2) - k.p[2]) * k.inv[2];
-  const float tmin = fminf(fminf(t0, t1), t2);
-  const int ax = t0 == tmin ? 0 : (t1 == tmin ? 1 : 2);
-  const float tex = fmaxf(tmin, 0.f);
-  const float dax = ax == 0 ? d0 : (ax == 1 ? d1 : d2);
-  const bool up = dax > 0.f;
-  const Kappa* kb = kap + k.bin * (kS > 0 ? kS : g.S);
-  float kx = c.kx;
-  if (kx < 0.f) kx = slot_ext<kS>(g, slot_row<kS>(g, c.slot), c.slot, bin_ext<kS>(kext, k.bin), kb);
-  const float dtau = kx * tex;
-  if (kx > 0.f && dtau > k.tau) {
-    const float sd = k.tau / kx;
-    k.p[0] = fminf(hi0, fmaxf(lo0, k.p[0] + sd * d0));
-    k.p[1] = fminf(hi1, fmaxf(lo1, k.p[1] + sd * d1));
-    k.p[2] = fminf(hi2, fmaxf(lo2, k.p[2] + sd * d2));
-    return kInteract;
-  }
+  const Exit e = exit_of(k, c);
+  const float dtau = c.kx * e.t;
+  if (dtau > k.tau) return kInteract;
   k.tau -= dtau;
-  const float f0 = d0 > 0.f ? hi0 : lo0, f1 = d1 > 0.f ? hi1 : lo1, f2 = d2 > 0.f ? hi2 : lo2;
-  k.p[0] = ax == 0 ? f0 : fminf(hi0, fmaxf(lo0, k.p[0] + tex * d0));
-  k.p[1] = ax == 1 ? f1 : fminf(hi1, fmaxf(lo1, k.p[1] + tex * d1));
-  k.p[2] = ax == 2 ? f2 : fminf(hi2, fmaxf(lo2, k.p[2] + tex * d2));
-  // integer coordinates of the same-size neighbour across face ax
-  const int L = c.level();
-  const int Iax = ax == 0 ? J0 : (ax == 1 ? J1 : J2);
-  const int Jax = up ? Iax + 1 : Iax - 1;
-  if (Jax < 0 || Jax >= (g.n_base << L)) return kEscaped;
-  if (ax == 0) J0 = Jax;
-  else if (ax == 1) J1 = Jax;
-  else J2 = Jax;
-  const int u = 32 - __clz(Iax ^ Jax);  // levels up to the common ancestor
-  int lev, slot;
-  if (u > L) {  // another base cube
-    lev = 0;
-    const int n = g.n_base;
-    slot = (J0 >> L) + n * ((J1 >> L) + n * (J2 >> L));
-  } else {      // the common ancestor's block holds the first node off the path
-    lev = L - u + 1;
-    const int sh = L - lev;
-    const int oct = ((J0 >> sh) & 1) | (((J1 >> sh) & 1) << 1) | (((J2 >> sh) & 1) << 2);
-    slot = g.n_base3 + c.blk(lev) * 8 + oct;
-  }
-  float4 row = slot_row<kS>(g, slot);
-  int K0 = J0 >> (L - lev), K1 = J1 >> (L - lev), K2 = J2 >> (L - lev);
-  int code = __float_as_int(row.x);
-  while (code < 0) {
-    const long long blk = -(long long)code - 1;
-    if (blk >= g.n_blocks || lev >= g.max_level || lev >= kPathLevels) return kError;
-    ++lev;
-    c.set_blk(lev, (int)blk);
-    if (lev <= L) {
+  const float Fax = e.ax0 ? e.F[0] : (e.ax1 ? e.F[1] : e.F[2]);
+  const int n = g.n_base;
+  // all ones where the exit axis is mirrored: the domain then ends at 0 and the base
+  // cubes' numbers fall
+  const int m = (int)pick_byte(k.dirs, e.ax0 ? 0x8888u : (e.ax1 ? 0x9999u : 0xAAAAu));
+  if (Fax >= __int_as_float(__float_as_int((float)n) & ~m)) return kEscaped;
+  cross(k, c, e);
+  const int stride = e.ax0 ? 1 : (e.ax1 ? n : n * n);
+  const int next = c.b0 + (stride ^ m) - m;
+  const float sz = c.sz;
+  int slot = next, lev = 0, L = 0;
+  int J[3];
+  if (sz != 1.f) {
+    L = c.level();
+    const float iz = __int_as_float((127 + L) << 23);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) J[a] = (int)(c.lo[a] * iz);
+    const int Jax = (int)(Fax * iz);
+    const int u = 32 - __clz(Jax ^ (Jax - 1));  // levels up to the common ancestor
+    if (u <= L) {  // the common ancestor's block holds the first node off the path
+      lev = L - u + 1;
       const int sh = L - lev;
-      K0 = J0 >> sh;
-      K1 = J1 >> sh;
-      K2 = J2 >> sh;
-    } else {  // a finer neighbour: the child holding the crossing point
-      const float sc = (float)(1 << lev);
-      K0 = min(max(cell_index(k.p[0] * sc, d0), 2 * K0), 2 * K0 + 1);
-      K1 = min(max(cell_index(k.p[1] * sc, d1), 2 * K1), 2 * K1 + 1);
-      K2 = min(max(cell_index(k.p[2] * sc, d2), 2 * K2), 2 * K2 + 1);
+      const unsigned oct = (unsigned)(((J[0] >> sh) & 1) | (((J[1] >> sh) & 1) << 1) |
+                                      (((J[2] >> sh) & 1) << 2)) ^ mirrored(k);
+      slot = g.n_base3 + c.blk(lev) * 8 + (int)oct;
     }
-    const int oct = (K0 & 1) | ((K1 & 1) << 1) | ((K2 & 1) << 2);
-    slot = g.n_base3 + (int)blk * 8 + oct;
-    row = slot_row<kS>(g, slot);
-    code = __float_as_int(row.x);
-    ++child_reads;
+  }
+  if (lev == 0) c.b0 = next;
+  float4 row = slot_row<kS>(g, slot);
+  int code = __float_as_int(row.x);
+  if (sz != 1.f || code < 0) {
+    if (sz == 1.f) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) J[a] = (int)c.lo[a];
+    }
+    int K[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) K[a] = J[a] >> (L - lev);
+    while (code < 0) {
+      const long long blk = -(long long)code - 1;
+      if (blk >= g.n_blocks || lev >= g.max_level || lev >= kPathLevels) return kError;
+      ++lev;
+      c.set_blk(lev, (int)blk);
+      unsigned oct = mirrored(k);
+      if (lev <= L) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) K[a] = J[a] >> (L - lev);
+      } else {  // a finer neighbour: the child holding the crossing point
+        const float sc = __int_as_float((127 + lev) << 23);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+          K[a] = min(max(__float2int_rd(k.p[a] * sc), 2 * K[a]), 2 * K[a] + 1);
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) oct ^= (unsigned)(K[a] & 1) << a;
+      slot = g.n_base3 + (int)blk * 8 + (int)oct;
+      row = slot_row<kS>(g, slot);
+      code = __float_as_int(row.x);
+      ++child_reads;
+    }
+    set_corner(c, K, lev);
   }
   c.slot = slot;
-  c.kx = slot_ext<kS>(g, row, slot, bin_ext<kS>(kext, k.bin), kb);
-  c.sz = __int_as_float((127 - lev) << 23);
-  c.J[0] = K0;
-  c.J[1] = K1;
-  c.J[2] = K2;
+  c.kx = slot_ext<kS>(g, row, slot, bin_vec<kS>(kext, k.bin), kap + k.bin * (kS > 0 ? kS : g.S));
   return kCrossed;
 }
 
@@ -707,7 +858,6 @@ __device__ __forceinline__ int interact(Pkg<R>& k, const DevGrid& g, const Kappa
     kext += rs * kb[s].kext;
     kabs += rs * kb[s].kabs;
   }
-  k.touched = true;
   const float xs = unit<float>(w0.y);
   int sp = S - 1;
   if (unit<float>(w0.x) * kext < ksca) {
@@ -744,7 +894,7 @@ template <typename R, int kS = 0>
 __device__ __forceinline__ void reemit(Pkg<R>& k, const DevGrid& g, const DevTables& t,
                                        const DevRun& r, int s, int leaf, int row, int level,
                                        unsigned long long n, const uint4& w1,
-                                       Tally& tl) {
+                                       unsigned& clamped) {
   float xu = unit<float>(w1.y), xb = unit<float>(w1.z);
   float rho = cell_rho<kS>(g, row, s);
   float u;
@@ -762,7 +912,7 @@ __device__ __forceinline__ void reemit(Pkg<R>& k, const DevGrid& g, const DevTab
   int i;
   if (u >= __ldg(&S[nI])) {
     i = nI - 1;
-    ++tl.clamped;
+    ++clamped;
   } else {
     // interval i with S[i] <= u < S[i+1]: start from the guide, finish by scanning
     float kf = (__logf(fmaxf(u, 1e-30f)) - t.u_ln0[s]) * t.u_inv[s];
@@ -830,6 +980,25 @@ __device__ __forceinline__ void flush_tally(Tally& tl, unsigned long long* c) {
   tl = Tally{};
 }
 
+__device__ __forceinline__ void flush_warp(LaneTally& tl, unsigned* wt, unsigned long long* c) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long cr = tl.crossings, lv = tl.levels;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    cr += __shfl_xor_sync(kFull, cr, o);
+    lv += __shfl_xor_sync(kFull, lv, o);
+  }
+  __syncwarp();
+  if (lane < kNumCounters) {
+    const unsigned long long x =
+        lane == kCCrossings ? cr : (lane == kCLevels ? lv : (unsigned long long)wt[lane]);
+    if (x) atomicAdd(&c[lane], x);
+    wt[lane] = 0;
+  }
+  __syncwarp();
+  tl = LaneTally{};
+}
+
 // ---------------------------------------------------------------- peel-off
 // Sight line from the point x (base-cube units) toward the observer at bin `bin`:
 // the pixel x projects to and the attenuation exp(-tau) to the boundary. Returns
@@ -859,9 +1028,7 @@ __device__ __forceinline__ bool sight_line(const DevGrid& g, const Kappa* kap,
   Cell c;
   unsigned lv = 0;
   float tau = 0.f;
-  int I0[3], lev0;
-  const int rc = locate<float>(g, k.p, k.d, c.leaf, lev0, I0);
-  if (rc == 0) set_corner(c, I0, lev0);
+  const int rc = enter(k, g, c, lv);
   if (rc < 0) {
     atomicOr(status, kStatusTree);
     return false;
@@ -870,7 +1037,7 @@ __device__ __forceinline__ bool sight_line(const DevGrid& g, const Kappa* kap,
     // a straight line crosses at most 3 n 2^L finest cells of the n^3 base grid
     const long long cap = 3ll * ((long long)g.n_base << g.max_level) + 8;
     for (long long i = 0;; ++i) {
-      const int a = advance_linked<true>(k, c, g, kap, lv, nullptr, &tau);
+      const int a = advance_linked<true>(k, c, g, kap, nullptr, lv, &tau);
       ++crossings;
       if (a == kEscaped) break;
       if (a == kError || i >= cap) {
@@ -977,7 +1144,7 @@ __global__ void __launch_bounds__(256) k_transport_plain(DevGrid g, DevTables t,
         ++tl.escaped;
         int db = dir_bin((float)k.d[2], g.n_dir);
         atomicAdd(&r.sed[(size_t)db * g.B + k.bin], 1ull);
-        if (!k.touched) atomicAdd(&r.sed[(size_t)(g.n_dir + db) * g.B + k.bin], 1ull);
+        if (k.event == 0) atomicAdd(&r.sed[(size_t)(g.n_dir + db) * g.B + k.bin], 1ull);
         break;
       }
       if (a == kError) {
@@ -993,7 +1160,7 @@ __global__ void __launch_bounds__(256) k_transport_plain(DevGrid g, DevTables t,
       if (t.pah_of[s] >= 0)
         pah_absorb<R>(k, g, t, r, t.pah_of[s], leaf, w1);
       else
-        reemit<R>(k, g, t, r, s, leaf, leaf, level, n, w1, tl);
+        reemit<R>(k, g, t, r, s, leaf, leaf, level, n, w1, tl.clamped);
       ++tl.absorptions;
     }
   }
@@ -1048,22 +1215,28 @@ struct ModelIds {
 // one atomic. `sed` is the escaped-spectrum histogram (shared or global memory).
 // kPeel: scatterings and re-emissions at image bins are recorded (position, w,
 // bin) in the peel-off event buffer, one slot range per warp and phase; point-source
-// emissions are counted per bin in s_nemit. Returns false when the time budget ran out.
-template <bool kPeel, class Ids, int kS = 0, bool kPath = false>
+// emissions are counted per bin in s_nemit. wt: the warp's counters (shared memory, zero
+// at the start; lane 0 or atomics). Returns false when the time budget ran out.
+template <bool kPeel, class Ids, int kS = 0, bool kPath = false, bool kTally = false>
 __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, const DevRun& r,
                                           const Kappa* kap, const float* star_cdf,
                                           unsigned long long* sed, unsigned long long n_end,
-                                          Ids& ids, Tally& tl, unsigned long long t0,
-                                          const DevPeel* pe = nullptr,
+                                          Ids& ids, LaneTally& tl, unsigned* wt,
+                                          unsigned long long t0, const DevPeel* pe = nullptr,
                                           unsigned long long* s_nemit = nullptr,
-                                          const float* kext = nullptr) {
+                                          const float* kext = nullptr,
+                                          const float* kabs = nullptr) {
   const int B = g.B;
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   Pkg<float> k;
   k.id = 0;
+  k.dirs = 0;
   bool alive = false;
   bool pending = false;  // reached an interaction point, waiting for the batch
+  // a lane that left the domain is put into the spectrum at the next refill, with the
+  // others: until then it is dead with tau = -1
+  k.tau = 0.f;
   // kPath: the path walk (densities from the density array, kI = -kS for the
   // interaction); otherwise the linked walk
   using CellT = typename std::conditional<kPath, PathCell, Cell>::type;
@@ -1074,15 +1247,22 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
   const int batch = r.interaction_batch > 0 ? r.interaction_batch : 8;
 
   for (;;) {
+    if (k.tau < 0.f) {
+      k.tau = 0.f;
+      const int db = dir_bin(true_component(k, k.d[2], 2), g.n_dir);
+      atomicAdd(&sed[db * B + k.bin], 1ull);
+      if (k.event == 0) atomicAdd(&sed[(g.n_dir + db) * B + k.bin], 1ull);
+    }
     unsigned dead = __ballot_sync(kFull, !alive);
     if (dead) {
       const int nd = __popc(dead);
       const unsigned long long j =
           ids.take(nd, __popc(dead & lt_mask), lane, __ffs(dead) - 1);
+      const unsigned fresh = __ballot_sync(kFull, !alive && j < n_end);
+      if (lane == 0) wt[kCEmitted] += __popc(fresh);
       if (!alive) {
         if (j < n_end) {
           emit<float>(k, r.first_id + j, r, star_cdf, B);
-          ++tl.emitted;
           if constexpr (kPeel) {
             if (r.source_kind != 1) atomicAdd(&s_nemit[k.bin], 1ull);
           }
@@ -1093,21 +1273,23 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
             rc = enter(k, g, cell, tl.levels);
           if (rc == 0) {
             alive = true;
+            if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kap, kext);
           } else if (rc == 1) {  // source outside the grid, moving away
-            ++tl.escaped;
+            atomicAdd(&wt[kCEscaped], 1u);
             const int db = dir_bin(k.d[2], g.n_dir);
             atomicAdd(&sed[db * B + k.bin], 1ull);
             atomicAdd(&sed[(g.n_dir + db) * B + k.bin], 1ull);
           } else {
-            ++tl.errors;
+            atomicAdd(&wt[kCErrors], 1u);
             atomicOr(r.status, kStatusTree);
           }
         }
       }
     }
     if (!__any_sync(kFull, alive)) return true;
-    if (__any_sync(kFull, tl.crossings >= kTallyFlushAt || tl.levels >= kTallyFlushAt))
-      flush_tally(tl, r.counters);
+    if (__any_sync(kFull, tl.crossings >= kTallyFlushAt || tl.levels >= kTallyFlushAt ||
+                              wt[lane & (kTallyWords - 1)] >= kTallyFlushAt))
+      flush_warp(tl, wt, r.counters);
     bool stop = false;
     if (lane == 0) stop = global_ns() - t0 > r.budget_ns;
     stop = __shfl_sync(kFull, stop, 0);
@@ -1118,29 +1300,26 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
     for (int step = 0; step < K; ++step) {
       // walk phase: lanes not waiting for an interaction cross one cell
       if (alive && !pending) {
-        // the two-species form and the path walk run without the path-length tally
-        // (launched only then)
         int a;
         if constexpr (kPath)
           a = advance_path<kS>(k, cell, g, kap, kext, tl.levels);
         else
-          a = advance_linked<false, kS>(k, cell, g, kap, tl.levels,
-                                        kS > 0 ? nullptr : r.pathabs);
+          a = advance_linked<false, kS, kTally>(k, cell, g, kap, kext, tl.levels, nullptr,
+                                                r.pathabs, kabs);
         if (a == kCrossed) {
           ++tl.crossings;
         } else if (a == kEscaped) {
           ++tl.crossings;  // the boundary face it left through
-          ++tl.escaped;
-          int db = dir_bin(k.d[2], g.n_dir);
-          atomicAdd(&sed[db * B + k.bin], 1ull);
-          if (!k.touched) atomicAdd(&sed[(g.n_dir + db) * B + k.bin], 1ull);
+          atomicAdd(&wt[kCEscaped], 1u);
+          k.tau = -1.f;
           alive = false;
         } else if (a == kError) {
-          ++tl.errors;
+          atomicAdd(&wt[kCErrors], 1u);
+          k.tau = 0.f;
           atomicOr(r.status, kStatusTree);
           alive = false;
         } else {
-          pending = true;  // at the interaction point inside the cell
+          pending = true;  // the optical depth runs out inside the cell
         }
       }
       // interaction phase, warp-uniform: once `batch` lanes wait, or nobody walks
@@ -1156,8 +1335,13 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
       int leaf = 0, row = 0;  // the cell's leaf id; its density row (leaf or slot)
       if (pending) {
         pending = false;
+        float kx;
+        if constexpr (kPath)
+          kx = cell.kx;
+        else
+          kx = leaf_ext<kS, kTally>(g, cell.leaf, leaf_rho<kS>(g, cell.leaf), k.bin, kap, kext);
+        to_point(k, cell, kx);
         if constexpr (kPath) {
-          cell.kx = -1.f;  // the bin may change: read the row again
           leaf = path_leaf(g, cell.slot);
           row = kI < 0 ? cell.slot : leaf;  // slot rows for 2 or 4 species
         } else {
@@ -1165,17 +1349,19 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
           row = leaf;
         }
         if (++k.event > r.max_events) {
-          ++tl.capped;
+          atomicAdd(&wt[kCCapped], 1u);
           alive = false;
         } else if (leaf < 0) {
-          ++tl.errors;
+          atomicAdd(&wt[kCErrors], 1u);
           atomicOr(r.status, kStatusTree);
           alive = false;
         } else {
+          const unsigned was = mirrored(k);
+          restore_direction(k);
           sp = interact<float, kI>(k, g, kap, row, r, w1, kPeel ? pe->o : nullptr,
                                    kPeel ? &wv : nullptr);
+          orient<kPath>(k, cell, was);
           if (sp < 0) {
-            ++tl.scatters;
             scattered = true;
           } else {
             absorbing = true;
@@ -1183,6 +1369,11 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
         }
       }
       const unsigned am = __ballot_sync(kFull, absorbing);
+      const unsigned sm = __ballot_sync(kFull, scattered);
+      if (lane == 0) {
+        wt[kCAbsorptions] += __popc(am);
+        wt[kCScatters] += __popc(sm);
+      }
       if (absorbing) {
         unsigned long long key = ((unsigned long long)sp << 48) | (unsigned long long)leaf;
         unsigned peers = __match_any_sync(am, key);
@@ -1194,10 +1385,13 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
         old = __shfl_sync(peers, old, leader);
         if (t.pah_of[sp] >= 0)
           pah_absorb<float>(k, g, t, r, t.pah_of[sp], leaf, w1);
-        else
+        else {
+          unsigned clamped = 0;
           reemit<float, kI>(k, g, t, r, sp, leaf, row, cell.level(), old + __popc(peers & lt_mask),
-                            w1, tl);
-        ++tl.absorptions;
+                            w1, clamped);
+          if (clamped) atomicAdd(&wt[kCClamped], 1u);
+        }
+        if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kap, kext);
       }
       if constexpr (kPeel) {
         // the event's share toward the observer, at the bin it leaves with
@@ -1211,48 +1405,63 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
           if (ev) {
             const unsigned long long slot = base + __popc(em & lt_mask);
             if (slot < pe->capacity) {
-              pe->ev[slot] = make_float4(k.p[0], k.p[1], k.p[2], wv);
+              pe->ev[slot] = make_float4(true_component(k, k.p[0], 0), true_component(k, k.p[1], 1),
+                                         true_component(k, k.p[2], 2), wv);
               pe->ev_bin[slot] = k.bin;
             }
-            ++tl.peel_events;
           }
+          if (lane == leader) wt[kCPeelEvents] += __popc(em);
         }
       }
     }
   }
 }
 
-// Shared-memory words (floats) of the path walk's per-bin extinction vectors: B x kS
-// for 2 or 4 species, rounded up to 16 bytes; none otherwise.
-template <int kS, bool kPath>
+// Shared-memory words (floats) of the per-bin extinction vectors: B x kS for the walks
+// compiled for 2 or 4 species, rounded up to 16 bytes; none otherwise.
+template <int kS>
 __host__ __device__ constexpr int kext_words(int B) {
-  return (kPath && (kS == 2 || kS == 4)) ? (B * kS + 3) / 4 * 4 : 0;
+  return kS == 2 || kS == 4 ? (B * kS + 3) / 4 * 4 : 0;
+}
+
+// Opacity records staged in shared memory: those of the generic walks, which read them at
+// every crossing. The walks compiled for 2 or 4 species need only the extinction vectors
+// there and take the records, read once per interaction, from L1.
+template <int kS>
+__host__ __device__ __forceinline__ int kap_records(const DevGrid& g) {
+  return kS > 2 ? 0 : g.B * g.S;
 }
 
 // ---------------------------------------------------------------- pool kernel
 // Persistent packet pool over one model: all warps draw package indices from one
 // global counter; the opacity table, the stellar CDF and (when it fits) the
 // escaped-spectrum histogram live in shared memory.
-template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false>
+template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false, bool kTally = false>
 __global__ void __launch_bounds__(256, kMinBlocks)
     k_transport_pool(DevGrid g, DevTables t, DevRun r, const __grid_constant__ DevPeel pe) {
   extern __shared__ unsigned long long smem_u64[];
   const int S = g.S, B = g.B;
   const int n_sed = 2 * g.n_dir * B;
   const bool sed_local = r.sed_in_smem != 0;
-  // the path walk with 2 or 4 species: the extinction opacities [B][S] first, one
-  // vector per bin (a multiple of 16 bytes)
+  // 2 or 4 species: the extinction opacities [B][S] first (with the path-length tally the
+  // absorption opacities after them), one vector per bin (a multiple of 16 bytes)
   float* s_kext = reinterpret_cast<float*>(smem_u64);
-  const int n_kext = kext_words<kS, kPath>(B);
-  unsigned long long* s_u64 = smem_u64 + n_kext / 2;
+  const int n_kext = kext_words<kS>(B);
+  float* s_kabs = s_kext + n_kext;
+  unsigned long long* s_u64 = smem_u64 + (kTally ? 2 : 1) * n_kext / 2;
   unsigned long long* s_sed = sed_local ? s_u64 : r.sed;   // [2][n_dir][B]
   Kappa* s_kap = reinterpret_cast<Kappa*>(s_u64 + (sed_local ? n_sed : 0));  // [B][S]
-  float* s_cdf = reinterpret_cast<float*>(s_kap + B * S);     // [B]
+  const int n_kap = kap_records<kS>(g);
+  float* s_cdf = reinterpret_cast<float*>(s_kap + n_kap);     // [B]
   if (sed_local)
     for (int i = threadIdx.x; i < n_sed; i += blockDim.x) s_sed[i] = 0ull;
-  for (int i = threadIdx.x; i < B * S; i += blockDim.x) s_kap[i] = t.kap[i];
+  if (n_kap)
+    for (int i = threadIdx.x; i < n_kap; i += blockDim.x) s_kap[i] = t.kap[i];
   if (n_kext)
-    for (int i = threadIdx.x; i < B * S; i += blockDim.x) s_kext[i] = t.kap[i].kext;
+    for (int i = threadIdx.x; i < B * S; i += blockDim.x) {
+      s_kext[i] = t.kext[i];
+      if (kTally) s_kabs[i] = t.kap[i].kabs;
+    }
   for (int i = threadIdx.x; i < B; i += blockDim.x) s_cdf[i] = t.star_cdf[i];
   // peel-off: the block's point-source emission counts per bin
   unsigned long long* s_nemit = nullptr;
@@ -1261,12 +1470,16 @@ __global__ void __launch_bounds__(256, kMinBlocks)
     s_nemit = reinterpret_cast<unsigned long long*>(a);
     for (int i = threadIdx.x; i < B; i += blockDim.x) s_nemit[i] = 0ull;
   }
+  __shared__ unsigned s_tally[8 * kTallyWords];
+  for (int i = threadIdx.x; i < 8 * kTallyWords; i += blockDim.x) s_tally[i] = 0u;
   __syncthreads();
-  Tally tl = {};
+  unsigned* wt = s_tally + (threadIdx.x >> 5) * kTallyWords;
+  LaneTally tl = {};
   GlobalIds ids{r.next};
-  pool_warp<kPeel, GlobalIds, kS, kPath>(g, t, r, s_kap, s_cdf, s_sed, r.n_packages, ids, tl,
-                                         global_ns(), &pe, s_nemit, s_kext);
-  flush_tally(tl, r.counters);
+  pool_warp<kPeel, GlobalIds, kS, kPath, kTally>(g, t, r, kS > 2 ? t.kap : s_kap, s_cdf, s_sed,
+                                                 r.n_packages, ids, tl, wt, global_ns(), &pe,
+                                                 s_nemit, s_kext, s_kabs);
+  flush_warp(tl, wt, r.counters);
   if (sed_local || kPeel) __syncthreads();
   if (sed_local) {
     for (int i = threadIdx.x; i < n_sed; i += blockDim.x)
@@ -1331,11 +1544,14 @@ __device__ __forceinline__ int pick_model(const ModelDesc* models, int n,
 
 // Two species: held to 64 registers (56 bytes of spills) for four blocks per SM, 8.0 ms
 // against 8.7 with the three blocks of 74 registers; the generic form would spill 180.
-template <int kS>
+template <int kS, bool kTally>
 __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const ModelDesc* models, int n_models,
                                                          unsigned long long* next, int chunk) {
   __shared__ ModelDesc sdesc[8];
+  __shared__ unsigned s_tally[8 * kTallyWords];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned* wt = s_tally + warp * kTallyWords;
+  if (lane < kTallyWords) wt[lane] = 0u;
   const unsigned per_block = blockDim.x >> 5;
   const unsigned long long t0 = global_ns();
   for (unsigned pick = 0;; ++pick) {
@@ -1347,12 +1563,13 @@ __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const 
     for (int i = lane; i < (int)(sizeof(ModelDesc) / sizeof(int)); i += 32) dst[i] = src[i];
     __syncwarp();
     const ModelDesc& md = sdesc[warp];
-    Tally tl = {};
+    LaneTally tl = {};
     ModelIds ids{next + m, 0ull, md.r.n_packages, 0, chunk};
     const bool in_time =
-        pool_warp<false, ModelIds, kS>(md.g, md.t, md.r, md.t.kap, md.t.star_cdf, md.r.sed,
-                                        md.r.n_packages, ids, tl, t0);
-    flush_tally(tl, md.r.counters);
+        pool_warp<false, ModelIds, kS, false, kTally>(md.g, md.t, md.r, md.t.kap, md.t.star_cdf, md.r.sed,
+                                        md.r.n_packages, ids, tl, wt, t0, nullptr, nullptr,
+                                        md.t.kext);
+    flush_warp(tl, wt, md.r.counters);
     __syncwarp();
     if (!in_time) break;
   }
@@ -1396,7 +1613,9 @@ __global__ void k_trace(DevGrid g, DevTables t, DevRun r, const unsigned long lo
   const unsigned long long t0 = global_ns();
   unsigned steps = 0;
   Cell c{0, {0.f, 0.f, 0.f}, 1.f};
+  k.dirs = 0;
   int rc = enter(k, g, c, tl.levels);
+  auto at = [&](int a) { return true_component(k, k.p[a], a); };
   if (rc == 1) rec[4] = 1;
   if (rc < 0) atomicOr(r.status, kStatusTree);
   while (rc == 0) {
@@ -1405,24 +1624,29 @@ __global__ void k_trace(DevGrid g, DevTables t, DevRun r, const unsigned long lo
       break;
     }
     const int lf = c.leaf;
-    const int a = advance_linked(k, c, g, t.kap, tl.levels, nullptr);
+    const int a = advance_linked(k, c, g, t.kap, nullptr, tl.levels);
     rec[8] = lf;
     if (a == kCrossed) { ++rec[3]; continue; }
     if (a == kEscaped) {
       ++rec[3];
       rec[4] = 1;
-      trace_event(my_ev, ev_cap, n_ev, 3, -1, lf, k.bin, k.p);
+      const float pe[3] = {at(0), at(1), at(2)};
+      trace_event(my_ev, ev_cap, n_ev, 3, -1, lf, k.bin, pe);
       break;
     }
     if (a == kError) { atomicOr(r.status, kStatusTree); break; }
+    to_point(k, c, leaf_ext<0>(g, c.leaf, float4{}, k.bin, t.kap, nullptr));
+    const float pi[3] = {at(0), at(1), at(2)};
     if (++k.event > r.max_events) {
       rec[5] = 1;
-      trace_event(my_ev, ev_cap, n_ev, 4, -1, c.leaf, k.bin, k.p);
+      trace_event(my_ev, ev_cap, n_ev, 4, -1, c.leaf, k.bin, pi);
       break;
     }
     uint4 w1;
-    const float pi[3] = {k.p[0], k.p[1], k.p[2]};
+    const unsigned was = mirrored(k);
+    restore_direction(k);
     int s = interact<float>(k, g, t.kap, c.leaf, r, w1);
+    orient<false>(k, c, was);
     if (s < 0) {
       ++rec[2];
       trace_event(my_ev, ev_cap, n_ev, 1, -1, c.leaf, k.bin, pi);
@@ -1431,7 +1655,7 @@ __global__ void k_trace(DevGrid g, DevTables t, DevRun r, const unsigned long lo
     if (t.pah_of[s] >= 0) {
       pah_bin(k, g, t, t.pah_of[s], c.leaf, w1);  // replay does not tally
     } else {
-      reemit<float>(k, g, t, r, s, c.leaf, c.leaf, c.level(), 0ull, w1, tl);
+      reemit<float>(k, g, t, r, s, c.leaf, c.leaf, c.level(), 0ull, w1, tl.clamped);
     }
     trace_event(my_ev, ev_cap, n_ev, 2, s, c.leaf, k.bin, pi);
     ++rec[1];
@@ -1439,7 +1663,7 @@ __global__ void k_trace(DevGrid g, DevTables t, DevRun r, const unsigned long lo
   if (ev_n) ev_n[i] = n_ev;
   rec[0] = k.event;
   rec[6] = k.bin;
-  rec[7] = dir_bin(k.d[2], g.n_dir);
+  rec[7] = dir_bin(true_component(k, k.d[2], 2), g.n_dir);
   for (int j = 0; j < 9; ++j) out[i * 9 + j] = rec[j];
 }
 
@@ -1483,7 +1707,7 @@ __global__ void k_build_links(DevGrid g, const int32_t* ijk, int32_t* links) {
       const int oct = ((J[0] >> sh) & 1) | (((J[1] >> sh) & 1) << 1) | (((J[2] >> sh) & 1) << 2);
       node = g.child[blk * 8 + oct];
     }
-    link = node >= 0 ? (node | (l << 28)) : node;
+    link = node >= 0 ? (node | ((lev - l) << 28)) : node;
   }
   int32_t* rec = links + leaf * kRec;
   rec[f] = link;
@@ -1508,8 +1732,10 @@ __global__ void k_philox(const unsigned long long* ids, long long n, unsigned ev
 
 constexpr size_t kSmemBudget = 200 * 1024;
 
+template <int kS, bool kTally>
 static size_t table_smem(const DevGrid& g) {
-  return sizeof(Kappa) * g.B * g.S + sizeof(float) * g.B;
+  return sizeof(Kappa) * kap_records<kS>(g) +
+         sizeof(float) * ((kTally ? 2 : 1) * kext_words<kS>(g.B) + g.B);
 }
 
 static size_t sed_smem(const DevGrid& g) {
@@ -1518,50 +1744,72 @@ static size_t sed_smem(const DevGrid& g) {
 
 static size_t peel_smem(const DevGrid& g) { return 16 + sizeof(unsigned long long) * g.B; }
 
-template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false>
+template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false, bool kTally = false>
 static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, const DevRun& r,
                                        const DevPeel& pe, int blocks_per_sm, int threads,
                                        int sms, cudaStream_t s) {
   DevRun rr = r;
-  const size_t extra = (kPeel ? peel_smem(g) : 0) + sizeof(float) * kext_words<kS, kPath>(g.B);
-  rr.sed_in_smem = table_smem(g) + extra + sed_smem(g) <= kSmemBudget ? 1 : 0;
-  size_t sm = table_smem(g) + extra + (rr.sed_in_smem ? sed_smem(g) : 0);
+  const size_t tables = table_smem<kS, kTally>(g) + (kPeel ? peel_smem(g) : 0);
+  rr.sed_in_smem = tables + sed_smem(g) <= kSmemBudget ? 1 : 0;
+  size_t sm = tables + (rr.sed_in_smem ? sed_smem(g) : 0);
   cudaError_t e;
+  const auto kernel = k_transport_pool<kMinBlocks, kPeel, kS, kPath, kTally>;
   if (sm > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_transport_pool<kMinBlocks, kPeel, kS, kPath>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ,
-                                                    k_transport_pool<kMinBlocks, kPeel, kS, kPath>,
-                                                    threads, sm);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, sm);
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   int bps = blocks_per_sm > 0 ? (blocks_per_sm < occ ? blocks_per_sm : occ) : occ;
-  k_transport_pool<kMinBlocks, kPeel, kS, kPath><<<sms * bps, threads, sm, s>>>(g, t, rr, pe);
+  kernel<<<sms * bps, threads, sm, s>>>(g, t, rr, pe);
   return cudaGetLastError();
 }
 
 // blocks_per_sm selects the register budget: 5 or 6 resident blocks of 256 threads
-// use variants compiled for that occupancy (fewer registers, more spills); other
-// values use the 4-block variants, capped at their occupancy: the two-species one
-// (no spills; used when the path-length tally is off) or the generic one (8 bytes
-// of spills). With peel-off images the 4-block variants are used.
+// use variants compiled for that occupancy (fewer registers, some spills); other
+// values use the 4-block variants, capped at their occupancy: the walks compiled for two
+// or four species or the generic one. With peel-off images or the path-length tally the
+// 4-block variants are used.
+//
+// Left to itself (0) the linked walk of two or four species takes five blocks per SM where
+// its records fit L2 and the launch has at least eight packages for every lane: more
+// warps hide the records' L2 latency, but spread fewer packages thinner over the lanes and,
+// once the records come from DRAM, widen the set of rows in use. Disk of 2.4e6 cells
+// (78 MB of records), four against five blocks: 5e6 packages 4.17 and 3.82 ms, 1.6e6 1.57
+// and 1.49, 8e5 0.95 and 0.95, 4e5 0.67 and 0.69, 1e5 0.40 and 0.43; disk of 1.9e7 cells
+// (0.6 GB), 1e7 packages: 22.9 and 27.5 ms.
 cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const DevRun& r,
                                   int blocks_per_sm, int threads, cudaStream_t s,
                                   const DevPeel* peel, bool path) {
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, l2 = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  if (peel && g.S == 2 && !r.pathabs)
+  e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+  if (e != cudaSuccess) return e;
+  if (peel && r.pathabs)
+    return launch_pool_variant<4, true, 0, false, true>(g, t, r, *peel, blocks_per_sm, threads,
+                                                        sms, s);
+  if (peel && g.S == 2)
     return launch_pool_variant<4, true, 2>(g, t, r, *peel, blocks_per_sm, threads, sms, s);
   if (peel) return launch_pool_variant<4, true>(g, t, r, *peel, blocks_per_sm, threads, sms, s);
   const DevPeel none{};
+  // the path-length tally: the linked walk, at four blocks per SM
+  if (r.pathabs) {
+    if (g.S == 2)
+      return launch_pool_variant<4, false, 2, false, true>(g, t, r, none, blocks_per_sm, threads,
+                                                           sms, s);
+    if (g.S == 4)
+      return launch_pool_variant<4, false, 4, false, true>(g, t, r, none, blocks_per_sm, threads,
+                                                           sms, s);
+    return launch_pool_variant<4, false, 0, false, true>(g, t, r, none, blocks_per_sm, threads,
+                                                         sms, s);
+  }
   // the path walk (no face links; grids of at most kPathLevels levels)
-  if (path && !r.pathabs && g.max_level <= kPathLevels) {
+  if (path && g.max_level <= kPathLevels) {
     if (g.S == 4)
       return launch_pool_variant<4, false, 4, true>(g, t, r, none, blocks_per_sm, threads, sms, s);
     if (g.S == 2)
@@ -1570,12 +1818,22 @@ cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const De
   }
   if (threads == 256 && blocks_per_sm == 6)
     return launch_pool_variant<6, false>(g, t, r, none, blocks_per_sm, threads, sms, s);
+  const bool in_l2 = (double)g.n_leaves * sizeof(int32_t) * kRec <= (double)l2;
+  const bool five =
+      threads == 256 && (blocks_per_sm == 5 || (blocks_per_sm == 0 && in_l2 &&
+                                                 r.n_packages >= 8ull * 5 * 256 * sms));
+  if (g.S == 2) {
+    if (five)
+      return launch_pool_variant<5, false, 2>(g, t, r, none, blocks_per_sm, threads, sms, s);
+    return launch_pool_variant<4, false, 2>(g, t, r, none, blocks_per_sm, threads, sms, s);
+  }
+  if (g.S == 4) {
+    if (five)
+      return launch_pool_variant<5, false, 4>(g, t, r, none, blocks_per_sm, threads, sms, s);
+    return launch_pool_variant<4, false, 4>(g, t, r, none, blocks_per_sm, threads, sms, s);
+  }
   if (threads == 256 && blocks_per_sm == 5)
     return launch_pool_variant<5, false>(g, t, r, none, blocks_per_sm, threads, sms, s);
-  // two species: a walk compiled for the densities in the face-link record (a
-  // variant for four species reading them as one 16-byte load measured 4 % slower)
-  if (g.S == 2 && !r.pathabs)
-    return launch_pool_variant<4, false, 2>(g, t, r, none, blocks_per_sm, threads, sms, s);
   return launch_pool_variant<4, false>(g, t, r, none, blocks_per_sm, threads, sms, s);
 }
 
@@ -1625,7 +1883,7 @@ cudaError_t launch_transport_plain(const DevGrid& g, const DevTables& t, const D
   return cudaGetLastError();
 }
 
-template <int kS>
+template <int kS, bool kTally>
 static cudaError_t launch_batch_variant(const ModelDesc* models, int n_models,
                                         unsigned long long* next, int chunk, int blocks_per_sm,
                                         int threads, cudaStream_t s) {
@@ -1635,22 +1893,25 @@ static cudaError_t launch_batch_variant(const ModelDesc* models, int n_models,
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_transport_batch<kS>, threads, 0);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_transport_batch<kS, kTally>, threads, 0);
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   int bps = blocks_per_sm > 0 && blocks_per_sm < occ ? blocks_per_sm : occ;
-  k_transport_batch<kS><<<sms * bps, threads, 0, s>>>(models, n_models, next, chunk);
+  k_transport_batch<kS, kTally><<<sms * bps, threads, 0, s>>>(models, n_models, next, chunk);
   return cudaGetLastError();
 }
 
 cudaError_t launch_transport_batch(const ModelDesc* models, int n_models,
                                    unsigned long long* next, int chunk, int blocks_per_sm,
-                                   int s_fixed, int threads, cudaStream_t s) {
+                                   int s_fixed, bool tally, int threads, cudaStream_t s) {
   if (threads <= 0) threads = 256;
   if (threads % 32 != 0 || threads > 256) return cudaErrorInvalidValue;
+  if (tally)
+    return launch_batch_variant<0, true>(models, n_models, next, chunk, blocks_per_sm, threads, s);
   if (s_fixed == 2)
-    return launch_batch_variant<2>(models, n_models, next, chunk, blocks_per_sm, threads, s);
-  return launch_batch_variant<0>(models, n_models, next, chunk, blocks_per_sm, threads, s);
+    return launch_batch_variant<2, false>(models, n_models, next, chunk, blocks_per_sm, threads,
+                                          s);
+  return launch_batch_variant<0, false>(models, n_models, next, chunk, blocks_per_sm, threads, s);
 }
 
 cudaError_t launch_trace(const DevGrid& g, const DevTables& t, const DevRun& r,
