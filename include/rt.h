@@ -465,7 +465,7 @@ rt_status rt_mlp_set_params(rt_mlp *m, const float *in);  /* host [n_params] */
  * the whole network runs per 128-row tile in one kernel on the 5th-generation tensor
  * cores (tcgen05.mma, FP32 accumulators in tensor memory, BF16 operands in shared
  * memory; an output layer wider than 256 in chunks of 256 columns); otherwise layer
- * by layer (one tcgen05 GEMM of 128 x 128 output tiles per layer, as in training). */
+ * by layer (one tcgen05 kernel per layer, as in training). */
 rt_status rt_mlp_forward(rt_mlp *m, const float *x, float *y, int64_t M, void *stream);
 
 /* Loss and gradients of a batch (device x [M][n_in], targets t [M][n_out]) into the

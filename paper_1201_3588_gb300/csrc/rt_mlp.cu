@@ -1,8 +1,8 @@
 // rt_mlp.cu -- the multilayer perceptron of the PAH emission surrogate: forward
 // pass, mean-squared-error gradients and Adam, on the 5th-generation tensor cores
 // (tcgen05.mma, FP32 accumulators in tensor memory) in BF16 with FP32 accumulation.
-// Inference runs the whole network per 128-row tile in one kernel; training runs
-// layer by layer, each GEMM on 128 x 128 output tiles.
+// Inference runs the whole network per 128-row tile in one kernel; training runs a
+// kernel per layer and direction, the element-wise work in the GEMMs' epilogues.
 //
 // Network: a_0 = x; z_l = a_{l-1} W_l^T + b_l; a_l = silu(z_l) for the hidden layers,
 // linear output. Loss = mean over rows and outputs of (y - t)^2. Master weights,
@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -26,7 +27,6 @@ typedef __nv_bfloat16 bf16;
 
 namespace {
 
-constexpr int kTile = 64;     // rows are padded to a multiple of this
 constexpr int kMaxLayers = 8;
 
 inline int pad16(int x) { return (x + 15) / 16 * 16; }
@@ -57,29 +57,17 @@ struct rt_mlp {
   float* d_loss = nullptr;
   long long step = 0;
   float x_lo = -1e30f, x_hi = 1e30f;  // admissible range of the second-to-last input
-  // activations for up to cap rows (padded to 64)
+  // activations for up to cap rows
   long long cap = 0;
-  bf16* d_a[kMaxLayers + 1] = {};   // a_l in BF16 [cap][dim_p]
-  float* d_z[kMaxLayers] = {};      // z_l in FP32 [cap][out_p]
-  float* d_dz = nullptr;            // FP32 scratch [cap][max_p]
-  bf16* d_dzb = nullptr;            // BF16 of dz
+  bf16* d_a[kMaxLayers] = {};   // the layers' inputs in BF16 [cap][in_p]
+  float* d_z[kMaxLayers] = {};  // z_l of the hidden layers in FP32 [cap][out_p]
+  bf16* d_dz[2] = {};           // dz of a layer and of the one below [cap][max_p]
   int max_p = 0;
 };
 
 namespace {
 
 // ---------------------------------------------------------------- kernels
-// x [M][n_in] FP32 -> a0 [Mp][in_p] BF16, zero padding
-__global__ void k_pack_input(const float* x, long long M, int n_in, long long Mp, int in_p,
-                             bf16* a0) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= Mp * in_p) return;
-  long long r = idx / in_p;
-  int c = (int)(idx % in_p);
-  float v = (r < M && c < n_in) ? x[r * n_in + c] : 0.0f;
-  a0[idx] = __float2bfloat16(v);
-}
-
 // logistic sigmoid as 1/2 + tanh(z/2)/2, with the hardware tanh approximation
 // (relative error about 2^-11, below the BF16 rounding of the activations); both the
 // layer-by-layer path and the fused forward use it, so their activations agree
@@ -96,99 +84,34 @@ __device__ __forceinline__ float silu_fast(float z) {
   return fmaf(h, t, h);
 }
 
-// z += b; a = silu(z) (hidden) or copy (output); padded columns forced to zero
-__global__ void k_bias_act(float* z, const float* b, long long Mp, int out_p, int n_out,
-                           int hidden, bf16* a) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= Mp * out_p) return;
-  int c = (int)(idx % out_p);
-  float v = c < n_out ? z[idx] + b[c] : 0.0f;
-  z[idx] = v;
-  if (a) {
-    float y = hidden ? silu_fast(v) : v;
-    a[idx] = __float2bfloat16(y);
-  }
-}
-
-// dz = 2 (y - t) / (M n_out) on valid rows/columns; loss accumulated
-__global__ void k_mse_grad(const float* y, const float* t, long long M, int n_out, long long Mp,
-                           int out_p, float* dz, bf16* dzb, float* loss) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  float l = 0.0f;
-  if (idx < Mp * out_p) {
-    long long r = idx / out_p;
-    int c = (int)(idx % out_p);
-    float d = 0.0f;
-    if (r < M && c < n_out) {
-      float e = y[idx] - t[r * n_out + c];
-      l = e * e;
-      d = 2.0f * e / ((float)M * (float)n_out);
-    }
-    dz[idx] = d;
-    dzb[idx] = __float2bfloat16(d);
-  }
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-  if ((threadIdx.x & 31) == 0 && l != 0.0f) atomicAdd(loss, l / ((float)M * (float)n_out));
-}
-
-// dz = da * silu'(z) (da in dz, in place) and its BF16 copy
-__global__ void k_act_back(float* dz, const float* z, long long Mp, int p, int n_valid, bf16* dzb) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= Mp * p) return;
-  int c = (int)(idx % p);
-  float v = 0.0f;
-  if (c < n_valid) {
-    float zz = z[idx];
-    float s = sigmoid_fast(zz);
-    v = dz[idx] * s * (1.0f + zz * (1.0f - s));
-  }
-  dz[idx] = v;
-  dzb[idx] = __float2bfloat16(v);
-}
-
-// db[c] += sum over rows of dz[r][c]
-__global__ void k_col_sums(const float* dz, long long Mp, int p, float* db) {
-  int c = blockIdx.x * 32 + (threadIdx.x & 31);
-  int r0 = threadIdx.x >> 5;
-  float s = 0.0f;
-  if (c < p)
-    for (long long r = r0 + (long long)blockIdx.y * 8; r < Mp; r += 8ll * gridDim.y) s += dz[r * p + c];
-  __shared__ float red[8][32];
-  red[r0][threadIdx.x & 31] = s;
-  __syncthreads();
-  if (r0 == 0 && c < p) {
-    float t = 0.0f;
-    for (int i = 0; i < 8; ++i) t += red[i][threadIdx.x & 31];
-    atomicAdd(&db[c], t);
-  }
-}
-
 __global__ void k_to_bf16(const float* p, bf16* q, size_t n) {
   size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i < n) q[i] = __float2bfloat16(p[i]);
 }
 
-__global__ void k_adam(float* p, const float* g, float* m, float* v, size_t n, float lr,
-                       float b1, float b2, float c1, float c2, float eps) {
-  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float gi = g[i];
-  float mi = b1 * m[i] + (1.0f - b1) * gi;
-  float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+// Adam, and the BF16 copy of the new weights. Four parameters a thread (the padded
+// count is a multiple of 16).
+__global__ void k_adam(float4* p, const float4* g, float4* m, float4* v, uint2* q, size_t n4,
+                       float lr, float b1, float b2, float c1, float c2, float eps) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= n4) return;
+  float4 pi = p[i], mi = m[i], vi = v[i];
+  const float4 gi = g[i];
+  auto step = [&](float& p1, float g1, float& m1, float& v1) {
+    m1 = b1 * m1 + (1.0f - b1) * g1;
+    v1 = b2 * v1 + (1.0f - b2) * g1 * g1;
+    p1 -= lr * (m1 / c1) / (sqrtf(v1 / c2) + eps);
+  };
+  step(pi.x, gi.x, mi.x, vi.x);
+  step(pi.y, gi.y, mi.y, vi.y);
+  step(pi.z, gi.z, mi.z, vi.z);
+  step(pi.w, gi.w, mi.w, vi.w);
   m[i] = mi;
   v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  p[i] = pi;
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(pi.x, pi.y), hi = __floats2bfloat162_rn(pi.z, pi.w);
+  q[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
-
-// y [M][n_out] <- z_last [Mp][out_p]
-__global__ void k_unpack_output(const float* z, long long M, int n_out, int out_p, float* y) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= M * n_out) return;
-  long long r = idx / n_out;
-  int c = (int)(idx % n_out);
-  y[idx] = z[r * out_p + c];
-}
-
 
 // ---------------------------------------------------------------- fused forward
 // The whole forward pass of a 128-row tile in one CTA on the 5th-generation tensor
@@ -208,7 +131,9 @@ constexpr int kTcThreads = 1024;  // 32 warps: each reads its lane quarter of th
                                   // accumulators, the column chunks shared by 8 warps
 constexpr int kTcMaxWidth = 256;
 constexpr int kTcMaxOut = 4096;  // output layer: up to 16 chunks of 256 columns
-constexpr unsigned long long kTcWaitNs = 2000000000ull;  // give up a wait after 2 s
+// give up a wait after 4e9 SM clocks: 2 s at full clock (the clock register is read in a
+// few cycles, the global timer only slowly)
+constexpr long long kTcWaitClocks = 4000000000ll;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -240,14 +165,8 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, 
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
-__device__ __forceinline__ unsigned long long tc_now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  const unsigned long long t0 = tc_now_ns();
+  const long long t0 = clock64();
   for (;;) {
     uint32_t done;
     asm volatile(
@@ -256,7 +175,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "=r"(done)
         : "r"(bar), "r"(parity));
     if (done) return true;
-    if (tc_now_ns() - t0 > kTcWaitNs) return false;
+    if (clock64() - t0 > kTcWaitClocks) return false;
   }
 }
 
@@ -291,166 +210,429 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-// ---------------------------------------------------------------- training GEMM
-// C[M][N] (=|+=) A[M][K] . B[K][N] on the 5th-generation tensor cores, for the
-// layer-by-layer passes of training: A row-major (lda) or column-major, B row-major
-// (ldb) or column-major; BF16 operands, FP32 accumulation in tensor memory. A CTA of
-// 4 warps owns a 128 x 128 tile of C. The contraction runs in chunks of 64: all
-// threads pack the chunk's A and B tiles from global memory (any layout) into the
-// K-major core-matrix layout in one of two shared-memory buffers, one thread issues
-// the chunk's four MMAs (K = 16 each) and commits them to that buffer's mbarrier, and
-// the packing of the next chunk overlaps them. gridDim.z splits K into chunks of
-// k_chunk (atomic adds). Every wait is bounded: after 2 s the tile's outputs are left
-// untouched and *err is set.
-constexpr int kGemmRows = 128, kGemmCols = 128, kGemmK = 64, kGemmThreads = 128;
+// ---------------------------------------------------------------- layer kernels
+// Training and the networks too wide for the fused forward run one kernel per layer and
+// direction on the 5th-generation tensor cores (BF16 operands, FP32 accumulators in tensor
+// memory). A minibatch of 1024 rows is a few megabytes in L2 and 0.1 GFLOP a layer, so a
+// step is a chain of short kernels whose launches, first loads and epilogues are all there
+// is: hence few kernels (a layer's bias, activation, loss, activation derivative and bias
+// gradient in the epilogue of its GEMM; the weight gradient of a layer in one launch with
+// the gradient passed down), small tiles (32 or more CTAs for 1024 rows) and all of a
+// tile's loads in flight at once instead of a pipeline. 28 launches with GEMMs that packed
+// column-major operands element by element took 307 us a step of 1024 rows (66 - 3x256 -
+// 200), these ten 90 us (16384 rows: 797 and 295; the 66 - 3x512 - 200 network forward over
+// 262144 rows: 4.3 and 3.1 ms). What bounds a step now is the latency within each kernel,
+// 7 us from its first load to its last store.
+//
+// layer tile: C [128 rows][64 columns] = A [rows][K] . B^T, K in chunks of 256:
+//   forward   A = the layer's input (or the FP32 input rows, converted), B = W
+//   backward  A = dz, B = W transposed while it is packed into shared memory
+// gradient tile: dW [128][128] += dz^T a over a range of rows, both operands transposed
+// while packed, by vector reductions.
+// A row-major operand with the contraction contiguous goes to its place in the core-matrix
+// layout by 16-byte asynchronous copies (8 rows x 64 bytes per warp instruction: whole
+// sectors, no bank conflicts). To transpose, a thread takes 8 columns of two rows and
+// writes 8 pairs; LBO is 144 bytes there so that a warp's 4-byte stores hit 32 banks.
+// Every wait is bounded: after 2 s the tile's outputs are left untouched and *err is set.
+constexpr int kLayRows = 128, kLayCols = 64, kLayK = 256, kLayThreads = 256;
+constexpr int kGradRows = 128;                       // rows of a gradient tile's chunk
+constexpr uint32_t kSbo = (kLayK / 8) * 128;         // packed by copies: LBO 128
+constexpr uint32_t kLboT = 144;                      // packed by transposing
+constexpr uint32_t kSboT = (kLayK / 8) * kLboT;      // K = 256
+constexpr uint32_t kSboG = (kGradRows / 8) * kLboT;  // K = 128
+constexpr uint32_t kLaySmem = (kLayRows / 8) * kSbo + (kLayCols / 8) * kSboT;
 
-template <bool kAcol, bool kBcol>
-__global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const bf16* A, int lda, const bf16* B,
-                                                          int ldb, float* C, int ldc, int M, int N,
-                                                          int K, int k_chunk, int atomic_out,
-                                                          unsigned* err) {
-  extern __shared__ __align__(128) unsigned char gemm_smem[];
-  bf16* sA0 = reinterpret_cast<bf16*>(gemm_smem);          // [2][128 x 64]: 2 x 16 KB
-  bf16* sB0 = sA0 + 2 * kGemmRows * kGemmK;                 // [2][128 x 64]: 2 x 16 KB
-  __shared__ uint64_t bar[2];
-  __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * kGemmRows, n0 = blockIdx.y * kGemmCols;
-  const int k_begin = blockIdx.z * k_chunk;
-  const int k_end = min(K, k_begin + k_chunk);
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     smem_addr(&tmem_slot)),
-                 "r"(kGemmCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+enum Epilogue { kHidden, kLoss, kOutput, kBack };
+
+struct LayerArgs {
+  long long M;            // rows
+  int N, K, n_valid;      // padded columns and contraction; valid columns
+  int n_in;               // columns of x
+  const float* x;         // [M][n_in] (first layer), else null
+  const bf16* a;          // [M][K] input, or dz (backward)
+  const bf16* w;          // forward W [N][K], backward W [K][N]
+  const float* bias;
+  float* z;               // hidden: [M][N] pre-activations (null: not kept); backward: read
+  bf16* out;              // hidden: activations [M][N]; backward and loss: dz [M][N]
+  bf16* a0;               // first layer: the converted input [M][K] (null: not kept)
+  const float* target;    // loss: [M][n_valid]
+  float* loss;
+  float* y;               // output: [M][n_valid]
+  float* db;              // loss, backward: [N] bias gradient, added to
+  float* zero;            // first layer of a training step: buffer to clear
+  long long n_zero;       // (a multiple of 4 floats) and the loss
+  unsigned* err;
+};
+
+struct GradArgs {
+  long long M;
+  int out_p, in_p;
+  const bf16* dz;   // [M][out_p]
+  const bf16* a;    // [M][in_p]
+  float* dw;        // [out_p][in_p], added to
+  int tiles_n;      // column tiles
+  int rows;         // rows of a CTA, a multiple of 64
+};
+
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, bool ok) {
+  const int n = ok ? 16 : 0;  // the rest is zeroed
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(n)
+               : "memory");
+}
+
+// [rows][kc] of src (row stride ld, rows below n_ok) -> core matrices, LBO 128, SBO kSbo
+__device__ __forceinline__ void pack_rows(uint32_t dst, const bf16* src, size_t ld,
+                                          long long n_ok, int rows, int kc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r = lane & 7, k8 = lane >> 3;  // 8 rows x 4 pieces of 8
+  const int nk = (kc / 8 + 3) / 4;
+  for (int u = warp; u < (rows / 8) * nk; u += kLayThreads / 32) {
+    const int g = u / nk, c = (u % nk) * 4 + k8, row = g * 8 + r;
+    if (c * 8 < kc)
+      copy16(dst + g * kSbo + c * 128u + r * 16u,
+             row < n_ok ? src + (size_t)row * ld + c * 8 : src, row < n_ok);
   }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(&bar[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(&bar[1])));
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+}
+
+// element (n, k) = src[k][n], n = 0 .. 8 kGroups - 1, k = 0 .. kc - 1 (a multiple of 16, at
+// most kMaxK), zero where k >= k_ok or n >= n_ok (a multiple of 8) -> core matrices, LBO kLboT, SBO sbo
+template <int kGroups, int kMaxK>
+__device__ __forceinline__ void pack_transposed(unsigned char* dst, uint32_t sbo, const bf16* src,
+                                                size_t ld, int n_ok, int kc, long long k_ok) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kUnits = kGroups * (kMaxK / 64) / (kLayThreads / 32);  // a warp's share
+  uint4 v0[kUnits], v1[kUnits];  // all of a thread's loads in flight
+#pragma unroll
+  for (int i = 0; i < kUnits; ++i) {
+    const int u = warp + i * (kLayThreads / 32), g = u % kGroups;
+    const int k = (u / kGroups) * 64 + (lane >> 2) * 8 + (lane & 3) * 2;
+    v0[i] = v1[i] = make_uint4(0, 0, 0, 0);
+    if (g * 8 < n_ok && k < kc) {
+      const bf16* p = src + (size_t)k * ld + g * 8;
+      if (k < k_ok) v0[i] = *reinterpret_cast<const uint4*>(p);
+      if (k + 1 < k_ok) v1[i] = *reinterpret_cast<const uint4*>(p + ld);
+    }
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = tc_idesc(kGemmRows, kGemmCols);
-  bool ok = true;
-  int n_chunks = 0;
-  for (int k0 = k_begin; k0 < k_end && ok; k0 += kGemmK, ++n_chunks) {
-    const int buf = n_chunks & 1;
-    // the buffer was last read by the MMAs of chunk n_chunks - 2
-    if (n_chunks >= 2) {
-      const bool got = mbar_wait(smem_addr(&bar[buf]), (uint32_t)(((n_chunks - 2) >> 1) & 1));
-      if (!__syncthreads_and(got)) {
-        if (tid == 0) atomicOr(err, 1u);
-        ok = false;
-        break;
-      }
-    }
-    const int kc = min(kGemmK, k_end - k0);  // a multiple of 16
-    // A tile: element (r, k) = A[m0 + r][k0 + k], zero outside; 8 k per item
-    bf16* a = sA0 + buf * kGemmRows * kGemmK;
-    for (int i = tid; i < kGemmRows * (kGemmK / 8); i += kGemmThreads) {
-      const int r = i / (kGemmK / 8), k8 = (i % (kGemmK / 8)) * 8;
-      const int m = m0 + r;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (m < M && k8 < kc) {
-        if (!kAcol) {
-          v = *reinterpret_cast<const uint4*>(A + (size_t)m * lda + k0 + k8);
-        } else {
-          uint32_t w[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            w[j] = (uint32_t)__bfloat16_as_ushort(A[(size_t)(k0 + k8 + 2 * j) * lda + m]) |
-                   ((uint32_t)__bfloat16_as_ushort(A[(size_t)(k0 + k8 + 2 * j + 1) * lda + m])
-                    << 16);
-          v = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-      *reinterpret_cast<uint4*>(&a[core_off(r, k8, kGemmK)]) = v;
-    }
-    // B tile as the MMA's [N][K] operand: element (n, k) = B[k0 + k][n0 + n]
-    bf16* b = sB0 + buf * kGemmCols * kGemmK;
-    for (int i = tid; i < kGemmCols * (kGemmK / 8); i += kGemmThreads) {
-      const int c = i / (kGemmK / 8), k8 = (i % (kGemmK / 8)) * 8;
-      const int n = n0 + c;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (n < N && k8 < kc) {
-        if (kBcol) {
-          v = *reinterpret_cast<const uint4*>(B + (size_t)n * ldb + k0 + k8);
-        } else {
-          uint32_t w[4];
+  for (int i = 0; i < kUnits; ++i) {
+    const int u = warp + i * (kLayThreads / 32), g = u % kGroups;
+    const int k = (u / kGroups) * 64 + (lane >> 2) * 8 + (lane & 3) * 2;
+    if (k >= kc) continue;
+    unsigned char* q = dst + g * sbo + (k >> 3) * kLboT + (k & 7) * 2;
+    const uint32_t a[4] = {v0[i].x, v0[i].y, v0[i].z, v0[i].w};
+    const uint32_t b[4] = {v1[i].x, v1[i].y, v1[i].z, v1[i].w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            w[j] = (uint32_t)__bfloat16_as_ushort(B[(size_t)(k0 + k8 + 2 * j) * ldb + n]) |
-                   ((uint32_t)__bfloat16_as_ushort(B[(size_t)(k0 + k8 + 2 * j + 1) * ldb + n])
-                    << 16);
-          v = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      }
-      *reinterpret_cast<uint4*>(&b[core_off(c, k8, kGemmK)]) = v;
+    for (int j = 0; j < 4; ++j) {
+      *reinterpret_cast<uint32_t*>(q + (2 * j) * 16) = __byte_perm(a[j], b[j], 0x5410);
+      *reinterpret_cast<uint32_t*>(q + (2 * j + 1) * 16) = __byte_perm(a[j], b[j], 0x7632);
     }
+  }
+}
+
+// The tensor memory and barrier of a CTA's single accumulator, and one accumulation step:
+// the packed chunk's MMAs, then the wait for them. All threads of the block.
+struct Accumulator {
+  uint32_t tmem, bar, parity;
+  const uint32_t* slot;
+  // no barrier: the first add() has one between the set-up and its use
+  __device__ __forceinline__ void open(uint64_t* bar_mem, uint32_t* slot_mem, int cols) {
+    slot = slot_mem;
+    if (threadIdx.x < 32) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                       smem_addr(slot_mem)),
+                   "r"(cols));
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    bar = smem_addr(bar_mem);
+    if (threadIdx.x == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar));
+      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    parity = 0;
+  }
+  // false when the wait ran out (the same in all threads)
+  __device__ __forceinline__ bool add(uint32_t a, uint32_t lbo_a, uint32_t sbo_a, uint32_t b,
+                                      uint32_t lbo_b, uint32_t sbo_b, uint32_t idesc, int kc,
+                                      bool first, unsigned* err) {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const uint32_t a0 = smem_addr(a), b0 = smem_addr(b);
-      const uint32_t sbo = (uint32_t)kGemmK * 16u;
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    tmem = *slot;
+    if (threadIdx.x == 0) {
       for (int kk = 0; kk < kc / 16; ++kk)
-        tc_mma(tmem, tc_desc(a0 + kk * 256u, 128u, sbo), tc_desc(b0 + kk * 256u, 128u, sbo), idesc,
-               (n_chunks > 0 || kk > 0) ? 1u : 0u);
+        tc_mma(tmem, tc_desc(a + kk * 2 * lbo_a, lbo_a, sbo_a),
+               tc_desc(b + kk * 2 * lbo_b, lbo_b, sbo_b), idesc, !first || kk > 0 ? 1u : 0u);
       asm volatile(
           "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-              smem_addr(&bar[buf]))
+              bar)
           : "memory");
     }
-  }
-  // the last chunk's MMAs (and with them all earlier ones) done
-  if (ok && n_chunks > 0) {
-    const int last = n_chunks - 1;
-    const bool got = mbar_wait(smem_addr(&bar[last & 1]), (uint32_t)((last >> 1) & 1));
+    const bool got = mbar_wait(bar, parity);
     if (!__syncthreads_and(got)) {
-      if (tid == 0) atomicOr(err, 1u);
-      ok = false;
+      if (threadIdx.x == 0) atomicOr(err, 1u);
+      mbar_wait(bar, parity);  // let the MMAs in flight land before the memory is released
+      return false;
+    }
+    parity ^= 1u;
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    return true;
+  }
+  __device__ __forceinline__ void close(int cols) {
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                   "r"(cols));
     }
   }
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (ok && n_chunks > 0) {
-    // warp w holds rows 32 w .. 32 w + 31 of the tile (tensor-memory lanes)
-    const int m = m0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < kGemmCols; c0 += 16) {
-      float v[16];
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-      if (m >= M || n0 + c0 >= N) continue;
-      float* cr = C + (size_t)m * ldc + n0 + c0;
-      const int nv = min(16, N - n0 - c0);
-      if (atomic_out) {
+};
+
+// Sums over the warp's lanes of v[0 .. 31]; lane c returns that of v[c] (v is used up).
+__device__ __forceinline__ float transpose_sum(float* v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (j < nv) atomicAdd(&cr[j], v[j]);
-      } else if (nv == 16 && ((reinterpret_cast<uintptr_t>(cr) & 15) == 0)) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool hi = (lane & o) != 0;
 #pragma unroll
-        for (int j = 0; j < 16; j += 4)
-          *reinterpret_cast<float4*>(&cr[j]) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-      } else {
+    for (int i = 0; i < o; ++i) {
+      const float send = hi ? v[i] : v[i + o], keep = hi ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return v[0];
+}
+
+__device__ __forceinline__ void store_bf16x16(bf16* dst, const float* v) {
+  uint32_t h[8];
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (j < nv) cr[j] = v[j];
+  for (int j = 0; j < 8; ++j) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+    h[j] = *reinterpret_cast<const uint32_t*>(&p);
+  }
+  uint4* q = reinterpret_cast<uint4*>(dst);
+  q[0] = make_uint4(h[0], h[1], h[2], h[3]);
+  q[1] = make_uint4(h[4], h[5], h[6], h[7]);
+}
+
+// The layer kernels of a pass are launched as dependents of one another: the next one's
+// blocks start, set up and fetch weights (which no kernel of a pass writes) while this one
+// finishes, and wait here for all of its results.
+__device__ __forceinline__ void after_previous_kernel() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+// One 128 x 64 tile of a layer. smem: kLaySmem bytes.
+template <int kEpi>
+__device__ void layer_tile(const LayerArgs& p, long long row_tile, int col_tile,
+                           unsigned char* smem, Accumulator& acc) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const long long m0 = row_tile * kLayRows;
+  const int n0 = col_tile * kLayCols;
+  const int n_cols = min(kLayCols, p.N - n0);  // a multiple of 16
+  const long long rows = p.M - m0 < kLayRows ? p.M - m0 : kLayRows;
+  unsigned char* sB = smem + (kLayRows / 8) * kSbo;
+  const uint32_t a_addr = smem_addr(smem), b_addr = smem_addr(sB);
+  const uint32_t idesc = tc_idesc(kLayRows, kLayCols);
+  constexpr bool kT = kEpi == kBack;
+  // warp w reads rows 32 (w & 3) .. + 31, columns 32 (w >> 2) .. + 31 of the tile
+  const int c0 = 32 * (warp >> 2);
+  const long long row = m0 + 32 * (warp & 3) + lane;
+  const bool live = row < p.M;
+  float pre[32];  // the epilogue's own input, fetched while the product is under way
+  __shared__ __align__(16) float s_bias[kLayCols];
+  if (kEpi != kBack && tid < kLayCols)
+    s_bias[tid] = n0 + tid < p.n_valid ? __ldg(&p.bias[n0 + tid]) : 0.0f;
+  bool ok = true;
+  for (int k0 = 0; k0 < p.K && ok; k0 += kLayK) {
+    const int kc = min(kLayK, p.K - k0);
+    if (!kT) pack_rows(b_addr, p.w + (size_t)n0 * p.K + k0, p.K, n_cols, kLayCols, kc);
+    if (kT)
+      pack_transposed<kLayCols / 8, kLayK>(sB, kSboT, p.w + (size_t)k0 * p.N + n0, p.N, n_cols,
+                                           kc, p.K - k0);
+    if (k0 == 0) after_previous_kernel();
+    if (!p.x) pack_rows(a_addr, p.a + (size_t)m0 * p.K + k0, p.K, rows, kLayRows, kc);
+    if (k0 == 0) {
+      if constexpr (kEpi == kBack) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          float4 z = make_float4(0, 0, 0, 0);
+          if (live && n0 + c0 + j < p.N)
+            z = *reinterpret_cast<const float4*>(p.z + row * p.N + n0 + c0 + j);
+          pre[j] = z.x;
+          pre[j + 1] = z.y;
+          pre[j + 2] = z.z;
+          pre[j + 3] = z.w;
+        }
+      } else if constexpr (kEpi == kLoss) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          pre[j] = live && n0 + c0 + j < p.n_valid
+                       ? __ldg(&p.target[row * p.n_valid + n0 + c0 + j]) : 0.0f;
       }
     }
-  } else if (!ok && n_chunks > 0 && warp == 0) {
-    // a wait ran out: let the MMAs still in flight land before releasing tensor memory
-    const int last = n_chunks - 1;
-    mbar_wait(smem_addr(&bar[last & 1]), (uint32_t)((last >> 1) & 1));
+    if (p.x) {  // the FP32 input rows: coalesced along a row, zero padding
+      const int valid = min(kc, p.n_in - k0);
+      for (int k = lane; k < kc; k += 32) {
+        float v[kLayRows / 8];  // all of a thread's rows in flight
+#pragma unroll
+        for (int i = 0; i < kLayRows / 8; ++i) {
+          const int r = warp + 8 * i;
+          v[i] = r < rows && k < valid ? __ldg(&p.x[(m0 + r) * p.n_in + k0 + k]) : 0.0f;
+        }
+#pragma unroll
+        for (int i = 0; i < kLayRows / 8; ++i) {
+          const int r = warp + 8 * i;
+          const bf16 h = __float2bfloat16(v[i]);
+          *reinterpret_cast<bf16*>(smem + (r >> 3) * kSbo + (k >> 3) * 128 + (r & 7) * 16 +
+                                   (k & 7) * 2) = h;
+          if (p.a0 && col_tile == 0 && r < rows) p.a0[(m0 + r) * p.K + k0 + k] = h;
+        }
+      }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    ok = acc.add(a_addr, 128, kSbo, b_addr, kT ? kLboT : 128, kT ? kSboT : kSbo, idesc, kc,
+                 k0 == 0, p.err);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"(kGemmCols));
+  if (!ok) return;
+  float v[32];
+  tmem_ld16(acc.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
+  tmem_ld16(acc.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0 + 16, v + 16);
+  float loss = 0.0f;
+#pragma unroll
+  for (int h = 0; h < 32; h += 16) {
+    const int col = n0 + c0 + h;
+    float* w = v + h;
+    if (col >= p.N) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) w[j] = 0.0f;
+      continue;
+    }
+    if constexpr (kEpi == kHidden || kEpi == kLoss || kEpi == kOutput) {
+#pragma unroll
+      for (int j = 0; j < 16; j += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(&s_bias[c0 + h + j]);
+        w[j] = col + j < p.n_valid ? w[j] + b.x : 0.0f;
+        w[j + 1] = col + j + 1 < p.n_valid ? w[j + 1] + b.y : 0.0f;
+        w[j + 2] = col + j + 2 < p.n_valid ? w[j + 2] + b.z : 0.0f;
+        w[j + 3] = col + j + 3 < p.n_valid ? w[j + 3] + b.w : 0.0f;
+      }
+    }
+    if constexpr (kEpi == kHidden) {
+      if (live && p.z) {
+        float4* q = reinterpret_cast<float4*>(p.z + row * p.N + col);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          q[j] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) w[j] = silu_fast(w[j]);
+    }
+    if constexpr (kEpi == kLoss) {
+      const float inv = (float)p.M * (float)p.n_valid;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float e = live && col + j < p.n_valid ? w[j] - pre[h + j] : 0.0f;
+        loss += e * e;
+        w[j] = 2.0f * e / inv;
+      }
+    }
+    if constexpr (kEpi == kBack) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float zz = pre[h + j], s = sigmoid_fast(zz);
+        w[j] = live && col + j < p.n_valid ? w[j] * s * (1.0f + zz * (1.0f - s)) : 0.0f;
+      }
+    }
+    if constexpr (kEpi == kOutput) {
+      if (live)
+        for (int j = 0; j < 16; ++j)
+          if (col + j < p.n_valid) p.y[row * p.n_valid + col + j] = w[j];
+    } else {
+      if (live) store_bf16x16(p.out + row * p.N + col, w);
+    }
   }
+  if constexpr (kEpi == kLoss) {
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    if (lane == 0 && loss != 0.0f)
+      atomicAdd(p.loss, loss / ((float)p.M * (float)p.n_valid));
+  }
+  if constexpr (kEpi == kLoss || kEpi == kBack) {
+    const float sum = transpose_sum(v);
+    if (n0 + c0 + lane < p.n_valid) atomicAdd(&p.db[n0 + c0 + lane], sum);
+  }
+}
+
+template <int kEpi>
+__global__ void __launch_bounds__(kLayThreads) k_layer(const __grid_constant__ LayerArgs p) {
+  extern __shared__ __align__(128) unsigned char lay_smem[];
+  __shared__ uint64_t bar;
+  __shared__ uint32_t slot;
+  Accumulator acc;
+  acc.open(&bar, &slot, kLayCols);
+  if (p.zero) {  // the pass's first kernel, an ordinary launch
+    const long long me = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kLayThreads + threadIdx.x;
+    for (long long i = me; i < p.n_zero / 4; i += (long long)gridDim.x * gridDim.y * kLayThreads)
+      reinterpret_cast<float4*>(p.zero)[i] = make_float4(0, 0, 0, 0);
+    if (me == 0) *p.loss = 0.0f;
+  }
+  layer_tile<kEpi>(p, blockIdx.x, blockIdx.y, lay_smem, acc);
+  acc.close(kLayCols);
+}
+
+// The backward kernel of a layer: the first n_layer blocks pass the gradient down (none
+// for the first layer), the others form the weight gradient.
+__global__ void __launch_bounds__(kLayThreads) k_layer_back(const __grid_constant__ LayerArgs p,
+                                                            const __grid_constant__ GradArgs q,
+                                                            int n_layer, int row_tiles) {
+  extern __shared__ __align__(128) unsigned char lay_smem[];
+  __shared__ uint64_t bar;
+  __shared__ uint32_t slot;
+  Accumulator acc;
+  acc.open(&bar, &slot, 128);
+  if ((int)blockIdx.x < n_layer) {
+    layer_tile<kBack>(p, blockIdx.x % row_tiles, blockIdx.x / row_tiles, lay_smem, acc);
+  } else {
+    after_previous_kernel();
+    const int i = blockIdx.x - n_layer;
+    const int tiles = q.tiles_n * ((q.out_p + 127) / 128);
+    const int t = i % tiles, m0 = (t / q.tiles_n) * 128, n0 = (t % q.tiles_n) * 128;
+    const long long r0 = (long long)(i / tiles) * q.rows;
+    const long long r1 = r0 + q.rows < q.M ? r0 + q.rows : q.M;
+    unsigned char* sB = lay_smem + 16 * kSboG;
+    bool ok = true;
+    for (long long r = r0; r < r1 && ok; r += kGradRows) {
+      const int kc = r1 - r < kGradRows ? ((int)(r1 - r) + 15) / 16 * 16 : kGradRows;
+      pack_transposed<16, kGradRows>(lay_smem, kSboG, q.dz + r * q.out_p + m0, q.out_p,
+                                     q.out_p - m0, kc, r1 - r);
+      pack_transposed<16, kGradRows>(sB, kSboG, q.a + r * q.in_p + n0, q.in_p, q.in_p - n0, kc,
+                                     r1 - r);
+      ok = acc.add(smem_addr(lay_smem), kLboT, kSboG, smem_addr(sB), kLboT, kSboG,
+                   tc_idesc(128, 128), kc, r == r0, p.err);
+    }
+    if (ok) {
+      // warp w: rows 32 (w & 3) .., columns 64 (w >> 2) .. of the tile
+      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      const int row = m0 + 32 * (warp & 3) + lane;
+      for (int c = 64 * (warp >> 2); c < 64 * (warp >> 2) + 64; c += 16) {
+        if (n0 + c >= q.in_p) break;
+        float v[16];
+        tmem_ld16(acc.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c, v);
+        if (row < q.out_p) {
+          float* dst = q.dw + (size_t)row * q.in_p + n0 + c;
+#pragma unroll
+          for (int j = 0; j < 16; j += 4)
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                             __cvta_generic_to_global(dst + j)),
+                         "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3])
+                         : "memory");
+        }
+      }
+    }
+  }
+  acc.close(128);
 }
 
 struct TcNet {
@@ -700,28 +882,46 @@ inline unsigned nb(long long n, int t);
 inline unsigned nb(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 // ---------------------------------------------------------------- host helpers
-template <bool Acol, bool Bcol>
-cudaError_t gemm(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, long long M,
-                 int N, int K, bool split, unsigned* err, cudaStream_t s) {
-  dim3 grid(nb(M, kGemmRows), nb(N, kGemmCols), 1);
-  int chunk = K;
-  if (split) {
-    // split the contraction so that the grid fills the GPU
-    long long tiles = (long long)grid.x * grid.y;
-    long long want = (152 * 2 + tiles - 1) / tiles;
-    long long ksteps = (K + kGemmK - 1) / kGemmK;
-    if (want > ksteps) want = ksteps;
-    if (want < 1) want = 1;
-    chunk = (int)(((ksteps + want - 1) / want) * kGemmK);
-    grid.z = (unsigned)((K + chunk - 1) / chunk);
-  }
-  const size_t smem = sizeof(bf16) * 2 * (kGemmRows + kGemmCols) * kGemmK;
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<Acol, Bcol>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// A kernel of a pass: `dependent` ones may start while the one before them finishes (they
+// wait in after_previous_kernel for its results).
+template <typename... P, typename... A>
+cudaError_t launch_pass_kernel(void (*kernel)(P...), dim3 grid, bool dependent, cudaStream_t s,
+                               A... args) {
+  const cudaError_t e = cudaFuncSetAttribute(
+      kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaySmem);
   if (e != cudaSuccess) return e;
-  k_gemm_tc<Acol, Bcol><<<grid, kGemmThreads, smem, s>>>(A, lda, B, ldb, C, ldc, (int)M, N, K,
-                                                         chunk, split ? 1 : 0, err);
-  return cudaGetLastError();
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(kLayThreads);
+  c.dynamicSmemBytes = kLaySmem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
+template <int kEpi>
+cudaError_t launch_layer(const LayerArgs& p, bool first, cudaStream_t s) {
+  return launch_pass_kernel(k_layer<kEpi>, dim3(nb(p.M, kLayRows), nb(p.N, kLayCols)), !first, s,
+                            p);
+}
+
+cudaError_t launch_layer_back(const LayerArgs& p, GradArgs q, bool down, cudaStream_t s) {
+  const int row_tiles = (int)nb(p.M, kLayRows);
+  const int n_layer = down ? row_tiles * (int)nb(p.N, kLayCols) : 0;
+  // rows split so that the gradient tiles are about two per SM (two CTAs fit an SM), in
+  // pieces of 64 rows at least
+  q.tiles_n = (int)nb(q.in_p, 128);
+  const long long tiles = (long long)q.tiles_n * nb(q.out_p, 128);
+  const long long chunks = (q.M + 63) / 64;
+  const long long splits = std::min(chunks, (304 + tiles - 1) / tiles);
+  q.rows = (int)((chunks + splits - 1) / splits) * 64;
+  const long long n_grad = tiles * ((q.M + q.rows - 1) / q.rows);
+  return launch_pass_kernel(k_layer_back, dim3((unsigned)(n_layer + n_grad)), true, s, p, q,
+                            n_layer, row_tiles);
 }
 
 uint64_t splitmix(uint64_t& x) {
@@ -749,26 +949,28 @@ void release(T*& p) {
 }
 
 void free_acts(rt_mlp* m) {
-  for (int l = 0; l <= kMaxLayers; ++l) release(m->d_a[l]);
+  for (int l = 0; l < kMaxLayers; ++l) release(m->d_a[l]);
   for (int l = 0; l < kMaxLayers; ++l) release(m->d_z[l]);
-  release(m->d_dz);
-  release(m->d_dzb);
+  for (int i = 0; i < 2; ++i) release(m->d_dz[i]);
   m->cap = 0;
 }
 
-rt_status ensure_rows(rt_mlp* m, long long Mp) {
-  if (Mp <= m->cap) return RT_OK;
+// Work arrays for `rows` rows: the layers' inputs, and for training the pre-activations
+// and two layers' dz.
+rt_status ensure_rows(rt_mlp* m, long long rows, bool train) {
+  if (rows <= m->cap && (!train || m->d_dz[0])) return RT_OK;
+  if (rows < m->cap) rows = m->cap;
   free_acts(m);
   rt_status st;
-  const int L = m->n_layers_total;
-  if ((st = alloc(&m->d_a[0], (size_t)Mp * m->layer[0].in_p)) != RT_OK) return st;
-  for (int l = 0; l < L; ++l) {
-    if ((st = alloc(&m->d_z[l], (size_t)Mp * m->layer[l].out_p)) != RT_OK) return st;
-    if ((st = alloc(&m->d_a[l + 1], (size_t)Mp * m->layer[l].out_p)) != RT_OK) return st;
+  for (int l = 0; l < m->n_layers_total; ++l) {
+    if ((st = alloc(&m->d_a[l], (size_t)rows * m->layer[l].in_p)) != RT_OK) return st;
+    if (train && l + 1 < m->n_layers_total &&
+        (st = alloc(&m->d_z[l], (size_t)rows * m->layer[l].out_p)) != RT_OK)
+      return st;
   }
-  if ((st = alloc(&m->d_dz, (size_t)Mp * m->max_p)) != RT_OK) return st;
-  if ((st = alloc(&m->d_dzb, (size_t)Mp * m->max_p)) != RT_OK) return st;
-  m->cap = Mp;
+  for (int i = 0; train && i < 2; ++i)
+    if ((st = alloc(&m->d_dz[i], (size_t)rows * m->max_p)) != RT_OK) return st;
+  m->cap = rows;
   return RT_OK;
 }
 
@@ -825,18 +1027,44 @@ rt_status forward_tc(rt_mlp* m, const float* x, float* y, long long M, cudaStrea
   return cudaGetLastError() == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }
 
-// forward over Mp padded rows of d_a[0]
-rt_status forward_rows(rt_mlp* m, long long Mp, cudaStream_t s) {
+// forward of M rows layer by layer: the last layer into y, or (t) its loss and dz
+rt_status forward_rows(rt_mlp* m, const float* x, long long M, float* y, const float* t,
+                       cudaStream_t s) {
   const int L = m->n_layers_total;
   for (int l = 0; l < L; ++l) {
     const Layer& ly = m->layer[l];
-    if (gemm<false, true>(m->d_a[l], ly.in_p, m->d_wbf + ly.w_off, ly.in_p, m->d_z[l], ly.out_p,
-                          Mp, ly.out_p, ly.in_p, false, m->d_err, s) != cudaSuccess)
-      return RT_ERR_CUDA;
-    k_bias_act<<<nb(Mp * ly.out_p, 256), 256, 0, s>>>(m->d_z[l], m->d_param + ly.b_off, Mp,
-                                                      ly.out_p, ly.n_out, l < L - 1,
-                                                      m->d_a[l + 1]);
-    if (cudaGetLastError() != cudaSuccess) return RT_ERR_CUDA;
+    LayerArgs p{};
+    p.M = M;
+    p.N = ly.out_p;
+    p.K = ly.in_p;
+    p.n_valid = ly.n_out;
+    p.n_in = m->n_in;
+    p.x = l == 0 ? x : nullptr;
+    p.a0 = l == 0 && t ? m->d_a[0] : nullptr;
+    p.a = m->d_a[l];
+    p.w = m->d_wbf + ly.w_off;
+    p.bias = m->d_param + ly.b_off;
+    p.err = m->d_err;
+    p.loss = m->d_loss;
+    if (l == 0 && t) {
+      p.zero = m->d_grad;
+      p.n_zero = (long long)m->n_padded;
+    }
+    cudaError_t e;
+    if (l + 1 < L) {
+      p.z = t ? m->d_z[l] : nullptr;
+      p.out = m->d_a[l + 1];
+      e = launch_layer<kHidden>(p, l == 0, s);
+    } else if (t) {
+      p.target = t;
+      p.out = m->d_dz[l & 1];
+      p.db = m->d_grad + ly.b_off;
+      e = launch_layer<kLoss>(p, l == 0, s);
+    } else {
+      p.y = y;
+      e = launch_layer<kOutput>(p, l == 0, s);
+    }
+    if (e != cudaSuccess) return RT_ERR_CUDA;
   }
   return RT_OK;
 }
@@ -1006,19 +1234,10 @@ rt_status rt_mlp_forward(rt_mlp* m, const float* x, float* y, int64_t M, void* s
   if (tc_eligible(m)) return forward_tc(m, x, y, M, s);
   const long long chunk = 1ll << 18;
   for (long long r0 = 0; r0 < M; r0 += chunk) {
-    long long Mc = M - r0 < chunk ? M - r0 : chunk;
-    long long Mp = (Mc + kTile - 1) / kTile * kTile;
-    rt_status st = ensure_rows(m, Mp);
+    const long long Mc = M - r0 < chunk ? M - r0 : chunk;
+    rt_status st = ensure_rows(m, Mc, false);
+    if (st == RT_OK) st = forward_rows(m, x + r0 * m->n_in, Mc, y + r0 * m->n_out, nullptr, s);
     if (st != RT_OK) return st;
-    const Layer& l0 = m->layer[0];
-    k_pack_input<<<nb(Mp * l0.in_p, 256), 256, 0, s>>>(x + r0 * m->n_in, Mc, m->n_in, Mp,
-                                                       l0.in_p, m->d_a[0]);
-    if ((st = forward_rows(m, Mp, s)) != RT_OK) return st;
-    const Layer& ll = m->layer[m->n_layers_total - 1];
-    k_unpack_output<<<nb(Mc * m->n_out, 256), 256, 0, s>>>(m->d_z[m->n_layers_total - 1], Mc,
-                                                           m->n_out, ll.out_p,
-                                                           y + r0 * m->n_out);
-    if (cudaGetLastError() != cudaSuccess) return RT_ERR_CUDA;
   }
   return RT_OK;
 }
@@ -1028,37 +1247,34 @@ rt_status rt_mlp_loss_grad(rt_mlp* m, const float* x, const float* t, int64_t M,
   if (!m || !x || !t || M < 1 || M > (1ll << 24)) return RT_ERR_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(m->dev) != cudaSuccess) return RT_ERR_CUDA;
-  const long long Mp = (M + kTile - 1) / kTile * kTile;
-  rt_status st = ensure_rows(m, Mp);
+  rt_status st = ensure_rows(m, M, true);
   if (st != RT_OK) return st;
   const int L = m->n_layers_total;
-  const Layer& l0 = m->layer[0];
-  if (cudaMemsetAsync(m->d_grad, 0, sizeof(float) * m->n_padded, s) != cudaSuccess ||
-      cudaMemsetAsync(m->d_loss, 0, sizeof(float), s) != cudaSuccess)
-    return RT_ERR_CUDA;
-  k_pack_input<<<nb(Mp * l0.in_p, 256), 256, 0, s>>>(x, M, m->n_in, Mp, l0.in_p, m->d_a[0]);
-  if ((st = forward_rows(m, Mp, s)) != RT_OK) return st;
-  const Layer& lo = m->layer[L - 1];
-  k_mse_grad<<<nb(Mp * lo.out_p, 256), 256, 0, s>>>(m->d_z[L - 1], t, M, m->n_out, Mp, lo.out_p,
-                                                    m->d_dz, m->d_dzb, m->d_loss);
+  if ((st = forward_rows(m, x, M, nullptr, t, s)) != RT_OK) return st;
   for (int l = L - 1; l >= 0; --l) {
     const Layer& ly = m->layer[l];
-    // dW_l = dz^T a_{l-1}: [out_p][in_p], contraction over rows (split)
-    if (gemm<true, false>(m->d_dzb, ly.out_p, m->d_a[l], ly.in_p, m->d_grad + ly.w_off, ly.in_p,
-                          ly.out_p, ly.in_p, (int)Mp, true, m->d_err, s) != cudaSuccess)
-      return RT_ERR_CUDA;
-    dim3 g2(nb(ly.out_p, 32), 64);
-    k_col_sums<<<g2, 256, 0, s>>>(m->d_dz, Mp, ly.out_p, m->d_grad + ly.b_off);
-    if (l > 0) {
-      // da_{l-1} = dz W_l: [Mp][in_p]; then through silu'
-      if (gemm<false, false>(m->d_dzb, ly.out_p, m->d_wbf + ly.w_off, ly.in_p, m->d_dz, ly.in_p,
-                             Mp, ly.in_p, ly.out_p, false, m->d_err, s) != cudaSuccess)
-        return RT_ERR_CUDA;
+    GradArgs q{};
+    q.M = M;
+    q.out_p = ly.out_p;
+    q.in_p = ly.in_p;
+    q.dz = m->d_dz[l & 1];
+    q.a = m->d_a[l];
+    q.dw = m->d_grad + ly.w_off;
+    LayerArgs p{};
+    p.M = M;
+    p.err = m->d_err;
+    if (l > 0) {  // da_{l-1} = dz W_l, through silu'
       const Layer& lp = m->layer[l - 1];
-      k_act_back<<<nb(Mp * ly.in_p, 256), 256, 0, s>>>(m->d_dz, m->d_z[l - 1], Mp, ly.in_p,
-                                                       lp.n_out, m->d_dzb);
+      p.N = ly.in_p;
+      p.K = ly.out_p;
+      p.n_valid = lp.n_out;
+      p.a = m->d_dz[l & 1];
+      p.w = m->d_wbf + ly.w_off;
+      p.z = m->d_z[l - 1];
+      p.out = m->d_dz[(l - 1) & 1];
+      p.db = m->d_grad + lp.b_off;
     }
-    if (cudaGetLastError() != cudaSuccess) return RT_ERR_CUDA;
+    if (launch_layer_back(p, q, l > 0, s) != cudaSuccess) return RT_ERR_CUDA;
   }
   if (loss_out &&
       cudaMemcpyAsync(loss_out, m->d_loss, sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess)
@@ -1077,10 +1293,13 @@ rt_status rt_mlp_adam_step(rt_mlp* m, float lr, void* stream) {
   m->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   float c1 = 1.0f - std::pow(b1, (float)m->step), c2 = 1.0f - std::pow(b2, (float)m->step);
-  k_adam<<<nb((long long)m->n_padded, 256), 256, 0, s>>>(m->d_param, m->d_grad, m->d_m, m->d_v,
-                                                         m->n_padded, lr, b1, b2, c1, c2, 1e-8f);
-  if (cudaGetLastError() != cudaSuccess) return RT_ERR_CUDA;
-  return refresh_bf16(m, s);
+  const long long n4 = (long long)m->n_padded / 4;
+  k_adam<<<nb(n4, 128), 128, 0, s>>>(
+      reinterpret_cast<float4*>(m->d_param), reinterpret_cast<const float4*>(m->d_grad),
+      reinterpret_cast<float4*>(m->d_m), reinterpret_cast<float4*>(m->d_v),
+      reinterpret_cast<uint2*>(m->d_wbf), (size_t)n4, lr, b1, b2, c1, c2, 1e-8f);
+  m->pk_stale = true;
+  return cudaGetLastError() == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }
 
 }  // extern "C"
