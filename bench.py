@@ -422,15 +422,15 @@ def train_surrogate(g, n, first, stream, dev):
     return net, info
 
 
-def pah_step_launches(n_active, n_fallback, n_pah):
+def pah_step_launches(n_active, n_fallback):
     """Kernels of one active-cell PAH emission pass: the compaction of PAH-active
-    cells; per batch of at most 2^20 of them and per PAH the features, the fused
-    network and the check, per PAH the add, and the compaction of failed cells;
-    then one exact launch for those."""
+    cells; per batch of at most 2^20 of them the features, the fused network and the
+    rows with their checks, all PAHs in each; then one exact launch for the cells that
+    failed them."""
     if n_active == 0:
         return 1
     batches = (n_active + (1 << 20) - 1) >> 20
-    return 1 + batches * (4 * n_pah + 1) + (1 if n_fallback else 0)
+    return 1 + 3 * batches + (1 if n_fallback else 0)
 
 
 def surrogate_error(g, net, cells_dev, j_dev, tol, stream):
@@ -573,7 +573,7 @@ def run_ours(args):
             # transport, temperatures, the reset's clearing of PAH rows; the PAH pass
             # (counted from its own sizes)
             launches += 2 + (1 if g.n_pah else 0) + (
-                pah_step_launches(pah_state["active"], pah_state["fallback"], g.n_pah)
+                pah_step_launches(pah_state["active"], pah_state["fallback"])
                 if pah else 0) + (4 if images else 0)
         t_end.record(stream)
         torch.cuda.nvtx.range_pop()

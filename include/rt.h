@@ -347,7 +347,7 @@ rt_status rt_pah_absorbed(rt_grid *g, uint32_t *out, int mem, void *stream);
  * number `pah` when pah >= 0). Exact (RT_PAH_EXACT): for each cell and PAH, the
  * thermal-discrete steady state under the photon absorption rates its absorbed
  * spectrum implies (count * eps / (h nu_k N_molecules)), then N_molecules
- * sum_f P_f 4 pi sigma_b P_b(T_f), a quad of four lanes per cell with FP32
+ * sum_f P_f 4 pi sigma_b P_b(T_f), eight lanes per cell with FP32
  * populations (the upward flux across each level boundary summed afresh from the
  * arrivals above it, so no cancellation); emitted power equals absorbed power. RT_PAH_SURROGATE: the network `surrogate` (an rt_mlp
  * with n_in = n_coarse + 2, n_out = n_bins, trained on rt_pah_training_pairs)

@@ -65,6 +65,8 @@ struct rt_grid {
   double* d_pah_wk = nullptr;
   float* d_pah_cf = nullptr;
   float* d_pah_wf = nullptr;
+  float* d_pah_ef = nullptr;
+  unsigned char* d_pah_first = nullptr;
   float* d_pah_cdf = nullptr;
   float* d_pah_cell_cdf = nullptr;  // [n_pah][N][B] per-cell re-emission spectra
   unsigned* d_pahabs = nullptr;
@@ -87,11 +89,10 @@ struct rt_grid {
   int64_t cells_scratch_n = 0;
   // surrogate scratch (rows per batch of active cells) and cell lists (per call)
   long long sur_cap = 0, list_cap = 0;
-  float* d_sx = nullptr;       // [batch][K+2]
+  float* d_sx = nullptr;       // [n_pah][batch][K+2]
   float* d_sy = nullptr;       // [n_pah][batch][B]
   float* d_spabs = nullptr;    // [n_pah][batch]
-  unsigned char* d_sflag = nullptr;  // [batch]
-  unsigned long long* d_scount = nullptr;
+  float* d_spower = nullptr;   // [n_pah][batch] absorbed power feature
   int* d_list = nullptr;       // [cells] PAH-active cells of the call
   int* d_list2 = nullptr;      // [cells] cells sent to the exact solution
   unsigned* d_ucount = nullptr;  // [2]
@@ -170,6 +171,8 @@ void free_tables(rt_grid* g) {
   dfree(g->d_pah_wk);
   dfree(g->d_pah_cf);
   dfree(g->d_pah_wf);
+  dfree(g->d_pah_ef);
+  dfree(g->d_pah_first);
   dfree(g->d_pah_cdf);
   g->tables_ready = false;
 }
@@ -233,8 +236,7 @@ void free_all(rt_grid* g) {
   dfree(g->d_sx);
   dfree(g->d_sy);
   dfree(g->d_spabs);
-  dfree(g->d_sflag);
-  dfree(g->d_scount);
+  dfree(g->d_spower);
   dfree(g->d_list);
   dfree(g->d_list2);
   dfree(g->d_ucount);
@@ -275,7 +277,8 @@ rt_status build_pah_tables(rt_grid* g, cudaStream_t s) {
   const int P = g->n_pah, M = g->pah_levels, K = g->tab.n_coarse;
   rt_status st;
   if ((st = dalloc(&g->d_pah_sigma, (size_t)P * B)) != RT_OK) return st;
-  if ((st = dalloc(&g->d_pah_s, (size_t)P * M * B)) != RT_OK) return st;
+  if ((st = dalloc(&g->d_pah_s, (size_t)P * ((M + 3) & ~3) * ((B + 3) & ~3))) != RT_OK)
+    return st;
   if ((st = dalloc(&g->d_pah_L, (size_t)P * M)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_T, (size_t)P * M)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_ek, (size_t)K)) != RT_OK) return st;
@@ -283,6 +286,8 @@ rt_status build_pah_tables(rt_grid* g, cudaStream_t s) {
   if ((st = dalloc(&g->d_pah_wk, (size_t)P * K)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_cf, (size_t)P * M)) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_wf, (size_t)P * K)) != RT_OK) return st;
+  if ((st = dalloc(&g->d_pah_ef, (size_t)K)) != RT_OK) return st;
+  if ((st = dalloc(&g->d_pah_first, (size_t)P * (M + 1))) != RT_OK) return st;
   if ((st = dalloc(&g->d_pah_cdf, (size_t)P * B)) != RT_OK) return st;
   if (!g->d_pahabs) {
     if ((st = dalloc(&g->d_pahabs, (size_t)P * g->desc.n_leaves * K)) != RT_OK) return st;
@@ -326,6 +331,8 @@ rt_status build_pah_tables(rt_grid* g, cudaStream_t s) {
   pb.template_cdf = g->d_pah_cdf;
   pb.c_f = g->d_pah_cf;
   pb.w_f = g->d_pah_wf;
+  pb.e_f = g->d_pah_ef;
+  pb.first_k = g->d_pah_first;
   pt.s = g->d_pah_s;
   pt.L = g->d_pah_L;
   pt.e_k = g->d_pah_ek;
@@ -333,6 +340,8 @@ rt_status build_pah_tables(rt_grid* g, cudaStream_t s) {
   pt.w_k = g->d_pah_wk;
   pt.c_f = g->d_pah_cf;
   pt.w_f = g->d_pah_wf;
+  pt.e_f = g->d_pah_ef;
+  pt.first_k = g->d_pah_first;
   RT_CUDA(launch_pah_tables(pb, pt, s));
   RT_CUDA(cudaStreamSynchronize(s));
   g->tab.pah_cdf = g->d_pah_cdf;
@@ -1463,15 +1472,14 @@ static rt_status surrogate_scratch(rt_grid* g, long long cells, long long batch,
     dfree(g->d_sx);
     dfree(g->d_sy);
     dfree(g->d_spabs);
-    dfree(g->d_sflag);
+    dfree(g->d_spower);
     g->sur_cap = 0;
-    if ((st = dalloc(&g->d_sflag, (size_t)batch)) != RT_OK) return st;
-    if ((st = dalloc(&g->d_sx, (size_t)batch * (K + 2))) != RT_OK) return st;
+    if ((st = dalloc(&g->d_spower, (size_t)P * batch)) != RT_OK) return st;
+    if ((st = dalloc(&g->d_sx, (size_t)P * batch * (K + 2))) != RT_OK) return st;
     if ((st = dalloc(&g->d_sy, (size_t)P * batch * B)) != RT_OK) return st;
     if ((st = dalloc(&g->d_spabs, (size_t)P * batch)) != RT_OK) return st;
     g->sur_cap = batch;
   }
-  if (!g->d_scount && (st = dalloc(&g->d_scount, 1)) != RT_OK) return st;
   if (!g->d_ucount && (st = dalloc(&g->d_ucount, 2)) != RT_OK) return st;
   return RT_OK;
 }
@@ -1528,8 +1536,7 @@ static rt_status pah_emission_impl(rt_grid* g, int64_t first_cell, int64_t n_cel
   }
   // the cells where a PAH absorbed anything, in one list for the whole range
   RT_CUDA(cudaMemsetAsync(g->d_ucount, 0, 2 * sizeof(unsigned), s));
-  RT_CUDA(launch_compact(g->ptab, g->d_pah_flag, g->desc.n_leaves, pah, first_cell, n_cells,
-                         nullptr, nullptr, g->d_list, g->d_ucount, s));
+  RT_CUDA(launch_compact(g->d_pah_flag, pah, first_cell, n_cells, g->d_list, g->d_ucount, s));
   unsigned na = 0;
   RT_CUDA(cudaMemcpyAsync(&na, g->d_ucount, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   RT_CUDA(cudaStreamSynchronize(s));
@@ -1548,36 +1555,25 @@ static rt_status pah_emission_impl(rt_grid* g, int64_t first_cell, int64_t n_cel
   const int* row_cells = compact ? g->d_list : nullptr;
   if (na > 0 && mode == RT_PAH_EXACT)
     RT_CUDA(launch_pah_exact(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, first_cell, na, dst,
-                             nullptr, pah, s, compact ? nullptr : g->d_list, row_cells));
+                             pah, s, compact ? nullptr : g->d_list, row_cells));
   if (na > 0 && mode != RT_PAH_EXACT) {
-    // the surrogate over batches of active cells; cells whose prediction fails its
-    // checks are appended to one fallback list, solved exactly in one launch
+    // the surrogate over batches of active cells, all PAHs in one pass of the network;
+    // cells whose prediction fails its checks are appended to one fallback list, solved
+    // exactly in one launch
+    const int pah0 = pah >= 0 ? pah : 0, np = pah >= 0 ? 1 : g->n_pah;
     const long long batch = na < (1u << 20) ? (long long)na : (1ll << 20);
     if ((st = surrogate_scratch(g, n_cells, batch, true)) != RT_OK) return st;
     for (long long b0 = 0; b0 < (long long)na; b0 += batch) {
       const long long nb = (long long)na - b0 < batch ? (long long)na - b0 : batch;
       const int* lst = g->d_list + b0;
-      RT_CUDA(cudaMemsetAsync(g->d_sflag, 0, (size_t)nb, s));
-      for (int p = 0; p < g->n_pah; ++p) {
-        if (pah >= 0 && p != pah) continue;
-        float* Y = g->d_sy + (size_t)p * batch * B;
-        float* pa = g->d_spabs + (size_t)p * batch;
-        RT_CUDA(launch_pah_features(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, p, first_cell,
-                                    nb, g->d_sx, pa, s, lst));
-        if ((st = rt_mlp_forward(m, g->d_sx, Y, nb, s)) != RT_OK) return st;
-        RT_CUDA(launch_surrogate_check(Y, g->d_sx, pa, nb, B, F, t, x_lo, x_hi, g->d_sflag, s));
-      }
-      for (int p = 0; p < g->n_pah; ++p) {
-        if (pah >= 0 && p != pah) continue;
-        RT_CUDA(launch_surrogate_add(g->d_sy + (size_t)p * batch * B,
-                                     g->d_spabs + (size_t)p * batch, nb, B,
-                                     mode == RT_PAH_AUTO ? g->d_sflag : nullptr,
-                                     compact ? dst + (size_t)b0 * B : dst, s,
-                                     compact ? nullptr : lst));
-      }
-      RT_CUDA(launch_compact(g->ptab, g->d_pah_flag, g->desc.n_leaves, pah, first_cell, nb,
-                             g->d_sflag, compact ? nullptr : lst, g->d_list2, g->d_ucount + 1,
-                             s, (int)b0));
+      RT_CUDA(launch_pah_features(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, pah0, np, first_cell,
+                                  nb, g->d_sx, g->d_spabs, g->d_spower, s, lst));
+      if ((st = rt_mlp_forward(m, g->d_sx, g->d_sy, np * nb, s)) != RT_OK) return st;
+      RT_CUDA(launch_surrogate_finish(g->d_sy, g->d_spower, g->d_spabs, nb, np, B,
+                                      t, x_lo, x_hi, mode == RT_PAH_AUTO,
+                                      compact ? dst + (size_t)b0 * B : dst,
+                                      compact ? nullptr : lst, (int)b0, g->d_list2,
+                                      g->d_ucount + 1, s));
     }
     unsigned nf = 0;
     RT_CUDA(cudaMemcpyAsync(&nf, g->d_ucount + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
@@ -1585,7 +1581,7 @@ static rt_status pah_emission_impl(rt_grid* g, int64_t first_cell, int64_t n_cel
     n_fallback = nf;
     if (mode == RT_PAH_AUTO && nf > 0)
       RT_CUDA(launch_pah_exact(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, first_cell, nf, dst,
-                               nullptr, pah, s, g->d_list2, row_cells));
+                               pah, s, g->d_list2, row_cells));
   }
   if (n_fallback_out) *n_fallback_out = n_fallback;
   return RT_OK;
@@ -1673,10 +1669,10 @@ rt_status rt_pah_training_pairs(rt_grid* g, int pah, int64_t first_cell, int64_t
   if (st != RT_OK) return st;
   if (pah < 0 || pah >= g->n_pah) return RT_ERR_ARG;
   if (n_cells == 0) return RT_OK;
-  RT_CUDA(launch_pah_features(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, pah, first_cell,
-                              n_cells, X, p_abs, s));
+  RT_CUDA(launch_pah_features(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, pah, 1, first_cell,
+                              n_cells, X, p_abs, nullptr, s));
   RT_CUDA(launch_pah_exact(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, first_cell, n_cells, Y,
-                           nullptr, pah, s));
+                           pah, s));
   RT_CUDA(launch_pah_encode(Y, p_abs, n_cells, g->desc.n_bins, Y, s));
   return RT_OK;
 }

@@ -234,7 +234,8 @@ struct PahBuild {
   PahSpec spec[kMaxPah];
   double dE[kMaxPah];        // level spacing, erg
   double T_star, f_ref;      // template heating: source blackbody at bolometric flux f_ref
-  float* s;                  // [n_pah][M][B] emission per level and bin, erg/s
+  float* s;                  // [n_pah][M/2][B][2] emission per level and bin, erg/s (M and
+                             // B padded to multiples of 4)
   double* L;                 // [n_pah][M] cooling rate per level, erg/s
   double* T;                 // [n_pah][M] level temperatures (work array)
   double* e_k;               // [K] photon energy of each coarse bin, erg
@@ -243,6 +244,8 @@ struct PahBuild {
   float* template_cdf;       // [n_pah][B]
   float* c_f;                // [n_pah][M] downward rate L_f / dE, 1/s (FP32 copy)
   float* w_f;                // [n_pah][K] w_k (FP32 copy)
+  float* e_f;                // [K] e_k (FP32 copy)
+  unsigned char* first_k;    // [n_pah][M + 1] coarse bins with q_k < d
 };
 
 struct PahTables {
@@ -254,6 +257,8 @@ struct PahTables {
   const double* w_k;
   const float* c_f;          // [n_pah][M] L_f / dE in FP32
   const float* w_f;          // [n_pah][K] w_k in FP32
+  const float* e_f;          // [K] e_k in FP32
+  const unsigned char* first_k;  // [n_pah][M + 1] coarse bins with q_k < d
   double dE[kMaxPah];
   double mol_mass[kMaxPah];  // g per molecule
   int species[kMaxPah];      // species index of each PAH
@@ -263,29 +268,23 @@ struct PahTables {
 cudaError_t launch_pah_tables(const PahBuild& pb, const PahTables& t, cudaStream_t s);
 cudaError_t launch_pah_exact(const DevGrid& g, const PahTables& t, const unsigned* pahabs,
                              double eps, double d0, long long first, long long n,
-                             float* j_out, const unsigned char* want, int pah_only,
-                             cudaStream_t s, const int* list = nullptr,
-                             const int* cell_of_row = nullptr);
+                             float* j_out, int pah_only, cudaStream_t s,
+                             const int* list = nullptr, const int* cell_of_row = nullptr);
 cudaError_t launch_pah_features(const DevGrid& g, const PahTables& t, const unsigned* pahabs,
-                                double eps, double d0, int p, long long first, long long n,
-                                float* X, float* p_abs, cudaStream_t s,
-                                const int* list = nullptr);
+                                double eps, double d0, int pah0, int n_pah, long long first,
+                                long long n, float* X, float* p_abs, float* power,
+                                cudaStream_t s, const int* list = nullptr);
 cudaError_t launch_pah_encode(const float* J, const float* p_abs, long long n, int B, float* Y,
                               cudaStream_t s);
-cudaError_t launch_surrogate_check(const float* Y, const float* X, const float* p_abs,
-                                   long long n, int B, int F, float tol, float x_lo, float x_hi,
-                                   unsigned char* flag, cudaStream_t s);
-cudaError_t launch_surrogate_add(const float* Y, const float* p_abs, long long n, int B,
-                                 const unsigned char* flag, float* j_out, cudaStream_t s,
-                                 const int* list = nullptr);
+cudaError_t launch_surrogate_finish(const float* Y, const float* power, const float* p_abs,
+                                    long long n, int n_pah, int B, float tol, float x_lo,
+                                    float x_hi, bool leave, float* j_out, const int* list,
+                                    int off, int* fallback, unsigned* n_fallback,
+                                    cudaStream_t s);
 cudaError_t launch_pah_clear(const unsigned* pah_flag, long long N, int K, int n_pah,
                              unsigned* pahabs, unsigned* pah_flag_out, cudaStream_t s);
-cudaError_t launch_compact(const PahTables& t, const unsigned* pah_flag, long long N, int pah,
-                           long long first, long long n, const unsigned char* flag,
-                           const int* list, int* out, unsigned* count, cudaStream_t s,
-                           int off = 0);
-cudaError_t launch_count_flags(const unsigned char* flag, long long n, unsigned long long* out,
-                               cudaStream_t s);
+cudaError_t launch_compact(const unsigned* pah_flag, int pah, long long first, long long n,
+                           int* out, unsigned* count, cudaStream_t s);
 cudaError_t launch_pah_cell_cdf(const float* J, long long n, int B, float* out, cudaStream_t s);
 
 // One P(T) problem: a PAH in a monochromatic field.
