@@ -114,34 +114,50 @@ __global__ void k_adam(float4* p, const float4* g, float4* m, float4* v, uint2* 
 }
 
 // ---------------------------------------------------------------- fused forward
-// The whole forward pass of a 128-row tile in one CTA on the 5th-generation tensor
-// cores: per layer, the activations (BF16, shared memory) times the layer's weights
-// (BF16, shared memory) accumulate in FP32 in tensor memory (tcgen05.mma, issued by
-// one thread), then 32 warps read the accumulators back (tcgen05.ld), add the
-// bias, apply silu and write the next layer's activations. Every padded input and
-// hidden width must be at most 256 (one MMA of M = 128, N = width per 16-wide K
-// step); a wider output layer runs in chunks of 256 output columns, each its own
-// weight copy, MMAs and epilogue.
+// The whole forward pass of 256 rows (two tiles of 128) in one CTA on the 5th-generation
+// tensor cores: per layer, the activations (BF16, shared memory) times the layer's weights
+// (BF16, streamed through shared memory) accumulate in FP32 in tensor memory, then 16 warps
+// read the accumulators back, add the bias, apply silu and write the next layer's
+// activations in place. Every padded input and hidden width must be at most 256; a wider
+// output layer runs in chunks of 256 output columns.
+//
+// Two things bound a layer of 256 columns: its products (2048 SM clocks per 128 rows) and
+// the activation function (one MUFU operation per element, 2048 clocks as well, with some
+// seven other instructions around it). To run them at the same time a layer is cut in halves of
+// 128 columns: while the second half's products run, the first half's activations are formed
+// (in registers: the products still read the layer's input, which they will replace), and
+// the next layer's products over its first 128 inputs run while the second half's
+// activations are formed. Weights come in pieces of 128 x 128 (32 KB) through a ring of
+// three, each piece used by both tiles; one warp issues the copies, one the products.
+// With one tile per CTA, a whole layer's weights at a time and the steps one after another,
+// 4.0e5 rows of 66 - 3x256 - 200 took 0.373 ms; now 0.262 ms (608 TFLOP/s of the 1863 that a
+// dense product reaches; 65536 rows 83 -> 62 us, up to 16384 rows 33 -> 29 us). Half of that
+// came from the halves and the ring (0.327 ms), half from one 32-column accumulator load per
+// wait, biases from shared memory and input rows converted 8 columns at a time, before the
+// previous step's last outputs are stored. What is left is the chain of a layer's products,
+// read-back and activations: tensor pipe 38 % busy, issue slots 32 %.
 //
 // Operand layout in shared memory (no swizzle, K-major): 8-row x 16-byte core
-// matrices; the core holding (row r, column k) starts at (r/8)*SBO + (k/8)*128 bytes,
-// with SBO = (K/8)*128; inside it row r%8 is 16 bytes at (r%8)*16.
+// matrices; the core holding (row r, column k) starts at (r/8)*SBO + (k/8)*128 bytes;
+// inside it row r%8 is 16 bytes at (r%8)*16. SBO is 4096 for the activations and
+// (columns/8)*128 for a piece of weights.
 constexpr int kTcRows = 128;
-constexpr int kTcThreads = 1024;  // 32 warps: each reads its lane quarter of the
-                                  // accumulators, the column chunks shared by 8 warps
+constexpr int kTcTiles = 2;
+constexpr int kTcEpiWarps = 16;  // 4 lane quarters of the accumulators x 4 column groups
+constexpr int kTcThreads = 32 * (kTcEpiWarps + 2);
 constexpr int kTcMaxWidth = 256;
+constexpr int kTcHalf = 128;
 constexpr int kTcMaxOut = 4096;  // output layer: up to 16 chunks of 256 columns
+constexpr uint32_t kTcActSbo = (kTcMaxWidth / 8) * 128;
+constexpr uint32_t kTcActBytes = (kTcRows / 8) * kTcActSbo;  // 64 KB a tile
+constexpr uint32_t kTcPieceBytes = kTcHalf * kTcHalf * 2;
+constexpr int kTcRing = 3;
 // give up a wait after 4e9 SM clocks: 2 s at full clock (the clock register is read in a
 // few cycles, the global timer only slowly)
 constexpr long long kTcWaitClocks = 4000000000ll;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// element offset of (r, k) in a [rows][K] operand in the core-matrix layout
-__device__ __forceinline__ int core_off(int r, int k, int K) {
-  return (r >> 3) * (K << 3) + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
 }
 
 // shared-memory matrix descriptor: start, LBO (K direction) and SBO (row direction)
@@ -208,6 +224,25 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// 32 columns of a lane quarter with one wait
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
+      "%28, %29, %30, %31}, [%32];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+        "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
+        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
+        "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 // ---------------------------------------------------------------- layer kernels
@@ -642,239 +677,395 @@ struct TcNet {
   const float* b[kMaxLayers];   // padded biases
 };
 
-// weights [out_p][in_p] row-major -> the core-matrix layout (one thread per element)
+// A layer's weights [out_p][in_p] are packed piece by piece: rows in halves of 128, columns
+// in halves of 128, the pieces of a half of rows one after the other (row halves of the
+// wide output layer just go on). Elements before piece (rows from n0, columns from k0):
+__host__ __device__ constexpr size_t piece_start(int n0, int k0, int out_p, int in_p) {
+  return (size_t)n0 * in_p + (size_t)(out_p - n0 < kTcHalf ? out_p - n0 : kTcHalf) * k0;
+}
+
 __global__ void k_pack_weights(const bf16* w, int out_p, int in_p, bf16* out) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= (long long)out_p * in_p) return;
-  const int r = (int)(i / in_p), k = (int)(i % in_p);
-  out[core_off(r, k, in_p)] = w[i];
+  const int n = (int)(i / in_p), k = (int)(i % in_p);
+  const int n0 = n & ~(kTcHalf - 1), k0 = k & ~(kTcHalf - 1), r = n - n0, c = k - k0;
+  const int kp = in_p - k0 < kTcHalf ? in_p - k0 : kTcHalf;
+  out[piece_start(n0, k0, out_p, in_p) + (r >> 3) * (kp << 3) + (c >> 3) * 64 + (r & 7) * 8 +
+      (c & 7)] = w[i];
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) k_mlp_forward_tc(const __grid_constant__ TcNet net,
-                                                           const float* x, long long M,
-                                                           float* y, unsigned* err) {
+// Barriers of the fused forward; each but the ring's completes once per stage (a layer, or
+// a chunk of the output layer).
+struct TcBars {
+  uint64_t full[kTcRing], empty[kTcRing];  // weight pieces arrived / read by their products
+  uint64_t acc[2];    // first half's products done; all of the stage's products done
+  uint64_t ready[2];  // a half of the activations written (and its accumulators read)
+  uint32_t tmem_slot, failed;
+  alignas(16) float bias[2][kTcMaxWidth];  // of this stage and the next
+};
+
+__device__ __forceinline__ void mbar_init(uint64_t* bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(count));
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}\n" ::"r"(
+                   smem_addr(bar))
+               : "memory");
+}
+
+// A wait that also ends when another of the CTA's waits ran out.
+__device__ __forceinline__ bool tc_wait(TcBars* bars, uint64_t* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  const uint32_t addr = smem_addr(bar);
+  for (;;) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (*reinterpret_cast<volatile uint32_t*>(&bars->failed)) return false;
+    if (clock64() - t0 > kTcWaitClocks) {
+      *reinterpret_cast<volatile uint32_t*>(&bars->failed) = 1u;
+      return false;
+    }
+  }
+}
+
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+          smem_addr(bar))
+      : "memory");
+}
+
+// y[0 .. 31] of a row: 32-byte stores where the rows allow them, whole sectors each
+__device__ __forceinline__ void store_outputs(float* y, const float* v, int n, bool vec8) {
+  if (vec8) {
+#pragma unroll
+    for (int j = 0; j < 32; j += 8)
+      if (j < n)
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                         __cvta_generic_to_global(y + j)),
+                     "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]), "f"(v[j + 4]),
+                     "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7])
+                     : "memory");
+  } else {
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (j < n) y[j] = v[j];
+  }
+}
+
+constexpr int kTcAhead = 3;  // input items (8 columns of a row) a thread has in flight
+
+// tiles: 1 or 2 of 128 rows per step of a CTA
+__global__ void __launch_bounds__(kTcThreads, 1)
+    k_mlp_forward_tc(const __grid_constant__ TcNet net, const float* x, long long M, float* y,
+                     int tiles, unsigned* err) {
   extern __shared__ __align__(128) unsigned char tc_smem[];
-  bf16* sA = reinterpret_cast<bf16*>(tc_smem);                       // [128][256]
-  bf16* sB = sA + kTcRows * kTcMaxWidth;                             // [256][256]
-  float* sBias = reinterpret_cast<float*>(sB + kTcMaxWidth * kTcMaxWidth);  // [layers][256]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sBias + kMaxLayers * kTcMaxWidth);  // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 2);
+  unsigned char* sW = tc_smem + kTcTiles * kTcActBytes;
+  TcBars* bars = reinterpret_cast<TcBars*>(sW + kTcRing * kTcPieceBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // biases of every layer, zero in the padding columns
-  for (int i = tid; i < net.n_layers * kTcMaxWidth; i += kTcThreads) {
-    const int l = i / kTcMaxWidth, c = i % kTcMaxWidth;
-    sBias[i] = c < net.n_valid[l] ? net.b[l][c] : 0.0f;
+  if (tid == 0) {
+    for (int i = 0; i < kTcRing; ++i) {
+      mbar_init(&bars->full[i], 1);
+      mbar_init(&bars->empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bars->acc[i], 1);
+      mbar_init(&bars->ready[i], kTcEpiWarps);
+    }
+    bars->failed = 0u;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     smem_addr(tmem_slot)),
-                 "r"(kTcMaxWidth));
+                     smem_addr(&bars->tmem_slot)),
+                 "r"(kTcTiles * kTcMaxWidth));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-  }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar + 1)));
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t bar_a = smem_addr(bar);      // MMAs done
-  const uint32_t bar_w = smem_addr(bar + 1);  // weights arrived
-  uint32_t parity = 0, wparity = 0;
-  bool ok = true;
-  uint32_t pend = 0;  // after a wait ran out: the barrier still owed a completion
-  const long long n_tiles = (M + kTcRows - 1) / kTcRows;
-  for (long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-    const long long r0 = tile * kTcRows;
-    // the first layer's weights stream in while the input is converted
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      const int n0 = net.out_p[0] < kTcMaxWidth ? net.out_p[0] : kTcMaxWidth;
-      bulk_load(smem_addr(sB), net.w[0], (uint32_t)(n0 * net.in_p[0] * 2), bar_w);
-    }
-    // input rows -> BF16 activations: the tile's rows are contiguous in x, read
-    // coalesced; zero beyond the valid rows and in the padding columns
-    {
-      const int K = net.in_p[0], F = net.n_in;
-      const long long valid = M - r0 < kTcRows ? M - r0 : kTcRows;
-      const float* xt = x + r0 * F;
-      const int total = kTcRows * F, n_ok = (int)valid * F;
-      // row of element i: (i + 1/2)/F lies at least 1/(2F) >= 2^-9 from an integer
-      // and i < 2^15, so the FP32 product truncates to floor(i/F) exactly
-      const float inv_f = 1.0f / (float)F;
-      for (int i0 = tid; i0 < total; i0 += 4 * kTcThreads) {
-        float v[4];  // four loads in flight before the stores
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + u * kTcThreads;
-          v[u] = i < n_ok ? __ldg(&xt[i]) : 0.0f;
+  const uint32_t tmem = bars->tmem_slot;
+  const int step_rows = tiles * kTcRows;
+  const long long n_steps = (M + step_rows - 1) / step_rows;
+  const int L = net.n_layers;
+
+  if (warp == kTcEpiWarps) {
+    // ---- weights: every step's pieces in the order of their products
+    if (lane == 0) {
+      uint32_t piece = 0;
+      bool ok = true;
+      for (long long step = blockIdx.x; step < n_steps && ok; step += gridDim.x)
+        for (int l = 0; l < L && ok; ++l) {
+          const int N = net.out_p[l], K = net.in_p[l];
+          for (int n0 = 0; n0 < N && ok; n0 += kTcHalf)
+            for (int k0 = 0; k0 < K && ok; k0 += kTcHalf, ++piece) {
+              const uint32_t slot = piece % kTcRing, round = piece / kTcRing;
+              if (round > 0) ok = tc_wait(bars, &bars->empty[slot], (round - 1) & 1u);
+              if (ok)
+                bulk_load(smem_addr(sW + slot * kTcPieceBytes),
+                          net.w[l] + piece_start(n0, k0, N, K),
+                          (uint32_t)(min(kTcHalf, N - n0) * min(kTcHalf, K - k0) * 2),
+                          smem_addr(&bars->full[slot]));
+            }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + u * kTcThreads;
-          if (i < total) {
-            const int r = (int)(((float)i + 0.5f) * inv_f), k = i - r * F;
-            sA[core_off(r, k, K)] = __float2bfloat16(v[u]);
+      // copies still in flight land before the memory is given up: the last of each slot
+      for (uint32_t i = piece > kTcRing ? piece - kTcRing : 0; i < piece; ++i)
+        mbar_wait(smem_addr(&bars->full[i % kTcRing]), (i / kTcRing) & 1u);
+    }
+  } else if (warp == kTcEpiWarps + 1) {
+    // ---- products
+    if (lane == 0) {
+      uint32_t piece = 0, stage = 0;
+      bool ok = true;
+      for (long long step = blockIdx.x; step < n_steps && ok; step += gridDim.x)
+        for (int l = 0; l < L && ok; ++l) {
+          const int K = net.in_p[l];
+          for (int col0 = 0; col0 < net.out_p[l] && ok; col0 += kTcMaxWidth, ++stage) {
+            const int N = min(kTcMaxWidth, net.out_p[l] - col0);
+            ok = tc_wait(bars, &bars->ready[0], stage & 1u);
+            bool second = false;  // the second half's readiness waited for
+            for (int h = 0; h * kTcHalf < N && ok; ++h) {
+              const uint32_t idesc = tc_idesc(kTcRows, min(kTcHalf, N - h * kTcHalf));
+              for (int k0 = 0; k0 < K && ok; k0 += kTcHalf, ++piece) {
+                if (!second && (h > 0 || k0 > 0)) {
+                  ok = tc_wait(bars, &bars->ready[1], stage & 1u);
+                  second = true;
+                }
+                const uint32_t slot = piece % kTcRing;
+                ok = ok && tc_wait(bars, &bars->full[slot], (piece / kTcRing) & 1u);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const int kp = min(kTcHalf, K - k0);
+                const uint32_t b0 = smem_addr(sW + slot * kTcPieceBytes);
+                for (int t = 0; t < tiles; ++t) {
+                  const uint32_t a0 = smem_addr(tc_smem + t * kTcActBytes) + (uint32_t)k0 * 16u;
+                  for (int kk = 0; kk < kp / 16; ++kk)
+                    tc_mma(tmem + (uint32_t)(t * kTcMaxWidth + h * kTcHalf),
+                           tc_desc(a0 + kk * 256u, 128u, kTcActSbo),
+                           tc_desc(b0 + kk * 256u, 128u, (uint32_t)kp * 16u), idesc,
+                           k0 > 0 || kk > 0 ? 1u : 0u);
+                }
+                tc_commit(&bars->empty[slot]);
+              }
+              if (ok && h == 0) tc_commit(&bars->acc[0]);
+            }
+            if (ok && !second) ok = tc_wait(bars, &bars->ready[1], stage & 1u);
+            if (ok) tc_commit(&bars->acc[1]);
           }
         }
+      if (!ok) {  // let the products in flight land before the memory is given up
+        tc_commit(&bars->acc[1]);
+        mbar_wait(smem_addr(&bars->acc[1]), stage & 1u);
       }
-      if (tid < kTcRows)
-        for (int k = F; k < K; ++k) sA[core_off(tid, k, K)] = __float2bfloat16(0.0f);
     }
-    // stages: (layer, chunk of at most 256 output columns); only the output layer
-    // may have more than one chunk (its packed weight rows are contiguous per chunk)
-    for (int l = 0; l < net.n_layers && ok; ++l) {
-      const int K = net.in_p[l], Np = net.out_p[l];
-      const bool hidden = l < net.n_layers - 1;
-      const int n_chunks = (Np + kTcMaxWidth - 1) / kTcMaxWidth;
-      for (int ch = 0; ch < n_chunks && ok; ++ch) {
-        const int col0 = ch * kTcMaxWidth;                    // first output column
-        const int N = Np - col0 < kTcMaxWidth ? Np - col0 : kTcMaxWidth;
-        // this stage's weights (bulk copy issued earlier)
-        const bool got_w = mbar_wait(bar_w, wparity);
-        if (!__syncthreads_and(got_w)) {
-          if (tid == 0) atomicOr(err, 1u);
-          ok = false;
-          pend = bar_w;
-          const long long gr = r0 + tid;
-          if (tid < kTcRows && gr < M)
-            for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
-          break;
-        }
-        wparity ^= 1u;
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-          const uint32_t idesc = tc_idesc(kTcRows, N);
-          const uint32_t a0 = smem_addr(sA), b0 = smem_addr(sB);
-          const uint32_t sbo = (uint32_t)K * 16u;  // (K/8) cores of 128 bytes
-          for (int kk = 0; kk < K / 16; ++kk)
-            tc_mma(tmem, tc_desc(a0 + kk * 256u, 128u, sbo), tc_desc(b0 + kk * 256u, 128u, sbo),
-                   idesc, kk > 0 ? 1u : 0u);
-          asm volatile(
-              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                  bar_a)
-              : "memory");
-        }
-        const bool waited = mbar_wait(bar_a, parity);
-        if (!__syncthreads_and(waited)) {  // the MMAs never signalled completion
-          if (tid == 0) atomicOr(err, 1u);
-          ok = false;
-          pend = bar_a;
-          const long long gr = r0 + tid;
-          if (tid < kTcRows && gr < M)
-            for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
-          break;
-        }
-        parity ^= 1u;
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        // the weight buffer is free: the next stage's weights stream in meanwhile
-        // (after a single-chunk output layer the buffer stages the outputs instead)
-        if (tid == 0) {
-          if (ch + 1 < n_chunks) {
-            const int n1 = Np - col0 - kTcMaxWidth < kTcMaxWidth ? Np - col0 - kTcMaxWidth
-                                                                : kTcMaxWidth;
-            bulk_load(smem_addr(sB), net.w[l] + (size_t)(col0 + kTcMaxWidth) * K,
-                      (uint32_t)(n1 * K * 2), bar_w);
-          } else if (hidden) {
-            const int n1 = net.out_p[l + 1] < kTcMaxWidth ? net.out_p[l + 1] : kTcMaxWidth;
-            bulk_load(smem_addr(sB), net.w[l + 1], (uint32_t)(n1 * net.in_p[l + 1] * 2), bar_w);
-          }
-        }
-        // accumulators of this warp's 32 rows: bias, activation, next operand or output
-        const int quarter = warp & 3;                 // lanes 32 quarter .. of the accumulators
-        const int row = quarter * 32 + lane;
-        const int group = warp >> 2, n_groups = kTcThreads / 128;
-        const float* bias = sBias + l * kTcMaxWidth;
-        // a single-chunk output layer is staged over both operand buffers (the last MMA
-        // is done) with an odd row stride, so that the 32 rows a warp stores hit 32
-        // different banks; wider output layers are stored from registers per chunk
-        const int o_stride = net.n_out | 1;
-        float* so = reinterpret_cast<float*>(sA);
-        const long long grow = r0 + row;
-        const bool vec4 = (net.n_out & 3) == 0;
-        for (int c0 = 16 * group; c0 < N; c0 += 16 * n_groups) {
-          float v[16];
-          tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
-          float bv[16];
-          if (n_chunks == 1) {
+  } else {
+    // ---- input, activations and outputs
+    const int quarter = warp & 3, row_in = quarter * 32 + lane, group = warp >> 2;
+    const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+    const int F = net.n_in, K0 = net.in_p[0];
+    const bool vec8 = (net.n_out & 7) == 0 && (reinterpret_cast<uintptr_t>(y) & 31) == 0;
+    const int total = step_rows * F;  // a step's rows are contiguous in x
+    const bool pairs = (F & 1) == 0 && (reinterpret_cast<uintptr_t>(x) & 7) == 0;
+    // an item is 8 columns of a row; the row of item i: (i + 1/2)/(K0/8) lies at least
+    // 1/(2 * 32) from an integer and i < 2^13, so the FP32 product truncates to it exactly
+    const int row_items = K0 >> 3;
+    const float inv_items = 1.0f / (float)row_items;
+    // the rows of a later step on their way to L2 meanwhile
+    auto fetch = [&](long long step) {
+      const char* xs = reinterpret_cast<const char*>(x + step * step_rows * F);
+      const long long left = (M - step * step_rows) * F;
+      const int bytes = 4 * (left < total ? (int)left : total);
+      for (int o = 128 * tid; o < bytes; o += 128 * 32 * kTcEpiWarps)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(xs + o)));
+    };
+    // input rows -> BF16 activations, zero beyond the valid rows and in the padding columns:
+    // 16 bytes of a core matrix at a time
+    auto input = [&](long long step) {
+      for (int i0 = tid; i0 < step_rows * row_items; i0 += kTcAhead * 32 * kTcEpiWarps) {
+        float v[kTcAhead][8];  // loads in flight before the stores
 #pragma unroll
-            for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(&bv[j]) =
-                *reinterpret_cast<const float4*>(&bias[c0 + j]);
-          } else {
+        for (int u = 0; u < kTcAhead; ++u) {
+          const int i = i0 + u * 32 * kTcEpiWarps;
+          const int r = (int)(((float)i + 0.5f) * inv_items), k = (i - r * row_items) * 8;
+          const bool in = r < step_rows && step * step_rows + r < M;
+          const float* xr = x + (step * step_rows + r) * F + k;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int c = col0 + c0 + j;
-              bv[j] = c < net.n_valid[l] ? __ldg(&net.b[l][c]) : 0.0f;
-            }
-          }
-          if (hidden) {
-            uint32_t h[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const __nv_bfloat162 p =
-                  __floats2bfloat162_rn(silu_fast(v[2 * j] + bv[2 * j]),
-                                        silu_fast(v[2 * j + 1] + bv[2 * j + 1]));
-              h[j] = *reinterpret_cast<const uint32_t*>(&p);
-            }
-            // columns c0..c0+15 of this row: two 16-byte pieces of the next operand
-            *reinterpret_cast<uint4*>(&sA[core_off(row, c0, N)]) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(&sA[core_off(row, c0 + 8, N)]) =
-                make_uint4(h[4], h[5], h[6], h[7]);
-          } else if (n_chunks == 1) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int c = c0 + j;
-              if (c < net.n_out) so[row * o_stride + c] = v[j] + bv[j];
-            }
-          } else if (grow < M) {
-            float* yr = y + grow * net.n_out + col0 + c0;
-            if (vec4 && col0 + c0 + 16 <= net.n_out) {
-#pragma unroll
-              for (int j = 0; j < 16; j += 4)
-                *reinterpret_cast<float4*>(&yr[j]) =
-                    make_float4(v[j] + bv[j], v[j + 1] + bv[j + 1], v[j + 2] + bv[j + 2],
-                                v[j + 3] + bv[j + 3]);
+          for (int j = 0; j < 8; j += 2) {
+            float2 e = make_float2(0.0f, 0.0f);
+            if (pairs) {
+              if (in && k + j < F) e = __ldg(reinterpret_cast<const float2*>(xr + j));
             } else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j)
-                if (col0 + c0 + j < net.n_out) yr[j] = v[j] + bv[j];
+              if (in && k + j < F) e.x = __ldg(xr + j);
+              if (in && k + j + 1 < F) e.y = __ldg(xr + j + 1);
             }
+            v[u][j] = e.x;
+            v[u][j + 1] = e.y;
           }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();
-        if (!hidden && n_chunks == 1) {  // the tile's output rows are contiguous in y
-          const long long valid = M - r0 < kTcRows ? M - r0 : kTcRows;
-          float* yt = y + r0 * net.n_out;
-          for (int r = warp; r < (int)valid; r += kTcThreads / 32)
-            for (int c = lane; c < net.n_out; c += 32)
-              yt[(long long)r * net.n_out + c] = so[r * o_stride + c];
-          __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kTcAhead; ++u) {
+          const int i = i0 + u * 32 * kTcEpiWarps;
+          const int r = (int)(((float)i + 0.5f) * inv_items), k = (i - r * row_items) * 8;
+          if (r >= step_rows) continue;
+          uint32_t h[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const __nv_bfloat162 p = __floats2bfloat162_rn(v[u][2 * j], v[u][2 * j + 1]);
+            h[j] = *reinterpret_cast<const uint32_t*>(&p);
+          }
+          *reinterpret_cast<uint4*>(tc_smem + (r >> 7) * kTcActBytes +
+                                    ((r & 127) >> 3) * kTcActSbo + (k >> 3) * 128 + (r & 7) * 16) =
+              make_uint4(h[0], h[1], h[2], h[3]);
         }
       }
+    };
+    auto written = [&](int half) {  // this warp's part of a half is in place
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->ready[half]);
+    };
+    uint32_t stage = 0;
+    bool ok = true;
+    long long step = blockIdx.x;
+    if (step < n_steps) {
+      input(step);
+      written(0);
+      written(1);
+    }
+    for (; step < n_steps && ok; step += gridDim.x) {
+      const bool more = step + gridDim.x < n_steps;
+      for (int l = 0; l < L && ok; ++l) {
+        const bool hidden = l + 1 < L;
+        if (l == 0 && more) fetch(step + gridDim.x);
+        for (int col0 = 0; col0 < net.out_p[l] && ok; col0 += kTcMaxWidth, ++stage) {
+          const int N = min(kTcMaxWidth, net.out_p[l] - col0);
+          const bool last = !hidden && col0 + kTcMaxWidth >= net.out_p[l];
+          // this warp's 32 columns of half h: accumulators + bias (zero in the padding)
+          auto columns = [&](int h, int t, float* v) {
+            const int c = h * kTcHalf + group * 32;
+            tmem_ld32(tmem + lanes + (uint32_t)(t * kTcMaxWidth + c), v);
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+              const float4 b = *reinterpret_cast<const float4*>(&bars->bias[stage & 1][c + j]);
+              v[j] += b.x;
+              v[j + 1] += b.y;
+              v[j + 2] += b.z;
+              v[j + 3] += b.w;
+            }
+          };
+          auto outputs = [&](int h) {
+            const int c = col0 + h * kTcHalf + group * 32;
+#pragma unroll 1
+            for (int t = 0; t < tiles; ++t) {
+              float v[32];
+              columns(h, t, v);
+              const long long row = step * step_rows + t * kTcRows + row_in;
+              if (row < M) store_outputs(y + row * net.n_out + c, v, net.n_out - c, vec8);
+            }
+          };
+          auto activations = [&](int h, uint32_t* q) {  // 16 pairs a tile
+#pragma unroll
+            for (int t = 0; t < kTcTiles; ++t) {
+              if (t >= tiles) break;
+              float v[32];
+              columns(h, t, v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const __nv_bfloat162 p =
+                    __floats2bfloat162_rn(silu_fast(v[2 * j]), silu_fast(v[2 * j + 1]));
+                q[16 * t + j] = *reinterpret_cast<const uint32_t*>(&p);
+              }
+            }
+          };
+          auto place = [&](int h, const uint32_t* q) {
+            const int c = h * kTcHalf + group * 32;
+#pragma unroll
+            for (int t = 0; t < kTcTiles; ++t) {
+              if (t >= tiles) break;
+              unsigned char* a = tc_smem + t * kTcActBytes + (row_in >> 3) * kTcActSbo +
+                                 (row_in & 7) * 16 + (c >> 3) * 128;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (c + 8 * j < N)
+                  *reinterpret_cast<uint4*>(a + j * 128) =
+                      make_uint4(q[16 * t + 4 * j], q[16 * t + 4 * j + 1], q[16 * t + 4 * j + 2],
+                                 q[16 * t + 4 * j + 3]);
+            }
+          };
+          const bool mine0 = group * 32 < N, mine1 = kTcHalf + group * 32 < N;
+          uint32_t q[32];
+          // the biases of this warp's columns (the four warps of a group write the same)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int c = h * kTcHalf + group * 32 + lane;
+            bars->bias[stage & 1][c] =
+                col0 + c < net.out_p[l] ? __ldg(&net.b[l][col0 + c]) : 0.0f;
+          }
+          __syncwarp();
+          ok = __all_sync(0xffffffffu, tc_wait(bars, &bars->acc[0], stage & 1u));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          if (hidden) {
+            if (mine0) activations(0, q);
+          } else {
+            if (mine0) outputs(0);
+            if (!last) written(0);
+          }
+          // the second half's products read the layer's input to their end
+          ok = __all_sync(0xffffffffu, tc_wait(bars, &bars->acc[1], stage & 1u));
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          if (hidden) {
+            if (mine0) place(0, q);
+            written(0);
+            if (mine1) {
+              activations(1, q);
+              place(1, q);
+            }
+            written(1);
+          } else {
+            // every product that read the activations is done: the next step's input goes in
+            // first, so that its products start while these outputs are stored
+            if (last && more) {
+              input(step + gridDim.x);
+              written(0);
+            }
+            if (mine1) outputs(1);
+            if (!last || more) written(1);
+          }
+        }
+      }
+    }
+    if (!ok) {  // a wait ran out: the rows of this and the later steps are not to be used
+      if (tid == 0) atomicOr(err, 1u);
+      for (long long s = step; s < n_steps; s += gridDim.x)
+        for (int t = 0; t < tiles; ++t) {
+          const long long row = s * step_rows + t * kTcRows + row_in;
+          if (group == 0 && row < M)
+            for (int c = 0; c < net.n_out; ++c)
+              y[row * net.n_out + c] = __int_as_float(0x7fc00000);
+        }
     }
   }
-  // after a wait that ran out: let the weight copy or the MMAs still in flight land
-  // (again with a time limit) before the shared and tensor memory are released
-  if (pend != 0 && warp == 0) mbar_wait(pend, pend == bar_w ? wparity : parity);
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
-                 "r"(kTcMaxWidth));
+                 "r"(kTcTiles * kTcMaxWidth));
   }
 }
 
 size_t tc_smem_bytes() {
-  return sizeof(bf16) * (size_t)(kTcRows + kTcMaxWidth) * kTcMaxWidth +
-         sizeof(float) * kMaxLayers * kTcMaxWidth + 32;
+  return kTcTiles * kTcActBytes + kTcRing * kTcPieceBytes + sizeof(TcBars);
 }
 
 inline unsigned nb(long long n, int t);
@@ -1021,9 +1212,13 @@ rt_status forward_tc(rt_mlp* m, const float* x, float* y, long long M, cudaStrea
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->dev) != cudaSuccess)
     return RT_ERR_CUDA;
-  const long long tiles = (M + kTcRows - 1) / kTcRows;
-  const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
-  k_mlp_forward_tc<<<grid, kTcThreads, smem, s>>>(net, x, M, y, m->d_err);
+  // two tiles a step where there are more tiles than SMs, else one (more CTAs, no overlap
+  // to gain between tiles)
+  const long long n_tiles = (M + kTcRows - 1) / kTcRows;
+  const int tiles = n_tiles > sms ? kTcTiles : 1;
+  const long long steps = (n_tiles + tiles - 1) / tiles;
+  const unsigned grid = (unsigned)(steps < sms ? steps : sms);
+  k_mlp_forward_tc<<<grid, kTcThreads, smem, s>>>(net, x, M, y, tiles, m->d_err);
   return cudaGetLastError() == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }
 
