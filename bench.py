@@ -383,8 +383,8 @@ def path_walk_runs(walk, N, S, L, n_slots, images=False):
         if 32 * N > 4e9:
             return True
         # a block turns one cell into eight: N = n^3 + 7 blocks, slots = n^3 + 8 blocks
-        refined = 8 * (n_slots - N) > 0.5 * N
-        return S == 4 and not (refined and 48 * N <= 0.5e9)
+        refined = 8 * (n_slots - N) / N
+        return S == 4 and (refined <= 0.5 or 48 * N > (0.7 * refined - 0.2) * 1e9)
     return walk == 2
 
 

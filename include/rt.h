@@ -91,9 +91,13 @@ typedef struct rt_run_opts {
     uint64_t max_events;    /* interactions per package before it is capped; 0: 1e7 */
     int32_t blocks_per_sm;  /* pool: resident blocks per SM; 0: from occupancy */
     int32_t threads;        /* threads per block, multiple of 32; 0: 256 */
-    int32_t refill_period;  /* pool: steps between refills of dead lanes; 0: 32 */
-    int32_t interaction_batch; /* pool: lanes of a warp waiting at an interaction
-                               point that start an interaction phase, 1..32; 0: 8 */
+    int32_t refill_period;  /* pool: rounds (of a few cells) between looks at the time
+                               budget, with path-length tallies also between refills of
+                               dead lanes; 0: 32 */
+    int32_t interaction_batch; /* pool: twice the idle lanes of a warp that make it look
+                               for work; with path-length tallies the lanes waiting at an
+                               interaction point that start an interaction phase, 1..32;
+                               0: 8 */
     double budget_s;        /* device time budget per launch in s; 0: 120 */
     int32_t estimators;     /* RT_EST_* bits: extra tallies kept during the launch */
     int32_t count_scale;    /* BW / no-correction: an absorption that finds n earlier

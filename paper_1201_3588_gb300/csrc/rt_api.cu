@@ -190,18 +190,19 @@ static bool path_walk_fits(const rt_grid_desc* d) {
 // reads 32-byte records and, for more than two species, a row of densities.
 //  - Two species (densities in the record), and species counts without a compiled path
 //    walk: linked until the records exceed 4 GB.
-//  - Four species: linked where most cells sit in refined blocks and records and densities
-//    are within 0.5 GB, a few times L2. 1e7 packages, linked and path: 8.0e6 cells, all but
-//    a tenth refined, 16.2 and 22.1 ms; 6.0e6 cells, a third refined, 21.8 and 21.0; 1.9e7
-//    cells, refined (0.9 GB), 40.7 and 34.6; 2.6e7 cells 46.8 and 36.0; 5.4e7 cells 84.6
-//    and 52.9.
+//  - Four species: linked where more than half of the cells, a fraction f, sit in refined
+//    blocks (where the path walk descends most) and the records and densities are within
+//    0.7 f - 0.2 GB. 1e7 packages, linked and path, ms: f = 1: 0.43 GB 15.2 and 17.6, 0.49 GB 18.4 and 18.4,
+//    0.61 GB 22.4 and 19.7, 0.94 GB 36.2 and 23.1, 2.5 GB 48.2 and 33.7; f = 0.55: 0.02 GB
+//    5.4 and 8.1, 0.16 GB 12.3 and 12.7, 0.23 GB 15.0 and 14.3, 0.31 GB 20.4 and 16.4;
+//    f = 0: 0.01 GB 4.6 and 4.6, 0.05 GB 7.1 and 6.2, 0.16 GB 14.9 and 8.1.
 static bool path_walk_auto(const rt_grid_desc* d) {
   if (!path_walk_fits(d)) return false;
   const double rec = 4.0 * kRec * (double)d->n_leaves;
   if (rec > 4.0e9) return true;
   if (d->n_species != 4) return false;
-  const bool refined = 8.0 * (double)d->n_blocks > 0.5 * (double)d->n_leaves;
-  return !(refined && rec + 16.0 * (double)d->n_leaves <= 0.5e9);
+  const double refined = 8.0 * (double)d->n_blocks / (double)d->n_leaves;
+  return refined <= 0.5 || rec + 16.0 * (double)d->n_leaves > (0.7 * refined - 0.2) * 1e9;
 }
 
 void free_all(rt_grid* g) {

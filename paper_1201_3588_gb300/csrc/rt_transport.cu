@@ -218,9 +218,17 @@ struct LaneTally {
 constexpr int kTallyWords = 16;  // per warp: kNumCounters words
 static_assert(kNumCounters <= kTallyWords, "the counters fit a warp's words");
 
-// a flush is forced once a counter passes 2^30: one round of the pool adds at most
-// 32 x refill_period to a warp's
+// a flush is forced once a counter passes 2^30: between two looks at them the pool adds at
+// most 32 x 2^24 to a warp's and kWalkSteps x 2^24 to a lane's
 constexpr unsigned kTallyFlushAt = 1u << 30;
+
+// Cells a lane crosses at most before the warp looks whether lanes are idle: looking costs
+// every lane some 25 instructions, waiting for the others costs the idle ones. 5e6 packages
+// through the disk of 2.4e6 cells, 1, 2, 4, 8 and 12 cells: 3.85, 3.59, 3.25, 3.13 and 3.13
+// ms (unrolled by two 3.21, which the grids beyond L2 gain from: 13.7 against 14.2 ms for
+// 8.0e6 cells of four species); 7.3 to 5.3 warp instructions per crossing. With the
+// path-length tally two: see pool_warp.
+constexpr int kWalkSteps = 8, kTallySteps = 2;
 
 enum Adv { kCrossed = 0, kInteract = 1, kEscaped = 2, kError = 3 };
 
@@ -575,42 +583,44 @@ __device__ __forceinline__ int advance_linked(Pkg<float>& k, Cell& c, const DevG
     c.leaf = link;
     return kCrossed;
   }
-  if (link >= 0) {  // a coarser leaf: round the corner down to its edge (exact)
+  if (link >= 0) {  // a leaf of the same size or coarser: round the corner down to its edge
     c.leaf = link & kLinkLeafMask;
     const int bits = __float_as_int(c.sz) + ((link >> 28) << 23);
     c.sz = __int_as_float(bits);
-    const float isz = __int_as_float((254 << 23) - bits);
+    // exact: adding 1.5 * 2^23 edges (corners lie below 2^18 of them) leaves multiples of one
+    const float big = __int_as_float(bits + (23 << 23) + (1 << 22));
 #pragma unroll
-    for (int a = 0; a < 3; ++a) c.lo[a] = floorf(c.lo[a] * isz) * c.sz;
+    for (int a = 0; a < 3; ++a) c.lo[a] = __fadd_rd(c.lo[a], big) - big;
     return kCrossed;
   }
   if (link == kLinkEscape) return kEscaped;
-  // the same-size neighbour is split: descend, staying inside that node
-  int lev = c.level();
-  const float iz = __int_as_float((127 + lev) << 23);  // 2^level
-  int J[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) J[a] = (int)(c.lo[a] * iz);
-  long long blk = -(long long)link - 1;
+  // the same-size neighbour is split: descend, staying inside that node (on the side of
+  // each middle that the position is on). A step of a warp has a lane here more often than
+  // not, so this is kept short: in integers with conversions, and floorf above, 5e6
+  // packages through the disk took 3.93 ms against 3.85.
+  int code = link, left = g.max_level - c.level();
+  float h = c.sz;
   for (;;) {
-    if (blk >= g.n_blocks || lev >= g.max_level) return kError;
-    ++lev;
+    const int blk = -code - 1;
+    if (blk >= g.n_blocks || left-- <= 0) return kError;
     ++child_reads;
-    const float sc = __int_as_float((127 + lev) << 23);
+    h *= 0.5f;
     unsigned oct = mirrored(k);  // a mirrored axis numbers its children backwards
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      J[a] = min(max(__float2int_rd(k.p[a] * sc), 2 * J[a]), 2 * J[a] + 1);
-      oct ^= (unsigned)(J[a] & 1) << a;
+      const float mid = c.lo[a] + h;
+      if (k.p[a] >= mid) {
+        c.lo[a] = mid;
+        oct ^= 1u << a;
+      }
     }
-    const int node = __ldg(&g.child[blk * 8 + oct]);
-    if (node >= 0) {
-      if ((long long)node >= g.n_leaves) return kError;
-      c.leaf = node;
-      set_corner(c, J, lev);
+    code = __ldg(&g.child[(size_t)blk * 8 + oct]);
+    if (code >= 0) {
+      if ((long long)code >= g.n_leaves) return kError;
+      c.leaf = code;
+      c.sz = h;
       return kCrossed;
     }
-    blk = -(long long)node - 1;
   }
 }
 
@@ -1206,22 +1216,125 @@ struct ModelIds {
   }
 };
 
-// One warp of the packet pool: each lane owns a package slot; dead lanes are refilled
-// with indices below n_end every `refill_period` steps. A lane that reaches its
-// interaction point waits; the warp runs the (long, divergent) interaction code only
-// once `interaction_batch` lanes wait or no lane is left walking, so both phases run
-// with most lanes active. Each package's history is unchanged by this schedule.
+// ---------------------------------------------------------------- parked packages
+// kPlaces places per warp in shared memory for packages that no lane is walking: a vector of
+// 16 bytes per place and part, so that lanes using neighbouring places never conflict.
+// Parts 0-3: position and tau; direction and bin; event, id, dirs and level; leaf and
+// corner. The path walk adds its block ids (part 4) and, in 8 bytes, the last of them and
+// the leaf's extinction. The reciprocals of the direction are computed again.
+constexpr int kPlaces = 32;
+
+template <bool kPath>
+__host__ __device__ constexpr int park_bytes() {  // per warp
+  return kPlaces * (kPath ? 16 * 5 + 8 : 16 * 4);
+}
+
+__device__ __forceinline__ uint4 park_pack(int v, const Pkg<float>& k, int leaf, const float lo[3],
+                                           int level) {
+  const auto u = [](float x) { return (unsigned)__float_as_int(x); };
+  if (v == 0) return make_uint4(u(k.p[0]), u(k.p[1]), u(k.p[2]), u(k.tau));
+  if (v == 1) return make_uint4(u(k.d[0]), u(k.d[1]), u(k.d[2]), (unsigned)k.bin);
+  if (v == 2)
+    return make_uint4(k.event, (unsigned)k.id, (unsigned)(k.id >> 32),
+                      k.dirs | (unsigned)level << 27);
+  return make_uint4((unsigned)leaf, u(lo[0]), u(lo[1]), u(lo[2]));
+}
+
+// A lane's package to place `dst` (store) and place `src` to the lane (load); places left
+// by loading lanes may be among those stored to.
+template <bool kPath, class CellT>
+__device__ __forceinline__ void park_exchange(uint4* park, Pkg<float>& k, CellT& c, bool load,
+                                              int src, bool store, int dst) {
+  const auto f = [](unsigned x) { return __int_as_float((int)x); };
+#pragma unroll
+  for (int v = 0; v < (kPath ? 6 : 4); ++v) {
+    uint4 x = make_uint4(0, 0, 0, 0), y = x;
+    uint2* last = reinterpret_cast<uint2*>(park + 5 * kPlaces);
+    if (load) {
+      if (v < 5) {
+        x = park[v * kPlaces + src];
+      } else {
+        const uint2 w = last[src];
+        x.x = w.x;
+        x.y = w.y;
+      }
+    }
+    __syncwarp();
+    if constexpr (kPath) {
+      if (v < 4) y = park_pack(v, k, c.slot, c.lo, c.level());
+      else if (v == 4) y = make_uint4(c.b0, c.b1, c.b2, c.b3);
+      else y = make_uint4(c.b4, (unsigned)__float_as_int(c.kx), 0, 0);
+    } else {
+      y = park_pack(v, k, c.leaf, c.lo, c.level());
+    }
+    if (store) {
+      if (v < 5)
+        park[v * kPlaces + dst] = y;
+      else
+        last[dst] = make_uint2(y.x, y.y);
+    }
+    if (load) {
+      if (v == 0) {
+        k.p[0] = f(x.x), k.p[1] = f(x.y), k.p[2] = f(x.z), k.tau = f(x.w);
+      } else if (v == 1) {
+        k.d[0] = f(x.x), k.d[1] = f(x.y), k.d[2] = f(x.z), k.bin = (int)x.w;
+      } else if (v == 2) {
+        k.event = x.x;
+        k.id = (unsigned long long)x.z << 32 | x.y;
+        k.dirs = x.w & 0x07ffffffu;
+      } else if (v == 3) {
+        c.lo[0] = f(x.y), c.lo[1] = f(x.z), c.lo[2] = f(x.w);
+        if constexpr (kPath) c.slot = (int)x.x;
+        else c.leaf = (int)x.x;
+      }
+      if constexpr (kPath) {
+        if (v == 4) c.b0 = (int)x.x, c.b1 = (int)x.y, c.b2 = (int)x.z, c.b3 = (int)x.w;
+        if (v == 5) c.b4 = (int)x.x, c.kx = f(x.y);
+      }
+    }
+    // the level travels in part 2, the edge it gives is read by the packing above
+    if (v == 2 && load) c.sz = __int_as_float((int)(127u - (x.w >> 27)) << 23);
+  }
+  __syncwarp();
+}
+
+// One warp of the packet pool. Lanes walk; a lane whose package reaches its interaction
+// point or leaves the domain is idle. Once `batch` lanes are idle (or none walks) the warp
+// finds them work, the first of these that applies:
+//  - 32 packages wait for their interaction, in lanes or parked: all lanes take one
+//    (walking packages are parked as ready) and the long, divergent interaction code runs
+//    with a full warp; afterwards every lane walks on with what it has;
+//  - packages are parked ready to walk: idle lanes take them, waiting ones are parked;
+//  - the source is not dry: waiting packages are parked, the idle lanes filled with new ones;
+//  - near the end of the source: interactions as soon as `batch` packages wait.
+// batch: half of `interaction_batch` (8: 4 idle lanes of 32). Each package's history is
+// unchanged by this schedule. With a package bound to its lane (waiting in place for eight
+// others, dead lanes refilled every 32 steps) half of the lanes idled, and the interaction
+// code ran with a quarter of them. Bound and parked, both walking eight cells at a time, ms:
+// disk of 2.4e6 cells, 5e6 packages 3.45 and 3.21; 8.0e6 cells of four species, 1e7
+// packages 15.4 and 13.7; disk with images 1.41 and 1.22; 24 models in a batch 6.44 and
+// 5.87; 1e5 packages in a small sphere 0.083 and 0.085. (Bound and one cell at a time: 4.06,
+// 17.7, 1.66, 7.09, 0.090.) 8, 16, 24 and 32 places, one cell at a time: 4.41, 4.09, 3.90
+// and 3.85 ms for the disk; 2 KB a warp for 32 still leave L1 most of its room.
+//
+// kTally: packages stay bound to their lanes, dead lanes are refilled every `refill_period`
+// rounds and `interaction_batch` lanes start an interaction phase. An FP32 tally of a cell
+// that 1e5 packages cross loses increments below half a unit of its last place (1e-3 of a
+// sum next to the source) unless the lanes that cross it together are combined first, as
+// they are when they start together: the parked schedule would change that sum by 1e-4 of
+// it. The tally's reductions bound these launches anyway (2.60 parked, 2.67 ms bound).
 // Absorptions of lanes hitting the same (species, cell) in one phase are merged into
 // one atomic. `sed` is the escaped-spectrum histogram (shared or global memory).
 // kPeel: scatterings and re-emissions at image bins are recorded (position, w,
 // bin) in the peel-off event buffer, one slot range per warp and phase; point-source
 // emissions are counted per bin in s_nemit. wt: the warp's counters (shared memory, zero
-// at the start; lane 0 or atomics). Returns false when the time budget ran out.
+// at the start; lane 0 or atomics). park: the warp's places. Time budget and counters are
+// looked at every `refill_period` steps. Returns false when the time budget ran out.
 template <bool kPeel, class Ids, int kS = 0, bool kPath = false, bool kTally = false>
 __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, const DevRun& r,
                                           const Kappa* kap, const float* star_cdf,
                                           unsigned long long* sed, unsigned long long n_end,
-                                          Ids& ids, LaneTally& tl, unsigned* wt,
+                                          Ids& ids, LaneTally& tl, unsigned* wt, uint4* park,
                                           unsigned long long t0, const DevPeel* pe = nullptr,
                                           unsigned long long* s_nemit = nullptr,
                                           const float* kext = nullptr,
@@ -1232,61 +1345,75 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
   Pkg<float> k;
   k.id = 0;
   k.dirs = 0;
-  bool alive = false;
-  bool pending = false;  // reached an interaction point, waiting for the batch
-  // a lane that left the domain is put into the spectrum at the next refill, with the
-  // others: until then it is dead with tau = -1
+  bool walking = false;
+  bool pending = false;  // reached an interaction point
+  // a lane that left the domain is put into the spectrum with the next ones to become
+  // idle: until then tau = -1
   k.tau = 0.f;
   // kPath: the path walk (densities from the density array, kI = -kS for the
   // interaction); otherwise the linked walk
   using CellT = typename std::conditional<kPath, PathCell, Cell>::type;
   constexpr int kI = kPath ? -kS : kS;
+  constexpr bool kPark = !kTally;
+  constexpr int kSteps = kTally ? kTallySteps : kWalkSteps;
   CellT cell{};
   cell.sz = 1.f;
-  const int K = r.refill_period > 0 ? r.refill_period : 32;
-  const int batch = r.interaction_batch > 0 ? r.interaction_batch : 8;
+  const int K = r.refill_period > 0 ? min(r.refill_period, 1 << 24) : 32;
+  const int n_lanes = r.interaction_batch > 0 ? r.interaction_batch : 8;
+  const int batch = kPark ? (n_lanes + 1) / 2 : n_lanes;
+  // parked: waiting for their interaction (places 0 ..), ready to walk (the last ones down)
+  int n_wait = 0, n_ready = 0;
+  bool dry = false;  // no packages left to draw
 
-  for (;;) {
+  // packages that left the domain since into the spectrum
+  auto book = [&]() {
     if (k.tau < 0.f) {
       k.tau = 0.f;
       const int db = dir_bin(true_component(k, k.d[2], 2), g.n_dir);
       atomicAdd(&sed[db * B + k.bin], 1ull);
       if (k.event == 0) atomicAdd(&sed[(g.n_dir + db) * B + k.bin], 1ull);
     }
-    unsigned dead = __ballot_sync(kFull, !alive);
-    if (dead) {
-      const int nd = __popc(dead);
-      const unsigned long long j =
-          ids.take(nd, __popc(dead & lt_mask), lane, __ffs(dead) - 1);
-      const unsigned fresh = __ballot_sync(kFull, !alive && j < n_end);
-      if (lane == 0) wt[kCEmitted] += __popc(fresh);
-      if (!alive) {
-        if (j < n_end) {
-          emit<float>(k, r.first_id + j, r, star_cdf, B);
-          if constexpr (kPeel) {
-            if (r.source_kind != 1) atomicAdd(&s_nemit[k.bin], 1ull);
-          }
-          int rc;
-          if constexpr (kPath)
-            rc = enter_path(k, g, cell, tl.levels);
-          else
-            rc = enter(k, g, cell, tl.levels);
-          if (rc == 0) {
-            alive = true;
-            if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kap, kext);
-          } else if (rc == 1) {  // source outside the grid, moving away
-            atomicAdd(&wt[kCEscaped], 1u);
-            const int db = dir_bin(k.d[2], g.n_dir);
-            atomicAdd(&sed[db * B + k.bin], 1ull);
-            atomicAdd(&sed[(g.n_dir + db) * B + k.bin], 1ull);
-          } else {
-            atomicAdd(&wt[kCErrors], 1u);
-            atomicOr(r.status, kStatusTree);
-          }
-        }
+  };
+  // new packages for the lanes `dead`
+  auto fill = [&](unsigned dead) {
+    const bool mine = (dead >> lane) & 1u;
+    const unsigned long long j =
+        ids.take(__popc(dead), __popc(dead & lt_mask), lane, __ffs(dead) - 1);
+    const unsigned fresh = __ballot_sync(kFull, mine && j < n_end);
+    dry = fresh != dead;
+    if (lane == 0) wt[kCEmitted] += __popc(fresh);
+    if (mine && j < n_end) {
+      emit<float>(k, r.first_id + j, r, star_cdf, B);
+      if constexpr (kPeel) {
+        if (r.source_kind != 1) atomicAdd(&s_nemit[k.bin], 1ull);
+      }
+      int rc;
+      if constexpr (kPath)
+        rc = enter_path(k, g, cell, tl.levels);
+      else
+        rc = enter(k, g, cell, tl.levels);
+      if (rc == 0) {
+        walking = true;
+        if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kap, kext);
+      } else if (rc == 1) {  // source outside the grid, moving away
+        atomicAdd(&wt[kCEscaped], 1u);
+        const int db = dir_bin(k.d[2], g.n_dir);
+        atomicAdd(&sed[db * B + k.bin], 1ull);
+        atomicAdd(&sed[(g.n_dir + db) * B + k.bin], 1ull);
+      } else {
+        atomicAdd(&wt[kCErrors], 1u);
+        atomicOr(r.status, kStatusTree);
       }
     }
-    if (!__any_sync(kFull, alive)) return true;
+  };
+
+  for (;;) {
+    if constexpr (!kPark) {
+      book();
+      const unsigned dead = __ballot_sync(kFull, !walking && !pending);
+      if (dead && !dry) fill(dead);
+      if (!__any_sync(kFull, walking || pending)) return true;
+    }
     if (__any_sync(kFull, tl.crossings >= kTallyFlushAt || tl.levels >= kTallyFlushAt ||
                               wt[lane & (kTallyWords - 1)] >= kTallyFlushAt))
       flush_warp(tl, wt, r.counters);
@@ -1298,35 +1425,89 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
       return false;
     }
     for (int step = 0; step < K; ++step) {
-      // walk phase: lanes not waiting for an interaction cross one cell
-      if (alive && !pending) {
-        int a;
-        if constexpr (kPath)
-          a = advance_path<kS>(k, cell, g, kap, kext, tl.levels);
-        else
-          a = advance_linked<false, kS, kTally>(k, cell, g, kap, kext, tl.levels, nullptr,
-                                                r.pathabs, kabs);
-        if (a == kCrossed) {
+      if (walking) {
+        int a = kCrossed;
+#pragma unroll 2
+        for (int u = 0; u < kSteps; ++u) {
+          if constexpr (kPath)
+            a = advance_path<kS>(k, cell, g, kap, kext, tl.levels);
+          else
+            a = advance_linked<false, kS, kTally>(k, cell, g, kap, kext, tl.levels, nullptr,
+                                                  r.pathabs, kabs);
+          if (a != kCrossed) break;
           ++tl.crossings;
-        } else if (a == kEscaped) {
-          ++tl.crossings;  // the boundary face it left through
-          atomicAdd(&wt[kCEscaped], 1u);
-          k.tau = -1.f;
-          alive = false;
-        } else if (a == kError) {
-          atomicAdd(&wt[kCErrors], 1u);
-          k.tau = 0.f;
-          atomicOr(r.status, kStatusTree);
-          alive = false;
-        } else {
-          pending = true;  // the optical depth runs out inside the cell
+        }
+        if (a != kCrossed) {
+          walking = false;
+          if (a == kEscaped) {
+            ++tl.crossings;  // the boundary face it left through
+            atomicAdd(&wt[kCEscaped], 1u);
+            k.tau = -1.f;
+          } else if (a == kError) {
+            atomicAdd(&wt[kCErrors], 1u);
+            k.tau = 0.f;
+            atomicOr(r.status, kStatusTree);
+          } else {
+            pending = true;  // the optical depth runs out inside the cell
+          }
         }
       }
-      // interaction phase, warp-uniform: once `batch` lanes wait, or nobody walks
-      const unsigned pm = __ballot_sync(kFull, pending);
-      if (pm == 0u) continue;
-      const unsigned walking = __ballot_sync(kFull, alive && !pending);
-      if (__popc(pm) < batch && walking != 0u) continue;
+      const unsigned wm = __ballot_sync(kFull, walking);
+      if constexpr (!kPark) {
+        const int np = __popc(__ballot_sync(kFull, pending));
+        if (np == 0 || (np < batch && wm)) continue;
+      } else {
+        if (__popc(wm) > 32 - batch && wm) continue;
+        book();
+        const unsigned pm = __ballot_sync(kFull, pending);
+        const int np = __popc(pm);
+        bool act = n_wait + np >= kPlaces;
+        if (!act && dry && n_ready == 0) {
+          if (wm == 0u && n_wait + np == 0) return true;
+          act = wm == 0u || n_wait + np >= batch;
+          if (!act) continue;
+        }
+        bool load = false, store = false, refill = false;
+        int src = 0, dst = 0;
+        if (act) {
+          const unsigned dm = ~(wm | pm);
+          const int nd = __popc(dm), n = min(n_wait, 32 - np);
+          const int rank = walking ? nd + __popc(wm & lt_mask) : __popc(dm & lt_mask);
+          load = !pending && rank < n;
+          store = load && walking;
+          src = n_wait - 1 - rank;
+          dst = kPlaces - 1 - n_ready - (rank - nd);
+          n_wait -= n;
+          n_ready += max(n - nd, 0);
+        } else if (n_ready > 0) {
+          const int rank = __popc(~wm & lt_mask), n = min(n_ready, 32 - __popc(wm));
+          load = !walking && rank < n;
+          store = load && pending;
+          const unsigned sm = __ballot_sync(kFull, store);
+          src = kPlaces - n_ready + rank;
+          dst = n_wait + __popc(sm & lt_mask);
+          n_ready -= n;
+          n_wait += __popc(sm);
+        } else {
+          store = pending;
+          dst = n_wait + __popc(pm & lt_mask);
+          n_wait += np;
+          refill = true;
+        }
+        if (__any_sync(kFull, load || store)) {
+          park_exchange<kPath>(park, k, cell, load, src, store, dst);
+          if (load) {
+            walking = !act;
+            pending = act;
+            set_inverse(k);
+          } else if (store) {
+            pending = false;
+          }
+        }
+        if (refill) fill(~wm);
+        if (!act) continue;
+      }
+      // interactions
       int sp = -1;
       uint4 w1 = make_uint4(0, 0, 0, 0);
       bool absorbing = false;
@@ -1335,6 +1516,7 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
       int leaf = 0, row = 0;  // the cell's leaf id; its density row (leaf or slot)
       if (pending) {
         pending = false;
+        walking = true;
         float kx;
         if constexpr (kPath)
           kx = cell.kx;
@@ -1350,11 +1532,13 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
         }
         if (++k.event > r.max_events) {
           atomicAdd(&wt[kCCapped], 1u);
-          alive = false;
+          walking = false;
+          k.tau = 0.f;
         } else if (leaf < 0) {
           atomicAdd(&wt[kCErrors], 1u);
           atomicOr(r.status, kStatusTree);
-          alive = false;
+          walking = false;
+          k.tau = 0.f;
         } else {
           const unsigned was = mirrored(k);
           restore_direction(k);
@@ -1471,13 +1655,16 @@ __global__ void __launch_bounds__(256, kMinBlocks)
     for (int i = threadIdx.x; i < B; i += blockDim.x) s_nemit[i] = 0ull;
   }
   __shared__ unsigned s_tally[8 * kTallyWords];
+  constexpr int kParkBytes = kTally ? 16 : park_bytes<kPath>();
+  __shared__ __align__(16) unsigned char s_park[8 * kParkBytes];
   for (int i = threadIdx.x; i < 8 * kTallyWords; i += blockDim.x) s_tally[i] = 0u;
   __syncthreads();
   unsigned* wt = s_tally + (threadIdx.x >> 5) * kTallyWords;
+  uint4* park = reinterpret_cast<uint4*>(s_park + (threadIdx.x >> 5) * kParkBytes);
   LaneTally tl = {};
   GlobalIds ids{r.next};
   pool_warp<kPeel, GlobalIds, kS, kPath, kTally>(g, t, r, kS > 2 ? t.kap : s_kap, s_cdf, s_sed,
-                                                 r.n_packages, ids, tl, wt, global_ns(), &pe,
+                                                 r.n_packages, ids, tl, wt, park, global_ns(), &pe,
                                                  s_nemit, s_kext, s_kabs);
   flush_warp(tl, wt, r.counters);
   if (sed_local || kPeel) __syncthreads();
@@ -1549,7 +1736,10 @@ __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const 
                                                          unsigned long long* next, int chunk) {
   __shared__ ModelDesc sdesc[8];
   __shared__ unsigned s_tally[8 * kTallyWords];
+  constexpr int kParkBytes = kTally ? 16 : park_bytes<false>();
+  __shared__ __align__(16) unsigned char s_park[8 * kParkBytes];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint4* park = reinterpret_cast<uint4*>(s_park + warp * kParkBytes);
   unsigned* wt = s_tally + warp * kTallyWords;
   if (lane < kTallyWords) wt[lane] = 0u;
   const unsigned per_block = blockDim.x >> 5;
@@ -1567,7 +1757,7 @@ __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const 
     ModelIds ids{next + m, 0ull, md.r.n_packages, 0, chunk};
     const bool in_time =
         pool_warp<false, ModelIds, kS, false, kTally>(md.g, md.t, md.r, md.t.kap, md.t.star_cdf, md.r.sed,
-                                        md.r.n_packages, ids, tl, wt, t0, nullptr, nullptr,
+                                        md.r.n_packages, ids, tl, wt, park, t0, nullptr, nullptr,
                                         md.t.kext);
     flush_warp(tl, wt, md.r.counters);
     __syncwarp();
@@ -1773,22 +1963,16 @@ static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, con
 // or four species or the generic one. With peel-off images or the path-length tally the
 // 4-block variants are used.
 //
-// Left to itself (0) the linked walk of two or four species takes five blocks per SM where
-// its records fit L2 and the launch has at least eight packages for every lane: more
-// warps hide the records' L2 latency, but spread fewer packages thinner over the lanes and,
-// once the records come from DRAM, widen the set of rows in use. Disk of 2.4e6 cells
-// (78 MB of records), four against five blocks: 5e6 packages 4.17 and 3.82 ms, 1.6e6 1.57
-// and 1.49, 8e5 0.95 and 0.95, 4e5 0.67 and 0.69, 1e5 0.40 and 0.43; disk of 1.9e7 cells
-// (0.6 GB), 1e7 packages: 22.9 and 27.5 ms.
+// Four is also what they take left to themselves (0): five blocks give the walks of two or
+// four species 48 registers, which spill now that packages move between lanes and places,
+// and their places take shared memory from L1 (2.4e6 cells, 5e6 packages: 3.40 ms against 3.21).
 cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const DevRun& r,
                                   int blocks_per_sm, int threads, cudaStream_t s,
                                   const DevPeel* peel, bool path) {
-  int dev = 0, sms = 0, l2 = 0;
+  int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
   if (e != cudaSuccess) return e;
   if (peel && r.pathabs)
     return launch_pool_variant<4, true, 0, false, true>(g, t, r, *peel, blocks_per_sm, threads,
@@ -1818,22 +2002,12 @@ cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const De
   }
   if (threads == 256 && blocks_per_sm == 6)
     return launch_pool_variant<6, false>(g, t, r, none, blocks_per_sm, threads, sms, s);
-  const bool in_l2 = (double)g.n_leaves * sizeof(int32_t) * kRec <= (double)l2;
-  const bool five =
-      threads == 256 && (blocks_per_sm == 5 || (blocks_per_sm == 0 && in_l2 &&
-                                                 r.n_packages >= 8ull * 5 * 256 * sms));
-  if (g.S == 2) {
-    if (five)
-      return launch_pool_variant<5, false, 2>(g, t, r, none, blocks_per_sm, threads, sms, s);
-    return launch_pool_variant<4, false, 2>(g, t, r, none, blocks_per_sm, threads, sms, s);
-  }
-  if (g.S == 4) {
-    if (five)
-      return launch_pool_variant<5, false, 4>(g, t, r, none, blocks_per_sm, threads, sms, s);
-    return launch_pool_variant<4, false, 4>(g, t, r, none, blocks_per_sm, threads, sms, s);
-  }
   if (threads == 256 && blocks_per_sm == 5)
     return launch_pool_variant<5, false>(g, t, r, none, blocks_per_sm, threads, sms, s);
+  if (g.S == 2)
+    return launch_pool_variant<4, false, 2>(g, t, r, none, blocks_per_sm, threads, sms, s);
+  if (g.S == 4)
+    return launch_pool_variant<4, false, 4>(g, t, r, none, blocks_per_sm, threads, sms, s);
   return launch_pool_variant<4, false>(g, t, r, none, blocks_per_sm, threads, sms, s);
 }
 
