@@ -11,44 +11,6 @@ namespace {
 
 using namespace planck;
 
-// One block per table row: the row's bin edges once each (FP64 is the cost: see
-// rt_planck.cuh), their differences into P, then S(T_i) = 4 pi sum_b kappa_abs P_b(T_i)
-// per species by one warp each from the row in shared memory.
-constexpr int kRowThreads = 128;
-
-__global__ void __launch_bounds__(kRowThreads) k_table_rows(TableBuild tb) {
-  __shared__ double edge[kMaxBins + 1];
-  __shared__ double P[kMaxBins];
-  const int i = blockIdx.x, B = tb.B;
-  const double T = table_T(i, tb.n_T, tb.t_min, tb.t_max);
-  const double a = T > 0.0 ? kH / (kK * T) : 0.0, pref = T > 0.0 ? planck_factor(T) : 0.0;
-  if (threadIdx.x == 0) tb.Tgrid[i] = T;
-  for (int b = threadIdx.x; b <= B; b += kRowThreads)
-    edge[b] = T > 0.0 ? planck_edge(a * tb.nu[b]) : 0.0;
-  __syncthreads();
-  for (int b = threadIdx.x; b < B; b += kRowThreads) {
-    const double v =
-        T > 0.0 ? pref * planck_between(a * tb.nu[b], edge[b], a * tb.nu[b + 1], edge[b + 1])
-                : 0.0;
-    P[b] = v;
-    tb.P[(size_t)i * B + b] = v;
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  for (int s = threadIdx.x >> 5; s < tb.S; s += kRowThreads / 32) {
-    const double* ka = tb.kabs + (size_t)s * B;
-    double acc = 0.0;
-    for (int b = lane; b < B; b += 32) acc += ka[b] * P[b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    acc *= 4.0 * kPi;
-    if (lane == 0) {
-      tb.S64[(size_t)s * tb.n_T + i] = acc;
-      tb.S32[(size_t)s * tb.n_T + i] = (float)acc;
-    }
-  }
-}
-
 // Inclusive sum over the warp's lanes.
 __device__ __forceinline__ double scan_add(double v) {
   const int lane = threadIdx.x & 31;
@@ -95,16 +57,109 @@ __device__ __forceinline__ double cumulative_warp(int B, F v, G out) {
   return tot;
 }
 
+// Opacity records of a bin.
+__device__ __forceinline__ void opacities(const TableBuild& tb, int b) {
+  for (int s = 0; s < tb.S; ++s) {
+    size_t j = (size_t)s * tb.B + b;
+    Kappa k;
+    k.kabs = (float)tb.kabs[j];
+    k.ksca = (float)tb.ksca[j];
+    k.kext = (float)(tb.kabs[j] + tb.ksca[j]);
+    k.g = (float)tb.ghg[j];
+    tb.kap[(size_t)b * tb.S + s] = k;
+    tb.kext[(size_t)b * tb.S + s] = k.kext;
+  }
+}
+
+// Stellar CDF and the in-range fraction of the blackbody: the bin edges in parallel
+// (one block), the cumulative by one warp. (The integrals bin by bin with the division
+// of every entry in one thread took 0.46 ms for 100 bins; this takes 0.03 ms.)
+__device__ __forceinline__ void star_spectrum(const TableBuild& tb, double* edge) {
+  const int B = tb.B;
+  const double a = kH / (kK * tb.T_star), pref = planck_factor(tb.T_star);
+  for (int b = threadIdx.x; b <= B; b += blockDim.x) edge[b] = planck_edge(a * tb.nu[b]);
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const double tot = cumulative_warp(
+      B,
+      [&](int b) {
+        return pref * planck_between(a * tb.nu[b], edge[b], a * tb.nu[b + 1], edge[b + 1]);
+      },
+      [&](int b, float c) { tb.star_cdf[b] = c; });
+  if (threadIdx.x == 0) {
+    // sigma = 2 pi^5 k^4 / (15 c^2 h^3)
+    double sigma = 2.0 * pow(kPi, 5.0) * pow(kK, 4.0) / (15.0 * kC * kC * pow(kH, 3.0));
+    double T4 = pow(tb.T_star, 4.0);
+    tb.star_frac[0] = kPi * tot / (sigma * T4);
+  }
+}
+
+// One block per table row: the row's bin edges once each (FP64 is the cost: see
+// rt_planck.cuh), their differences into P, then S(T_i) = 4 pi sum_b kappa_abs P_b(T_i)
+// per species by one warp each from the row in shared memory. The star's spectrum (the
+// first block, so that its serial chain runs beside the rows) and the opacities need
+// nothing of the rows: with launches of their own, as the guides below, the tables of 2
+// species x 100 bins took 122 us, in two launches 83.
+constexpr int kRowThreads = 128;
+
+__global__ void __launch_bounds__(kRowThreads) k_table_rows(TableBuild tb) {
+  __shared__ double edge[kMaxBins + 1];
+  __shared__ double P[kMaxBins];
+  const int B = tb.B, i = (int)blockIdx.x - 1;
+  if (i < 0) {
+    star_spectrum(tb, edge);
+    return;
+  }
+  if (i >= tb.n_T) {
+    const int b = (i - tb.n_T) * kRowThreads + threadIdx.x;
+    if (b < B) opacities(tb, b);
+    return;
+  }
+  const double T = table_T(i, tb.n_T, tb.t_min, tb.t_max);
+  const double a = T > 0.0 ? kH / (kK * T) : 0.0, pref = T > 0.0 ? planck_factor(T) : 0.0;
+  if (threadIdx.x == 0) tb.Tgrid[i] = T;
+  for (int b = threadIdx.x; b <= B; b += kRowThreads)
+    edge[b] = T > 0.0 ? planck_edge(a * tb.nu[b]) : 0.0;
+  __syncthreads();
+  for (int b = threadIdx.x; b < B; b += kRowThreads) {
+    const double v =
+        T > 0.0 ? pref * planck_between(a * tb.nu[b], edge[b], a * tb.nu[b + 1], edge[b + 1])
+                : 0.0;
+    P[b] = v;
+    tb.P[(size_t)i * B + b] = v;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int s = threadIdx.x >> 5; s < tb.S; s += kRowThreads / 32) {
+    const double* ka = tb.kabs + (size_t)s * B;
+    double acc = 0.0;
+    for (int b = lane; b < B; b += 32) acc += ka[b] * P[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    acc *= 4.0 * kPi;
+    if (lane == 0) {
+      tb.S64[(size_t)s * tb.n_T + i] = acc;
+      tb.S32[(size_t)s * tb.n_T + i] = (float)acc;
+    }
+  }
+}
+
 // One warp per (species, interval): the normalised cumulative of
 // kappa_abs(b) [P_b(T_{i+1}) - P_b(T_i)] over the bins, and the row's search guide: the
 // first bin whose cumulative value exceeds k/B, k = 0 .. B-1 (at most the last bin) --
 // a starting point only, the draws finish by scanning. A thread per row walking its
 // bins serially, with rows B doubles apart, took 88 + 45 us for 2 species x 100 bins;
-// the warp reads them coalesced and takes 21 us.
+// the warp reads them coalesced and takes 21 us (the guides u_k beside them).
 constexpr int kCdfWarps = 4;
 
-__global__ void __launch_bounds__(32 * kCdfWarps) k_difference_cdfs(TableBuild tb) {
+__device__ __forceinline__ void u_guide(const TableBuild& tb, int idx);
+
+__global__ void __launch_bounds__(32 * kCdfWarps) k_difference_cdfs(TableBuild tb, int n_cdf) {
   __shared__ float rows[kCdfWarps][kMaxBins];
+  if ((int)blockIdx.x >= n_cdf) {
+    u_guide(tb, ((int)blockIdx.x - n_cdf) * 32 * kCdfWarps + threadIdx.x);
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int idx = blockIdx.x * kCdfWarps + warp, nI = tb.n_T - 1, B = tb.B;
   if (idx >= tb.S * nI) return;
@@ -135,8 +190,7 @@ __global__ void __launch_bounds__(32 * kCdfWarps) k_difference_cdfs(TableBuild t
 
 // Per species: for u_k = exp(ln S(T_1) + k (ln S(T_last) - ln S(T_1)) / (n_T - 1)),
 // the largest interval i <= n_T - 2 with S(T_i) <= u_k. One thread per (s, k).
-__global__ void k_u_guides(TableBuild tb) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void u_guide(const TableBuild& tb, int idx) {
   if (idx >= tb.S * tb.n_T) return;
   int s = idx / tb.n_T, k = idx % tb.n_T;
   const double* S = tb.S64 + (size_t)s * tb.n_T;
@@ -149,46 +203,6 @@ __global__ void k_u_guides(TableBuild tb) {
     if (S[mid] <= u) lo = mid; else hi = mid;
   }
   tb.u_guide[idx] = lo;
-}
-
-__global__ void k_opacity(TableBuild tb) {
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < tb.B) {
-    for (int s = 0; s < tb.S; ++s) {
-      size_t j = (size_t)s * tb.B + b;
-      Kappa k;
-      k.kabs = (float)tb.kabs[j];
-      k.ksca = (float)tb.ksca[j];
-      k.kext = (float)(tb.kabs[j] + tb.ksca[j]);
-      k.g = (float)tb.ghg[j];
-      tb.kap[(size_t)b * tb.S + s] = k;
-      tb.kext[(size_t)b * tb.S + s] = k.kext;
-    }
-  }
-}
-
-// Stellar CDF and the in-range fraction of the blackbody: the bin edges in parallel
-// (one block), the cumulative by one warp. (The integrals bin by bin with the division
-// of every entry in one thread took 0.46 ms for 100 bins, now 0.03 ms.)
-__global__ void __launch_bounds__(256) k_star_cdf(TableBuild tb) {
-  __shared__ double edge[kMaxBins + 1];
-  const int B = tb.B;
-  const double a = kH / (kK * tb.T_star), pref = planck_factor(tb.T_star);
-  for (int b = threadIdx.x; b <= B; b += blockDim.x) edge[b] = planck_edge(a * tb.nu[b]);
-  __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const double tot = cumulative_warp(
-      B,
-      [&](int b) {
-        return pref * planck_between(a * tb.nu[b], edge[b], a * tb.nu[b + 1], edge[b + 1]);
-      },
-      [&](int b, float c) { tb.star_cdf[b] = c; });
-  if (threadIdx.x == 0) {
-    // sigma = 2 pi^5 k^4 / (15 c^2 h^3)
-    double sigma = 2.0 * pow(kPi, 5.0) * pow(kK, 4.0) / (15.0 * kC * kC * pow(kH, 3.0));
-    double T4 = pow(tb.T_star, 4.0);
-    tb.star_frac[0] = kPi * tot / (sigma * T4);
-  }
 }
 
 // S at temperature T by linear interpolation in T between table rows (the same
@@ -283,12 +297,11 @@ inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 }  // namespace
 
 cudaError_t launch_build_tables(const TableBuild& tb, cudaStream_t s) {
-  k_table_rows<<<(unsigned)tb.n_T, kRowThreads, 0, s>>>(tb);
-  k_difference_cdfs<<<nblk((long long)tb.S * (tb.n_T - 1), kCdfWarps), 32 * kCdfWarps, 0, s>>>(
-      tb);
-  k_u_guides<<<nblk((long long)tb.S * tb.n_T, 128), 128, 0, s>>>(tb);
-  k_opacity<<<nblk(tb.B, 128), 128, 0, s>>>(tb);
-  k_star_cdf<<<1, 256, 0, s>>>(tb);
+  k_table_rows<<<1 + (unsigned)tb.n_T + nblk(tb.B, kRowThreads), kRowThreads, 0, s>>>(tb);
+  // the guides' blocks after those of the rows
+  const unsigned n_cdf = nblk((long long)tb.S * (tb.n_T - 1), kCdfWarps);
+  k_difference_cdfs<<<n_cdf + nblk((long long)tb.S * tb.n_T, 32 * kCdfWarps), 32 * kCdfWarps, 0,
+                      s>>>(tb, (int)n_cdf);
   return cudaGetLastError();
 }
 
