@@ -839,7 +839,8 @@ rt_status rt_set_frozen_temperatures(rt_grid* g, const float* T, int mem, void* 
                           mem == RT_MEM_DEVICE ? cudaMemcpyDeviceToDevice
                                                : cudaMemcpyHostToDevice,
                           s));
-  RT_CUDA(launch_frozen_u(g->g, g->tab, g->d_Tfrozen, g->d_ufrozen, (float)g->desc.t_min, s));
+  RT_CUDA(launch_frozen_u(g->g, g->tab, g->d_Tfrozen, g->d_ufrozen, (float)g->desc.t_min,
+                          (float)g->desc.t_max, s));
   if (mem != RT_MEM_DEVICE) RT_CUDA(cudaStreamSynchronize(s));
   g->frozen_ready = true;
   return RT_OK;

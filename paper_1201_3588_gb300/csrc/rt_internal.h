@@ -301,7 +301,7 @@ cudaError_t launch_pah_pt(const PtCase* cases, int n_cases, const double* nu, in
 size_t pt_scratch_doubles(int n_cases, int M, int B);
 
 cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T_frozen,
-                            float* u_frozen, float t_min, cudaStream_t s);
+                            float* u_frozen, float t_min, float t_max, cudaStream_t s);
 // out [S][n_leaves] from tallies [n_leaves][S]
 cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out, cudaStream_t s);
 cudaError_t launch_temperatures(const DevGrid& g, const DevTables& t,

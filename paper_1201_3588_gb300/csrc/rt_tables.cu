@@ -205,84 +205,149 @@ __device__ __forceinline__ void u_guide(const TableBuild& tb, int idx) {
   tb.u_guide[idx] = lo;
 }
 
+// 1/x to 4e-15 from its FP32 value: a reciprocal there and one Newton step (the FP64 division
+// is some ten operations of a pipe that does two a clock). For x well inside FP32's range.
+__device__ __forceinline__ double reciprocal(float x32, double x) {
+  const double r = (double)__frcp_rn(x32);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
 // S at temperature T by linear interpolation in T between table rows (the same
 // piecewise-linear model the transport samples from).
+// a < b for doubles that are not negative: their bits as integers (a compare is an FP64
+// operation too)
+__device__ __forceinline__ bool below(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+// A binary search of FP64 rows, then an FP64 division: 3.2e7 entries 1.46 ms, now 0.65; FP64
+// operations, some twelve an entry, still bound it.
 __global__ void k_frozen_u(DevGrid g, DevTables t, const float* T_frozen, float* u_frozen,
-                           float t_min) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long tot = (long long)g.S * g.n_leaves;
-  if (idx >= tot) return;
-  int s = (int)(idx / g.n_leaves);
-  double T = fmax((double)T_frozen[idx], (double)t_min);
+                           float t_min, float t_max) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (c >= g.n_leaves) return;
+  const int s = blockIdx.y;
+  const long long idx = s * g.n_leaves + c;
+  const float T32 = fmaxf(T_frozen[idx], t_min);
+  const double T = (double)T32;
   const double* Tg = t.Tgrid;
   const double* S = t.S64 + (size_t)s * g.n_T;
-  int n_T = g.n_T;
+  const int n_T = g.n_T;
   double u;
-  if (T >= Tg[n_T - 1]) {
+  if (!below(T, Tg[n_T - 1])) {
     u = S[n_T - 1];
   } else {
-    int lo = 0, hi = n_T - 1;  // Tg[lo] <= T < Tg[hi]
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (Tg[mid] <= T) lo = mid; else hi = mid;
+    // Tg[lo] <= T < Tg[lo + 1]: the rows from the second on are evenly spaced in ln T, so
+    // start there and finish by scanning
+    const float l1 = __logf(t_min), step = (__logf(t_max) - l1) / (float)(n_T - 2);
+    const float k = (__logf(T32) - l1) / step + 1.0f;
+    int lo = (int)fminf(fmaxf(k, 0.0f), (float)(n_T - 2));
+    while (lo > 0 && below(T, Tg[lo])) --lo;
+    while (lo + 2 < n_T && !below(T, Tg[lo + 1])) ++lo;
+    const double dT = Tg[lo + 1] - Tg[lo];
+    double w = T - Tg[lo];
+    if ((float)dT > 1e-30f && (float)dT < 1e30f) {
+      w *= reciprocal((float)dT, dT);  // to 4e-15; w makes up a few per cent of u at most
+    } else {
+      w /= dT;
     }
-    double w = (T - Tg[lo]) / (Tg[hi] - Tg[lo]);
-    u = S[lo] + w * (S[hi] - S[lo]);
+    u = S[lo] + w * (S[lo + 1] - S[lo]);
   }
   u_frozen[idx] = (float)u;
 }
 
 // T from n eps = M S(T): the FP64 S table's interval (guide + scan), then power-law
 // (log-log) interpolation between rows; linear from T = 0 in the first interval.
-__global__ void k_temperatures(DevGrid g, DevTables t, const unsigned long long* count,
-                               float* T_out, unsigned long long* counters,
-                               const float* pathabs) {
-  long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long tot = (long long)g.S * g.n_leaves;
-  bool clamped = false;
-  if (idx < tot) {
-    int s = (int)(idx / g.n_leaves);
-    long long c = idx - (long long)s * g.n_leaves;
-    // absorbed energy in units of eps: the count, or the path-length tally
-    const double n = pathabs ? (double)pathabs[c * g.S + s] : (double)count[idx];
-    float rho_d0 = g.rho[c * g.S + s];
-    float Tv = 0.0f;
-    if (n > 0.0 && rho_d0 > 0.0f) {
-      int lev = g.level[c];
-      double rho = (double)rho_d0 / t.d0;
-      double u = n * t.eps_over_V[lev] / rho;
-      const double* S = t.S64 + (size_t)s * g.n_T;
-      const double* Tg = t.Tgrid;
-      int n_T = g.n_T;
-      if (u >= S[n_T - 1]) {
-        Tv = (float)Tg[n_T - 1];
-        clamped = true;
-      } else {
-        // interval i with S[i] <= u < S[i+1]: start from the guide of ln S (the
-        // re-emission draws use the same one), finish by scanning
-        const int nI = n_T - 1;
-        float kf = (__logf(fmaxf((float)u, 1e-30f)) - t.u_ln0[s]) * t.u_inv[s];
-        int kk = (int)fminf(fmaxf(kf, 0.0f), (float)nI);
-        int i = t.u_guide[s * n_T + kk];
-        while (i > 0 && S[i] > u) --i;
-        while (i + 1 < nI && S[i + 1] <= u) ++i;
-        double T;
-        if (i == 0 || !(S[i] > 0.0)) {
-          T = Tg[i + 1] * u / S[i + 1];
-        } else {
-          // power law between the rows: ln(T/T_i) = ln(u/S_i) ln(T_i+1/T_i) / ln(S_i+1/S_i);
-          // the ratios are formed in FP64, their logarithms (of numbers near 1) in FP32
-          const double inv = 1.0 / S[i];
-          const float a = log1pf((float)(u * inv - 1.0)) / log1pf((float)(S[i + 1] * inv - 1.0));
-          T = Tg[i] * (double)expf(a * logf((float)(Tg[i + 1] / Tg[i])));
-        }
-        Tv = (float)T;
-      }
-    }
-    T_out[idx] = Tv;
+//
+// FP64 operations bound it (two a clock per SM): four divisions an entry before. u needs
+// FP64 against the rows (they differ by a few per cent, T by less than one), but the place
+// within an interval does not: differences in FP64, their quotients (of numbers well above
+// rounding) in FP32, as the new T is T_i plus at most a per cent of it. Against 80 bits: 2.6e-8 RMS, 6.1e-8 at most (the
+// rounding of the FP32 result; with divisions 6.4e-8 and 2.4e-7, from the quotient of
+// neighbouring T in FP32).
+__device__ __forceinline__ float cell_temperature(const DevTables& t, int n_T, int s, double n,
+                                                  float rho_d0, int lev, unsigned& clamped) {
+  if (!(n > 0.0) || !(rho_d0 > 0.0f)) return 0.0f;
+  const double rho = (double)rho_d0, k = t.eps_over_V[lev] * t.d0;
+  double u;
+  if (rho_d0 > 1e-30f && rho_d0 < 1e30f) {
+    u = n * k * reciprocal(rho_d0, rho);
+  } else {
+    u = n * k / rho;
   }
-  unsigned m = __ballot_sync(0xffffffffu, clamped);
-  if ((threadIdx.x & 31) == 0 && m) atomicAdd(&counters[kCClamped], (unsigned long long)__popc(m));
+  const double* S = t.S64 + (size_t)s * n_T;
+  const double* Tg = t.Tgrid;
+  const int nI = n_T - 1;
+  if (!below(u, S[nI])) {
+    ++clamped;
+    return (float)Tg[nI];
+  }
+  // interval i with S[i] <= u < S[i+1]: start from the guide of ln S (the re-emission
+  // draws use the same one), finish by scanning
+  const float kf = (__logf(fmaxf((float)u, 1e-30f)) - t.u_ln0[s]) * t.u_inv[s];
+  int i = t.u_guide[s * n_T + (int)fminf(fmaxf(kf, 0.0f), (float)nI)];
+  double Si = S[i], Sn = S[i + 1];
+  while (i > 0 && below(u, Si)) {
+    Sn = Si;
+    Si = S[--i];
+  }
+  while (i + 1 < nI && !below(u, Sn)) {
+    Si = Sn;
+    Sn = S[++i + 1];
+  }
+  const double T0 = Tg[i], T1 = Tg[i + 1];
+  if (i == 0 || !(Si > 0.0)) return (float)(T1 * u / Sn);
+  // power law between the rows: ln(T/T_i) = ln(u/S_i) ln(T_i+1/T_i) / ln(S_i+1/S_i)
+  float x = (float)(u - Si), xs = (float)(Sn - Si);
+  const float S32 = (float)Si;
+  if (S32 > 1e-28f && S32 < 1e30f) {
+    x /= S32;
+    xs /= S32;
+  } else {
+    x = (float)((u - Si) / Si);
+    xs = (float)((Sn - Si) / Si);
+  }
+  const float y = log1pf(x) / log1pf(xs) * log1pf((float)(T1 - T0) / (float)T0);
+  return (float)fma(T0, (double)expm1f(y), T0);
+}
+
+// One thread a cell: its densities (and path-length tallies) lie side by side, while a
+// thread per species and cell read them in as many passes. With
+// the arithmetic above: 8.0e6 cells of four species 0.60 -> 0.31 ms, 2.4e6 of two 0.20 -> 0.11.
+template <int kS>
+__global__ void __launch_bounds__(256) k_temperatures(DevGrid g, DevTables t,
+                                                      const unsigned long long* count,
+                                                      float* T_out, unsigned long long* counters,
+                                                      const float* pathabs) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int S = kS > 0 ? kS : g.S;
+  unsigned clamped = 0;
+  if (c < g.n_leaves) {
+    const int lev = g.level[c];
+    // absorbed energy in units of eps: the count, or the path-length tally
+    const auto absorbed = [&](int s) {
+      return pathabs ? (double)pathabs[c * S + s] : (double)count[s * g.n_leaves + c];
+    };
+    if constexpr (kS > 0) {
+      double n[kS];
+      float rho[kS];
+#pragma unroll
+      for (int s = 0; s < kS; ++s) {
+        n[s] = absorbed(s);
+        rho[s] = g.rho[c * kS + s];
+      }
+#pragma unroll
+      for (int s = 0; s < kS; ++s)
+        T_out[s * g.n_leaves + c] = cell_temperature(t, g.n_T, s, n[s], rho[s], lev, clamped);
+    } else {
+      for (int s = 0; s < S; ++s)
+        T_out[s * g.n_leaves + c] =
+            cell_temperature(t, g.n_T, s, absorbed(s), g.rho[c * S + s], lev, clamped);
+    }
+  }
+  clamped = __reduce_add_sync(0xffffffffu, clamped);
+  if ((threadIdx.x & 31) == 0 && clamped)
+    atomicAdd(&counters[kCClamped], (unsigned long long)clamped);
 }
 
 // Path-length tallies, species within a cell adjacent, to one array per species.
@@ -306,9 +371,9 @@ cudaError_t launch_build_tables(const TableBuild& tb, cudaStream_t s) {
 }
 
 cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T_frozen,
-                            float* u_frozen, float t_min, cudaStream_t s) {
-  long long n = (long long)g.S * g.n_leaves;
-  k_frozen_u<<<nblk(n, 256), 256, 0, s>>>(g, t, T_frozen, u_frozen, t_min);
+                            float* u_frozen, float t_min, float t_max, cudaStream_t s) {
+  const dim3 grid(nblk(g.n_leaves, 256), (unsigned)g.S);
+  k_frozen_u<<<grid, 256, 0, s>>>(g, t, T_frozen, u_frozen, t_min, t_max);
   return cudaGetLastError();
 }
 
@@ -322,8 +387,9 @@ cudaError_t launch_temperatures(const DevGrid& g, const DevTables& t,
                                 const unsigned long long* count, float* T_out,
                                 unsigned long long* counters, cudaStream_t s,
                                 const float* pathabs) {
-  long long n = (long long)g.S * g.n_leaves;
-  k_temperatures<<<nblk(n, 256), 256, 0, s>>>(g, t, count, T_out, counters, pathabs);
+  const auto kernel = g.S == 2 ? k_temperatures<2> : (g.S == 4 ? k_temperatures<4>
+                                                              : k_temperatures<0>);
+  kernel<<<nblk(g.n_leaves, 256), 256, 0, s>>>(g, t, count, T_out, counters, pathabs);
   return cudaGetLastError();
 }
 
