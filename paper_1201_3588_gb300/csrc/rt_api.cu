@@ -497,6 +497,22 @@ rt_status build_tables(rt_grid* g, cudaStream_t s) {
   return RT_OK;
 }
 
+// the tallies that not every grid has
+rt_status reset_optional(rt_grid* g, cudaStream_t s) {
+  const size_t S = g->desc.n_species, N = g->desc.n_leaves;
+  // only the rows of PAH-active cells hold counts: clear those and their flags
+  if (g->d_pahabs)
+    RT_CUDA(launch_pah_clear(g->d_pah_flag, (long long)N, g->tab.n_coarse, g->n_pah,
+                             g->d_pahabs, g->d_pah_flag, s));
+  if (g->d_pathabs) RT_CUDA(cudaMemsetAsync(g->d_pathabs, 0, sizeof(float) * S * N, s));
+  if (g->images) {
+    const size_t n = (size_t)g->peel.n_planes * g->peel.ny * g->peel.nx;
+    RT_CUDA(cudaMemsetAsync(g->d_image, 0, sizeof(double) * n, s));
+    RT_CUDA(cudaMemsetAsync(g->d_nemit, 0, sizeof(unsigned long long) * g->desc.n_bins, s));
+  }
+  return RT_OK;
+}
+
 cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 bool finite3(const double* v) {
@@ -850,24 +866,12 @@ rt_status rt_reset(rt_grid* g, void* stream) {
   if (!g) return RT_ERR_ARG;
   cudaStream_t s = as_stream(stream);
   RT_CUDA(cudaSetDevice(g->dev));
-  const size_t S = g->desc.n_species, N = g->desc.n_leaves;
-  RT_CUDA(cudaMemsetAsync(g->d_count, 0, sizeof(unsigned long long) * S * N, s));
-  RT_CUDA(cudaMemsetAsync(g->d_sed, 0,
-                          sizeof(unsigned long long) * 2 * g->desc.n_sed_dirs * g->desc.n_bins,
+  // counts, spectrum, counters and status end the grid's allocation
+  RT_CUDA(cudaMemsetAsync(g->d_count, 0,
+                          (size_t)(g->grid_slab + g->grid_bytes -
+                                   reinterpret_cast<char*>(g->d_count)),
                           s));
-  RT_CUDA(cudaMemsetAsync(g->d_counters, 0, sizeof(unsigned long long) * kNumCounters, s));
-  RT_CUDA(cudaMemsetAsync(g->d_status, 0, sizeof(unsigned), s));
-  // only the rows of PAH-active cells hold counts: clear those and their flags
-  if (g->d_pahabs)
-    RT_CUDA(launch_pah_clear(g->d_pah_flag, (long long)N, g->tab.n_coarse, g->n_pah,
-                             g->d_pahabs, g->d_pah_flag, s));
-  if (g->d_pathabs) RT_CUDA(cudaMemsetAsync(g->d_pathabs, 0, sizeof(float) * S * N, s));
-  if (g->images) {
-    const size_t n = (size_t)g->peel.n_planes * g->peel.ny * g->peel.nx;
-    RT_CUDA(cudaMemsetAsync(g->d_image, 0, sizeof(double) * n, s));
-    RT_CUDA(cudaMemsetAsync(g->d_nemit, 0, sizeof(unsigned long long) * g->desc.n_bins, s));
-  }
-  return RT_OK;
+  return reset_optional(g, s);
 }
 
 // The path-length tallies are allocated (and zeroed) the first time a launch asks
@@ -1741,6 +1745,7 @@ struct rt_batch {
   int blocks_per_sm = 0;
   int threads = 256;  // threads per block of the batched launch
   int s_fixed = 0;  // the species count every model shares (walk compiled for it), else 0
+  long long max_cells = 0;  // of the largest model
   bool tally = false;  // path-length tallies kept
   cudaStream_t capture_stream = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -1794,6 +1799,8 @@ rt_status rt_batch_create(rt_grid* const* grids, int n, const uint64_t* n_packag
     desc[(size_t)m].t.u_frozen = g->d_ufrozen;
     desc[(size_t)m].t.pah_cell_cdf = g->d_pah_cell_cdf;
     desc[(size_t)m].r = r;
+    desc[(size_t)m].T_out = g->d_Tscratch;
+    b->max_cells = std::max(b->max_cells, (long long)g->desc.n_leaves);
     b->grids.push_back(g);
     b->n_pk.push_back(n_packages[m]);
   }
@@ -1830,17 +1837,19 @@ rt_status rt_batch_run(rt_batch* b, int reset, int temperatures, void* stream) {
   if (!b) return RT_ERR_ARG;
   cudaStream_t s = as_stream(stream);
   RT_CUDA(cudaSetDevice(b->dev));
-  if (reset)
+  const int n = (int)b->grids.size();
+  if (reset) {
+    RT_CUDA(launch_batch_reset(b->d_models, n, b->max_cells, s));
     for (rt_grid* g : b->grids) {
-      rt_status st = rt_reset(g, stream);
+      rt_status st = reset_optional(g, s);
       if (st != RT_OK) return st;
     }
-  RT_CUDA(cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long) * b->grids.size(), s));
-  RT_CUDA(launch_transport_batch(b->d_models, (int)b->grids.size(), b->d_next, b->chunk,
+  }
+  RT_CUDA(cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long) * n, s));
+  RT_CUDA(launch_transport_batch(b->d_models, n, b->d_next, b->chunk,
                                  b->blocks_per_sm, b->s_fixed, b->tally, b->threads, s));
   if (temperatures)
-    for (rt_grid* g : b->grids)
-      RT_CUDA(launch_temperatures(g->g, g->tab, g->d_count, g->d_Tscratch, g->d_counters, s));
+    RT_CUDA(launch_batch_temperatures(b->d_models, n, b->max_cells, b->s_fixed, s));
   return RT_OK;
 }
 

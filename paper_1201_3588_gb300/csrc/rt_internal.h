@@ -138,6 +138,7 @@ struct ModelDesc {
   DevGrid g;
   DevTables t;
   DevRun r;
+  float* T_out;  // temperatures [S][n_leaves] of the model
 };
 
 // Kernel launchers (rt_transport.cu, rt_tables.cu).
@@ -304,6 +305,12 @@ cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T
                             float* u_frozen, float t_min, float t_max, cudaStream_t s);
 // out [S][n_leaves] from tallies [n_leaves][S]
 cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out, cudaStream_t s);
+// Every model of a batch in one launch (max_cells: of the largest): temperatures from the
+// counts into T_out; counts, spectra, counters and status to zero.
+cudaError_t launch_batch_temperatures(const ModelDesc* models, int n_models, long long max_cells,
+                                      int s_fixed, cudaStream_t s);
+cudaError_t launch_batch_reset(const ModelDesc* models, int n_models, long long max_cells,
+                               cudaStream_t s);
 cudaError_t launch_temperatures(const DevGrid& g, const DevTables& t,
                                 const unsigned long long* count, float* T_out,
                                 unsigned long long* counters, cudaStream_t s,
