@@ -1225,7 +1225,7 @@ struct ModelIds {
 constexpr int kPlaces = 32;
 
 template <bool kPath>
-__host__ __device__ constexpr int park_bytes() {  // per warp
+__host__ __device__ constexpr int park_bytes() {  // per warp (bound schedule: none)
   return kPlaces * (kPath ? 16 * 5 + 8 : 16 * 4);
 }
 
@@ -1620,6 +1620,10 @@ __host__ __device__ __forceinline__ int kap_records(const DevGrid& g) {
 // Persistent packet pool over one model: all warps draw package indices from one
 // global counter; the opacity table, the stellar CDF and (when it fits) the
 // escaped-spectrum histogram live in shared memory.
+// shared memory of a block beside what the launch asks for
+template <bool kPath, bool kTally>
+constexpr size_t kPoolStatic = 8 * ((kTally ? 16 : park_bytes<kPath>()) + 4 * kTallyWords);
+
 template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false, bool kTally = false>
 __global__ void __launch_bounds__(256, kMinBlocks)
     k_transport_pool(DevGrid g, DevTables t, DevRun r, const __grid_constant__ DevPeel pe) {
@@ -1657,6 +1661,8 @@ __global__ void __launch_bounds__(256, kMinBlocks)
   __shared__ unsigned s_tally[8 * kTallyWords];
   constexpr int kParkBytes = kTally ? 16 : park_bytes<kPath>();
   __shared__ __align__(16) unsigned char s_park[8 * kParkBytes];
+  static_assert(sizeof(s_tally) + sizeof(s_park) <= kPoolStatic<kPath, kTally>,
+                "the launch counts the kernel's own shared memory");
   for (int i = threadIdx.x; i < 8 * kTallyWords; i += blockDim.x) s_tally[i] = 0u;
   __syncthreads();
   unsigned* wt = s_tally + (threadIdx.x >> 5) * kTallyWords;
@@ -1687,8 +1693,9 @@ __global__ void __launch_bounds__(256, kMinBlocks)
 // random. A warp's lanes therefore run dry once per model it works on. (Fixed chunks of
 // 4096 packages, a warp's lanes drained at the end of each, left three quarters of the
 // warps without work for a batch of 24 models and 6.5e6 packages -- 1600 chunks for 4864
-// warps -- and took 28.7 ms; this takes 8.0.) Tables in global memory / L2, spectrum by global atomics;
-// counters are flushed to the model when the warp leaves it.
+// warps -- and took 28.7 ms against 8.0 for this, and 4.8 with the walk as it is now.) Tables
+// in global memory / L2, spectrum by global atomics; counters are flushed to the model when
+// the warp leaves it.
 __device__ __forceinline__ int pick_model(const ModelDesc* models, int n,
                                           const unsigned long long* next, unsigned warp_id,
                                           unsigned n_warps, unsigned pick) {
@@ -1729,8 +1736,9 @@ __device__ __forceinline__ int pick_model(const ModelDesc* models, int n,
   return last;
 }
 
-// Two species: held to 64 registers (56 bytes of spills) for four blocks per SM, 8.0 ms
-// against 8.7 with the three blocks of 74 registers; the generic form would spill 180.
+// Two species: held to 64 registers (58 bytes of spills) for four blocks per SM; when this
+// was decided 8.0 ms against 8.7 with three blocks of 74 registers, and 180 bytes of spills in
+// the generic form.
 template <int kS, bool kTally>
 __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const ModelDesc* models, int n_models,
                                                          unsigned long long* next, int chunk) {
@@ -1944,7 +1952,8 @@ static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, con
   size_t sm = tables + (rr.sed_in_smem ? sed_smem(g) : 0);
   cudaError_t e;
   const auto kernel = k_transport_pool<kMinBlocks, kPeel, kS, kPath, kTally>;
-  if (sm > 48 * 1024) {
+  // beyond 48 KB a block with the kernel's own shared memory (places and counters)
+  if (sm + kPoolStatic<kPath, kTally> > 48 * 1024) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }

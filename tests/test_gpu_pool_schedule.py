@@ -64,3 +64,30 @@ def test_every_schedule_gives_the_replayed_histories(S, walk, star):
                 parted = 0 if S in (1, 3) else 2 + c["crossings"] // 10**6
                 slack = parted * int(tr[:, col].max())
                 assert abs(c[name] - int(tr[:, col].sum())) <= slack, (n, kw, name)
+
+
+@pytest.mark.parametrize("S,bins,dirs,walk", [
+    (1, 1024, 1, "LINKED"), (2, 1024, 1, "LINKED"), (6, 300, 1, "LINKED"), (6, 300, 1, "PATH"),
+    (8, 1024, 3, "LINKED"), (3, 1024, 9, "PATH"), (3, 1024, 64, "LINKED")])
+def test_tables_of_every_size_beside_the_places(S, bins, dirs, walk):
+    # the places are part of the block's shared memory: launches whose tables alone stay
+    # below 48 KB, or fill what the spectrum's choice of memory allows (200 KB)
+    nu = w.frequency_edges(bins)
+    sp = w.two_species(nu)[:S] + [w.grey_species(bins, 0.2 + 0.1 * s, 0.3)
+                                  for s in range(max(S - 2, 0))]
+    m = w.uniform_box_model(4, bins, 3.0, sp, max_level=1, refine=w.sphere_refine_fn(4, 0.5),
+                            n_sed_dirs=dirs)
+    n = 3000
+    with rt.Grid(m) as g:
+        g.emit_star(n)
+        g.set_frozen_temperatures(frozen_field(m))
+        tr = g.trace(np.arange(n), seed=8)
+        for est in (0, rt.EST_PATHLENGTH):
+            g.reset()
+            g.transport(n, seed=8, mode=rt.REEMIT_FROZEN, walk=getattr(rt, "WALK_" + walk),
+                        estimators=est)
+            c, sed = g.counters(), g.sed()[0][0]
+            assert c["errors"] == 0 and c["escaped"] == n == int(sed.sum())
+            slack = 0 if S != 2 else 2 * int(tr[:, 1].max())
+            assert abs(c["absorptions"] - int(tr[:, 1].sum())) <= slack
+            assert c["absorptions"] == int(g.counts().sum())
