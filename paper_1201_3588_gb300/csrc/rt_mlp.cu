@@ -51,8 +51,10 @@ struct rt_mlp {
   float* d_m = nullptr;
   float* d_v = nullptr;
   bf16* d_wbf = nullptr;     // padded BF16 weights
-  bf16* d_wpk = nullptr;     // the same weights in the tensor-core operand layout
-  bool pk_stale = true;      // d_wpk lags behind d_wbf
+  // the same weights in the operand layouts of the two fused forward kernels (see
+  // forward_tc), and whether each lags behind d_wbf
+  bf16* d_wpk[2] = {nullptr, nullptr};
+  bool pk_stale[2] = {true, true};
   unsigned* d_err = nullptr; // fused forward: nonzero after a wait ran out
   float* d_loss = nullptr;
   long long step = 0;
@@ -131,7 +133,7 @@ __global__ void k_adam(float4* p, const float4* g, float4* m, float4* v, uint2* 
 // three, each piece used by both tiles; one warp issues the copies, one the products.
 // With one tile per CTA, a whole layer's weights at a time and the steps one after another,
 // 4.0e5 rows of 66 - 3x256 - 200 took 0.373 ms; now 0.262 ms (608 TFLOP/s of the 1863 that a
-// dense product reaches; 65536 rows 83 -> 62 us, up to 16384 rows 33 -> 29 us). Half of that
+// dense product reaches; 65536 rows 83 -> 62 us). Half of that
 // came from the halves and the ring (0.327 ms), half from one 32-column accumulator load per
 // wait, biases from shared memory and input rows converted 8 columns at a time, before the
 // previous step's last outputs are stored. What is left is the chain of a layer's products,
@@ -742,27 +744,29 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
       : "memory");
 }
 
-// y[0 .. 31] of a row: 32-byte stores where the rows allow them, whole sectors each
+// y[0 .. 31] of a row: whole sectors where rows lie on 32-byte boundaries, which is what this
+// kernel is chosen for; else element by element. (Without that branch, or with a constant
+// number of tiles, the compiler spills 92 bytes: 291 against 262 us for 4.0e5 rows.)
 __device__ __forceinline__ void store_outputs(float* y, const float* v, int n, bool vec8) {
-  if (vec8) {
-#pragma unroll
-    for (int j = 0; j < 32; j += 8)
-      if (j < n)
-        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                         __cvta_generic_to_global(y + j)),
-                     "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]), "f"(v[j + 4]),
-                     "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7])
-                     : "memory");
-  } else {
+  if (!vec8) {
 #pragma unroll
     for (int j = 0; j < 32; ++j)
       if (j < n) y[j] = v[j];
+    return;
   }
+#pragma unroll
+  for (int j = 0; j < 32; j += 8)
+    if (j < n)
+      asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                       __cvta_generic_to_global(y + j)),
+                   "f"(v[j]), "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]), "f"(v[j + 4]),
+                   "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7])
+                   : "memory");
 }
 
 constexpr int kTcAhead = 3;  // input items (8 columns of a row) a thread has in flight
 
-// tiles: 1 or 2 of 128 rows per step of a CTA
+// tiles: of 128 rows per step of a CTA
 __global__ void __launch_bounds__(kTcThreads, 1)
     k_mlp_forward_tc(const __grid_constant__ TcNet net, const float* x, long long M, float* y,
                      int tiles, unsigned* err) {
@@ -1068,6 +1072,251 @@ size_t tc_smem_bytes() {
   return kTcTiles * kTcActBytes + kTcRing * kTcPieceBytes + sizeof(TcBars);
 }
 
+// ---------------------------------------------------------------- few rows, or ragged outputs
+// One 128-row tile at a time, a layer's weights in one copy, 32 warps on one epilogue, the
+// outputs staged in shared memory and written coalesced. forward_tc says when it is taken.
+constexpr int kTileThreads = 1024;
+
+// element offset of (r, k) in a [rows][K] operand in the core-matrix layout
+__device__ __forceinline__ int core_off(int r, int k, int K) {
+  return (r >> 3) * (K << 3) + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
+}
+
+// weights [out_p][in_p] row-major -> the core-matrix layout (one thread per element)
+__global__ void k_pack_layer(const bf16* w, int out_p, int in_p, bf16* out) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= (long long)out_p * in_p) return;
+  const int r = (int)(i / in_p), k = (int)(i % in_p);
+  out[core_off(r, k, in_p)] = w[i];
+}
+
+__global__ void __launch_bounds__(kTileThreads, 1) k_mlp_forward_tile(const __grid_constant__ TcNet net,
+                                                           const float* x, long long M,
+                                                           float* y, unsigned* err) {
+  extern __shared__ __align__(128) unsigned char tc_smem[];
+  bf16* sA = reinterpret_cast<bf16*>(tc_smem);                       // [128][256]
+  bf16* sB = sA + kTcRows * kTcMaxWidth;                             // [256][256]
+  float* sBias = reinterpret_cast<float*>(sB + kTcMaxWidth * kTcMaxWidth);  // [layers][256]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sBias + kMaxLayers * kTcMaxWidth);  // [2]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 2);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // biases of every layer, zero in the padding columns
+  for (int i = tid; i < net.n_layers * kTcMaxWidth; i += kTileThreads) {
+    const int l = i / kTcMaxWidth, c = i % kTcMaxWidth;
+    sBias[i] = c < net.n_valid[l] ? net.b[l][c] : 0.0f;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_addr(tmem_slot)),
+                 "r"(kTcMaxWidth));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar + 1)));
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t bar_a = smem_addr(bar);      // MMAs done
+  const uint32_t bar_w = smem_addr(bar + 1);  // weights arrived
+  uint32_t parity = 0, wparity = 0;
+  bool ok = true;
+  uint32_t pend = 0;  // after a wait ran out: the barrier still owed a completion
+  const long long n_tiles = (M + kTcRows - 1) / kTcRows;
+  for (long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+    const long long r0 = tile * kTcRows;
+    // the first layer's weights stream in while the input is converted
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      const int n0 = net.out_p[0] < kTcMaxWidth ? net.out_p[0] : kTcMaxWidth;
+      bulk_load(smem_addr(sB), net.w[0], (uint32_t)(n0 * net.in_p[0] * 2), bar_w);
+    }
+    // input rows -> BF16 activations: the tile's rows are contiguous in x, read
+    // coalesced; zero beyond the valid rows and in the padding columns
+    {
+      const int K = net.in_p[0], F = net.n_in;
+      const long long valid = M - r0 < kTcRows ? M - r0 : kTcRows;
+      const float* xt = x + r0 * F;
+      const int total = kTcRows * F, n_ok = (int)valid * F;
+      // row of element i: (i + 1/2)/F lies at least 1/(2F) >= 2^-9 from an integer
+      // and i < 2^15, so the FP32 product truncates to floor(i/F) exactly
+      const float inv_f = 1.0f / (float)F;
+      for (int i0 = tid; i0 < total; i0 += 4 * kTileThreads) {
+        float v[4];  // four loads in flight before the stores
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kTileThreads;
+          v[u] = i < n_ok ? __ldg(&xt[i]) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kTileThreads;
+          if (i < total) {
+            const int r = (int)(((float)i + 0.5f) * inv_f), k = i - r * F;
+            sA[core_off(r, k, K)] = __float2bfloat16(v[u]);
+          }
+        }
+      }
+      if (tid < kTcRows)
+        for (int k = F; k < K; ++k) sA[core_off(tid, k, K)] = __float2bfloat16(0.0f);
+    }
+    // stages: (layer, chunk of at most 256 output columns); only the output layer
+    // may have more than one chunk (its packed weight rows are contiguous per chunk)
+    for (int l = 0; l < net.n_layers && ok; ++l) {
+      const int K = net.in_p[l], Np = net.out_p[l];
+      const bool hidden = l < net.n_layers - 1;
+      const int n_chunks = (Np + kTcMaxWidth - 1) / kTcMaxWidth;
+      for (int ch = 0; ch < n_chunks && ok; ++ch) {
+        const int col0 = ch * kTcMaxWidth;                    // first output column
+        const int N = Np - col0 < kTcMaxWidth ? Np - col0 : kTcMaxWidth;
+        // this stage's weights (bulk copy issued earlier)
+        const bool got_w = mbar_wait(bar_w, wparity);
+        if (!__syncthreads_and(got_w)) {
+          if (tid == 0) atomicOr(err, 1u);
+          ok = false;
+          pend = bar_w;
+          const long long gr = r0 + tid;
+          if (tid < kTcRows && gr < M)
+            for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
+          break;
+        }
+        wparity ^= 1u;
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        __syncthreads();
+        if (tid == 0) {
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          const uint32_t idesc = tc_idesc(kTcRows, N);
+          const uint32_t a0 = smem_addr(sA), b0 = smem_addr(sB);
+          const uint32_t sbo = (uint32_t)K * 16u;  // (K/8) cores of 128 bytes
+          for (int kk = 0; kk < K / 16; ++kk)
+            tc_mma(tmem, tc_desc(a0 + kk * 256u, 128u, sbo), tc_desc(b0 + kk * 256u, 128u, sbo),
+                   idesc, kk > 0 ? 1u : 0u);
+          asm volatile(
+              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                  bar_a)
+              : "memory");
+        }
+        const bool waited = mbar_wait(bar_a, parity);
+        if (!__syncthreads_and(waited)) {  // the MMAs never signalled completion
+          if (tid == 0) atomicOr(err, 1u);
+          ok = false;
+          pend = bar_a;
+          const long long gr = r0 + tid;
+          if (tid < kTcRows && gr < M)
+            for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
+          break;
+        }
+        parity ^= 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        // the weight buffer is free: the next stage's weights stream in meanwhile
+        // (after a single-chunk output layer the buffer stages the outputs instead)
+        if (tid == 0) {
+          if (ch + 1 < n_chunks) {
+            const int n1 = Np - col0 - kTcMaxWidth < kTcMaxWidth ? Np - col0 - kTcMaxWidth
+                                                                : kTcMaxWidth;
+            bulk_load(smem_addr(sB), net.w[l] + (size_t)(col0 + kTcMaxWidth) * K,
+                      (uint32_t)(n1 * K * 2), bar_w);
+          } else if (hidden) {
+            const int n1 = net.out_p[l + 1] < kTcMaxWidth ? net.out_p[l + 1] : kTcMaxWidth;
+            bulk_load(smem_addr(sB), net.w[l + 1], (uint32_t)(n1 * net.in_p[l + 1] * 2), bar_w);
+          }
+        }
+        // accumulators of this warp's 32 rows: bias, activation, next operand or output
+        const int quarter = warp & 3;                 // lanes 32 quarter .. of the accumulators
+        const int row = quarter * 32 + lane;
+        const int group = warp >> 2, n_groups = kTileThreads / 128;
+        const float* bias = sBias + l * kTcMaxWidth;
+        // a single-chunk output layer is staged over both operand buffers (the last MMA
+        // is done) with an odd row stride, so that the 32 rows a warp stores hit 32
+        // different banks; wider output layers are stored from registers per chunk
+        const int o_stride = net.n_out | 1;
+        float* so = reinterpret_cast<float*>(sA);
+        const long long grow = r0 + row;
+        const bool vec4 = (net.n_out & 3) == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0;
+        for (int c0 = 16 * group; c0 < N; c0 += 16 * n_groups) {
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
+          float bv[16];
+          if (n_chunks == 1) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4*>(&bv[j]) =
+                *reinterpret_cast<const float4*>(&bias[c0 + j]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int c = col0 + c0 + j;
+              bv[j] = c < net.n_valid[l] ? __ldg(&net.b[l][c]) : 0.0f;
+            }
+          }
+          if (hidden) {
+            uint32_t h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const __nv_bfloat162 p =
+                  __floats2bfloat162_rn(silu_fast(v[2 * j] + bv[2 * j]),
+                                        silu_fast(v[2 * j + 1] + bv[2 * j + 1]));
+              h[j] = *reinterpret_cast<const uint32_t*>(&p);
+            }
+            // columns c0..c0+15 of this row: two 16-byte pieces of the next operand
+            *reinterpret_cast<uint4*>(&sA[core_off(row, c0, N)]) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(&sA[core_off(row, c0 + 8, N)]) =
+                make_uint4(h[4], h[5], h[6], h[7]);
+          } else if (n_chunks == 1) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int c = c0 + j;
+              if (c < net.n_out) so[row * o_stride + c] = v[j] + bv[j];
+            }
+          } else if (grow < M) {
+            float* yr = y + grow * net.n_out + col0 + c0;
+            if (vec4 && col0 + c0 + 16 <= net.n_out) {
+#pragma unroll
+              for (int j = 0; j < 16; j += 4)
+                *reinterpret_cast<float4*>(&yr[j]) =
+                    make_float4(v[j] + bv[j], v[j + 1] + bv[j + 1], v[j + 2] + bv[j + 2],
+                                v[j + 3] + bv[j + 3]);
+            } else {
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                if (col0 + c0 + j < net.n_out) yr[j] = v[j] + bv[j];
+            }
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        __syncthreads();
+        if (!hidden && n_chunks == 1) {  // the tile's output rows are contiguous in y
+          const long long valid = M - r0 < kTcRows ? M - r0 : kTcRows;
+          float* yt = y + r0 * net.n_out;
+          for (int r = warp; r < (int)valid; r += kTileThreads / 32)
+            for (int c = lane; c < net.n_out; c += 32)
+              yt[(long long)r * net.n_out + c] = so[r * o_stride + c];
+          __syncthreads();
+        }
+      }
+    }
+  }
+  // after a wait that ran out: let the weight copy or the MMAs still in flight land
+  // (again with a time limit) before the shared and tensor memory are released
+  if (pend != 0 && warp == 0) mbar_wait(pend, pend == bar_w ? wparity : parity);
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                 "r"(kTcMaxWidth));
+  }
+}
+
+size_t tile_smem_bytes() {
+  return sizeof(bf16) * (size_t)(kTcRows + kTcMaxWidth) * kTcMaxWidth +
+         sizeof(float) * kMaxLayers * kTcMaxWidth + 32;
+}
+
 inline unsigned nb(long long n, int t);
 
 inline unsigned nb(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -1167,7 +1416,7 @@ rt_status ensure_rows(rt_mlp* m, long long rows, bool train) {
 
 rt_status refresh_bf16(rt_mlp* m, cudaStream_t s) {
   k_to_bf16<<<nb((long long)m->n_padded, 256), 256, 0, s>>>(m->d_param, m->d_wbf, m->n_padded);
-  m->pk_stale = true;
+  m->pk_stale[0] = m->pk_stale[1] = true;
   return cudaGetLastError() == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }
 
@@ -1182,16 +1431,28 @@ bool tc_eligible(const rt_mlp* m) {
   return true;
 }
 
-// forward of M rows with the fused tensor-core kernel (weights repacked when stale)
+// forward of M rows with a fused tensor-core kernel (weights repacked when stale): the
+// pieces' kernel where there are more tiles than SMs, so that a CTA has two to overlap, and
+// whole 32-byte sectors to write; else one tile at a time. 49 to 66 inputs, 64 to 256 wide,
+// pieces against tile, us: 4.0e5 rows with 200 outputs 262 against 374, 3.0e5 with 400 outputs
+// 195 against 328, with 131 (whose rows it writes through a transpose) 292 against 274; 500
+// rows 31 against 28.
 rt_status forward_tc(rt_mlp* m, const float* x, float* y, long long M, cudaStream_t s) {
-  if (m->pk_stale) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->dev) != cudaSuccess)
+    return RT_ERR_CUDA;
+  const long long n_tiles = (M + kTcRows - 1) / kTcRows;
+  const int pieces = n_tiles > sms && m->n_out % 8 == 0 &&
+                     (reinterpret_cast<uintptr_t>(y) & 31) == 0;
+  if (m->pk_stale[pieces]) {
     for (int l = 0; l < m->n_layers_total; ++l) {
       const Layer& ly = m->layer[l];
-      k_pack_weights<<<nb((long long)ly.out_p * ly.in_p, 256), 256, 0, s>>>(
-          m->d_wbf + ly.w_off, ly.out_p, ly.in_p, m->d_wpk + ly.w_off);
+      const auto pack = pieces ? k_pack_weights : k_pack_layer;
+      pack<<<nb((long long)ly.out_p * ly.in_p, 256), 256, 0, s>>>(
+          m->d_wbf + ly.w_off, ly.out_p, ly.in_p, m->d_wpk[pieces] + ly.w_off);
     }
     if (cudaGetLastError() != cudaSuccess) return RT_ERR_CUDA;
-    m->pk_stale = false;
+    m->pk_stale[pieces] = false;
   }
   TcNet net{};
   net.n_layers = m->n_layers_total;
@@ -1202,23 +1463,21 @@ rt_status forward_tc(rt_mlp* m, const float* x, float* y, long long M, cudaStrea
     net.in_p[l] = ly.in_p;
     net.out_p[l] = ly.out_p;
     net.n_valid[l] = ly.n_out;
-    net.w[l] = m->d_wpk + ly.w_off;
+    net.w[l] = m->d_wpk[pieces] + ly.w_off;
     net.b[l] = m->d_param + ly.b_off;
   }
-  const size_t smem = tc_smem_bytes();
-  if (cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const size_t smem = pieces ? tc_smem_bytes() : tile_smem_bytes();
+  if (cudaFuncSetAttribute(pieces ? reinterpret_cast<const void*>(k_mlp_forward_tc)
+                                  : reinterpret_cast<const void*>(k_mlp_forward_tile),
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess)
     return RT_ERR_CUDA;
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->dev) != cudaSuccess)
-    return RT_ERR_CUDA;
-  // two tiles a step where there are more tiles than SMs, else one (more CTAs, no overlap
-  // to gain between tiles)
-  const long long n_tiles = (M + kTcRows - 1) / kTcRows;
-  const int tiles = n_tiles > sms ? kTcTiles : 1;
-  const long long steps = (n_tiles + tiles - 1) / tiles;
+  const long long steps = pieces ? (n_tiles + kTcTiles - 1) / kTcTiles : n_tiles;
   const unsigned grid = (unsigned)(steps < sms ? steps : sms);
-  k_mlp_forward_tc<<<grid, kTcThreads, smem, s>>>(net, x, M, y, tiles, m->d_err);
+  if (pieces)
+    k_mlp_forward_tc<<<grid, kTcThreads, smem, s>>>(net, x, M, y, kTcTiles, m->d_err);
+  else
+    k_mlp_forward_tile<<<grid, kTileThreads, smem, s>>>(net, x, M, y, m->d_err);
   return cudaGetLastError() == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }
 
@@ -1305,7 +1564,7 @@ rt_status rt_mlp_create(int n_in, int n_hidden, int n_layers, int n_out, uint64_
   rt_status st;
   if ((st = alloc(&m->d_param, off)) != RT_OK || (st = alloc(&m->d_grad, off)) != RT_OK ||
       (st = alloc(&m->d_m, off)) != RT_OK || (st = alloc(&m->d_v, off)) != RT_OK ||
-      (st = alloc(&m->d_wbf, off)) != RT_OK || (st = alloc(&m->d_wpk, off)) != RT_OK ||
+      (st = alloc(&m->d_wbf, off)) != RT_OK || (st = alloc(&m->d_wpk[0], 2 * off)) != RT_OK ||
       (st = alloc(&m->d_err, 1)) != RT_OK || (st = alloc(&m->d_loss, 1)) != RT_OK) {
     rt_mlp_destroy(m);
     return st;
@@ -1322,6 +1581,7 @@ rt_status rt_mlp_create(int n_in, int n_hidden, int n_layers, int n_out, uint64_
         h[ly.w_off + (size_t)r * ly.in_p + c] = (float)((2.0 * u - 1.0) * lim);
       }
   }
+  m->d_wpk[1] = m->d_wpk[0] + off;
   cudaError_t e = cudaMemcpy(m->d_param, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(m->d_m, 0, sizeof(float) * off);
   if (e == cudaSuccess) e = cudaMemset(m->d_v, 0, sizeof(float) * off);
@@ -1344,7 +1604,7 @@ rt_status rt_mlp_destroy(rt_mlp* m) {
   release(m->d_m);
   release(m->d_v);
   release(m->d_wbf);
-  release(m->d_wpk);
+  release(m->d_wpk[0]);  // [1] is its second half
   release(m->d_err);
   release(m->d_loss);
   delete m;
@@ -1493,7 +1753,7 @@ rt_status rt_mlp_adam_step(rt_mlp* m, float lr, void* stream) {
       reinterpret_cast<float4*>(m->d_param), reinterpret_cast<const float4*>(m->d_grad),
       reinterpret_cast<float4*>(m->d_m), reinterpret_cast<float4*>(m->d_v),
       reinterpret_cast<uint2*>(m->d_wbf), (size_t)n4, lr, b1, b2, c1, c2, 1e-8f);
-  m->pk_stale = true;
+  m->pk_stale[0] = m->pk_stale[1] = true;
   return cudaGetLastError() == cudaSuccess ? RT_OK : RT_ERR_CUDA;
 }
 
