@@ -1769,7 +1769,15 @@ __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const 
                                         md.t.kext);
     flush_warp(tl, wt, md.r.counters);
     __syncwarp();
-    if (!in_time) break;
+    if (!in_time) {
+      // the budget is the launch's: what is left of any model stays undone, and its status
+      // says so, also where no warp was on it (models with few packages wait for the large)
+      for (int j = lane; j < n_models; j += 32)
+        if (*reinterpret_cast<const volatile unsigned long long*>(&next[j]) <
+            models[j].r.n_packages)
+          atomicOr(models[j].r.status, kStatusTimeout);
+      break;
+    }
   }
 }
 
