@@ -58,6 +58,7 @@ struct rt_mlp {
   unsigned* d_err = nullptr; // fused forward: nonzero after a wait ran out
   float* d_loss = nullptr;
   long long step = 0;
+  long long wait_clocks = 4000000000ll;  // of the fused forward's waits (see kTcWaitClocks)
   float x_lo = -1e30f, x_hi = 1e30f;  // admissible range of the second-to-last input
   // activations for up to cap rows
   long long cap = 0;
@@ -677,6 +678,7 @@ struct TcNet {
   int in_p[kMaxLayers], out_p[kMaxLayers], n_valid[kMaxLayers];
   const bf16* w[kMaxLayers];    // packed weights of each layer
   const float* b[kMaxLayers];   // padded biases
+  long long wait_clocks;        // limit of the epilogue's waits; 0: give up without waiting
 };
 
 // A layer's weights [out_p][in_p] are packed piece by piece: rows in halves of 128, columns
@@ -702,6 +704,7 @@ struct TcBars {
   uint64_t full[kTcRing], empty[kTcRing];  // weight pieces arrived / read by their products
   uint64_t acc[2];    // first half's products done; all of the stage's products done
   uint64_t ready[2];  // a half of the activations written (and its accumulators read)
+  uint64_t drained;   // once: all products issued are done
   uint32_t tmem_slot, failed;
   alignas(16) float bias[2][kTcMaxWidth];  // of this stage and the next
 };
@@ -717,7 +720,12 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 // A wait that also ends when another of the CTA's waits ran out.
-__device__ __forceinline__ bool tc_wait(TcBars* bars, uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool tc_wait(TcBars* bars, uint64_t* bar, uint32_t parity,
+                                        long long limit = kTcWaitClocks) {
+  if (limit <= 0) {
+    *reinterpret_cast<volatile uint32_t*>(&bars->failed) = 1u;
+    return false;
+  }
   const long long t0 = clock64();
   const uint32_t addr = smem_addr(bar);
   for (;;) {
@@ -730,7 +738,7 @@ __device__ __forceinline__ bool tc_wait(TcBars* bars, uint64_t* bar, uint32_t pa
         : "memory");
     if (done) return true;
     if (*reinterpret_cast<volatile uint32_t*>(&bars->failed)) return false;
-    if (clock64() - t0 > kTcWaitClocks) {
+    if (clock64() - t0 > limit) {
       *reinterpret_cast<volatile uint32_t*>(&bars->failed) = 1u;
       return false;
     }
@@ -783,6 +791,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       mbar_init(&bars->acc[i], 1);
       mbar_init(&bars->ready[i], kTcEpiWarps);
     }
+    mbar_init(&bars->drained, 1);
     bars->failed = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -809,14 +818,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int l = 0; l < L && ok; ++l) {
           const int N = net.out_p[l], K = net.in_p[l];
           for (int n0 = 0; n0 < N && ok; n0 += kTcHalf)
-            for (int k0 = 0; k0 < K && ok; k0 += kTcHalf, ++piece) {
+            for (int k0 = 0; k0 < K; k0 += kTcHalf) {
               const uint32_t slot = piece % kTcRing, round = piece / kTcRing;
               if (round > 0) ok = tc_wait(bars, &bars->empty[slot], (round - 1) & 1u);
-              if (ok)
-                bulk_load(smem_addr(sW + slot * kTcPieceBytes),
-                          net.w[l] + piece_start(n0, k0, N, K),
-                          (uint32_t)(min(kTcHalf, N - n0) * min(kTcHalf, K - k0) * 2),
-                          smem_addr(&bars->full[slot]));
+              if (!ok) break;  // this piece was not copied
+              bulk_load(smem_addr(sW + slot * kTcPieceBytes),
+                        net.w[l] + piece_start(n0, k0, N, K),
+                        (uint32_t)(min(kTcHalf, N - n0) * min(kTcHalf, K - k0) * 2),
+                        smem_addr(&bars->full[slot]));
+              ++piece;
             }
         }
       // copies still in flight land before the memory is given up: the last of each slot
@@ -864,10 +874,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (ok) tc_commit(&bars->acc[1]);
           }
         }
-      if (!ok) {  // let the products in flight land before the memory is given up
-        tc_commit(&bars->acc[1]);
-        mbar_wait(smem_addr(&bars->acc[1]), stage & 1u);
-      }
+      // the products in flight land before the memory is given up, whichever warp's wait ran
+      // out: a barrier of its own, whose one phase no other commit completes
+      tc_commit(&bars->drained);
+      mbar_wait(smem_addr(&bars->drained), 0u);
     }
   } else {
     // ---- input, activations and outputs
@@ -1014,7 +1024,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 col0 + c < net.out_p[l] ? __ldg(&net.b[l][col0 + c]) : 0.0f;
           }
           __syncwarp();
-          ok = __all_sync(0xffffffffu, tc_wait(bars, &bars->acc[0], stage & 1u));
+          ok = __all_sync(0xffffffffu,
+                          tc_wait(bars, &bars->acc[0], stage & 1u, net.wait_clocks));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           if (hidden) {
@@ -1024,7 +1035,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (!last) written(0);
           }
           // the second half's products read the layer's input to their end
-          ok = __all_sync(0xffffffffu, tc_wait(bars, &bars->acc[1], stage & 1u));
+          ok = __all_sync(0xffffffffu,
+                          tc_wait(bars, &bars->acc[1], stage & 1u, net.wait_clocks));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           if (hidden) {
@@ -1466,6 +1478,7 @@ rt_status forward_tc(rt_mlp* m, const float* x, float* y, long long M, cudaStrea
     net.w[l] = m->d_wpk[pieces] + ly.w_off;
     net.b[l] = m->d_param + ly.b_off;
   }
+  net.wait_clocks = m->wait_clocks;
   const size_t smem = pieces ? tc_smem_bytes() : tile_smem_bytes();
   if (cudaFuncSetAttribute(pieces ? reinterpret_cast<const void*>(k_mlp_forward_tc)
                                   : reinterpret_cast<const void*>(k_mlp_forward_tile),
@@ -1629,6 +1642,12 @@ rt_status rt_mlp_get_range(const rt_mlp* m, float* lo, float* hi) {
   if (!m || !lo || !hi) return RT_ERR_ARG;
   *lo = m->x_lo;
   *hi = m->x_hi;
+  return RT_OK;
+}
+
+rt_status rt_mlp_set_wait_limit(rt_mlp* m, double seconds) {
+  if (!m || !(seconds >= 0) || seconds > 60) return RT_ERR_ARG;
+  m->wait_clocks = (long long)(seconds * 2e9);
   return RT_OK;
 }
 

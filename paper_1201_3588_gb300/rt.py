@@ -137,6 +137,7 @@ SIGNATURES = {
                               C.c_void_p, C.c_void_p, C.c_void_p],
     "rt_mlp_dims": [C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_int)],
     "rt_mlp_set_range": [C.c_void_p, C.c_float, C.c_float],
+    "rt_mlp_set_wait_limit": [C.c_void_p, C.c_double],
     "rt_mlp_get_range": [C.c_void_p, C.POINTER(C.c_float), C.POINTER(C.c_float)],
     "rt_cell_temperatures_noalloc": [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                      C.c_void_p, C.c_int, C.c_int64, C.c_int, C.c_double,
@@ -645,6 +646,10 @@ class MLP:
 
     def set_range(self, lo: float, hi: float):
         _check(load().rt_mlp_set_range(self._h, float(lo), float(hi)), "rt_mlp_set_range")
+
+    def set_wait_limit(self, seconds: float):
+        """Limit of the forward pass's waits for the tensor cores (2 s; 0: give up at once)."""
+        _check(load().rt_mlp_set_wait_limit(self._h, float(seconds)), "rt_mlp_set_wait_limit")
 
     def adam_step(self, lr: float, stream=None):
         _check(load().rt_mlp_adam_step(self._h, float(lr), _stream(stream)), "rt_mlp_adam_step")

@@ -1,0 +1,51 @@
+"""The forward pass when a wait for the tensor cores runs out (a limit of 0 gives up every
+wait of the epilogue at once, while weight copies and products are on their way): the kernel
+ends by itself with its copies and products landed and its tensor memory given back, the next
+read of the handle reports the timeout, and the GPU goes on computing as before."""
+import pytest
+
+from paper_1201_3588_gb300 import rt
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+RT_ERR_TIMEOUT = 4
+# rows for the kernel of many rows (more than 152 tiles of 128, output rows on 32-byte
+# boundaries): one and several steps a CTA, one and several layers and output chunks
+MANY = [(39_000, 66, 256, 3, 200), (150_001, 66, 256, 3, 200), (90_000, 34, 64, 1, 8),
+        (60_000, 128, 128, 2, 400)]
+
+
+def _net(n_in, hidden, layers, n_out):
+    return rt.MLP(n_in, hidden, layers, n_out, seed=3)
+
+
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", MANY)
+def test_gives_up_reports_and_goes_on(M, n_in, hidden, layers, n_out):
+    x = torch.randn((M, n_in), generator=torch.Generator().manual_seed(1)).cuda()
+    good, bad = _net(n_in, hidden, layers, n_out), _net(n_in, hidden, layers, n_out)
+    want = good.forward(x, torch.empty((M, n_out), device="cuda")).clone()
+    bad.set_wait_limit(0.0)
+    y = torch.zeros((M, n_out), device="cuda")
+    for _ in range(3):
+        bad.forward(x, y)
+    torch.cuda.synchronize()
+    with pytest.raises(rt.RTError) as e:
+        bad.get_params()
+    assert e.value.code == RT_ERR_TIMEOUT
+    # tensor memory that was not given back would leave none for these
+    for net in (good, _net(n_in, hidden, layers, n_out)):
+        got = net.forward(x, torch.zeros((M, n_out), device="cuda"))
+        torch.cuda.synchronize()
+        net.get_params()
+        assert torch.equal(got, want)
+    # within the limit again: the outputs are those of any other handle
+    bad.set_wait_limit(2.0)
+    assert torch.equal(bad.forward(x, y), want)
+
+
+def test_limit_is_checked():
+    net = _net(8, 16, 1, 8)
+    for s in (-1.0, float("nan"), 61.0):
+        with pytest.raises(rt.RTError):
+            net.set_wait_limit(s)
