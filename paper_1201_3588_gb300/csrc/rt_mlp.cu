@@ -1060,12 +1060,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
       }
     }
-    if (!ok) {  // a wait ran out: the rows of this and the later steps are not to be used
-      if (tid == 0) atomicOr(err, 1u);
-      for (long long s = step; s < n_steps; s += gridDim.x)
+    // a wait ran out: the rows of that step (the loop has gone one past it) and the later ones
+    // are not to be used. Every warp that gave up marks its rows: another may have found the
+    // same barrier complete.
+    if (!ok) {
+      if (lane == 0) atomicOr(err, 1u);
+      for (long long s = step - gridDim.x; s < n_steps; s += gridDim.x)
         for (int t = 0; t < tiles; ++t) {
           const long long row = s * step_rows + t * kTcRows + row_in;
-          if (group == 0 && row < M)
+          if (row < M)
             for (int c = 0; c < net.n_out; ++c)
               y[row * net.n_out + c] = __int_as_float(0x7fc00000);
         }

@@ -44,6 +44,20 @@ def test_gives_up_reports_and_goes_on(M, n_in, hidden, layers, n_out):
     assert torch.equal(bad.forward(x, y), want)
 
 
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", MANY)
+def test_no_row_keeps_what_it_held(M, n_in, hidden, layers, n_out):
+    x = torch.randn((M, n_in), generator=torch.Generator().manual_seed(1)).cuda()
+    net = _net(n_in, hidden, layers, n_out)
+    net.set_wait_limit(0.0)
+    # y as an earlier, plausible result, between guards
+    buf = torch.full((M * n_out + 16,), 0.5, device="cuda")
+    y = buf[8:8 + M * n_out].view(M, n_out)
+    net.forward(x, y)
+    torch.cuda.synchronize()
+    assert torch.isnan(y).all()
+    assert (buf[:8] == 0.5).all() and (buf[8 + M * n_out:] == 0.5).all()
+
+
 def test_limit_is_checked():
     net = _net(8, 16, 1, 8)
     for s in (-1.0, float("nan"), 61.0):
