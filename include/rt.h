@@ -459,12 +459,12 @@ rt_status rt_mlp_dims(const rt_mlp *m, int *n_in, int *n_out);
  * solution. Default: unbounded. */
 rt_status rt_mlp_set_range(rt_mlp *m, float lo, float hi);
 rt_status rt_mlp_get_range(const rt_mlp *m, float *lo, float *hi);
-/* Limit of the waits for the tensor cores in rt_mlp_forward's fused kernel for many rows,
- * 0 to 60 s of SM clocks at 2 GHz (default 2). 0: every wait gives up at once, for
+/* Limit of the waits for the tensor cores in rt_mlp_forward's fused kernels, 0 to
+ * 60 s of SM clocks at 2 GHz (default 2). 0: every wait gives up at once, for
  * callers' tests of what they do with the RT_ERR_TIMEOUT that follows. */
 rt_status rt_mlp_set_wait_limit(rt_mlp *m, double seconds);
-/* host [n_params]; RT_ERR_TIMEOUT when a tensor-core forward pass gave up waiting for
- * its MMAs since the handle was created (its outputs were set to NaN) */
+/* host [n_params]; RT_ERR_TIMEOUT when a pass gave up waiting for its MMAs since the
+ * handle was created (a fused forward sets the rows from there on to NaN) */
 rt_status rt_mlp_get_params(rt_mlp *m, float *out);
 rt_status rt_mlp_set_params(rt_mlp *m, const float *in);  /* host [n_params] */
 

@@ -184,7 +184,9 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, 
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
+                                          long long limit = kTcWaitClocks) {
+  if (limit <= 0) return false;
   const long long t0 = clock64();
   for (;;) {
     uint32_t done;
@@ -194,7 +196,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         : "=r"(done)
         : "r"(bar), "r"(parity));
     if (done) return true;
-    if (clock64() - t0 > kTcWaitClocks) return false;
+    if (clock64() - t0 > limit) return false;
   }
 }
 
@@ -678,7 +680,7 @@ struct TcNet {
   int in_p[kMaxLayers], out_p[kMaxLayers], n_valid[kMaxLayers];
   const bf16* w[kMaxLayers];    // packed weights of each layer
   const float* b[kMaxLayers];   // padded biases
-  long long wait_clocks;        // limit of the epilogue's waits; 0: give up without waiting
+  long long wait_clocks;        // limit of the waits for results; 0: give up without waiting
 };
 
 // A layer's weights [out_p][in_p] are packed piece by piece: rows in halves of 128, columns
@@ -1141,7 +1143,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_mlp_forward_tile(const __gr
   bool ok = true;
   uint32_t pend = 0;  // after a wait ran out: the barrier still owed a completion
   const long long n_tiles = (M + kTcRows - 1) / kTcRows;
-  for (long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+  long long tile = blockIdx.x;
+  for (; tile < n_tiles && ok; tile += gridDim.x) {
     const long long r0 = tile * kTcRows;
     // the first layer's weights stream in while the input is converted
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -1189,14 +1192,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_mlp_forward_tile(const __gr
         const int col0 = ch * kTcMaxWidth;                    // first output column
         const int N = Np - col0 < kTcMaxWidth ? Np - col0 : kTcMaxWidth;
         // this stage's weights (bulk copy issued earlier)
-        const bool got_w = mbar_wait(bar_w, wparity);
+        const bool got_w = mbar_wait(bar_w, wparity, net.wait_clocks);
         if (!__syncthreads_and(got_w)) {
           if (tid == 0) atomicOr(err, 1u);
           ok = false;
           pend = bar_w;
-          const long long gr = r0 + tid;
-          if (tid < kTcRows && gr < M)
-            for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
           break;
         }
         wparity ^= 1u;
@@ -1216,14 +1216,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_mlp_forward_tile(const __gr
                   bar_a)
               : "memory");
         }
-        const bool waited = mbar_wait(bar_a, parity);
+        const bool waited = mbar_wait(bar_a, parity, net.wait_clocks);
         if (!__syncthreads_and(waited)) {  // the MMAs never signalled completion
           if (tid == 0) atomicOr(err, 1u);
           ok = false;
           pend = bar_a;
-          const long long gr = r0 + tid;
-          if (tid < kTcRows && gr < M)
-            for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
           break;
         }
         parity ^= 1u;
@@ -1318,6 +1315,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_mlp_forward_tile(const __gr
   // after a wait that ran out: let the weight copy or the MMAs still in flight land
   // (again with a time limit) before the shared and tensor memory are released
   if (pend != 0 && warp == 0) mbar_wait(pend, pend == bar_w ? wparity : parity);
+  // and the rows of that tile (the loop has gone one past it) and the later ones are not to
+  // be used
+  if (!ok)
+    for (long long t = tile - gridDim.x; t < n_tiles; t += gridDim.x) {
+      const long long gr = t * kTcRows + tid;
+      if (tid < kTcRows && gr < M)
+        for (int c = 0; c < net.n_out; ++c) y[gr * net.n_out + c] = __int_as_float(0x7fc00000);
+    }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   if (warp == 0) {

@@ -15,12 +15,16 @@ RT_ERR_TIMEOUT = 4
 MANY = [(39_000, 66, 256, 3, 200), (150_001, 66, 256, 3, 200), (90_000, 34, 64, 1, 8),
         (60_000, 128, 128, 2, 400)]
 
+# and for the one of few rows or ragged outputs: one and several tiles a CTA
+FEW = [(100, 66, 256, 3, 200), (45_001, 66, 256, 3, 131), (60_000, 34, 64, 1, 7),
+       (30_000, 128, 128, 2, 333)]
+
 
 def _net(n_in, hidden, layers, n_out):
     return rt.MLP(n_in, hidden, layers, n_out, seed=3)
 
 
-@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", MANY)
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", MANY + FEW)
 def test_gives_up_reports_and_goes_on(M, n_in, hidden, layers, n_out):
     x = torch.randn((M, n_in), generator=torch.Generator().manual_seed(1)).cuda()
     good, bad = _net(n_in, hidden, layers, n_out), _net(n_in, hidden, layers, n_out)
@@ -44,7 +48,7 @@ def test_gives_up_reports_and_goes_on(M, n_in, hidden, layers, n_out):
     assert torch.equal(bad.forward(x, y), want)
 
 
-@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", MANY)
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", MANY + FEW)
 def test_no_row_keeps_what_it_held(M, n_in, hidden, layers, n_out):
     x = torch.randn((M, n_in), generator=torch.Generator().manual_seed(1)).cuda()
     net = _net(n_in, hidden, layers, n_out)
