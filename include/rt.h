@@ -364,7 +364,9 @@ rt_status rt_pah_absorbed(rt_grid *g, uint32_t *out, int mem, void *stream);
  * number of such cells. The PAH-active cells of the range are listed first; the
  * surrogate runs over them in batches of up to 2^20 and the cells sent to the exact
  * solution are solved in one launch at the end. Synchronises the stream to size that
- * work (after listing the active cells and after the checks) and for a host output. */
+ * work (after listing the active cells and after the checks) and for a host output.
+ * RT_ERR_TIMEOUT (the rows are not to be used) when a wait of the network's has run out
+ * since it was created, as rt_mlp_get_params reports it. */
 typedef struct rt_mlp rt_mlp;
 rt_status rt_pah_emission(rt_grid *g, int64_t first_cell, int64_t n_cells, int pah, int mode,
                           const rt_mlp *surrogate, float tol, float *j_out, int mem,

@@ -101,7 +101,7 @@ struct rt_grid {
   float* d_spower = nullptr;   // [n_pah][batch] absorbed power feature
   int* d_list = nullptr;       // [cells] PAH-active cells of the call
   int* d_list2 = nullptr;      // [cells] cells sent to the exact solution
-  unsigned* d_ucount = nullptr;  // [2]
+  unsigned* d_ucount = nullptr;  // [3] active cells, cells to solve exactly, network error
   // host state
   std::vector<double> nu, kabs, ksca, ghg;   // [S][B]
   std::vector<char> dust_set;
@@ -1536,7 +1536,7 @@ static rt_status surrogate_scratch(rt_grid* g, long long cells, long long batch,
     if ((st = dalloc(&g->d_spabs, (size_t)P * batch)) != RT_OK) return st;
     g->sur_cap = batch;
   }
-  if (!g->d_ucount && (st = dalloc(&g->d_ucount, 2)) != RT_OK) return st;
+  if (!g->d_ucount && (st = dalloc(&g->d_ucount, 3)) != RT_OK) return st;
   return RT_OK;
 }
 
@@ -1591,7 +1591,7 @@ static rt_status pah_emission_impl(rt_grid* g, int64_t first_cell, int64_t n_cel
     RT_CUDA(cudaMemsetAsync(dst, 0, sizeof(float) * (size_t)n_cells * B, s));
   }
   // the cells where a PAH absorbed anything, in one list for the whole range
-  RT_CUDA(cudaMemsetAsync(g->d_ucount, 0, 2 * sizeof(unsigned), s));
+  RT_CUDA(cudaMemsetAsync(g->d_ucount, 0, 3 * sizeof(unsigned), s));
   RT_CUDA(launch_compact(g->d_pah_flag, pah, first_cell, n_cells, g->d_list, g->d_ucount, s));
   unsigned na = 0;
   RT_CUDA(cudaMemcpyAsync(&na, g->d_ucount, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
@@ -1629,11 +1629,13 @@ static rt_status pah_emission_impl(rt_grid* g, int64_t first_cell, int64_t n_cel
                                       t, x_lo, x_hi, mode == RT_PAH_AUTO,
                                       compact ? dst + (size_t)b0 * B : dst,
                                       compact ? nullptr : lst, (int)b0, g->d_list2,
-                                      g->d_ucount + 1, s));
+                                      g->d_ucount + 1, mlp_error_word(m), s));
     }
-    unsigned nf = 0;
-    RT_CUDA(cudaMemcpyAsync(&nf, g->d_ucount + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    unsigned got[2] = {0, 0};
+    RT_CUDA(cudaMemcpyAsync(got, g->d_ucount + 1, sizeof(got), cudaMemcpyDeviceToHost, s));
     RT_CUDA(cudaStreamSynchronize(s));
+    if (got[1]) return RT_ERR_TIMEOUT;
+    const unsigned nf = got[0];
     n_fallback = nf;
     if (mode == RT_PAH_AUTO && nf > 0)
       RT_CUDA(launch_pah_exact(g->g, g->ptab, g->d_pahabs, g->eps, g->d0, first_cell, nf, dst,

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+struct rt_mlp;  // the network (rt_mlp.cu)
+
 namespace rt {
 
 constexpr int kMaxSpecies = 8;
@@ -281,12 +283,15 @@ cudaError_t launch_surrogate_finish(const float* Y, const float* power, const fl
                                     long long n, int n_pah, int B, float tol, float x_lo,
                                     float x_hi, bool leave, float* j_out, const int* list,
                                     int off, int* fallback, unsigned* n_fallback,
-                                    cudaStream_t s);
+                                    const unsigned* net_err, cudaStream_t s);
 cudaError_t launch_pah_clear(const unsigned* pah_flag, long long N, int K, int n_pah,
                              unsigned* pahabs, unsigned* pah_flag_out, cudaStream_t s);
 cudaError_t launch_compact(const unsigned* pah_flag, int pah, long long first, long long n,
                            int* out, unsigned* count, cudaStream_t s);
 cudaError_t launch_pah_cell_cdf(const float* J, long long n, int B, float* out, cudaStream_t s);
+
+// The network's device word that a wait that ran out sets.
+const unsigned* mlp_error_word(const rt_mlp* m);
 
 // One P(T) problem: a PAH in a monochromatic field.
 struct PtCase {

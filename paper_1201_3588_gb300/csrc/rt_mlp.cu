@@ -1546,6 +1546,8 @@ rt_status forward_rows(rt_mlp* m, const float* x, long long M, float* y, const f
 
 }  // namespace
 
+const unsigned* rt::mlp_error_word(const rt_mlp* m) { return m->d_err; }
+
 extern "C" {
 
 rt_status rt_mlp_create(int n_in, int n_hidden, int n_layers, int n_out, uint64_t seed,

@@ -762,7 +762,8 @@ __device__ __forceinline__ float decode_q(float y) {
 // (or c) of j_out. A PAH whose energy residual |sum_b q_b - 1| (before scaling) exceeds tol or
 // whose power feature lies outside [x_lo, x_hi] flags the cell: it is appended to
 // fallback[*n_fallback ..] (list[c], or off + c without a list), and with `leave` its row is
-// left alone for the exact solution. One warp per cell; Y is read once,
+// left alone for the exact solution. n_fallback[1] becomes nonzero where the network's error
+// word is (a wait of its pass ran out: Y is not to be used). One warp per cell; Y is read once,
 // a lane's bins of every PAH in flight together. (Separate passes for the checks and for
 // each PAH's sum, decoding twice and adding into j_out, took 170 us for 2.7e4 cells, two
 // PAHs and 200 bins; this 32.)
@@ -771,10 +772,12 @@ constexpr int kFinishBins = 8;  // bins of a lane held in registers at a time
 __global__ void k_surrogate_finish(const float* Y, const float* power, const float* p_abs,
                                    long long n, int n_pah, int B, float tol, float x_lo,
                                    float x_hi, bool leave, float* j_out, const int* list,
-                                   int off, int* fallback, unsigned* n_fallback) {
+                                   int off, int* fallback, unsigned* n_fallback,
+                                   const unsigned* net_err) {
   const long long c = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= n) return;
+  if (c == 0 && lane == 0 && *net_err) n_fallback[1] = 1u;
   float scale[kMaxPah];
   bool flagged = false;
 #pragma unroll
@@ -961,11 +964,11 @@ cudaError_t launch_surrogate_finish(const float* Y, const float* power, const fl
                                     long long n, int n_pah, int B, float tol, float x_lo,
                                     float x_hi, bool leave, float* j_out, const int* list,
                                     int off, int* fallback, unsigned* n_fallback,
-                                    cudaStream_t s) {
+                                    const unsigned* net_err, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   k_surrogate_finish<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(Y, power, p_abs, n, n_pah, B, tol,
                                                              x_lo, x_hi, leave, j_out, list, off,
-                                                             fallback, n_fallback);
+                                                             fallback, n_fallback, net_err);
   return cudaGetLastError();
 }
 

@@ -4,7 +4,7 @@ ends by itself with its copies and products landed and its tensor memory given b
 read of the handle reports the timeout, and the GPU goes on computing as before."""
 import pytest
 
-from paper_1201_3588_gb300 import rt
+from paper_1201_3588_gb300 import rt, workloads as w
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -60,6 +60,34 @@ def test_no_row_keeps_what_it_held(M, n_in, hidden, layers, n_out):
     torch.cuda.synchronize()
     assert torch.isnan(y).all()
     assert (buf[:8] == 0.5).all() and (buf[8 + M * n_out:] == 0.5).all()
+
+
+@pytest.mark.parametrize("mode", [rt.PAH_SURROGATE, rt.PAH_AUTO])
+@pytest.mark.parametrize("n_base", [4, 36])        # few rows, and enough for the other kernel
+def test_emission_reports_it(mode, n_base):
+    nu = w.frequency_edges(64)
+    sp = w.two_species(nu) + [w.pah_species(nu, n) for n in (30, 200)]
+    m = w.sphere_model(n_base=n_base, n_bins=64, tau_v=3.0, species=sp,
+                       fractions=[0.7, 0.25, 0.025, 0.025])
+    net = rt.MLP(64 + 2, 64, 2, 64, seed=3)
+    n = 1_000_000 if n_base > 4 else 100_000
+    with rt.Grid(m) as g:
+        g.emit_star(n)
+        g.transport(n, seed=3)
+        rows = 2 * len(g.pah_emission_active(mode=rt.PAH_EXACT)[0])
+        assert (rows > 152 * 128) == (n_base > 4)
+        want, _ = g.pah_emission(mode=mode, surrogate=net, tol=1e9)
+        again, _ = g.pah_emission(mode=mode, surrogate=net, tol=1e9)
+        assert (want == again).all()
+        net.set_wait_limit(0.0)
+        for call in (g.pah_emission, g.pah_emission_active):
+            with pytest.raises(rt.RTError) as e:
+                call(mode=mode, surrogate=net, tol=1e9)
+            assert e.value.code == RT_ERR_TIMEOUT
+        # another handle, and the exact solution, are not affected
+        fresh, _ = g.pah_emission(mode=mode, surrogate=rt.MLP(64 + 2, 64, 2, 64, seed=3), tol=1e9)
+        assert (fresh == want).all()
+        g.pah_emission()
 
 
 def test_limit_is_checked():
