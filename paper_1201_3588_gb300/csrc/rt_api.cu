@@ -1741,8 +1741,10 @@ struct rt_batch {
   int dev = 0;
   std::vector<rt_grid*> grids;
   std::vector<unsigned long long> n_pk;
+  char* slab = nullptr;  // holds the next two and every model's temperatures
   ModelDesc* d_models = nullptr;
   unsigned long long* d_next = nullptr;  // [models] packages handed out
+  std::vector<float*> d_T;               // of each model, [S][n_leaves]
   int chunk = 0;                         // packages a warp takes at a time
   int blocks_per_sm = 0;
   int threads = 256;  // threads per block of the batched launch
@@ -1762,8 +1764,7 @@ rt_status rt_batch_destroy(rt_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   if (b->capture_stream) cudaStreamDestroy(b->capture_stream);
-  dfree(b->d_models);
-  dfree(b->d_next);
+  dfree(b->slab);
   delete b;
   return RT_OK;
 }
@@ -1794,14 +1795,11 @@ rt_status rt_batch_create(rt_grid* const* grids, int n, const uint64_t* n_packag
     if (n_packages[m] > g->n_total) { st = RT_ERR_RANGE; break; }
     DevRun r;
     if ((st = fill_run(g, n_packages[m], seed + (uint64_t)m, 0, o, &r)) != RT_OK) break;
-    const size_t nT = (size_t)g->desc.n_species * g->desc.n_leaves;
-    if (!g->d_Tscratch && (st = dalloc(&g->d_Tscratch, nT)) != RT_OK) break;
     desc[(size_t)m].g = g->g;
     desc[(size_t)m].t = g->tab;
     desc[(size_t)m].t.u_frozen = g->d_ufrozen;
     desc[(size_t)m].t.pah_cell_cdf = g->d_pah_cell_cdf;
     desc[(size_t)m].r = r;
-    desc[(size_t)m].T_out = g->d_Tscratch;
     b->max_cells = std::max(b->max_cells, (long long)g->desc.n_leaves);
     b->grids.push_back(g);
     b->n_pk.push_back(n_packages[m]);
@@ -1820,11 +1818,19 @@ rt_status rt_batch_create(rt_grid* const* grids, int n, const uint64_t* n_packag
   b->tally = desc[0].r.pathabs != nullptr;  // one choice of estimators for all models
   for (int m = 0; m < n; ++m)
     if (grids[m]->desc.n_species != b->s_fixed) b->s_fixed = 0;
-  if ((st = dalloc(&b->d_models, (size_t)n)) != RT_OK ||
-      (st = dalloc(&b->d_next, (size_t)n)) != RT_OK) {
+  // the temperatures are the batch's own: a grid's scratch serves every host read of that grid
+  Slab slab;
+  b->d_T.assign((size_t)n, nullptr);
+  slab.add(&b->d_models, (size_t)n);
+  slab.add(&b->d_next, (size_t)n);
+  for (int m = 0; m < n; ++m)
+    slab.add(&b->d_T[(size_t)m],
+             (size_t)grids[m]->desc.n_species * (size_t)grids[m]->desc.n_leaves);
+  if ((st = slab.allocate(&b->slab)) != RT_OK) {
     rt_batch_destroy(b);
     return st;
   }
+  for (int m = 0; m < n; ++m) desc[(size_t)m].T_out = b->d_T[(size_t)m];
   cudaError_t e = cudaMemcpy(b->d_models, desc.data(), sizeof(ModelDesc) * n,
                              cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
@@ -1883,7 +1889,7 @@ rt_status rt_batch_temperatures(rt_batch* b, int model, float* T_out, int mem, v
   cudaStream_t s = as_stream(stream);
   RT_CUDA(cudaSetDevice(b->dev));
   const size_t n = (size_t)g->desc.n_species * g->desc.n_leaves;
-  RT_CUDA(cudaMemcpyAsync(T_out, g->d_Tscratch, sizeof(float) * n,
+  RT_CUDA(cudaMemcpyAsync(T_out, b->d_T[(size_t)model], sizeof(float) * n,
                           mem == RT_MEM_DEVICE ? cudaMemcpyDeviceToDevice
                                                : cudaMemcpyDeviceToHost,
                           s));
