@@ -1412,7 +1412,7 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
       book();
       const unsigned dead = __ballot_sync(kFull, !walking && !pending);
       if (dead && !dry) fill(dead);
-      if (!__any_sync(kFull, walking || pending)) return true;
+      if (dry && !__any_sync(kFull, walking || pending)) return true;
     }
     if (__any_sync(kFull, tl.crossings >= kTallyFlushAt || tl.levels >= kTallyFlushAt ||
                               wt[lane & (kTallyWords - 1)] >= kTallyFlushAt))
@@ -1423,6 +1423,9 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
     if (stop) {
       if (lane == 0) atomicOr(r.status, kStatusTimeout);
       return false;
+    }
+    if constexpr (!kPark) {  // all packages just drawn left the domain at once: draw again
+      if (!__any_sync(kFull, walking || pending)) continue;
     }
     for (int step = 0; step < K; ++step) {
       if (walking) {
