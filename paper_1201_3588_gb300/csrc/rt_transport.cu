@@ -1421,6 +1421,7 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
     if (lane == 0) stop = global_ns() - t0 > r.budget_ns;
     stop = __shfl_sync(kFull, stop, 0);
     if (stop) {
+      book();  // what has escaped so far is counted as escaped
       if (lane == 0) atomicOr(r.status, kStatusTimeout);
       return false;
     }
