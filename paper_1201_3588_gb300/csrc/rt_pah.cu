@@ -475,21 +475,25 @@ __device__ float solve_levels_f32(const float* cf, int M, const Halves& P, const
       q = C > 0.0f ? fmaf(fmaf(-q, C, sum), rC, q) : 0.0f;
       if (fb == 0 && i == 0) q = 1.0f;
       float pi = __shfl_sync(0xffffffffu, q, i, 8);
-      if (!(pi <= kTopPopulation)) {  // rescale what there is so that this level is 1e20
+      if (!(pi <= kTopPopulation)) {
         const float sc = __shfl_sync(group, (kTopPopulation * C) / sum, i, 8);
-        for (int jb = l; jb < fb; jb += 8) {
-          float p[8];
-          P.read(jb, p);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) p[k] *= sc;
-          P.write(jb, p);
-        }
-        __syncwarp(group);
-        own *= sc;
-        flux *= sc;
-        lost *= sc;
-        tot *= sc;
         pi = kTopPopulation;
+        if (sc >= 1.0f) {  // the reciprocal of a rate below 3e-39 (the coldest levels) overflowed
+          pi = kTopPopulation / sc;
+        } else {  // rescale what there is so that this level is 1e20
+          for (int jb = l; jb < fb; jb += 8) {
+            float p[8];
+            P.read(jb, p);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) p[k] *= sc;
+            P.write(jb, p);
+          }
+          __syncwarp(group);
+          own *= sc;
+          flux *= sc;
+          lost *= sc;
+          tot *= sc;
+        }
       }
       if (l == i) own = pi;
       if (i < 7) {
