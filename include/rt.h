@@ -362,7 +362,8 @@ rt_status rt_pah_absorbed(rt_grid *g, uint32_t *out, int mem, void *stream);
  * before rescaling exceeds `tol`, or its absorbed power per molecule lies outside
  * the range set with rt_mlp_set_range. *n_fallback_out (may be NULL) receives the
  * number of such cells. The PAH-active cells of the range are listed first; the
- * surrogate runs over them in batches of up to 2^20 and the cells sent to the exact
+ * surrogate runs over them in batches of up to 2^20 (fewer where device memory is short)
+ * and the cells sent to the exact
  * solution are solved in one launch at the end. Synchronises the stream to size that
  * work (after listing the active cells and after the checks) and for a host output.
  * RT_ERR_TIMEOUT (the rows are not to be used) when a wait of the network's has run out

@@ -1511,8 +1511,8 @@ rt_status rt_pah_temperature_distribution(const rt_pah_pt_case* cases, int n_cas
   return st != RT_OK ? st : cuda_status(e);
 }
 
-// Work arrays of rt_pah_emission: cell lists for `cells` cells; the network's
-// inputs, outputs and flags for `batch` rows only when a surrogate is used.
+// Work arrays of rt_pah_emission: cell lists for `cells` cells; the network's inputs and
+// outputs and the absorbed powers of every PAH in `batch` cells only when a surrogate is used.
 static rt_status surrogate_scratch(rt_grid* g, long long cells, long long batch, bool with_net) {
   const int K = g->tab.n_coarse, B = g->desc.n_bins, P = g->n_pah;
   rt_status st;
@@ -1617,8 +1617,11 @@ static rt_status pah_emission_impl(rt_grid* g, int64_t first_cell, int64_t n_cel
     // cells whose prediction fails its checks are appended to one fallback list, solved
     // exactly in one launch
     const int pah0 = pah >= 0 ? pah : 0, np = pah >= 0 ? 1 : g->n_pah;
-    const long long batch = na < (1u << 20) ? (long long)na : (1ll << 20);
-    if ((st = surrogate_scratch(g, n_cells, batch, true)) != RT_OK) return st;
+    long long batch = na < (1u << 20) ? (long long)na : (1ll << 20);
+    // smaller batches where the device has no room for that many rows of all PAHs
+    while ((st = surrogate_scratch(g, n_cells, batch, true)) == RT_ERR_OOM && batch > 512)
+      batch = (batch + 1) / 2;
+    if (st != RT_OK) return st;
     for (long long b0 = 0; b0 < (long long)na; b0 += batch) {
       const long long nb = (long long)na - b0 < batch ? (long long)na - b0 : batch;
       const int* lst = g->d_list + b0;
