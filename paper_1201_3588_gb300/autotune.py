@@ -2,9 +2,9 @@
 transport of a package prefix under each candidate (resident blocks per SM, threads
 per block, interaction batch, refill period, and for a single grid the walk) with CUDA
 events and keep the fastest.
-Results are cached in a JSON file keyed by the workload class (cells to the nearest
-power of two, species, levels, bins, optical-depth decade; for a batch, its models'
-classes)."""
+Results are cached in a JSON file keyed by the pool's schedule and the workload class
+(cells to the nearest power of two, species, levels, bins, optical-depth decade; for a
+batch, its models' classes)."""
 from __future__ import annotations
 
 import itertools
@@ -14,6 +14,12 @@ import os
 from typing import Dict, Optional
 
 from . import rt
+
+# What the options mean to the pool: raised whenever its schedule changes, so that options
+# found under another are measured again. 2: packages parked in shared memory
+# (interaction_batch is twice the idle lanes that start a search); 1, which keys did not
+# name: packages bound to their lanes.
+SCHEDULE = 2
 
 # the batched launch runs the linked walk; a single grid also tries the path walk
 BATCH_CANDIDATES = dict(blocks_per_sm=(0, 5), threads=(128, 256), interaction_batch=(4, 8, 12),
@@ -37,7 +43,7 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_1201_3588
 
 
 def workload_key(grid: "rt.Grid", tau_v: float) -> str:
-    return (f"cells2^{int(round(math.log2(max(grid.N, 1))))}-S{grid.S}-"
+    return (f"pool{SCHEDULE}-cells2^{int(round(math.log2(max(grid.N, 1))))}-S{grid.S}-"
             f"L{grid.model.tree.max_level}-bins{grid.B}-"
             f"tau1e{int(math.floor(math.log10(max(tau_v, 1e-30))))}")
 
@@ -96,7 +102,7 @@ def batch_key(grids, tau_vs, n_packages) -> str:
         for ch in c.encode():
             h = (h * 131 + ch) % (1 << 61)
     pk = int(round(math.log2(max(sum(n_packages), 1))))
-    return f"batch{len(grids)}-pk2^{pk}-{h:016x}"
+    return f"pool{SCHEDULE}-batch{len(grids)}-pk2^{pk}-{h:016x}"
 
 
 def tune_batch(grids, tau_vs, n_packages, fraction: float = 0.05, seed: int = 0,
