@@ -1941,6 +1941,7 @@ __global__ void k_philox(const unsigned long long* ids, long long n, unsigned ev
 }  // namespace
 
 constexpr size_t kSmemBudget = 200 * 1024;
+constexpr size_t kSmemSm = 228 * 1024, kSmemBlock = 1024;  // of an SM; kept by each block
 
 template <int kS, bool kTally>
 static size_t table_smem(const DevGrid& g) {
@@ -1972,6 +1973,24 @@ static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, con
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, sm);
   if (e != cudaSuccess) return e;
+  // The spectrum in shared memory is worth a few per cent, a block per SM far more: it goes to
+  // global memory where, beside the places, it would cost one that the launch would have (asked
+  // for only where shared memory can be what limits the blocks). 5.3e5 cells of two species,
+  // 3e6 packages, in shared and in global memory, ms: 200 bins, one direction (four blocks
+  // both) 1.28 and 1.30; eight directions of 257 bins (three and four) 1.57 and 1.29, path
+  // walk 2.69 and 2.27; of 333 bins (two and four) 2.28 and 1.29, path walk 3.53 and 2.28; of
+  // 1024 bins (one and four) 3.61 and 1.58.
+  if (rr.sed_in_smem &&
+      (sm + kPoolStatic<kPath, kTally> + kSmemBlock) * kMinBlocks * 256 > kSmemSm * threads) {
+    int most = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, kernel, threads, tables);
+    if (e != cudaSuccess) return e;
+    if (occ < (blocks_per_sm > 0 && blocks_per_sm < most ? blocks_per_sm : most)) {
+      rr.sed_in_smem = 0;
+      sm = tables;
+      occ = most;
+    }
+  }
   if (occ < 1) occ = 1;
   int bps = blocks_per_sm > 0 ? (blocks_per_sm < occ ? blocks_per_sm : occ) : occ;
   kernel<<<sms * bps, threads, sm, s>>>(g, t, rr, pe);
