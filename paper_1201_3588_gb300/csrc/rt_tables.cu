@@ -311,14 +311,15 @@ __device__ __forceinline__ float cell_temperature(const DevTables& t, int n_T, i
   return (float)fma(T0, (double)expm1f(y), T0);
 }
 
-// Temperatures of one cell. A thread takes all its species: their densities (and path-length
-// tallies) lie side by side, a thread per species and cell read them in as many passes. With
-// the arithmetic above: 8.0e6 cells of four species 0.60 -> 0.31 ms, 2.4e6 of two 0.20 -> 0.11.
+// Temperatures of one cell. A thread takes all its species (from s0 on in steps of s_step):
+// their densities (and path-length tallies) lie side by side, a thread per species and cell
+// read them in as many passes. With the arithmetic above: 8.0e6 cells of four species 0.60 ->
+// 0.31 ms, 2.4e6 of two 0.20 -> 0.11.
 template <int kS>
 __device__ __forceinline__ void cell_temperatures(const DevGrid& g, const DevTables& t,
                                                   const unsigned long long* count, float* T_out,
                                                   const float* pathabs, long long c,
-                                                  unsigned& clamped) {
+                                                  unsigned& clamped, int s0 = 0, int s_step = 1) {
   const int S = kS > 0 ? kS : g.S;
   const int lev = g.level[c];
   // absorbed energy in units of eps: the count, or the path-length tally
@@ -337,7 +338,7 @@ __device__ __forceinline__ void cell_temperatures(const DevGrid& g, const DevTab
     for (int s = 0; s < kS; ++s)
       T_out[s * g.n_leaves + c] = cell_temperature(t, g.n_T, s, n[s], rho[s], lev, clamped);
   } else {
-    for (int s = 0; s < S; ++s)
+    for (int s = s0; s < S; s += s_step)
       T_out[s * g.n_leaves + c] =
           cell_temperature(t, g.n_T, s, absorbed(s), g.rho[c * S + s], lev, clamped);
   }
@@ -356,7 +357,8 @@ __global__ void __launch_bounds__(256) k_temperatures(DevGrid g, DevTables t,
                                                       const float* pathabs) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   unsigned clamped = 0;
-  if (c < g.n_leaves) cell_temperatures<kS>(g, t, count, T_out, pathabs, c, clamped);
+  if (c < g.n_leaves)
+    cell_temperatures<kS>(g, t, count, T_out, pathabs, c, clamped, blockIdx.y, gridDim.y);
   add_clamped(clamped, counters);
 }
 
@@ -432,9 +434,15 @@ cudaError_t launch_temperatures(const DevGrid& g, const DevTables& t,
                                 const unsigned long long* count, float* T_out,
                                 unsigned long long* counters, cudaStream_t s,
                                 const float* pathabs) {
-  const auto kernel = g.S == 2 ? k_temperatures<2> : (g.S == 4 ? k_temperatures<4>
-                                                              : k_temperatures<0>);
-  kernel<<<nblk(g.n_leaves, 256), 256, 0, s>>>(g, t, count, T_out, counters, pathabs);
+  // A thread per cell where a cell's species are one vector and the cells fill the chip, else a
+  // thread per species and cell. Cell and species, us: two species, 512 cells 8.2 and 6.2,
+  // 2.6e5 26.7 and 26.7; four, 512 cells 11.4 and 6.2, 2.6e5 31.2 and 30.0, 8.8e5 78 and 84;
+  // eight (no vector), 512 cells 18.5 and 6.2, 8.8e5 109 and 108.
+  const bool cells = (g.S == 2 || g.S == 4) && g.n_leaves > 1 << 18;
+  const auto kernel = !cells ? k_temperatures<0> : (g.S == 2 ? k_temperatures<2>
+                                                             : k_temperatures<4>);
+  kernel<<<dim3(nblk(g.n_leaves, 256), cells ? 1 : (unsigned)g.S), 256, 0, s>>>(
+      g, t, count, T_out, counters, pathabs);
   return cudaGetLastError();
 }
 
