@@ -36,6 +36,10 @@ constexpr int32_t kLinkLeafMask = 0x0FFFFFFF;
 constexpr int32_t kLinkSame = 1 << 28;
 constexpr long long kMaxLinkedLeaves = 1ll << 28;
 
+// Path-length tallies lie species by species within a cell, in rows of this many floats: whole
+// vectors for the reductions (see tally_segment).
+__host__ __device__ constexpr int tally_row(int S) { return S <= 2 ? S : (S + 3) & ~3; }
+
 // Geometry and densities (device pointers), passed by value.
 struct DevGrid {
   const int32_t* base;     // [n^3]
@@ -95,7 +99,7 @@ struct DevRun {
   unsigned int* status;
   unsigned* pahabs;               // [n_pah][n_leaves][n_coarse] PAH absorptions
   unsigned* pah_flag;             // [n_leaves] bit p set: PAH p absorbed in the cell
-  float* pathabs;                 // [n_leaves][S] path-length tallies, or null
+  float* pathabs;                 // [n_leaves][tally_row(S)] path-length tallies, or null
   float src[3];                   // source position, base-cube units
   float beam[3];
   double src64[3];
@@ -308,7 +312,7 @@ size_t pt_scratch_doubles(int n_cases, int M, int B);
 
 cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T_frozen,
                             float* u_frozen, float t_min, float t_max, cudaStream_t s);
-// out [S][n_leaves] from tallies [n_leaves][S]
+// out [S][n_leaves] from tallies [n_leaves][tally_row(S)]
 cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out, cudaStream_t s);
 // Every model of a batch in one launch (max_cells: of the largest): temperatures from the
 // counts into T_out; counts, spectra, counters and status to zero.

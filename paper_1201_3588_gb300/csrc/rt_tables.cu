@@ -324,7 +324,7 @@ __device__ __forceinline__ void cell_temperatures(const DevGrid& g, const DevTab
   const int lev = g.level[c];
   // absorbed energy in units of eps: the count, or the path-length tally
   const auto absorbed = [&](int s) {
-    return pathabs ? (double)pathabs[c * S + s] : (double)count[s * g.n_leaves + c];
+    return pathabs ? (double)pathabs[c * tally_row(S) + s] : (double)count[s * g.n_leaves + c];
   };
   if constexpr (kS > 0) {
     double n[kS];
@@ -401,7 +401,8 @@ __global__ void __launch_bounds__(256) k_batch_reset(const ModelDesc* models) {
 __global__ void k_tally_out(const float* pathabs, long long N, int S, float* out) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
-  for (int s = 0; s < S; ++s) out[(size_t)s * N + c] = pathabs[(size_t)c * S + s];
+  const float* row = pathabs + (size_t)c * tally_row(S);
+  for (int s = 0; s < S; ++s) out[(size_t)s * N + c] = row[s];
 }
 
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }

@@ -297,7 +297,7 @@ __device__ __forceinline__ int advance(Pkg<R>& k, const DevGrid& g, const Kappa*
     const R seg = (kx > (R)0 && dtau > k.tau) ? k.tau / kx : tex;
     for (int s = 0; s < g.S; ++s) {
       const float v = (float)((R)__ldg(&rho[s]) * (R)kb[s].kabs * seg);
-      if (v > 0.f) atomicAdd(&pathabs[(size_t)leaf * g.S + s], v);
+      if (v > 0.f) atomicAdd(&pathabs[(size_t)leaf * tally_row(g.S) + s], v);
     }
   }
   if (kx > (R)0 && dtau > k.tau) {
@@ -509,38 +509,59 @@ __device__ __forceinline__ float leaf_ext(const DevGrid& g, int leaf, float4 r, 
   }
 }
 
-// Path-length tallies of a segment of length seg in a leaf, [n_leaves][S]: rho_s
+// Vector additions to memory, left out where nothing is to be added.
+__device__ __forceinline__ void red_add2(float* p, float v0, float v1) {
+  if (v0 > 0.f || v1 > 0.f)
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)),
+                 "f"(v0), "f"(v1)
+                 : "memory");
+}
+
+__device__ __forceinline__ void red_add4(float* p, const float* v) {
+  if (v[0] > 0.f || v[1] > 0.f || v[2] > 0.f || v[3] > 0.f)
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                     __cvta_generic_to_global(p)),
+                 "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+}
+
+// Path-length tallies of a segment of length seg in a leaf, [n_leaves][tally_row(S)]: rho_s
 // kappa_abs,s seg is added for every species. With the species of a cell side by side two
 // or four of them are one vector reduction to one sector. 2e6 packages through 1.06e6
 // cells of two species: 3.9 ms with an atomic per species into arrays apart (and the
-// generic species loop), 2.7 ms.
+// generic species loop), 2.7 ms. Other species counts need rows of whole vectors: 1e6
+// packages through 6.4e4 cells of three, five and eight species took 2.27, 2.83 and 5.06 ms
+// with an array per species, 2.78, 3.96 and 5.32 with single atomics into rows of S, and 1.16,
+// 1.78 and 3.57 so.
 template <int kS>
 __device__ __forceinline__ void tally_segment(const DevGrid& g, float* pathabs, int leaf,
                                               float4 r, int bin, float seg, const Kappa* kap,
                                               const float* kabs) {
   if constexpr (kS == 2) {
     const float4 a = bin_vec<2>(kabs, bin);
-    const float v0 = r.x * a.x * seg, v1 = r.y * a.y * seg;
-    if (v0 > 0.f || v1 > 0.f)
-      asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(
-                       __cvta_generic_to_global(pathabs + 2 * (size_t)leaf)),
-                   "f"(v0), "f"(v1)
-                   : "memory");
+    red_add2(pathabs + 2 * (size_t)leaf, r.x * a.x * seg, r.y * a.y * seg);
   } else if constexpr (kS == 4) {
     const float4 a = bin_vec<4>(kabs, bin);
-    const float v0 = r.x * a.x * seg, v1 = r.y * a.y * seg, v2 = r.z * a.z * seg,
-                v3 = r.w * a.w * seg;
-    if (v0 > 0.f || v1 > 0.f || v2 > 0.f || v3 > 0.f)
-      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
-                       __cvta_generic_to_global(pathabs + 4 * (size_t)leaf)),
-                   "f"(v0), "f"(v1), "f"(v2), "f"(v3)
-                   : "memory");
+    const float v[4] = {r.x * a.x * seg, r.y * a.y * seg, r.z * a.z * seg, r.w * a.w * seg};
+    red_add4(pathabs + 4 * (size_t)leaf, v);
   } else {
-    const float* rho = g.rho + (size_t)leaf * g.S;
-    const Kappa* kb = kap + bin * g.S;
-    for (int s = 0; s < g.S; ++s) {
-      const float v = __ldg(&rho[s]) * kb[s].kabs * seg;
-      if (v > 0.f) atomicAdd(&pathabs[(size_t)leaf * g.S + s], v);
+    const int S = g.S;
+    const float* rho = g.rho + (size_t)leaf * S;
+    const Kappa* kb = kap + bin * S;
+    float* row = pathabs + (size_t)leaf * tally_row(S);
+    if (S == 1) {
+      const float v = __ldg(rho) * kb[0].kabs * seg;
+      if (v > 0.f) atomicAdd(row, v);
+      return;
+    }
+    for (int s = 0; s < S; s += 4) {
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = s + j < S ? __ldg(&rho[s + j]) * kb[s + j].kabs * seg : 0.f;
+      if (S == 2)
+        red_add2(row, v[0], v[1]);
+      else
+        red_add4(row + s, v);
     }
   }
 }
