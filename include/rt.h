@@ -119,8 +119,8 @@ typedef struct rt_run_opts {
  * of the block below it) -- one read per crossing, one more per level descended (no
  * link records; grids of at most 4 levels whose base cells plus 8 x blocks fit an
  * int32). Both give the same histories. AUTO takes the path walk when the link records
- * exceed 4 GB, and for four species unless the grid is small (link records and densities
- * within 0.5 GB) with most of its cells in refined blocks: its randomly read array,
+ * exceed 4 GB, and for four species unless more than half of the cells, a fraction f, sit in
+ * refined blocks and link records and densities are within 0.7 f - 0.2 GB: its randomly read array,
  * (n^3 + 8 n_blocks) x S floats, is smaller, which costs less address translation on
  * large grids. */
 enum { RT_WALK_AUTO = 0, RT_WALK_LINKED = 1, RT_WALK_PATH = 2 };

@@ -226,8 +226,11 @@ static bool path_walk_fits(const rt_grid_desc* d) {
 // neighbour is not finer; the path walk descends through the tree at every change of a
 // refined block, but reads one array of (slots x species) floats where the linked walk
 // reads 32-byte records and, for more than two species, a row of densities.
-//  - Two species (densities in the record), and species counts without a compiled path
-//    walk: linked until the records exceed 4 GB.
+//  - Two species (densities in the record): linked until the records exceed 4 GB. 1e7
+//    packages, linked and path, ms: f = 1 (see below): 0.08 GB 6.0 and 11.8, 0.29 GB 9.5 and
+//    16.1, 0.96 GB 19.8 and 23.4, 2.2 GB 35.7 and 33.0; f = 0: 0.26 GB 15.4 and 9.5 -- large
+//    unrefined grids would gain from the path walk, which a caller can ask for. Species counts
+//    without a compiled path walk: the same line, not measured.
 //  - Four species: linked where more than half of the cells, a fraction f, sit in refined
 //    blocks (where the path walk descends most) and the records and densities are within
 //    0.7 f - 0.2 GB. 1e7 packages, linked and path, ms: f = 1: 0.43 GB 15.2 and 17.6, 0.49 GB 18.4 and 18.4,

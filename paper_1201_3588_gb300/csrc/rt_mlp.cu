@@ -260,7 +260,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // the gradient passed down), small tiles (32 or more CTAs for 1024 rows) and all of a
 // tile's loads in flight at once instead of a pipeline. 28 launches with GEMMs that packed
 // column-major operands element by element took 307 us a step of 1024 rows (66 - 3x256 -
-// 200), these ten 90 us (16384 rows: 797 and 295; the 66 - 3x512 - 200 network forward over
+// 200), these nine and Adam 90 us (16384 rows: 797 and 295; the 66 - 3x512 - 200 network forward over
 // 262144 rows: 4.3 and 3.1 ms). What bounds a step now is the latency within each kernel,
 // 7 us from its first load to its last store.
 //
@@ -1336,8 +1336,6 @@ size_t tile_smem_bytes() {
   return sizeof(bf16) * (size_t)(kTcRows + kTcMaxWidth) * kTcMaxWidth +
          sizeof(float) * kMaxLayers * kTcMaxWidth + 32;
 }
-
-inline unsigned nb(long long n, int t);
 
 inline unsigned nb(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 

@@ -212,14 +212,14 @@ __device__ __forceinline__ double reciprocal(float x32, double x) {
   return fma(r, fma(-x, r, 1.0), r);
 }
 
-// S at temperature T by linear interpolation in T between table rows (the same
-// piecewise-linear model the transport samples from).
 // a < b for doubles that are not negative: their bits as integers (a compare is an FP64
 // operation too)
 __device__ __forceinline__ bool below(double a, double b) {
   return __double_as_longlong(a) < __double_as_longlong(b);
 }
 
+// S at temperature T by linear interpolation in T between table rows (the same
+// piecewise-linear model the transport samples from), a thread per species and cell.
 // A binary search of FP64 rows, then an FP64 division: 3.2e7 entries 1.46 ms, now 0.65; FP64
 // operations, some twelve an entry, still bound it.
 __global__ void k_frozen_u(DevGrid g, DevTables t, const float* T_frozen, float* u_frozen,

@@ -1642,13 +1642,13 @@ __host__ __device__ __forceinline__ int kap_records(const DevGrid& g) {
 }
 
 // ---------------------------------------------------------------- pool kernel
-// Persistent packet pool over one model: all warps draw package indices from one
-// global counter; the opacity table, the stellar CDF and (when it fits) the
-// escaped-spectrum histogram live in shared memory.
-// shared memory of a block beside what the launch asks for
+// Shared memory of a block beside what the launch asks for: places and counters of 8 warps.
 template <bool kPath, bool kTally>
 constexpr size_t kPoolStatic = 8 * ((kTally ? 16 : park_bytes<kPath>()) + 4 * kTallyWords);
 
+// Persistent packet pool over one model: all warps draw package indices from one
+// global counter; the opacity table, the stellar CDF and (where that costs no resident
+// block: launch_pool_variant) the escaped-spectrum histogram live in shared memory.
 template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false, bool kTally = false>
 __global__ void __launch_bounds__(256, kMinBlocks)
     k_transport_pool(DevGrid g, DevTables t, DevRun r, const __grid_constant__ DevPeel pe) {
