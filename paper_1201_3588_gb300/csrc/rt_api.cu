@@ -77,7 +77,7 @@ struct rt_grid {
   float* d_pah_cell_cdf = nullptr;  // [n_pah][N][B] per-cell re-emission spectra
   unsigned* d_pahabs = nullptr;
   unsigned* d_pah_flag = nullptr;  // [N] PAH-active bits per cell (bit p: PAH p)
-  float* d_pathabs = nullptr;  // path-length tallies [N][tally_row(S)]
+  float* d_pathabs = nullptr;  // path-length tallies, rows tally_place(leaf)
   // peel-off images
   int* d_plane_of_bin = nullptr;         // [B]
   double* d_image = nullptr;             // [n_planes][ny][nx]
@@ -508,7 +508,8 @@ rt_status reset_optional(rt_grid* g, cudaStream_t s) {
     RT_CUDA(launch_pah_clear(g->d_pah_flag, (long long)N, g->tab.n_coarse, g->n_pah,
                              g->d_pahabs, g->d_pah_flag, s));
   if (g->d_pathabs)
-    RT_CUDA(cudaMemsetAsync(g->d_pathabs, 0, sizeof(float) * tally_row((int)S) * N, s));
+    RT_CUDA(cudaMemsetAsync(g->d_pathabs, 0,
+                            sizeof(float) * tally_floats((int)S, (long long)N), s));
   if (g->images) {
     const size_t n = (size_t)g->peel.n_planes * g->peel.ny * g->peel.nx;
     RT_CUDA(cudaMemsetAsync(g->d_image, 0, sizeof(double) * n, s));
@@ -882,7 +883,7 @@ rt_status rt_reset(rt_grid* g, void* stream) {
 // for them.
 static rt_status ensure_pathabs(rt_grid* g, const rt_run_opts* o, cudaStream_t s) {
   if (!o || !(o->estimators & RT_EST_PATHLENGTH) || g->d_pathabs) return RT_OK;
-  const size_t n = (size_t)tally_row(g->desc.n_species) * g->desc.n_leaves;
+  const size_t n = tally_floats(g->desc.n_species, g->desc.n_leaves);
   rt_status st = dalloc(&g->d_pathabs, n);
   if (st != RT_OK) return st;
   RT_CUDA(cudaMemsetAsync(g->d_pathabs, 0, sizeof(float) * n, s));

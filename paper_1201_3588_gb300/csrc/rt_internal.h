@@ -40,6 +40,24 @@ constexpr long long kMaxLinkedLeaves = 1ll << 28;
 // vectors for the reductions (see tally_segment).
 __host__ __device__ constexpr int tally_row(int S) { return S <= 2 ? S : (S + 3) & ~3; }
 
+// The row of a leaf: within blocks of 4096 leaves the two 6-bit halves of the number trade
+// places (which undoes itself), so that cells close together lie 64 rows apart. Reductions to one
+// memory line are done one after another, and leaves are numbered along a space-filling curve:
+// in order, the cells that every package crosses next to the source share a few lines, and the
+// time of a launch went by which parts of L2 those lines fell into. 2e6 packages through 1.06e6
+// cells of two species, the array moved by 0 to 32 MB: 2.28 to 3.25 ms in order, 1.90 to 1.98 so
+// (blocks of 1024 1.97 to 2.10, of 16384 1.91 to 2.06); 4e6 through 1.9e7 cells 16.5 and 14.4;
+// 1e6 through 5.9e4 1.83 and 0.85.
+constexpr int kTallyBits = 6;
+constexpr long long kTallyBlock = 1ll << (2 * kTallyBits);
+__host__ __device__ constexpr size_t tally_place(long long leaf) {
+  constexpr long long m = (1ll << kTallyBits) - 1;
+  return (size_t)((leaf & ~(kTallyBlock - 1)) | (leaf & m) << kTallyBits | (leaf >> kTallyBits & m));
+}
+__host__ __device__ constexpr size_t tally_floats(int S, long long n_leaves) {
+  return (size_t)((n_leaves + kTallyBlock - 1) / kTallyBlock * kTallyBlock) * tally_row(S);
+}
+
 // Geometry and densities (device pointers), passed by value.
 struct DevGrid {
   const int32_t* base;     // [n^3]
@@ -99,7 +117,7 @@ struct DevRun {
   unsigned int* status;
   unsigned* pahabs;               // [n_pah][n_leaves][n_coarse] PAH absorptions
   unsigned* pah_flag;             // [n_leaves] bit p set: PAH p absorbed in the cell
-  float* pathabs;                 // [n_leaves][tally_row(S)] path-length tallies, or null
+  float* pathabs;                 // path-length tallies, rows tally_place(leaf), or null
   float src[3];                   // source position, base-cube units
   float beam[3];
   double src64[3];
@@ -312,7 +330,7 @@ size_t pt_scratch_doubles(int n_cases, int M, int B);
 
 cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T_frozen,
                             float* u_frozen, float t_min, float t_max, cudaStream_t s);
-// out [S][n_leaves] from tallies [n_leaves][tally_row(S)]
+// out [S][n_leaves] from tallies in rows tally_place(leaf)
 cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out, cudaStream_t s);
 // Every model of a batch in one launch (max_cells: of the largest): temperatures from the
 // counts into T_out; counts, spectra, counters and status to zero.

@@ -324,7 +324,7 @@ __device__ __forceinline__ void cell_temperatures(const DevGrid& g, const DevTab
   const int lev = g.level[c];
   // absorbed energy in units of eps: the count, or the path-length tally
   const auto absorbed = [&](int s) {
-    return pathabs ? (double)pathabs[c * tally_row(S) + s] : (double)count[s * g.n_leaves + c];
+    return pathabs ? (double)pathabs[tally_place(c) * tally_row(S) + s] : (double)count[s * g.n_leaves + c];
   };
   if constexpr (kS > 0) {
     double n[kS];
@@ -397,11 +397,12 @@ __global__ void __launch_bounds__(256) k_batch_reset(const ModelDesc* models) {
   if (first == 0) *md.r.status = 0u;
 }
 
-// Path-length tallies, species within a cell adjacent, to one array per species.
+// Path-length tallies, species within a cell adjacent, to one array per species (the rows of a
+// block of leaves come from L1 and L2 but for the first).
 __global__ void k_tally_out(const float* pathabs, long long N, int S, float* out) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= N) return;
-  const float* row = pathabs + (size_t)c * tally_row(S);
+  const float* row = pathabs + tally_place(c) * tally_row(S);
   for (int s = 0; s < S; ++s) out[(size_t)s * N + c] = row[s];
 }
 

@@ -297,7 +297,7 @@ __device__ __forceinline__ int advance(Pkg<R>& k, const DevGrid& g, const Kappa*
     const R seg = (kx > (R)0 && dtau > k.tau) ? k.tau / kx : tex;
     for (int s = 0; s < g.S; ++s) {
       const float v = (float)((R)__ldg(&rho[s]) * (R)kb[s].kabs * seg);
-      if (v > 0.f) atomicAdd(&pathabs[(size_t)leaf * tally_row(g.S) + s], v);
+      if (v > 0.f) atomicAdd(&pathabs[tally_place(leaf) * tally_row(g.S) + s], v);
     }
   }
   if (kx > (R)0 && dtau > k.tau) {
@@ -525,8 +525,8 @@ __device__ __forceinline__ void red_add4(float* p, const float* v) {
                  : "memory");
 }
 
-// Path-length tallies of a segment of length seg in a leaf, [n_leaves][tally_row(S)]: rho_s
-// kappa_abs,s seg is added for every species. With the species of a cell side by side two
+// Path-length tallies of a segment of length seg in a leaf, in its row: rho_s kappa_abs,s seg is
+// added for every species. With the species of a cell side by side two
 // or four of them are one vector reduction to one sector. 2e6 packages through 1.06e6
 // cells of two species: 3.9 ms with an atomic per species into arrays apart (and the
 // generic species loop), 2.7 ms. Other species counts need rows of whole vectors: 1e6
@@ -539,16 +539,16 @@ __device__ __forceinline__ void tally_segment(const DevGrid& g, float* pathabs, 
                                               const float* kabs) {
   if constexpr (kS == 2) {
     const float4 a = bin_vec<2>(kabs, bin);
-    red_add2(pathabs + 2 * (size_t)leaf, r.x * a.x * seg, r.y * a.y * seg);
+    red_add2(pathabs + 2 * tally_place(leaf), r.x * a.x * seg, r.y * a.y * seg);
   } else if constexpr (kS == 4) {
     const float4 a = bin_vec<4>(kabs, bin);
     const float v[4] = {r.x * a.x * seg, r.y * a.y * seg, r.z * a.z * seg, r.w * a.w * seg};
-    red_add4(pathabs + 4 * (size_t)leaf, v);
+    red_add4(pathabs + 4 * tally_place(leaf), v);
   } else {
     const int S = g.S;
     const float* rho = g.rho + (size_t)leaf * S;
     const Kappa* kb = kap + bin * S;
-    float* row = pathabs + (size_t)leaf * tally_row(S);
+    float* row = pathabs + tally_place(leaf) * tally_row(S);
     if (S == 1) {
       const float v = __ldg(rho) * kb[0].kabs * seg;
       if (v > 0.f) atomicAdd(row, v);
