@@ -397,13 +397,43 @@ __global__ void __launch_bounds__(256) k_batch_reset(const ModelDesc* models) {
   if (first == 0) *md.r.status = 0u;
 }
 
-// Path-length tallies, species within a cell adjacent, to one array per species (the rows of a
-// block of leaves come from L1 and L2 but for the first).
-__global__ void k_tally_out(const float* pathabs, long long N, int S, float* out) {
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  const float* row = pathabs + tally_place(c) * tally_row(S);
-  for (int s = 0; s < S; ++s) out[(size_t)s * N + c] = row[s];
+// Path-length tallies, species within a cell adjacent, to one array per species: a block of
+// rows is a 64 x 64 transposition (tally_place), done in tiles of 32 x 32 through shared memory
+// so that reads and writes are whole sectors, kV species at a time. 8.0e6 cells, us, a cell per
+// thread and in tiles: one species 33 and 12, two 60 and 25, four 119 and 42 (51 with kV = 4).
+constexpr int kTile = 32, kTileRows = 8;
+constexpr int kTilesAcross = (1 << kTallyBits) / kTile;
+
+template <int kV>
+__global__ void __launch_bounds__(kTile * kTileRows) k_tally_out(const float* pathabs,
+                                                                 long long N, int S, float* out) {
+  struct alignas(4 * kV) Vec {
+    float v[kV];
+  };
+  __shared__ float tile[kV][kTile][kTile + 1];
+  const int x = threadIdx.x & (kTile - 1), y = threadIdx.x / kTile;
+  const int t = blockIdx.x % (kTilesAcross * kTilesAcross);
+  const long long first = (long long)(blockIdx.x / (kTilesAcross * kTilesAcross)) * kTallyBlock;
+  const int a0 = t % kTilesAcross * kTile, b0 = t / kTilesAcross * kTile;
+  const int row = tally_row(S);  // a multiple of kV
+  for (int s0 = 0; s0 < S; s0 += kV) {
+#pragma unroll
+    for (int i = y; i < kTile; i += kTileRows) {  // place first + (b0 + i) 64 + a0 + x
+      const Vec r = *reinterpret_cast<const Vec*>(
+          pathabs + (size_t)(first + ((b0 + i) << kTallyBits) + a0 + x) * row + s0);
+#pragma unroll
+      for (int v = 0; v < kV; ++v) tile[v][i][x] = r.v[v];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = y; i < kTile; i += kTileRows) {
+      const long long leaf = first + ((a0 + i) << kTallyBits) + b0 + x;
+#pragma unroll
+      for (int v = 0; v < kV; ++v)
+        if (leaf < N && s0 + v < S) out[(size_t)(s0 + v) * N + leaf] = tile[v][x][i];
+    }
+    __syncthreads();
+  }
 }
 
 inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -428,7 +458,10 @@ cudaError_t launch_frozen_u(const DevGrid& g, const DevTables& t, const float* T
 
 cudaError_t launch_tally_out(const DevGrid& g, const float* pathabs, float* out,
                              cudaStream_t s) {
-  k_tally_out<<<nblk(g.n_leaves, 256), 256, 0, s>>>(pathabs, g.n_leaves, g.S, out);
+  const long long blocks = (g.n_leaves + kTallyBlock - 1) / kTallyBlock;
+  const auto kernel = g.S == 1 ? k_tally_out<1> : k_tally_out<2>;
+  kernel<<<(unsigned)(blocks * kTilesAcross * kTilesAcross), kTile * kTileRows, 0, s>>>(
+      pathabs, g.n_leaves, g.S, out);
   return cudaGetLastError();
 }
 
