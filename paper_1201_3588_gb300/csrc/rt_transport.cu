@@ -258,8 +258,8 @@ __device__ __forceinline__ void emit(Pkg<R>& k, unsigned long long id, const Dev
 }
 
 // One cell: cross it, or move to the interaction point inside it (the leaf is found
-// from the base cube each time: the plain walk).
-template <typename R>
+// from the base cube each time: the plain walk). kTally: path lengths into pathabs.
+template <typename R, bool kTally>
 __device__ __forceinline__ int advance(Pkg<R>& k, const DevGrid& g, const Kappa* kap,
                                        int& leaf, int& level, float* pathabs) {
   int I[3];
@@ -293,11 +293,12 @@ __device__ __forceinline__ int advance(Pkg<R>& k, const DevGrid& g, const Kappa*
   R kx = (R)0;
   for (int s = 0; s < g.S; ++s) kx += (R)__ldg(&rho[s]) * (R)kb[s].kext;
   const R dtau = kx * tex;
-  if (pathabs) {  // path-length tally of the segment inside this cell
+  if constexpr (kTally) {  // path-length tally of the segment inside this cell
     const R seg = (kx > (R)0 && dtau > k.tau) ? k.tau / kx : tex;
+    float* row = pathabs + tally_place(leaf) * tally_row(g.S);
     for (int s = 0; s < g.S; ++s) {
       const float v = (float)((R)__ldg(&rho[s]) * (R)kb[s].kabs * seg);
-      if (v > 0.f) atomicAdd(&pathabs[tally_place(leaf) * tally_row(g.S) + s], v);
+      if (v > 0.f) atomicAdd(row + s, v);
     }
   }
   if (kx > (R)0 && dtau > k.tau) {
@@ -1152,7 +1153,7 @@ __global__ void k_image_profile(const double* image, int nx, int ny, int plane_a
 // ---------------------------------------------------------------- plain kernel
 // One thread per package, tables read from global memory, one global atomic per
 // absorption and per escape.
-template <typename R>
+template <typename R, bool kTally>
 __global__ void __launch_bounds__(256) k_transport_plain(DevGrid g, DevTables t, DevRun r) {
   Tally tl = {};
   unsigned long long idx = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
@@ -1168,7 +1169,7 @@ __global__ void __launch_bounds__(256) k_transport_plain(DevGrid g, DevTables t,
         break;
       }
       int leaf, level;
-      int a = advance<R>(k, g, t.kap, leaf, level, r.pathabs);
+      int a = advance<R, kTally>(k, g, t.kap, leaf, level, r.pathabs);
       if (a <= kInteract) tl.levels += level;
       if (a == kCrossed) { ++tl.crossings; continue; }
       if (a == kEscaped) {
@@ -2111,10 +2112,11 @@ cudaError_t launch_transport_plain(const DevGrid& g, const DevTables& t, const D
   unsigned long long nb = (r.n_packages + threads - 1) / threads;
   if (nb == 0) return cudaSuccess;
   if (nb > 0x7fffffffull) return cudaErrorInvalidValue;
-  if (fp64)
-    k_transport_plain<double><<<(unsigned)nb, threads, 0, s>>>(g, t, r);
-  else
-    k_transport_plain<float><<<(unsigned)nb, threads, 0, s>>>(g, t, r);
+  const auto kernel = r.pathabs ? (fp64 ? k_transport_plain<double, true>
+                                        : k_transport_plain<float, true>)
+                                : (fp64 ? k_transport_plain<double, false>
+                                        : k_transport_plain<float, false>);
+  kernel<<<(unsigned)nb, threads, 0, s>>>(g, t, r);
   return cudaGetLastError();
 }
 
