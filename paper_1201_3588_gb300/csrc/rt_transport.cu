@@ -1643,9 +1643,11 @@ __host__ __device__ __forceinline__ int kap_records(const DevGrid& g) {
 }
 
 // ---------------------------------------------------------------- pool kernel
-// Shared memory of a block beside what the launch asks for: places and counters of 8 warps.
+// Shared memory of a warp: its places and its counters.
 template <bool kPath, bool kTally>
-constexpr size_t kPoolStatic = 8 * ((kTally ? 16 : park_bytes<kPath>()) + 4 * kTallyWords);
+__host__ __device__ constexpr int pool_warp_bytes() {
+  return (kTally ? 0 : park_bytes<kPath>()) + 4 * kTallyWords;
+}
 
 // Persistent packet pool over one model: all warps draw package indices from one
 // global counter; the opacity table, the stellar CDF and (where that costs no resident
@@ -1653,7 +1655,17 @@ constexpr size_t kPoolStatic = 8 * ((kTally ? 16 : park_bytes<kPath>()) + 4 * kT
 template <int kMinBlocks, bool kPeel, int kS = 0, bool kPath = false, bool kTally = false>
 __global__ void __launch_bounds__(256, kMinBlocks)
     k_transport_pool(DevGrid g, DevTables t, DevRun r, const __grid_constant__ DevPeel pe) {
-  extern __shared__ unsigned long long smem_u64[];
+  extern __shared__ __align__(16) unsigned char smem[];
+  // the warps' places and counters (as many as the block has warps: eight for blocks of any
+  // size left the smaller ones a few KB of L1; 1e6 packages through 1.1e5 cells, blocks of 128:
+  // five species 1.77 against 1.13 ms), then the launch's tables
+  constexpr int kWarpBytes = pool_warp_bytes<kPath, kTally>();
+  unsigned char* mine = smem + (threadIdx.x >> 5) * kWarpBytes;
+  unsigned* wt = reinterpret_cast<unsigned*>(mine + kWarpBytes - 4 * kTallyWords);
+  uint4* park = reinterpret_cast<uint4*>(mine);
+  if ((threadIdx.x & 31) < kTallyWords) wt[threadIdx.x & 31] = 0u;
+  unsigned long long* smem_u64 =
+      reinterpret_cast<unsigned long long*>(smem + (blockDim.x >> 5) * kWarpBytes);
   const int S = g.S, B = g.B;
   const int n_sed = 2 * g.n_dir * B;
   const bool sed_local = r.sed_in_smem != 0;
@@ -1684,15 +1696,7 @@ __global__ void __launch_bounds__(256, kMinBlocks)
     s_nemit = reinterpret_cast<unsigned long long*>(a);
     for (int i = threadIdx.x; i < B; i += blockDim.x) s_nemit[i] = 0ull;
   }
-  __shared__ unsigned s_tally[8 * kTallyWords];
-  constexpr int kParkBytes = kTally ? 16 : park_bytes<kPath>();
-  __shared__ __align__(16) unsigned char s_park[8 * kParkBytes];
-  static_assert(sizeof(s_tally) + sizeof(s_park) <= kPoolStatic<kPath, kTally>,
-                "the launch counts the kernel's own shared memory");
-  for (int i = threadIdx.x; i < 8 * kTallyWords; i += blockDim.x) s_tally[i] = 0u;
   __syncthreads();
-  unsigned* wt = s_tally + (threadIdx.x >> 5) * kTallyWords;
-  uint4* park = reinterpret_cast<uint4*>(s_park + (threadIdx.x >> 5) * kParkBytes);
   LaneTally tl = {};
   GlobalIds ids{r.next};
   pool_warp<kPeel, GlobalIds, kS, kPath, kTally>(g, t, r, kS > 2 ? t.kap : s_kap, s_cdf, s_sed,
@@ -1983,12 +1987,12 @@ static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, con
                                        int sms, cudaStream_t s) {
   DevRun rr = r;
   const size_t tables = table_smem<kS, kTally>(g) + (kPeel ? peel_smem(g) : 0);
+  const size_t warps = threads / 32 * pool_warp_bytes<kPath, kTally>();
   rr.sed_in_smem = tables + sed_smem(g) <= kSmemBudget ? 1 : 0;
-  size_t sm = tables + (rr.sed_in_smem ? sed_smem(g) : 0);
+  size_t sm = warps + tables + (rr.sed_in_smem ? sed_smem(g) : 0);
   cudaError_t e;
   const auto kernel = k_transport_pool<kMinBlocks, kPeel, kS, kPath, kTally>;
-  // beyond 48 KB a block with the kernel's own shared memory (places and counters)
-  if (sm + kPoolStatic<kPath, kTally> > 48 * 1024) {
+  if (sm > 48 * 1024) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
@@ -2002,14 +2006,13 @@ static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, con
   // both) 1.28 and 1.30; eight directions of 257 bins (three and four) 1.57 and 1.29, path
   // walk 2.69 and 2.27; of 333 bins (two and four) 2.28 and 1.29, path walk 3.53 and 2.28; of
   // 1024 bins (one and four) 3.61 and 1.58.
-  if (rr.sed_in_smem &&
-      (sm + kPoolStatic<kPath, kTally> + kSmemBlock) * kMinBlocks * 256 > kSmemSm * threads) {
+  if (rr.sed_in_smem && (sm + kSmemBlock) * kMinBlocks * 256 > kSmemSm * threads) {
     int most = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, kernel, threads, tables);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, kernel, threads, warps + tables);
     if (e != cudaSuccess) return e;
     if (occ < (blocks_per_sm > 0 && blocks_per_sm < most ? blocks_per_sm : most)) {
       rr.sed_in_smem = 0;
-      sm = tables;
+      sm = warps + tables;
       occ = most;
     }
   }
