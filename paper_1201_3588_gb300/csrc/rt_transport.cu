@@ -479,10 +479,11 @@ __device__ __forceinline__ float4 bin_vec(const float* table, int bin) {
 }
 
 // Extinction of a leaf per base-cube unit of path at a bin. kS: the species count when
-// fixed at compile time (2 or 4: the densities r, the bin's opacities as one vector from
-// kext), 0 when read from the grid (densities from the face-link record for one or two
-// species). kInOrder: summed species by species as the generic form does (the launches with
-// the path-length tally, whose histories are those of the generic walk to the last bit).
+// fixed at compile time (2 or 4: the densities r, the bin's opacities as one vector), 0 when
+// read from the grid (densities from the face-link record for one or two species). The
+// opacities come from kext [B][S]. kInOrder: the launches with the path-length tally, summed
+// species by species as the generic form does (their histories are those of the generic walk
+// to the last bit), the generic form's opacities from the records kap it reads anyway.
 template <int kS, bool kInOrder = false>
 __device__ __forceinline__ float leaf_ext(const DevGrid& g, int leaf, float4 r, int bin,
                                           const Kappa* kap, const float* kext) {
@@ -497,15 +498,17 @@ __device__ __forceinline__ float leaf_ext(const DevGrid& g, int leaf, float4 r, 
     return r.x * e.x + r.y * e.y + r.z * e.z + r.w * e.w;
   } else {
     const Kappa* kb = kap + bin * g.S;
+    const float* eb = kext + bin * g.S;
+    const auto e = [&](int s) { return kInOrder ? kb[s].kext : eb[s]; };
     if (g.S <= 2) {
       const int* rec = g.links + (size_t)leaf * kRec;
-      float kx = __int_as_float(__ldg(rec + 6)) * kb[0].kext;
-      if (g.S == 2) kx += __int_as_float(__ldg(rec + 7)) * kb[1].kext;
+      float kx = __int_as_float(__ldg(rec + 6)) * e(0);
+      if (g.S == 2) kx += __int_as_float(__ldg(rec + 7)) * e(1);
       return kx;
     }
     const float* rho = g.rho + (size_t)leaf * g.S;
     float kx = 0.f;
-    for (int s = 0; s < g.S; ++s) kx += __ldg(&rho[s]) * kb[s].kext;
+    for (int s = 0; s < g.S; ++s) kx += __ldg(&rho[s]) * e(s);
     return kx;
   }
 }
@@ -747,7 +750,7 @@ __device__ __forceinline__ int path_leaf(const DevGrid& g, int slot) {
 
 template <int kS>
 __device__ __forceinline__ float slot_ext(const DevGrid& g, float4 v, int slot, float4 e,
-                                          const Kappa* kb) {
+                                          const float* eb) {
   if constexpr (kS == 4) {
     return v.x * e.x + v.y * e.y + v.z * e.z + v.w * e.w;
   } else if constexpr (kS == 2) {
@@ -755,17 +758,17 @@ __device__ __forceinline__ float slot_ext(const DevGrid& g, float4 v, int slot, 
   } else {
     const float* rho = g.rho_slot + (size_t)slot * g.S;
     float kx = 0.f;
-    for (int s = 0; s < g.S; ++s) kx += __ldg(&rho[s]) * kb[s].kext;
+    for (int s = 0; s < g.S; ++s) kx += __ldg(&rho[s]) * eb[s];
     return kx;
   }
 }
 
 // The extinction of the cell a package is in, at its bin.
 template <int kS>
-__device__ __forceinline__ float path_ext(const DevGrid& g, int slot, int bin, const Kappa* kap,
+__device__ __forceinline__ float path_ext(const DevGrid& g, int slot, int bin,
                                           const float* kext) {
   return slot_ext<kS>(g, slot_row<kS>(g, slot), slot, bin_vec<kS>(kext, bin),
-                      kap + bin * (kS > 0 ? kS : g.S));
+                      kext + bin * (kS > 0 ? kS : g.S));
 }
 
 // One cell of the path walk (kS: 2 or 4 species read as one vector, 0 the generic
@@ -778,8 +781,7 @@ __device__ __forceinline__ float path_ext(const DevGrid& g, int slot, int bin, c
 // is kept in the cell for the next step.
 template <int kS>
 __device__ __forceinline__ int advance_path(Pkg<float>& k, PathCell& c, const DevGrid& g,
-                                            const Kappa* kap, const float* kext,
-                                            unsigned& child_reads) {
+                                            const float* kext, unsigned& child_reads) {
   const Exit e = exit_of(k, c);
   const float dtau = c.kx * e.t;
   if (dtau > k.tau) return kInteract;
@@ -847,7 +849,7 @@ __device__ __forceinline__ int advance_path(Pkg<float>& k, PathCell& c, const De
     set_corner(c, K, lev);
   }
   c.slot = slot;
-  c.kx = slot_ext<kS>(g, row, slot, bin_vec<kS>(kext, k.bin), kap + k.bin * (kS > 0 ? kS : g.S));
+  c.kx = slot_ext<kS>(g, row, slot, bin_vec<kS>(kext, k.bin), kext + k.bin * (kS > 0 ? kS : g.S));
   return kCrossed;
 }
 
@@ -1036,7 +1038,7 @@ __device__ __forceinline__ void flush_warp(LaneTally& tl, unsigned* wt, unsigned
 // the pixel x projects to and the attenuation exp(-tau) to the boundary. Returns
 // false when x falls outside the image, tau passes pe.tau_max, or the walk fails
 // (then the tree status bit is set).
-__device__ __forceinline__ bool sight_line(const DevGrid& g, const Kappa* kap,
+__device__ __forceinline__ bool sight_line(const DevGrid& g, const float* kext,
                                            const DevPeel& pe, float x0, float x1, float x2,
                                            int bin, float& att, size_t& pix,
                                            unsigned& crossings, unsigned* status) {
@@ -1069,7 +1071,7 @@ __device__ __forceinline__ bool sight_line(const DevGrid& g, const Kappa* kap,
     // a straight line crosses at most 3 n 2^L finest cells of the n^3 base grid
     const long long cap = 3ll * ((long long)g.n_base << g.max_level) + 8;
     for (long long i = 0;; ++i) {
-      const int a = advance_linked<true>(k, c, g, kap, nullptr, lv, &tau);
+      const int a = advance_linked<true>(k, c, g, nullptr, kext, lv, &tau);
       ++crossings;
       if (a == kEscaped) break;
       if (a == kError || i >= cap) {
@@ -1096,7 +1098,7 @@ __global__ void k_peel_source(DevGrid g, DevTables t, DevRun r, DevPeel pe) {
   float att;
   size_t pix;
   unsigned cr = 0;
-  if (sight_line(g, t.kap, pe, r.src[0], r.src[1], r.src[2], b, att, pix, cr, r.status))
+  if (sight_line(g, t.kext, pe, r.src[0], r.src[1], r.src[2], b, att, pix, cr, r.status))
     atomicAdd(&pe.image[pix], (double)n * (double)kInv4Pi * (double)att);
   if (cr) atomicAdd(&r.counters[kCPeelCrossings], (unsigned long long)cr);
 }
@@ -1117,7 +1119,7 @@ __global__ void __launch_bounds__(256) k_peel_trace(DevGrid g, DevTables t, DevR
     const int bin = pe.ev_bin[i];
     float att;
     size_t pix;
-    if (sight_line(g, t.kap, pe, e.x, e.y, e.z, bin, att, pix, cr, r.status))
+    if (sight_line(g, t.kext, pe, e.x, e.y, e.z, bin, att, pix, cr, r.status))
       atomicAdd(&pe.image[pix], (double)(e.w * att));
   }
   unsigned long long x = cr;
@@ -1416,7 +1418,7 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
         rc = enter(k, g, cell, tl.levels);
       if (rc == 0) {
         walking = true;
-        if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kap, kext);
+        if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kext);
       } else if (rc == 1) {  // source outside the grid, moving away
         atomicAdd(&wt[kCEscaped], 1u);
         const int db = dir_bin(k.d[2], g.n_dir);
@@ -1456,7 +1458,7 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
 #pragma unroll 2
         for (int u = 0; u < kSteps; ++u) {
           if constexpr (kPath)
-            a = advance_path<kS>(k, cell, g, kap, kext, tl.levels);
+            a = advance_path<kS>(k, cell, g, kext, tl.levels);
           else
             a = advance_linked<false, kS, kTally>(k, cell, g, kap, kext, tl.levels, nullptr,
                                                   r.pathabs, kabs);
@@ -1601,7 +1603,7 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
                             w1, clamped);
           if (clamped) atomicAdd(&wt[kCClamped], 1u);
         }
-        if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kap, kext);
+        if constexpr (kPath) cell.kx = path_ext<kS>(g, cell.slot, k.bin, kext);
       }
       if constexpr (kPeel) {
         // the event's share toward the observer, at the bin it leaves with
@@ -1627,19 +1629,22 @@ __device__ __forceinline__ bool pool_warp(const DevGrid& g, const DevTables& t, 
   }
 }
 
-// Shared-memory words (floats) of the per-bin extinction vectors: B x kS for the walks
-// compiled for 2 or 4 species, rounded up to 16 bytes; none otherwise.
-template <int kS>
-__host__ __device__ constexpr int kext_words(int B) {
-  return kS == 2 || kS == 4 ? (B * kS + 3) / 4 * 4 : 0;
+// Shared-memory words (floats) of the extinction opacities [B][S], rounded up to 16 bytes, and
+// the opacity records staged there too. A crossing needs the extinctions alone: with the
+// records of a generic walk's species in every block, beside the places, nothing was left of L1
+// (1e6 packages through 1.1e5 cells, ms, records and extinctions in shared memory: five
+// species, 400 bins 1.78 and 1.01; six 1.92 and 1.28; eight, 200 bins 2.74 and 2.33; five, 100
+// bins 0.98 and 0.95). Records are read at interactions, from L1, but for two species (4.11 ms
+// in shared memory against 4.17 for the disk of 2.4e6 cells) and for the generic walk with the
+// path-length tally, which reads them at every crossing and has no places.
+template <int kS, bool kTally>
+__host__ __device__ __forceinline__ int kext_words(const DevGrid& g) {
+  return kS == 0 && kTally ? 0 : (g.B * (kS > 0 ? kS : g.S) + 3) / 4 * 4;
 }
 
-// Opacity records staged in shared memory: those of the generic walks, which read them at
-// every crossing. The walks compiled for 2 or 4 species need only the extinction vectors
-// there and take the records, read once per interaction, from L1.
-template <int kS>
+template <int kS, bool kTally>
 __host__ __device__ __forceinline__ int kap_records(const DevGrid& g) {
-  return kS > 2 ? 0 : g.B * g.S;
+  return kS == 2 || (kS == 0 && kTally) ? g.B * g.S : 0;
 }
 
 // ---------------------------------------------------------------- pool kernel
@@ -1669,15 +1674,15 @@ __global__ void __launch_bounds__(256, kMinBlocks)
   const int S = g.S, B = g.B;
   const int n_sed = 2 * g.n_dir * B;
   const bool sed_local = r.sed_in_smem != 0;
-  // 2 or 4 species: the extinction opacities [B][S] first (with the path-length tally the
-  // absorption opacities after them), one vector per bin (a multiple of 16 bytes)
+  // the extinction opacities [B][S] first (with the path-length tally of 2 or 4 species the
+  // absorption opacities after them), for 2 or 4 one vector per bin (a multiple of 16 bytes)
   float* s_kext = reinterpret_cast<float*>(smem_u64);
-  const int n_kext = kext_words<kS>(B);
+  const int n_kext = kext_words<kS, kTally>(g);
   float* s_kabs = s_kext + n_kext;
   unsigned long long* s_u64 = smem_u64 + (kTally ? 2 : 1) * n_kext / 2;
   unsigned long long* s_sed = sed_local ? s_u64 : r.sed;   // [2][n_dir][B]
   Kappa* s_kap = reinterpret_cast<Kappa*>(s_u64 + (sed_local ? n_sed : 0));  // [B][S]
-  const int n_kap = kap_records<kS>(g);
+  const int n_kap = kap_records<kS, kTally>(g);
   float* s_cdf = reinterpret_cast<float*>(s_kap + n_kap);     // [B]
   if (sed_local)
     for (int i = threadIdx.x; i < n_sed; i += blockDim.x) s_sed[i] = 0ull;
@@ -1699,7 +1704,7 @@ __global__ void __launch_bounds__(256, kMinBlocks)
   __syncthreads();
   LaneTally tl = {};
   GlobalIds ids{r.next};
-  pool_warp<kPeel, GlobalIds, kS, kPath, kTally>(g, t, r, kS > 2 ? t.kap : s_kap, s_cdf, s_sed,
+  pool_warp<kPeel, GlobalIds, kS, kPath, kTally>(g, t, r, kS == 2 || (kS == 0 && kTally) ? s_kap : t.kap, s_cdf, s_sed,
                                                  r.n_packages, ids, tl, wt, park, global_ns(), &pe,
                                                  s_nemit, s_kext, s_kabs);
   flush_warp(tl, wt, r.counters);
@@ -1860,7 +1865,7 @@ __global__ void k_trace(DevGrid g, DevTables t, DevRun r, const unsigned long lo
       break;
     }
     const int lf = c.leaf;
-    const int a = advance_linked(k, c, g, t.kap, nullptr, tl.levels);
+    const int a = advance_linked(k, c, g, t.kap, t.kext, tl.levels);
     rec[8] = lf;
     if (a == kCrossed) { ++rec[3]; continue; }
     if (a == kEscaped) {
@@ -1871,7 +1876,7 @@ __global__ void k_trace(DevGrid g, DevTables t, DevRun r, const unsigned long lo
       break;
     }
     if (a == kError) { atomicOr(r.status, kStatusTree); break; }
-    to_point(k, c, leaf_ext<0>(g, c.leaf, float4{}, k.bin, t.kap, nullptr));
+    to_point(k, c, leaf_ext<0>(g, c.leaf, float4{}, k.bin, t.kap, t.kext));
     const float pi[3] = {at(0), at(1), at(2)};
     if (++k.event > r.max_events) {
       rec[5] = 1;
@@ -1971,8 +1976,8 @@ constexpr size_t kSmemSm = 228 * 1024, kSmemBlock = 1024;  // of an SM; kept by 
 
 template <int kS, bool kTally>
 static size_t table_smem(const DevGrid& g) {
-  return sizeof(Kappa) * kap_records<kS>(g) +
-         sizeof(float) * ((kTally ? 2 : 1) * kext_words<kS>(g.B) + g.B);
+  return sizeof(Kappa) * kap_records<kS, kTally>(g) +
+         sizeof(float) * ((kTally ? 2 : 1) * kext_words<kS, kTally>(g) + g.B);
 }
 
 static size_t sed_smem(const DevGrid& g) {
