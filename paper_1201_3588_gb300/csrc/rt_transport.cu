@@ -1972,7 +1972,9 @@ __global__ void k_philox(const unsigned long long* ids, long long n, unsigned ev
 }  // namespace
 
 constexpr size_t kSmemBudget = 200 * 1024;
-constexpr size_t kSmemSm = 228 * 1024, kSmemBlock = 1024;  // of an SM; kept by each block
+constexpr size_t kSmemBlock = 1024;  // kept by each block beside what it asks for
+// shared memory of an SM beyond which the next carve-outs leave L1 a quarter or less of the 256 KB
+constexpr size_t kSmemKeep = 164 * 1024;
 
 template <int kS, bool kTally>
 static size_t table_smem(const DevGrid& g) {
@@ -2004,18 +2006,20 @@ static cudaError_t launch_pool_variant(const DevGrid& g, const DevTables& t, con
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, sm);
   if (e != cudaSuccess) return e;
-  // The spectrum in shared memory is worth a few per cent, a block per SM far more: it goes to
-  // global memory where, beside the places, it would cost one that the launch would have (asked
-  // for only where shared memory can be what limits the blocks). 5.3e5 cells of two species,
+  // The spectrum in shared memory is worth a few per cent, a block per SM or L1 far more: it goes
+  // to global memory where, beside the places, it would cost a block that the launch would have,
+  // or L1 (asked only where shared memory can be what limits). 5.3e5 cells of two species,
   // 3e6 packages, in shared and in global memory, ms: 200 bins, one direction (four blocks
   // both) 1.28 and 1.30; eight directions of 257 bins (three and four) 1.57 and 1.29, path
   // walk 2.69 and 2.27; of 333 bins (two and four) 2.28 and 1.29, path walk 3.53 and 2.28; of
-  // 1024 bins (one and four) 3.61 and 1.58.
-  if (rr.sed_in_smem && (sm + kSmemBlock) * kMinBlocks * 256 > kSmemSm * threads) {
+  // 1024 bins (one and four) 3.61 and 1.58. Four blocks both, 1e6 packages through 1.1e5 cells:
+  // three species, 1024 bins 1.45 and 0.81, two species, 600 bins 0.86 and 0.59.
+  if (rr.sed_in_smem && (sm + kSmemBlock) * kMinBlocks * 256 > kSmemKeep * threads) {
     int most = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, kernel, threads, warps + tables);
     if (e != cudaSuccess) return e;
-    if (occ < (blocks_per_sm > 0 && blocks_per_sm < most ? blocks_per_sm : most)) {
+    const int want = blocks_per_sm > 0 && blocks_per_sm < most ? blocks_per_sm : most;
+    if (occ < want || (sm + kSmemBlock) * want > kSmemKeep) {
       rr.sed_in_smem = 0;
       sm = warps + tables;
       occ = most;
