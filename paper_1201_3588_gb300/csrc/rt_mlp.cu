@@ -876,10 +876,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (ok) tc_commit(&bars->acc[1]);
           }
         }
-      // the products in flight land before the memory is given up, whichever warp's wait ran
-      // out: a barrier of its own, whose one phase no other commit completes
       tc_commit(&bars->drained);
-      mbar_wait(smem_addr(&bars->drained), 0u);
     }
   } else {
     // ---- input, activations and outputs
@@ -1079,6 +1076,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   if (warp == 0) {
+    // the products in flight land before the memory is given up, whichever warp's wait ran
+    // out: a barrier of its own, whose one phase no other commit completes (long complete
+    // where none did)
+    mbar_wait(smem_addr(&bars->drained), 0u);
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
                  "r"(kTcTiles * kTcMaxWidth));
