@@ -297,18 +297,18 @@ PROFILE_SOURCES = ("paper_1201_3588_gb300/csrc/rt_transport.cu",
                    "paper_1201_3588_gb300/csrc/rt_internal.h")
 PROFILE = {
     # 1-pass counters of one 2e7-package launch on the full large disk (path walk):
-    # dram 174.27 GB read + 0.11 GB written; 6.759e10 warp and 1.053e12 thread
+    # dram 175.18 GB read + 0.11 GB written; 3.543e10 warp and 5.801e11 thread
     # instructions over 5.24e9 crossings
-    "large_disk": {"sha256": "37df585bc0db86db4b62d16c47608a40489a74d084f398b36c592e962be6373b",
-                   "dram_bytes_per_package": 8718.9, "warp_lanes_active": 15.58,
-                   "warp_instr_per_crossing": 12.89,
+    "large_disk": {"sha256": "13489e331a0a4d4380a29b82e0c0791a31f034beddd9dab0ff8d92b87d9234c4",
+                   "dram_bytes_per_package": 8764.2, "warp_lanes_active": 16.37,
+                   "warp_instr_per_crossing": 6.76,
                    "file": "profiles/k_transport_pool_large_disk.md"},
     # the same counters of one 1e8-package launch on the flared disk (linked walk):
-    # dram 103.92 GB read + 0.24 GB written; 1.496e11 warp and 2.543e12 thread
+    # dram 113.57 GB read + 0.24 GB written; 6.928e10 warp and 1.370e12 thread
     # instructions over 1.41e10 crossings
-    "disk": {"sha256": "37df585bc0db86db4b62d16c47608a40489a74d084f398b36c592e962be6373b",
-             "dram_bytes_per_package": 1041.6, "warp_lanes_active": 17.0,
-             "warp_instr_per_crossing": 10.62, "file": "profiles/k_transport_pool_disk.md"},
+    "disk": {"sha256": "13489e331a0a4d4380a29b82e0c0791a31f034beddd9dab0ff8d92b87d9234c4",
+             "dram_bytes_per_package": 1138.0, "warp_lanes_active": 19.77,
+             "warp_instr_per_crossing": 4.92, "file": "profiles/k_transport_pool_disk.md"},
 }
 
 
