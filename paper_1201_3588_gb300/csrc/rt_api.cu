@@ -1749,11 +1749,14 @@ struct rt_batch {
   int dev = 0;
   std::vector<rt_grid*> grids;
   std::vector<unsigned long long> n_pk;
-  char* slab = nullptr;  // holds the next two and every model's temperatures
+  char* slab = nullptr;  // holds the next four and every model's temperatures
   ModelDesc* d_models = nullptr;
-  unsigned long long* d_next = nullptr;  // [models] packages handed out
+  unsigned long long* d_plan = nullptr;    // see BatchQueue
+  unsigned long long* d_before = nullptr;
+  unsigned long long* d_next = nullptr;
   std::vector<float*> d_T;               // of each model, [S][n_leaves]
   int chunk = 0;                         // packages a warp takes at a time
+  int n_live = 0;                        // models with packages
   int blocks_per_sm = 0;
   int threads = 256;  // threads per block of the batched launch
   int s_fixed = 0;  // the species count every model shares (walk compiled for it), else 0
@@ -1830,7 +1833,9 @@ rt_status rt_batch_create(rt_grid* const* grids, int n, const uint64_t* n_packag
   Slab slab;
   b->d_T.assign((size_t)n, nullptr);
   slab.add(&b->d_models, (size_t)n);
-  slab.add(&b->d_next, (size_t)n);
+  slab.add(&b->d_plan, (size_t)n);
+  slab.add(&b->d_before, (size_t)n + 1);
+  slab.add(&b->d_next, (size_t)n + 1);
   for (int m = 0; m < n; ++m)
     slab.add(&b->d_T[(size_t)m],
              (size_t)grids[m]->desc.n_species * (size_t)grids[m]->desc.n_leaves);
@@ -1839,8 +1844,19 @@ rt_status rt_batch_create(rt_grid* const* grids, int n, const uint64_t* n_packag
     return st;
   }
   for (int m = 0; m < n; ++m) desc[(size_t)m].T_out = b->d_T[(size_t)m];
+  std::vector<unsigned long long> before((size_t)n + 1, 0);
+  for (int m = 0; m < n; ++m) {
+    before[(size_t)m + 1] = before[(size_t)m] + b->n_pk[(size_t)m];
+    b->n_live += b->n_pk[(size_t)m] > 0;
+  }
   cudaError_t e = cudaMemcpy(b->d_models, desc.data(), sizeof(ModelDesc) * n,
                              cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(b->d_plan, b->n_pk.data(), sizeof(unsigned long long) * n,
+                   cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(b->d_before, before.data(), sizeof(unsigned long long) * (n + 1),
+                   cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     rt_batch_destroy(b);
     return RT_ERR_CUDA;
@@ -1861,9 +1877,10 @@ rt_status rt_batch_run(rt_batch* b, int reset, int temperatures, void* stream) {
       if (st != RT_OK) return st;
     }
   }
-  RT_CUDA(cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long) * n, s));
-  RT_CUDA(launch_transport_batch(b->d_models, n, b->d_next, b->chunk,
-                                 b->blocks_per_sm, b->s_fixed, b->tally, b->threads, s));
+  RT_CUDA(cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long) * (n + 1), s));
+  const BatchQueue q{b->d_plan, b->d_before, b->d_next, n, b->n_live};
+  RT_CUDA(launch_transport_batch(b->d_models, q, b->chunk, b->blocks_per_sm, b->s_fixed, b->tally,
+                                 b->threads, s));
   if (temperatures)
     RT_CUDA(launch_batch_temperatures(b->d_models, n, b->max_cells, b->s_fixed, s));
   return RT_OK;

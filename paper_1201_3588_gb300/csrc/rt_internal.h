@@ -165,13 +165,23 @@ struct ModelDesc {
   float* T_out;  // temperatures [S][n_leaves] of the model
 };
 
+// The packages of a batched launch.
+struct BatchQueue {
+  const unsigned long long* plan;    // [n] of each model
+  const unsigned long long* before;  // [n + 1] of the models before it
+  unsigned long long* next;          // [n] of each model handed out so far, then the number of
+                                     // models found exhausted (zeros at the start)
+  int n, n_live;                     // models, and those with packages
+};
+constexpr unsigned long long kExhausted = 1ull << 63;  // set in next[m] by the first to find it so
+
 // Kernel launchers (rt_transport.cu, rt_tables.cu).
-// next [n_models]: packages of each model handed out so far (zeros); chunk >= 32: how
-// many a warp takes at a time. s_fixed: the species count all models share (2 has a walk
-// compiled for it), 0 otherwise; tally: the path-length tallies (of every model)
-cudaError_t launch_transport_batch(const ModelDesc* models, int n_models,
-                                   unsigned long long* next, int chunk, int blocks_per_sm,
-                                   int s_fixed, bool tally, int threads, cudaStream_t s);
+// chunk >= 32: how many packages a warp takes at a time. s_fixed: the species count all
+// models share (2 has a walk compiled for it), 0 otherwise; tally: the path-length tallies
+// (of every model)
+cudaError_t launch_transport_batch(const ModelDesc* models, const BatchQueue& q, int chunk,
+                                   int blocks_per_sm, int s_fixed, bool tally, int threads,
+                                   cudaStream_t s);
 cudaError_t launch_transport_pool(const DevGrid& g, const DevTables& t, const DevRun& r,
                                   int blocks_per_sm, int threads, cudaStream_t s,
                                   const DevPeel* peel = nullptr, bool path = false);

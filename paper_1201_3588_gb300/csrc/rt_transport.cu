@@ -1723,7 +1723,7 @@ __global__ void __launch_bounds__(256, kMinBlocks)
 // Many models in one persistent launch. A warp picks a model, stages its descriptor in
 // shared memory and runs the pool loop on it, drawing packages from the model's counter
 // until that is exhausted and its own lanes have run dry; then it picks the next. The
-// pick is weighted by the packages each model has left: the first one stratified over
+// pick is weighted by the packages each model has left (pick_model): the first one stratified over
 // the warps (so that neighbouring warps share a model's rows in L1), later ones at
 // random. A warp's lanes therefore run dry once per model it works on. (Fixed chunks of
 // 4096 packages, a warp's lanes drained at the end of each, left three quarters of the
@@ -1731,52 +1731,84 @@ __global__ void __launch_bounds__(256, kMinBlocks)
 // warps -- and took 28.7 ms against 8.0 for this, and 4.8 with the walk as it is now.) Tables
 // in global memory / L2, spectrum by global atomics; counters are flushed to the model when
 // the warp leaves it.
-__device__ __forceinline__ int pick_model(const ModelDesc* models, int n,
-                                          const unsigned long long* next, unsigned warp_id,
-                                          unsigned n_warps, unsigned pick) {
+//
+// Up to kPickWindow models are weighed together by what each has left. Of more, one is drawn by
+// the plan (its packages at the start) and taken if it has any left, else the window of models
+// from it on is weighed, and so on round the batch: a pick's cost does not grow with the batch
+// until its end, and then only while some model has packages. (Weighing all models at every pick, with their descriptors read for it, 4000 and
+// 8000 models of 50 packages took 565 and 1427 us beside 87 and 148 for chunks of one model; now
+// 96 and 182.)
+constexpr int kPickWindow = 256;
+
+__device__ __forceinline__ int pick_model(const BatchQueue& q, unsigned warp_id, unsigned n_warps,
+                                          unsigned pick) {
   const int lane = threadIdx.x & 31;
   auto remaining = [&](int m) {
-    if (m >= n) return 0ull;
-    const unsigned long long all = models[m].r.n_packages;
-    const unsigned long long out = *reinterpret_cast<const volatile unsigned long long*>(&next[m]);
+    const unsigned long long all = q.plan[m];
+    const unsigned long long out =
+        *reinterpret_cast<const volatile unsigned long long*>(&q.next[m]);
     return out < all ? all - out : 0ull;
   };
-  unsigned long long tot = 0;
-  for (int m = lane; m < n; m += 32) tot += remaining(m);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(kFull, tot, o);
-  if (tot == 0) return -1;
-  // a point in [0, tot) as a 64-bit fraction: the warp's place, or a hash
+  // a point as a 64-bit fraction: the warp's place, or a hash
   unsigned long long frac = (((unsigned long long)warp_id << 1 | 1) << 31) / n_warps << 32;
   if (pick > 0) {
     frac = ((unsigned long long)warp_id << 32 | pick) * 0x9E3779B97F4A7C15ull;
     frac ^= frac >> 29;
     frac *= 0xBF58476D1CE4E5B9ull;
   }
-  unsigned long long point = __umul64hi(frac, tot);
-  int last = -1;  // the counters move meanwhile: the last model that had any left
-  for (int m0 = 0; m0 < n; m0 += 32) {
-    const unsigned long long r = remaining(m0 + lane);
-    unsigned long long c = r;  // inclusive sum over the lanes
+  int first = 0;
+  if (q.n > kPickWindow) {
+    const unsigned long long point = __umul64hi(frac, q.before[q.n]);
+    int hi = q.n;  // before[first] <= point < before[hi]
+    while (hi - first > 1) {
+      const int mid = (first + hi) >> 1;
+      if (q.before[mid] <= point) first = mid; else hi = mid;
+    }
+    if (__shfl_sync(kFull, remaining(first), 0) > 0) return first;
+    const unsigned long long done =
+        *reinterpret_cast<const volatile unsigned long long*>(&q.next[q.n]);
+    if (__shfl_sync(kFull, done, 0) >= (unsigned long long)q.n_live) return -1;
+    frac = (frac ^ frac >> 31) * 0x94D049BB133111EBull;
+  }
+  for (int off = 0; off < q.n; off += kPickWindow) {
+    constexpr int kEach = kPickWindow / 32;
+    unsigned long long r[kEach], sum = 0;
+#pragma unroll
+    for (int j = 0; j < kEach; ++j) {
+      const int i = off + 32 * j + lane, m = first + i;
+      r[j] = i < q.n ? remaining(m < q.n ? m : m - q.n) : 0ull;
+      sum += r[j];
+    }
+    unsigned long long c = sum;  // inclusive sum over the lanes
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned long long u = __shfl_up_sync(kFull, c, o);
       if (lane >= o) c += u;
     }
-    const unsigned above = __ballot_sync(kFull, c > point), any = __ballot_sync(kFull, r > 0);
-    if (above) return m0 + __ffs(above) - 1;
-    if (any) last = m0 + 31 - __clz(any);
-    point -= __shfl_sync(kFull, c, 31);
+    const unsigned long long tot = __shfl_sync(kFull, c, 31);
+    if (tot == 0) continue;
+    const unsigned long long point = __umul64hi(frac, tot);
+    const int src = __ffs(__ballot_sync(kFull, c > point)) - 1;
+    unsigned long long p = point - (c - sum);  // within the lane src
+    int at = off + lane;
+#pragma unroll
+    for (int j = 0; j + 1 < kEach; ++j)
+      if (at == off + 32 * j + lane && p >= r[j]) {
+        p -= r[j];
+        at += 32;
+      }
+    const int m = first + __shfl_sync(kFull, at, src);
+    return m < q.n ? m : m - q.n;
   }
-  return last;
+  return -1;
 }
 
 // Two species: held to 64 registers (58 bytes of spills) for four blocks per SM; when this
 // was decided 8.0 ms against 8.7 with three blocks of 74 registers, and 180 bytes of spills in
 // the generic form.
 template <int kS, bool kTally>
-__global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const ModelDesc* models, int n_models,
-                                                         unsigned long long* next, int chunk) {
+__global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const ModelDesc* models,
+                                                         BatchQueue q, int chunk) {
   __shared__ ModelDesc sdesc[8];
   __shared__ unsigned s_tally[8 * kTallyWords];
   constexpr int kParkBytes = kTally ? 16 : park_bytes<false>();
@@ -1788,8 +1820,7 @@ __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const 
   const unsigned per_block = blockDim.x >> 5;
   const unsigned long long t0 = global_ns();
   for (unsigned pick = 0;; ++pick) {
-    const int m = pick_model(models, n_models, next, blockIdx.x * per_block + warp,
-                             gridDim.x * per_block, pick);
+    const int m = pick_model(q, blockIdx.x * per_block + warp, gridDim.x * per_block, pick);
     if (m < 0) break;
     const int* src = reinterpret_cast<const int*>(&models[m]);
     int* dst = reinterpret_cast<int*>(&sdesc[warp]);
@@ -1797,19 +1828,20 @@ __global__ void __launch_bounds__(256, kS == 2 ? 4 : 3) k_transport_batch(const 
     __syncwarp();
     const ModelDesc& md = sdesc[warp];
     LaneTally tl = {};
-    ModelIds ids{next + m, 0ull, md.r.n_packages, 0, chunk};
+    ModelIds ids{q.next + m, 0ull, md.r.n_packages, 0, chunk};
     const bool in_time =
         pool_warp<false, ModelIds, kS, false, kTally>(md.g, md.t, md.r, md.t.kap, md.t.star_cdf, md.r.sed,
                                         md.r.n_packages, ids, tl, wt, park, t0, nullptr, nullptr,
                                         md.t.kext);
     flush_warp(tl, wt, md.r.counters);
     __syncwarp();
+    if (in_time && lane == 0 && !(atomicOr(&q.next[m], kExhausted) & kExhausted))
+      atomicAdd(&q.next[q.n], 1ull);
     if (!in_time) {
       // the budget is the launch's: what is left of any model stays undone, and its status
       // says so, also where no warp was on it (models with few packages wait for the large)
-      for (int j = lane; j < n_models; j += 32)
-        if (*reinterpret_cast<const volatile unsigned long long*>(&next[j]) <
-            models[j].r.n_packages)
+      for (int j = lane; j < q.n; j += 32)
+        if (*reinterpret_cast<const volatile unsigned long long*>(&q.next[j]) < q.plan[j])
           atomicOr(models[j].r.status, kStatusTimeout);
       break;
     }
@@ -2133,9 +2165,8 @@ cudaError_t launch_transport_plain(const DevGrid& g, const DevTables& t, const D
 }
 
 template <int kS, bool kTally>
-static cudaError_t launch_batch_variant(const ModelDesc* models, int n_models,
-                                        unsigned long long* next, int chunk, int blocks_per_sm,
-                                        int threads, cudaStream_t s) {
+static cudaError_t launch_batch_variant(const ModelDesc* models, const BatchQueue& q, int chunk,
+                                        int blocks_per_sm, int threads, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -2146,21 +2177,20 @@ static cudaError_t launch_batch_variant(const ModelDesc* models, int n_models,
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   int bps = blocks_per_sm > 0 && blocks_per_sm < occ ? blocks_per_sm : occ;
-  k_transport_batch<kS, kTally><<<sms * bps, threads, 0, s>>>(models, n_models, next, chunk);
+  k_transport_batch<kS, kTally><<<sms * bps, threads, 0, s>>>(models, q, chunk);
   return cudaGetLastError();
 }
 
-cudaError_t launch_transport_batch(const ModelDesc* models, int n_models,
-                                   unsigned long long* next, int chunk, int blocks_per_sm,
-                                   int s_fixed, bool tally, int threads, cudaStream_t s) {
+cudaError_t launch_transport_batch(const ModelDesc* models, const BatchQueue& q, int chunk,
+                                   int blocks_per_sm, int s_fixed, bool tally, int threads,
+                                   cudaStream_t s) {
   if (threads <= 0) threads = 256;
   if (threads % 32 != 0 || threads > 256) return cudaErrorInvalidValue;
   if (tally)
-    return launch_batch_variant<0, true>(models, n_models, next, chunk, blocks_per_sm, threads, s);
+    return launch_batch_variant<0, true>(models, q, chunk, blocks_per_sm, threads, s);
   if (s_fixed == 2)
-    return launch_batch_variant<2, false>(models, n_models, next, chunk, blocks_per_sm, threads,
-                                          s);
-  return launch_batch_variant<0, false>(models, n_models, next, chunk, blocks_per_sm, threads, s);
+    return launch_batch_variant<2, false>(models, q, chunk, blocks_per_sm, threads, s);
+  return launch_batch_variant<0, false>(models, q, chunk, blocks_per_sm, threads, s);
 }
 
 cudaError_t launch_trace(const DevGrid& g, const DevTables& t, const DevRun& r,
