@@ -46,6 +46,7 @@ struct rt_mlp {
   int n_in = 0, n_out = 0;
   size_t n_padded = 0;     // padded parameter count
   int64_t n_params = 0;    // unpadded
+  char* slab = nullptr;      // holds the arrays down to d_loss
   float* d_param = nullptr;  // padded FP32 master
   float* d_grad = nullptr;
   float* d_m = nullptr;
@@ -1583,14 +1584,23 @@ rt_status rt_mlp_create(int n_in, int n_hidden, int n_layers, int n_out, uint64_
   // keep BF16 weight offsets 16-element aligned: offsets are sums of multiples of 16
   m->n_padded = off;
   m->n_params = np;
+  // one allocation, as each takes some 30 us from 1 MB on: a network of 66 - 3x256 - 200 made and
+  // closed in 569 us with eight, 380 with one. Four FP32 and three BF16 arrays of `off`, a
+  // multiple of 16, the error word and the loss.
   rt_status st;
-  if ((st = alloc(&m->d_param, off)) != RT_OK || (st = alloc(&m->d_grad, off)) != RT_OK ||
-      (st = alloc(&m->d_m, off)) != RT_OK || (st = alloc(&m->d_v, off)) != RT_OK ||
-      (st = alloc(&m->d_wbf, off)) != RT_OK || (st = alloc(&m->d_wpk[0], 2 * off)) != RT_OK ||
-      (st = alloc(&m->d_err, 1)) != RT_OK || (st = alloc(&m->d_loss, 1)) != RT_OK) {
+  if ((st = alloc(&m->slab, (4 * sizeof(float) + 3 * sizeof(bf16)) * off + 32)) != RT_OK) {
     rt_mlp_destroy(m);
     return st;
   }
+  m->d_param = reinterpret_cast<float*>(m->slab);
+  m->d_grad = m->d_param + off;
+  m->d_m = m->d_grad + off;
+  m->d_v = m->d_m + off;
+  m->d_wbf = reinterpret_cast<bf16*>(m->d_v + off);
+  m->d_wpk[0] = m->d_wbf + off;
+  m->d_wpk[1] = m->d_wpk[0] + off;
+  m->d_err = reinterpret_cast<unsigned*>(m->d_wpk[1] + off);
+  m->d_loss = reinterpret_cast<float*>(m->d_err + 1);
   // He-uniform weights from a seeded splitmix64 stream, zero biases
   std::vector<float> h(off, 0.0f);
   uint64_t x = seed;
@@ -1603,11 +1613,8 @@ rt_status rt_mlp_create(int n_in, int n_hidden, int n_layers, int n_out, uint64_
         h[ly.w_off + (size_t)r * ly.in_p + c] = (float)((2.0 * u - 1.0) * lim);
       }
   }
-  m->d_wpk[1] = m->d_wpk[0] + off;
   cudaError_t e = cudaMemcpy(m->d_param, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemset(m->d_m, 0, sizeof(float) * off);
-  if (e == cudaSuccess) e = cudaMemset(m->d_v, 0, sizeof(float) * off);
-  if (e == cudaSuccess) e = cudaMemset(m->d_grad, 0, sizeof(float) * off);
+  if (e == cudaSuccess) e = cudaMemset(m->d_grad, 0, sizeof(float) * 3 * off);  // and moments
   if (e == cudaSuccess) e = cudaMemset(m->d_err, 0, sizeof(unsigned));
   if (e != cudaSuccess || refresh_bf16(m, nullptr) != RT_OK) {
     rt_mlp_destroy(m);
@@ -1621,14 +1628,7 @@ rt_status rt_mlp_destroy(rt_mlp* m) {
   if (!m) return RT_OK;
   cudaSetDevice(m->dev);
   free_acts(m);
-  release(m->d_param);
-  release(m->d_grad);
-  release(m->d_m);
-  release(m->d_v);
-  release(m->d_wbf);
-  release(m->d_wpk[0]);  // [1] is its second half
-  release(m->d_err);
-  release(m->d_loss);
+  release(m->slab);
   delete m;
   return RT_OK;
 }
