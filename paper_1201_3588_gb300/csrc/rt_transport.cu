@@ -1805,7 +1805,7 @@ __device__ __forceinline__ int pick_model(const BatchQueue& q, unsigned warp_id,
   return -1;
 }
 
-// Two species: held to 64 registers (58 bytes of spills) for four blocks per SM; when this
+// Two species: held to 64 registers (46 bytes of spills) for four blocks per SM; when this
 // was decided 8.0 ms against 8.7 with three blocks of 74 registers, and 180 bytes of spills in
 // the generic form.
 template <int kS, bool kTally>
