@@ -297,16 +297,16 @@ PROFILE_SOURCES = ("paper_1201_3588_gb300/csrc/rt_transport.cu",
                    "paper_1201_3588_gb300/csrc/rt_internal.h")
 PROFILE = {
     # 1-pass counters of one 2e7-package launch on the full large disk (path walk):
-    # dram 175.18 GB read + 0.11 GB written; 3.543e10 warp and 5.801e11 thread
+    # dram 175.16 GB read + 0.11 GB written; 3.543e10 warp and 5.801e11 thread
     # instructions over 5.24e9 crossings
-    "large_disk": {"sha256": "13489e331a0a4d4380a29b82e0c0791a31f034beddd9dab0ff8d92b87d9234c4",
-                   "dram_bytes_per_package": 8764.2, "warp_lanes_active": 16.37,
+    "large_disk": {"sha256": "23c29546ae79219abb6a4966b4f0c874495142d330b159deb50dbcab74bc6d51",
+                   "dram_bytes_per_package": 8763.2, "warp_lanes_active": 16.37,
                    "warp_instr_per_crossing": 6.76,
                    "file": "profiles/k_transport_pool_large_disk.md"},
     # the same counters of one 1e8-package launch on the flared disk (linked walk):
-    # dram 113.57 GB read + 0.24 GB written; 6.928e10 warp and 1.370e12 thread
+    # dram 113.56 GB read + 0.24 GB written; 6.928e10 warp and 1.370e12 thread
     # instructions over 1.41e10 crossings
-    "disk": {"sha256": "13489e331a0a4d4380a29b82e0c0791a31f034beddd9dab0ff8d92b87d9234c4",
+    "disk": {"sha256": "23c29546ae79219abb6a4966b4f0c874495142d330b159deb50dbcab74bc6d51",
              "dram_bytes_per_package": 1138.0, "warp_lanes_active": 19.77,
              "warp_instr_per_crossing": 4.92, "file": "profiles/k_transport_pool_disk.md"},
 }
